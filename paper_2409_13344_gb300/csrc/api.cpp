@@ -61,6 +61,7 @@ void free_csr(DevCSR& c) {
   cudaFree(c.col);
   cudaFree(c.val);
   cudaFree(c.val_bf16);
+  cudaFree(c.order);
   c = DevCSR();
 }
 
@@ -170,6 +171,13 @@ appga_status upload_csr(const appga::HostCSR& h, bool bf16, DevCSR* out, int64_t
   }
   *out = c;
   return APPGA_OK;
+}
+
+appga_status upload_order(const std::vector<int32_t>& order, DevCSR* c, int64_t* bytes) {
+  cudaError_t e = dalloc(&c->order, order.size(), bytes);
+  if (e == cudaSuccess)
+    e = cudaMemcpy(c->order, order.data(), order.size() * 4, cudaMemcpyHostToDevice);
+  return e == cudaSuccess ? APPGA_OK : cuda_fail(e, "row order");
 }
 
 appga_status ensure_workspace(appga_matrix* M) {
@@ -958,6 +966,11 @@ appga_status appga_matrix_create(appga_ctx* ctx, int32_t m, int32_t d, int32_t n
   M->npfov = appga::disk_pixels(n_side);
   rc = upload_csr(pa, M->has_bf16, &M->A, &M->bytes);
   if (rc == APPGA_OK) rc = upload_csr(pt, M->has_bf16, &M->At, &M->bytes);
+  // the batched projectors' row orders: pixels by tiles, and rays by tiles of
+  // (angle, bin) when the rows are angle-major
+  if (rc == APPGA_OK) rc = upload_order(appga::zorder(n_side, n_side), &M->At, &M->bytes);
+  if (rc == APPGA_OK && m % n_angles == 0)
+    rc = upload_order(appga::zorder(n_angles, m / n_angles), &M->A, &M->bytes);
   if (rc == APPGA_OK) {
     // A's column indices in the 8 x 8-tiled pixel order (row_ptr and values shared)
     std::vector<int32_t> ct(pa.col.size());

@@ -73,6 +73,8 @@ __host__ __device__ inline void orbit_pixel(int32_t o, int32_t r, int32_t n, int
 }
 
 struct DevCSR {
+  // order in which the batched projectors take the rows (NULL: ascending)
+  int32_t* order = nullptr;
   int32_t rows = 0, cols = 0;
   int64_t nnz_padded = 0;
   int32_t* row_ptr = nullptr;    // rows + 1 padded offsets
@@ -295,6 +297,12 @@ bool quarter_turn_symmetric(int32_t m, int32_t n, int32_t n_angles, const int32_
 // (i, A[i, p]) with i < half of pixel p = orbit_pixel(o, r), in ascending i,
 // from the stable transpose `at` of the whole A.
 void fold_transpose(const HostCSR& at, int32_t half, int32_t n, HostCSR* out);
+
+// The points (y, x) of an ny x nx grid, as y * nx + x, along the Z-order curve:
+// every aligned run of 16 (64, ...) of the full square is a 4 x 4 (8 x 8, ...)
+// tile, so consecutive rows of a projector are neighbouring pixels, or rays
+// of neighbouring bins and angles, which share most of what they gather.
+std::vector<int32_t> zorder(int32_t ny, int32_t nx);
 
 // Round-to-nearest-even FP32 -> BF16 bits.
 uint16_t float_to_bf16(float x);

@@ -31,7 +31,6 @@ void free_batch_workspace(BatchWorkspace* bw) {
   cudaFree(bw->bst);
   cudaFree(bw->partial);
   cudaFree(bw->fpartial);
-  cudaFree(bw->gtick);
   cudaFree(bw->flag);
   for (auto& p : bw->fsm) cudaFree(p);
   cudaFree(bw->gsm);
@@ -75,15 +74,16 @@ cudaError_t alloc_batch_workspace(BatchWorkspace& b, int m, int d, int Kp) {
   if (e == cudaSuccess) e = dalloc(&b.bst, 1);
   if (e == cudaSuccess) e = dalloc(&b.partial, (size_t)(maxb + ngroups + 2) * Kp);
   if (e == cudaSuccess) e = dalloc(&b.fpartial, (size_t)maxb * Kp);
-  if (e == cudaSuccess) e = dalloc(&b.gtick, (size_t)ngroups);
   if (e == cudaSuccess) e = dalloc(&b.flag, 1);
   if (e == cudaSuccess) e = dalloc(&b.vscal, (size_t)2 * Kp + 2);
   if (e == cudaSuccess) e = cudaMallocHost((void**)&b.vscal_host, (2 * Kp + 2) * sizeof(double));
-  if (e == cudaSuccess) e = cudaMemset(b.gtick, 0, (size_t)ngroups * sizeof(unsigned int));
   if (e == cudaSuccess) e = cudaMemset(b.bst, 0, sizeof(BatchState));
   if (e == cudaSuccess) e = cudaMallocHost((void**)&b.slots_host, Kp * sizeof(SlotState));
   if (e == cudaSuccess) e = cudaMallocHost((void**)&b.bst_host, sizeof(BatchState));
   if (e == cudaSuccess) e = cudaMallocHost((void**)&b.flag_host, sizeof(int));
+  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b.side, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b.ev_fork, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b.ev_join, cudaEventDisableTiming);
   if (e != cudaSuccess) {
     free_batch_workspace(&b);
     return e;
@@ -100,15 +100,16 @@ BatchSchedule tuned_schedule(const appga_matrix* M, int Kp, bool bf16) {
 }
 
 void make_batch_args(const DevCSR& A, const DevCSR& At, const float* inv_lambda, int n,
-                     BatchWorkspace& b, bool bf16, bool track, const BatchSchedule& sch,
-                     BFwdArgs* fa, BPixArgs* pa) {
+                     BatchWorkspace& b, int stride, bool bf16, bool track,
+                     const BatchSchedule& sch, BFwdArgs* fa, BPixArgs* pa) {
   *fa = BFwdArgs{};
   fa->spmv_per_sm = sch.spmv_per_sm;
   fa->stencil_per_sm = sch.stencil_per_sm;
   fa->gather_rows = sch.gather_rows_fw;
   fa->A = A;
   fa->n = n;
-  fa->Kp = b.Kp;
+  fa->Kp = stride;
+  fa->width = stride;
   fa->track = track ? 1 : 0;
   fa->use_bf16 = bf16 ? 1 : 0;
   for (int i = 0; i < 3; ++i) fa->f[i] = b.f[i];
@@ -126,7 +127,8 @@ void make_batch_args(const DevCSR& A, const DevCSR& At, const float* inv_lambda,
   pa->gather_rows = sch.gather_rows_px;
   pa->At = At;
   pa->n = n;
-  pa->Kp = b.Kp;
+  pa->Kp = stride;
+  pa->width = stride;
   pa->use_bf16 = bf16 ? 1 : 0;
   for (int i = 0; i < 3; ++i) pa->f[i] = b.f[i];
   pa->w = b.w;
@@ -136,14 +138,14 @@ void make_batch_args(const DevCSR& A, const DevCSR& At, const float* inv_lambda,
   pa->slots = b.slots;
   pa->bst = b.bst;
   pa->partial = b.partial;
-  pa->gtick = b.gtick;
   pa->fpartial = b.fpartial;
   pa->n_fpartial = bforward_grid(*fa);
   pa->track = track ? 1 : 0;
 }
 
-cudaError_t capture_batch_graph(const BFwdArgs& fa, const BPixArgs& pa, int S, cudaStream_t s,
-                                cudaGraphExec_t* out, const VolumeSteps* vb) {
+cudaError_t capture_batch_graph(const BFwdArgs& fa, const BPixArgs& pa, int S,
+                                const BatchWorkspace& b, cudaStream_t s, cudaGraphExec_t* out,
+                                const VolumeSteps* vb) {
   *out = nullptr;
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
@@ -153,20 +155,17 @@ cudaError_t capture_batch_graph(const BFwdArgs& fa, const BPixArgs& pa, int S, c
     if (e == cudaSuccess && vb)
       e = launch_slots_to_slices(vb->slot_ring, vb->slice_ring, vb->d, vb->Kp, vb->nz,
                                  vb->va.bst, 0, s);
-    if (vb) {
-      // the 3-D stencil needs only the iterate: its branch runs beside the
-      // forward phase (which reads the same iterate and writes w, y and the
-      // objective rows before the stencil's) and joins before the update
-      if (e == cudaSuccess) e = cudaEventRecord(vb->ev_fork, s);
-      if (e == cudaSuccess) e = cudaStreamWaitEvent(vb->side, vb->ev_fork, 0);
-      if (e == cudaSuccess) e = launch_stencil3d(vb->va, vb->side);
-      if (e == cudaSuccess)
-        e = launch_slices_to_slots(vb->va.gR, fa.gR, vb->d, vb->Kp, vb->nz, vb->va.bst,
-                                   vb->side);
-      if (e == cudaSuccess) e = cudaEventRecord(vb->ev_join, vb->side);
-    }
+    // the stencil (2-D or 3-D) needs only the iterate: its branch runs beside
+    // the forward phase (which reads the same iterate and writes w, y and the
+    // objective rows before the stencil's) and joins before the update
+    if (e == cudaSuccess) e = cudaEventRecord(b.ev_fork, s);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(b.side, b.ev_fork, 0);
+    if (e == cudaSuccess) e = vb ? launch_stencil3d(vb->va, b.side) : launch_bstencil(fa, b.side);
+    if (e == cudaSuccess && vb)
+      e = launch_slices_to_slots(vb->va.gR, fa.gR, vb->d, vb->Kp, vb->nz, vb->va.bst, b.side);
+    if (e == cudaSuccess) e = cudaEventRecord(b.ev_join, b.side);
     if (e == cudaSuccess) e = launch_bforward(fa, s);
-    if (e == cudaSuccess && vb) e = cudaStreamWaitEvent(s, vb->ev_join, 0);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, b.ev_join, 0);
   }
   const cudaError_t e2 = cudaStreamEndCapture(s, &graph);
   if (e == cudaSuccess) e = e2;
@@ -202,20 +201,6 @@ SlotState slot_from_params(const appga_params* p, int k0, bool active) {
 namespace {
 
 constexpr int kBatchGraphIters = 8;
-// forward-phase blocks per SM in volume mode: 5 (one resident wave at 48
-// registers per thread) measured fastest with the 3-D stencil's branch
-// beside it (680.6 us per 64 x 256^2 volume iteration; 4: 725.9, 3: 842.7,
-// the batched default of 8: 727.3); 0 keeps the batched default
-#ifndef APPGA_VOL_SPMV_PER_SM
-#define APPGA_VOL_SPMV_PER_SM 5
-#endif
-// pixel-phase blocks per SM in volume mode (0: the batched default): 5, the
-// 2-D autotuner's choice for 64 slices of 256^2, measured fastest here too
-// (650.7 us per 64 x 256^2 volume iteration; 4: 682.6, 6: 736.4, default:
-// 679.3)
-#ifndef APPGA_VOL_PIXEL_PER_SM
-#define APPGA_VOL_PIXEL_PER_SM 5
-#endif
 
 int padded_width(int K) { return K <= 32 ? 32 : (K <= 64 ? 64 : 128); }
 
@@ -253,8 +238,10 @@ appga_status batched_solve(appga_ctx* ctx, appga_matrix* M, int32_t K, const flo
                            float* f_out, appga_stats* stats_host, const BatchSchedule& sch,
                            void* stream, int min_width = 0, bool volume = false) {
   appga_status rc = APPGA_OK;
-  const int Kp = std::max(padded_width(K), min_width);
-  if ((rc = ensure_batch_workspace(M, Kp)) != APPGA_OK) return rc;
+  // the workspace holds 32, 64 or 128 slots; the run uses as many as the
+  // slices need, 8 or 16 among them, as its row stride
+  if ((rc = ensure_batch_workspace(M, std::max(padded_width(K), min_width))) != APPGA_OK) return rc;
+  const int Kp = std::max(slot_width(K), min_width);
   if ((rc = enter_stream(ctx, stream)) != APPGA_OK) return rc;
   BatchWorkspace& b = *M->bw;
   cudaStream_t s = ctx->stream;
@@ -301,8 +288,8 @@ appga_status batched_solve(appga_ctx* ctx, appga_matrix* M, int32_t K, const flo
 
   BFwdArgs fa;
   BPixArgs pa;
-  make_batch_args(M->A, M->At, bf16 ? M->inv_lambda_bf16 : M->inv_lambda, n, b, bf16, track, sch,
-                  &fa, &pa);
+  make_batch_args(M->A, M->At, bf16 ? M->inv_lambda_bf16 : M->inv_lambda, n, b, Kp, bf16, track,
+                  sch, &fa, &pa);
   // volume: the K slots are the slices of one volume.  The 3-D stencil runs
   // on slice-major copies of the iterates after the forward phase, leaves
   // its per-slice regulariser sums after the forward phase's rows, and its
@@ -310,18 +297,9 @@ appga_status batched_solve(appga_ctx* ctx, appga_matrix* M, int32_t K, const flo
   VolumeSteps vb{};
   if (volume) {
     for (int i = 0; i < 3; ++i)
-      if (!b.fsm[i]) CK(cudaMalloc((void**)&b.fsm[i], (size_t)d * Kp * sizeof(float)));
-    if (!b.gsm) CK(cudaMalloc((void**)&b.gsm, (size_t)d * Kp * sizeof(float)));
-    if (!b.side) CK(cudaStreamCreateWithFlags(&b.side, cudaStreamNonBlocking));
-    if (!b.ev_fork) CK(cudaEventCreateWithFlags(&b.ev_fork, cudaEventDisableTiming));
-    if (!b.ev_join) CK(cudaEventCreateWithFlags(&b.ev_join, cudaEventDisableTiming));
-    vb.side = b.side;
-    vb.ev_fork = b.ev_fork;
-    vb.ev_join = b.ev_join;
+      if (!b.fsm[i]) CK(cudaMalloc((void**)&b.fsm[i], (size_t)d * b.Kp * sizeof(float)));
+    if (!b.gsm) CK(cudaMalloc((void**)&b.gsm, (size_t)d * b.Kp * sizeof(float)));
     fa.no_stencil = 1;
-    // leave room on each SM for a stencil block beside the forward phase's
-    if (sch.spmv_per_sm == 0) fa.spmv_per_sm = APPGA_VOL_SPMV_PER_SM;
-    if (sch.pixel_per_sm == 0 && APPGA_VOL_PIXEL_PER_SM > 0) pa.blocks_per_sm = APPGA_VOL_PIXEL_PER_SM;
     pa.joint = 1;
     const int nfw = bforward_grid(fa);
     Vol3Args& va = vb.va;
@@ -344,11 +322,12 @@ appga_status batched_solve(appga_ctx* ctx, appga_matrix* M, int32_t K, const flo
     pa.n_fpartial = nfw + (track ? stencil3d_grid(n, K) : 0);
   }
 
-  // y^{k0-1}, then the first forward phase (w, y, stencil, Phi of f^{k0})
+  // the first forward phase (w, y, stencil, Phi of f^{k0}); with f^{k0-1} =
+  // f^{k0} it needs no projection of the previous iterate
   BFwdArgs init = fa;
   init.mode = 1;
   CK(launch_bforward(init, s));
-  CK(launch_bforward(fa, s));
+  CK(launch_bstencil(init, s));
   if (volume) {
     CK(launch_slots_to_slices(vb.slot_ring, vb.slice_ring, d, Kp, K, b.bst, 1, s));
     CK(launch_stencil3d(vb.va, s));
@@ -359,15 +338,16 @@ appga_status batched_solve(appga_ctx* ctx, appga_matrix* M, int32_t K, const flo
     const int S = params->graph_iters > 0 ? params->graph_iters : kBatchGraphIters;
     char key[256];
     // the graph's kernels see only the workspace, never K or the caller's buffers
-    std::snprintf(key, sizeof key, "%d|%d|%d|%d|%d|%d|%d|%d|%d", Kp, (int)track, (int)bf16, S,
-                  sch.spmv_per_sm, sch.stencil_per_sm, sch.pixel_per_sm, (int)volume,
-                  volume ? K : 0);
+    std::snprintf(key, sizeof key, "%d|%d|%d|%d|%d|%d|%d|%d|%d|%d|%d", Kp, (int)track, (int)bf16,
+                  S, sch.spmv_per_sm, sch.stencil_per_sm, sch.pixel_per_sm, sch.gather_rows_fw,
+                  sch.gather_rows_px, (int)volume, volume ? K : 0);
     if (b.gexec == nullptr || b.gkey != key) {
       if (b.gexec) {
         cudaGraphExecDestroy(b.gexec);
         b.gexec = nullptr;
       }
-      const cudaError_t e = capture_batch_graph(fa, pa, S, s, &b.gexec, volume ? &vb : nullptr);
+      const cudaError_t e =
+          capture_batch_graph(fa, pa, S, b, s, &b.gexec, volume ? &vb : nullptr);
       if (e != cudaSuccess) return cuda_fail(e, "batched graph capture");
       b.gkey = key;
     }
@@ -517,19 +497,19 @@ namespace appga {
 namespace {
 // best gathered GB/s over launch shapes for the column stream `col` (nnz
 // entries) into the slot-minor block x of `width` floats per row
-appga_status probe_best(const DevCSR& M, bool forward, const float* x, int width, float* sink,
-                        int launches, cudaStream_t s, double* best) {
+appga_status probe_best(const DevCSR& M, const float* x, int width, float* sink, int launches,
+                        cudaStream_t s, double* best) {
   const long long nnz = M.nnz_padded;
   *best = 0.0;
   cudaEvent_t ev[2] = {nullptr, nullptr};
   CK(cudaEventCreate(&ev[0]));
   cudaError_t e = cudaEventCreate(&ev[1]);
-  for (const int per_sm : {3, 4, 5, 6, 8}) {
+  for (const int per_sm : {2, 4, 6, 8, 12}) {
     for (int i = 0; i < 2 && e == cudaSuccess; ++i)
-      e = launch_gather_probe(M, forward, x, width, sink, per_sm, s);
+      e = launch_gather_probe(M, x, width, sink, per_sm, s);
     if (e == cudaSuccess) e = cudaEventRecord(ev[0], s);
     for (int i = 0; i < launches && e == cudaSuccess; ++i)
-      e = launch_gather_probe(M, forward, x, width, sink, per_sm, s);
+      e = launch_gather_probe(M, x, width, sink, per_sm, s);
     if (e == cudaSuccess) e = cudaEventRecord(ev[1], s);
     if (e == cudaSuccess) e = cudaEventSynchronize(ev[1]);
     float ms = 0.f;
@@ -567,8 +547,8 @@ extern "C" appga_status appga_gather_probe(appga_ctx* ctx, const appga_matrix* m
   // back-projection: A^T's columns into the weight block [m][width]
   CK(cudaMemsetAsync(b.f[0], 0, (size_t)M->d * width * sizeof(float), s));
   CK(cudaMemsetAsync(b.w, 0, (size_t)M->m * width * sizeof(float), s));
-  rc = probe_best(M->A, true, b.f[0], width, sink, launches, s, gbs_fwd);
-  if (rc == APPGA_OK) rc = probe_best(M->At, false, b.w, width, sink, launches, s, gbs_bwd);
+  rc = probe_best(M->A, b.f[0], width, sink, launches, s, gbs_fwd);
+  if (rc == APPGA_OK) rc = probe_best(M->At, b.w, width, sink, launches, s, gbs_bwd);
   return rc;
 }
 

@@ -42,16 +42,18 @@ struct BatchState {
 
 struct BFwdArgs {
   DevCSR A;
-  int32_t n, Kp;
-  int32_t mode;  // 0: solver step; 1: project the previous iterate only;
-                 // 2: first forward phase of the fresh slots only (admission)
+  int32_t n;
+  int32_t Kp;     // row stride of the slot-minor arrays
+  int32_t width;  // slots worked on: 8, 16, 32, 64 or 128, every live slot below it
+  int32_t mode;   // 0: solver step; 1: first forward phase of a run (f^{k-1} = f^k);
+                  // 2: first forward phase of the fresh slots only (admission)
   int32_t track;
   int32_t use_bf16;
-  int32_t n_spmv_blocks;  // set by the launcher
-  int32_t spmv_per_sm;    // SpMV blocks per SM (0: default); tuned by the autotuner
+  int32_t n_spmv_blocks;  // virtual blocks of the projection, set by the launcher
+  int32_t spmv_per_sm;    // virtual blocks per SM (0: default); tuned by the autotuner
   int32_t stencil_per_sm; // stencil blocks per SM (0: default)
-  int32_t no_stencil;     // volume mode: the 3-D stencil runs in its own kernel
-  int32_t gather_rows;    // image rows gathered per step: 8 (0: default) or 4; tuned
+  int32_t no_stencil;     // volume mode: the 3-D stencil takes the 2-D one's place
+  int32_t gather_rows;    // image rows a lane gathers per step: 8 (0: default) or 4; tuned
   float* f[3];
   float* y[2];
   float* w;
@@ -65,11 +67,13 @@ struct BFwdArgs {
 
 struct BPixArgs {
   DevCSR At;
-  int32_t n, Kp;
+  int32_t n;
+  int32_t Kp;             // row stride of the slot-minor arrays
+  int32_t width;          // slots worked on (as BFwdArgs)
   int32_t use_bf16;
+  int32_t n_blocks;       // virtual blocks, set by the launcher
   int32_t blocks_per_sm;  // 0: default; tuned by the autotuner
-  int32_t gather_rows;    // weight rows gathered per step: 8 (0: default) or 4; tuned
-  int32_t pad;
+  int32_t gather_rows;    // weight rows a lane gathers per step: 8 (0: default) or 4; tuned
   float* f[3];
   const float* w;
   const float* gR;
@@ -77,8 +81,7 @@ struct BPixArgs {
   float* pfreeze;
   SlotState* slots;
   BatchState* bst;
-  float2* partial;
-  unsigned int* gtick;
+  float2* partial;  // group sums of the objective partials
   // objective partials left by the forward phase of the same step (track):
   // reduced here, where the stopping test runs
   const float2* fpartial;
@@ -121,19 +124,29 @@ cudaError_t launch_slices_to_slots(const float* in, float* out, int d, int Kp, i
                                    const BatchState* bst, cudaStream_t s);
 
 int batch_max_blocks();
-// Grid of the forward phase for these arguments (the launcher's own choice).
+// Rows of objective partials a forward phase with these arguments leaves
+// (its projection's virtual blocks, then its stencil blocks).
 int bforward_grid(const BFwdArgs& a);
 // Slots whose result sits one ring entry back (stopped by the test in the
 // last pixel phase): copy it into the current entry and clear the mark.
 cudaError_t launch_resolve_rollback(const BFwdArgs& a, cudaStream_t s);
 cudaError_t launch_bforward(const BFwdArgs& a, cudaStream_t s);
+// The forward phase's 2-D stencil, on the same arguments; independent of
+// launch_bforward (they may overlap).
+cudaError_t launch_bstencil(const BFwdArgs& a, cudaStream_t s);
 // The batched projectors' inner loop alone over M (rows reduced against the
-// Kp-wide rows of x, [cols][Kp]; no epilogue) in the row order of the forward
-// projection (forward) or of the back-projection, with blocks_per_sm (1..16)
+// Kp-wide rows of x, [cols][Kp]; no epilogue) with blocks_per_sm (1..16)
 // blocks per SM; sink: at least (SMs x 16) floats, written only in a case
 // that does not arise.
-cudaError_t launch_gather_probe(const DevCSR& M, bool forward, const float* x, int Kp,
-                                float* sink, int blocks_per_sm, cudaStream_t s);
+cudaError_t launch_gather_probe(const DevCSR& M, const float* x, int Kp, float* sink,
+                                int blocks_per_sm, cudaStream_t s);
+// Slots the kernels work on for K slices: the narrowest of 8, 16, 32, 64 and
+// 128 that holds them.
+inline int slot_width(int K) {
+  int w = 8;
+  while (w < K) w *= 2;
+  return w;
+}
 cudaError_t launch_bpixel(const BPixArgs& a, cudaStream_t s);
 // Slot lists: where `ids` is given, slice k goes to slot ids[k] (a device
 // array of K ints); otherwise to slot s0 + k.

@@ -217,6 +217,33 @@ void fold_transpose(const HostCSR& at, int32_t half, int32_t n, HostCSR* out) {
   }
 }
 
+std::vector<int32_t> zorder(int32_t ny, int32_t nx) {
+  std::vector<int32_t> out;
+  out.reserve((size_t)ny * nx);
+  int64_t side = 1;
+  while (side < ny || side < nx) side *= 2;
+  // squares of the curve that still meet the grid, as (y, x, side) on a stack
+  struct Square {
+    int64_t y, x, side;
+  };
+  std::vector<Square> todo = {{0, 0, side}};
+  while (!todo.empty()) {
+    const Square q = todo.back();
+    todo.pop_back();
+    if (q.y >= ny || q.x >= nx) continue;
+    if (q.side == 1) {
+      out.push_back((int32_t)(q.y * nx + q.x));
+      continue;
+    }
+    const int64_t h = q.side / 2;
+    todo.push_back({q.y + h, q.x + h, h});
+    todo.push_back({q.y + h, q.x, h});
+    todo.push_back({q.y, q.x + h, h});
+    todo.push_back({q.y, q.x, h});
+  }
+  return out;
+}
+
 uint16_t float_to_bf16(float x) {
   uint32_t u;
   std::memcpy(&u, &x, 4);

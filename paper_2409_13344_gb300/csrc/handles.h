@@ -93,7 +93,6 @@ struct BatchWorkspace {
   BatchState* bst_host = nullptr;             // pinned
   float2* partial = nullptr;                  // (blocks + groups) x Kp
   float2* fpartial = nullptr;                 // forward-phase objective partials, blocks x Kp
-  unsigned int* gtick = nullptr;
   int* flag = nullptr;
   int* flag_host = nullptr;
   float* fsm[3] = {nullptr, nullptr, nullptr};  // volume mode: slice-major iterate ring [Kp][d]
@@ -102,8 +101,8 @@ struct BatchWorkspace {
   double* vscal_host = nullptr;  // pinned mirror
   cudaGraphExec_t gexec = nullptr;
   std::string gkey;
-  // volume mode: the 3-D stencil's branch of the captured step (a second
-  // stream forked from and joined to the solver's stream by two events)
+  // the stencil's branch of the captured step (a second stream forked from
+  // and joined to the solver's stream by two events)
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
 };
@@ -113,31 +112,30 @@ void free_batch_workspace(BatchWorkspace* bw);
 int64_t batch_workspace_bytes(int m, int d, int Kp);
 // Allocates every array of a width-Kp workspace (frees what it made on error).
 cudaError_t alloc_batch_workspace(BatchWorkspace& b, int m, int d, int Kp);
-// Kernel arguments of one batched step over workspace b with matrix arrays
-// from (A, At, inv_lambda).
+// Kernel arguments of one batched step over workspace b, `stride` (at most
+// b.Kp) slots per row, with matrix arrays from (A, At, inv_lambda).
 void make_batch_args(const DevCSR& A, const DevCSR& At, const float* inv_lambda, int n,
-                     BatchWorkspace& b, bool bf16, bool track, const BatchSchedule& sch,
-                     BFwdArgs* fa, BPixArgs* pa);
+                     BatchWorkspace& b, int stride, bool bf16, bool track,
+                     const BatchSchedule& sch, BFwdArgs* fa, BPixArgs* pa);
 // Tuned schedule of matrix M for padded width Kp and precision (defaults if none).
 BatchSchedule tuned_schedule(const appga_matrix* M, int Kp, bool bf16);
 // Slot state of a problem run with `p` from iterate index k0 (active), or an
 // empty slot that holds no problem (inactive).
 SlotState slot_from_params(const appga_params* p, int k0, bool active);
-// Captures S x (pixel update, forward phase) into an executable graph; with
-// vb (volume mode) each step is pixel update, transpose of the new iterate to
-// the slice-major ring, forward phase, 3-D stencil, transpose of its gradient.
+// Captures S x (pixel update, forward phase beside the 2-D stencil) into an
+// executable graph; with vb (volume mode) each step is pixel update, transpose
+// of the new iterate to the slice-major ring, forward phase beside the 3-D
+// stencil and the transpose of its gradient.  The stencil's branch runs on
+// b.side.
 struct VolumeSteps {
   Vol3Args va;
   float* slot_ring[3];
   float* slice_ring[3];
   int d, Kp, nz;
-  // the stencil branch runs on `side`, forked after the iterate's transpose
-  // and joined before the next pixel update, beside the forward phase
-  cudaStream_t side;
-  cudaEvent_t ev_fork, ev_join;
 };
-cudaError_t capture_batch_graph(const BFwdArgs& fa, const BPixArgs& pa, int S, cudaStream_t s,
-                                cudaGraphExec_t* out, const VolumeSteps* vb = nullptr);
+cudaError_t capture_batch_graph(const BFwdArgs& fa, const BPixArgs& pa, int S,
+                                const BatchWorkspace& b, cudaStream_t s, cudaGraphExec_t* out,
+                                const VolumeSteps* vb = nullptr);
 // APPGA on a volume of K <= 128 slices sharing the matrix (the batched solver
 // in volume mode): device buffers as in appga_reconstruct_batched; on return
 // the workspace's pinned slot and batch states hold the final states.

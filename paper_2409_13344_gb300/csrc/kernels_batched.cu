@@ -2,19 +2,17 @@
 // matrix run the APPGA iteration together, so every nonzero of A and A^T is
 // read once per iteration for all K right-hand sides (CSR SpMM).
 //
-// Layout (slot-minor): images f[j][s], sinograms y[i][s], w[i][s], g[i][s]
-// with K padded to Kp = 32 V (V = 1, 2 or 4 slots per lane).  One warp owns
-// a CSR row: lanes load 32 (column, value) pairs at a time and stage them in
-// shared memory; every lane reads them back with broadcast loads and, for
-// each nonzero, gathers its 4V-byte piece of the Kp-wide image row (one
-// coalesced row per warp) and accumulates V products in FP32.  The
-// back-projection's blocks own contiguous runs of pixels, whose rays overlap,
-// so the gathered weight rows are reused from L1; the forward projection
-// deals rays to the warps of the whole grid in turn, so the grid works on
-// neighbouring rays at once and the image rows they gather stay in L2 (each
-// order is a per-projection switch).  The per-(row, slot) epilogues match the
-// single-slice kernels (Eq. APPGAiter, Eq. EM, Sec. 2.2); the SHOITV stencil
-// runs on shared-memory tiles of 2 x 32 pixels x 8 slots.
+// Layout (slot-minor): images f[j][s], sinograms y[i][s], w[i][s], g[i][s],
+// rows of Kp slots.  A launch works on the first W = 8, 16, 32, 64 or 128 of
+// them; the lanes of a warp share a row's products as Team<W> says.  The bound
+// is the L1 pipe: each nonzero takes W/32 passes of 128 bytes for its gathered
+// row, plus its share of the matrix's broadcast loads.  Rows are dealt to
+// warps along a Z-order curve (pixels, or rays by angle and bin), so a block
+// gathers for neighbouring rows and half to three quarters of the sectors hit
+// L1 (64 slots of 256 x 256: 1.8 and 1.2 GB from L2 per projection, 3.5 and
+// 2.6 GB in row order).  The per-(row, slot) epilogues match the single-slice
+// kernels (Eq. APPGAiter, Eq. EM, Sec. 2.2); the SHOITV stencil is a kernel of
+// its own that runs beside the forward projection.
 //
 // Every slot carries its own device state (iteration index, momentum scalar,
 // objective, stop flag, parameters), so slots may sit at different
@@ -25,6 +23,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <algorithm>
+
 #include "appga_internal.h"
 #include "batched_internal.h"
 #include "device_common.cuh"
@@ -32,366 +32,221 @@
 namespace appga {
 namespace {
 
-constexpr int B_THREADS = 256;
-constexpr int B_WARPS = B_THREADS / 32;
-constexpr int MAXK = 128;                    // largest padded batch (V = 4)
-// Default grids: more blocks than fit at once (measured faster on GB300 than
-// grids that are all resident: blocks own contiguous row ranges, and the
-// block scheduler balances the tail).
-constexpr int kSpmvPerSm = 8;                // SpMV / back-projection blocks per SM
-constexpr int kStencilPerSm = 4;             // stencil blocks per SM
-constexpr int kMaxPerSm = 16;                // upper bound of either tuned value
+constexpr int B_THREADS = 256;               // stencil blocks (and set-up kernels)
+constexpr int MAXK = 128;                    // largest padded batch
+// Projector blocks: 16 warps, two blocks per SM (64 registers per thread).  A
+// block's warps work on a compact bundle of rows (DevCSR::order), so the wider
+// the block the more of its gathers meet in L1.
+constexpr int P_THREADS = 512;
+constexpr int P_WARPS = P_THREADS / 32;
+constexpr int kMaxPerSm = 16;                // upper bound of the tuned values
 __host__ __forceinline__ int clamp_per_sm(int v, int dflt) {
   return v <= 0 ? dflt : (v > kMaxPerSm ? kMaxPerSm : v);
 }
-// Blocks per SM when no tuned schedule is given: at 64 slots the
-// autotuner's choice on 64 slices of 256^2 (forward 4, pixel 5, stencil 8),
-// other widths the caps above.
-__host__ __forceinline__ int default_spmv_per_sm(int Kp) { return Kp == 64 ? 4 : kSpmvPerSm; }
-__host__ __forceinline__ int default_pixel_per_sm(int Kp) { return Kp == 64 ? 5 : kSpmvPerSm; }
-__host__ __forceinline__ int default_stencil_per_sm(int Kp) {
-  return Kp == 64 ? 8 : kStencilPerSm;
-}
-constexpr int BST_R = 2, BST_C = 32, BST_S = 8;  // stencil item: 2 x 32 pixels x 8 slots
-constexpr int BTW = BST_C + 4, BVW = BST_C + 2;
-static_assert(BST_C * BST_S == B_THREADS, "stencil: one thread per (column, slot)");
+// Row groups per SM when no tuned schedule is given: more than are resident
+// at once, so the block scheduler levels the tail.
+constexpr int kSpmvPerSm = 8;
+constexpr int kPixelPerSm = 8;
+constexpr int kStencilPerSm = 8;
+// Stencil blocks: 8 slots x 32 image columns (the outer two on each side are
+// halo), marching down runs of BST_R rows.
+constexpr int BST_S = 8, BST_C = B_THREADS / BST_S, BST_OUT = BST_C - 4, BST_R = 16;
+static_assert(BST_S == 8 && BST_C % 4 == 0, "a warp holds four columns of eight slots");
 
-template <int V>
-__device__ __forceinline__ void vload(const float* p, float (&x)[V]) {
-  if constexpr (V == 1) {
-    x[0] = __ldg(p);
-  } else if constexpr (V == 2) {
-    const float2 t = __ldg(reinterpret_cast<const float2*>(p));
+template <int E>
+__device__ __forceinline__ void vload(const float* p, float (&x)[E]) {
+  if constexpr (E == 1) {
+    x[0] = *p;
+  } else if constexpr (E == 2) {
+    const float2 t = *reinterpret_cast<const float2*>(p);
     x[0] = t.x;
     x[1] = t.y;
   } else {
-    const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+    const float4 t = *reinterpret_cast<const float4*>(p);
     x[0] = t.x;
     x[1] = t.y;
     x[2] = t.z;
     x[3] = t.w;
   }
 }
-template <int V>
-__device__ __forceinline__ void vstore(float* p, const float (&x)[V]) {
-  if constexpr (V == 1) {
-    p[0] = x[0];
-  } else if constexpr (V == 2) {
-    *reinterpret_cast<float2*>(p) = make_float2(x[0], x[1]);
+// Stores the elements whose on[] is set (one vector store when all are).
+template <int E>
+__device__ __forceinline__ void vstore_on(float* p, const float (&x)[E], const int (&on)[E]) {
+  int all = 1;
+#pragma unroll
+  for (int t = 0; t < E; ++t) all &= on[t] ? 1 : 0;
+  if (all) {
+    if constexpr (E == 1) {
+      *p = x[0];
+    } else if constexpr (E == 2) {
+      *reinterpret_cast<float2*>(p) = make_float2(x[0], x[1]);
+    } else {
+      *reinterpret_cast<float4*>(p) = make_float4(x[0], x[1], x[2], x[3]);
+    }
   } else {
-    *reinterpret_cast<float4*>(p) = make_float4(x[0], x[1], x[2], x[3]);
+#pragma unroll
+    for (int t = 0; t < E; ++t)
+      if (on[t]) p[t] = x[t];
   }
 }
 
-#ifndef APPGA_BDOT
-#define APPGA_BDOT 2
-#endif
-// Row order of each projection: a contiguous run of rows per block (1) or
-// rows dealt to the warps of the whole grid in turn (0).  The forward
-// projection gathers image rows faster dealt in turn (the whole grid works
-// on neighbouring rays at once, so the rows it gathers stay in L2); the
-// back-projection keeps contiguous runs of pixels (their weight rows are
-// reused from L1).
-#ifndef APPGA_BCONTIG_FW
-#define APPGA_BCONTIG_FW 0
-#endif
-#ifndef APPGA_BCONTIG_PX
-#define APPGA_BCONTIG_PX 1
-#endif
-
-// One CSR row of M times the Kp-wide columns of X ([cols][Kp]): lane holds
-// the V sums of slots lane*V .. lane*V + V - 1.  Each lane loads one of 32
-// (column, value) pairs; the warp stages them in shared memory (the column
-// as an element offset col * Kp) and every lane reads them back four at a
-// time with broadcast loads, gathering GR image rows per step (8 or 4: more
-// loads in flight against fewer registers; a launch-schedule choice).  The
-// next 32 pairs are loaded while the current ones are consumed.  Products
-// are accumulated in the row's entry order whatever GR, so the sums do not
-// depend on it.
-template <int V, bool BF16, int GR = 8>
-__device__ __forceinline__ void brow_dot(const DevCSR& M, int row, const float* __restrict__ X,
-                                         int Kp, int lane, bool lane_on, uint64_t pol,
-                                         int* s_off, float* s_val, float (&acc)[V]) {
-#if APPGA_BDOT == 2
-#pragma unroll
-  for (int t = 0; t < V; ++t) acc[t] = 0.f;
-  const int s = __ldg(M.row_ptr + row), e = __ldg(M.row_ptr + row + 1);
-  const float* xl = X + lane * V;
-  int c = 0;
-  float v = 0.f;
-  if (s + lane < e) {
-    c = ld_stream_i1(M.col + s + lane, pol);
-    v = BF16 ? ld_stream_bf16_1(M.val_bf16 + s + lane, pol) : ld_stream_f1(M.val + s + lane, pol);
-  }
-  for (int p0 = s; p0 < e; p0 += 32) {
-    const int cnt = min(32, e - p0);  // a multiple of 4 (rows are padded)
-    __syncwarp();
-    s_off[lane] = c * Kp;
-    s_val[lane] = v;
-    __syncwarp();
-    const int pn = p0 + 32 + lane;
-    if (pn < e) {
-      c = ld_stream_i1(M.col + pn, pol);
-      v = BF16 ? ld_stream_bf16_1(M.val_bf16 + pn, pol) : ld_stream_f1(M.val + pn, pol);
-    }
-    if (!lane_on) continue;
-    int q = 0;
-    if constexpr (GR == 8) {
-      for (; q + 8 <= cnt; q += 8) {
-        const int4 o0 = *reinterpret_cast<const int4*>(s_off + q);
-        const int4 o1 = *reinterpret_cast<const int4*>(s_off + q + 4);
-        const float4 w0 = *reinterpret_cast<const float4*>(s_val + q);
-        const float4 w1 = *reinterpret_cast<const float4*>(s_val + q + 4);
-        float x[8][V];
-        vload<V>(xl + o0.x, x[0]);
-        vload<V>(xl + o0.y, x[1]);
-        vload<V>(xl + o0.z, x[2]);
-        vload<V>(xl + o0.w, x[3]);
-        vload<V>(xl + o1.x, x[4]);
-        vload<V>(xl + o1.y, x[5]);
-        vload<V>(xl + o1.z, x[6]);
-        vload<V>(xl + o1.w, x[7]);
-        const float w[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-#pragma unroll
-          for (int t = 0; t < V; ++t) acc[t] = fmaf(w[u], x[u][t], acc[t]);
-      }
-    }
-    static_assert(GR == 8 || GR == 4, "image rows gathered per step");
-    for (; q < cnt; q += 4) {  // cnt is a multiple of 4 (rows are padded)
-      const int4 o0 = *reinterpret_cast<const int4*>(s_off + q);
-      const float4 w0 = *reinterpret_cast<const float4*>(s_val + q);
-      float x[4][V];
-      vload<V>(xl + o0.x, x[0]);
-      vload<V>(xl + o0.y, x[1]);
-      vload<V>(xl + o0.z, x[2]);
-      vload<V>(xl + o0.w, x[3]);
-      const float w[4] = {w0.x, w0.y, w0.z, w0.w};
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int t = 0; t < V; ++t) acc[t] = fmaf(w[u], x[u][t], acc[t]);
-    }
-  }
-#else
-  (void)s_off;
-  (void)s_val;
-#pragma unroll
-  for (int t = 0; t < V; ++t) acc[t] = 0.f;
-  const int s = __ldg(M.row_ptr + row), e = __ldg(M.row_ptr + row + 1);
-  const float* xl = X + lane * V;
-  for (int p0 = s; p0 < e; p0 += 32) {
-    const int p = p0 + lane;
-    int c = 0;
-    float v = 0.f;
-    if (p < e) {
-      c = ld_stream_i1(M.col + p, pol);
-      v = BF16 ? ld_stream_bf16_1(M.val_bf16 + p, pol) : ld_stream_f1(M.val + p, pol);
-    }
-    const int cnt = min(32, e - p0);  // a multiple of 4 (rows are padded)
-    for (int q = 0; q < cnt; q += 4) {
-      int cq[4];
-      float vq[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        cq[u] = __shfl_sync(0xffffffffu, c, q + u);
-        vq[u] = __shfl_sync(0xffffffffu, v, q + u);
-      }
-      float x[4][V];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (lane_on) {
-          vload<V>(xl + (size_t)cq[u] * Kp, x[u]);
-        } else {
-#pragma unroll
-          for (int t = 0; t < V; ++t) x[u][t] = 0.f;
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int t = 0; t < V; ++t) acc[t] = fmaf(vq[u], x[u][t], acc[t]);
-    }
-  }
-#endif
-}
-
-// ------------------------------------------------- per-slot grid reduction
-// Two-level deterministic reduction of Kp double-float values per block
-// (p_hi/p_lo in shared memory).  True in the final block, where tot_hi /
-// tot_lo (shared) hold the per-slot totals.  Partial layout: block b at
-// partial[b*Kp .. ), group g result at partial[(nb + g)*Kp .. ).
-__device__ bool grid_reduce_slots(float2* partial, unsigned int* gtick, unsigned int* ftick,
-                                  const float* p_hi, const float* p_lo, int Kp, float* tot_hi,
-                                  float* tot_lo) {
-  __shared__ int s_flag;
-  __shared__ float r_hi[B_THREADS], r_lo[B_THREADS];
-  const int nb = gridDim.x, b = blockIdx.x, g = b / RED_GROUP, tid = threadIdx.x;
-  const int ngroups = (nb + RED_GROUP - 1) / RED_GROUP;
-  const int gsize = min(RED_GROUP, nb - g * RED_GROUP);
-  for (int s = tid; s < Kp; s += blockDim.x) partial[(size_t)b * Kp + s] = make_float2(p_hi[s], p_lo[s]);
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) s_flag = (atomicAdd(&gtick[g], 1u) == (unsigned)(gsize - 1));
-  __syncthreads();
-  if (!s_flag) return false;
-  __threadfence();
-  const int P = blockDim.x / Kp;  // parts per slot
-  auto reduce_rows = [&](const float2* base, int count) {
-    const int s = tid % Kp, part = tid / Kp;
-    float h = 0.f, l = 0.f;
-    if (part < P) {
-      for (int i = part; i < count; i += P) {
-        const float2 v = __ldcg(base + (size_t)i * Kp + s);
-        acc_add(h, l, v.x, v.y);
-      }
-    }
-    r_hi[tid] = h;
-    r_lo[tid] = l;
-    __syncthreads();
-    if (tid < Kp) {
-      float hh = 0.f, ll = 0.f;
-      for (int q = 0; q < P; ++q) acc_add(hh, ll, r_hi[q * Kp + tid], r_lo[q * Kp + tid]);
-      tot_hi[tid] = hh;
-      tot_lo[tid] = ll;
-    }
-    __syncthreads();
-  };
-  reduce_rows(partial + (size_t)g * RED_GROUP * Kp, gsize);
-  for (int s = tid; s < Kp; s += blockDim.x)
-    partial[(size_t)(nb + g) * Kp + s] = make_float2(tot_hi[s], tot_lo[s]);
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) {
-    gtick[g] = 0;
-    s_flag = (atomicAdd(ftick, 1u) == (unsigned)(ngroups - 1));
-  }
-  __syncthreads();
-  if (!s_flag) return false;
-  __threadfence();
-  reduce_rows(partial + (size_t)nb * Kp, ngroups);
-  if (tid == 0) *ftick = 0;
-  return true;
-}
-
-// --------------------------------------------------------------- stencil
-
-struct BStencilSmem {
-  float T[BST_R + 4][BTW][BST_S];
-  float K[BST_R + 4][BTW][BST_S];
-  float V[6][BST_R + 2][BVW][BST_S];
+// How the lanes of a warp share a row whose products fill W slots.  A lane
+// holds Q slots (Q/4 16-byte loads per gathered row), L lanes make a group
+// that covers the W slots, and the G groups of a row's team take the row's
+// 4-entry packs in turn.  The row's sum is always that of four partial sums,
+// p_i over the packs k = i (mod 4) in order, as (p0 + p1) + (p2 + p3), so the
+// results do not depend on W: the widest team holds several of the four in
+// one lane (A), the narrow ones work on RW rows of the warp at a time.
+// Eight slots per lane because the load of a pack's columns or values, which
+// a group's lanes make at one address, still takes the L1 pipe four passes
+// (a 16-byte load is served in quarter warps): with four groups a warp those
+// passes feed 16 entries.
+template <int W>
+struct Team {
+  static constexpr int Q = W >= 16 ? 8 : 4;
+  static constexpr int L = W / Q;
+  static constexpr int G = L <= 8 ? 4 : 32 / L;
+  static constexpr int A = 4 / G;
+  static constexpr int LANES = L * G;
+  static constexpr int RW = 32 / LANES;
+  static constexpr int E = Q / G;  // slots a lane owns after the reduction
+  static constexpr int GSTRIDE = 4 * L;
 };
-
-// One stencil item: tile (r0, c0) for slots s0 .. s0+7.  Thread (col, q) =
-// (tid % 32, tid / 32).  Writes gR and returns this thread's regulariser
-// share of Phi(f^k) for slot s0 + q (both tile rows).
-__device__ float bstencil_item(BStencilSmem& S, const float* __restrict__ fk,
-                               const float* __restrict__ fkm, const SlotState* slots, int Kp,
-                               int r0, int c0, int s0, int n, float* __restrict__ gR,
-                               bool want_reg, int mode) {
-  const int tid = threadIdx.x;
-  // load the halo tile, slots fastest (32-byte runs)
-  for (int t = tid; t < (BST_R + 4) * BTW * BST_S; t += blockDim.x) {
-    const int q = t % BST_S, pix = t / BST_S;
-    const int ii = pix / BTW, jj = pix % BTW;
-    const int r = r0 - 2 + ii, c = c0 - 2 + jj;
-    float vk = 0.f, vt = 0.f;
-    if (r >= 0 && r < n && c >= 0 && c < n) {
-      const size_t o = (size_t)(r * n + c) * Kp + s0 + q;
-      vk = fk[o];
-      vt = mode == 2 ? vk : fmaf(slots[s0 + q].theta_hi, vk - fkm[o], vk);
-    }
-    S.K[ii][jj][q] = vk;
-    S.T[ii][jj][q] = vt;
-  }
-  __syncthreads();
-  for (int t = tid; t < (BST_R + 2) * BVW * BST_S; t += blockDim.x) {
-    const int q = t % BST_S, pix = t / BST_S;
-    const int ii = pix / BVW, jj = pix % BVW;
-    const int r = r0 - 1 + ii, c = c0 - 1 + jj;
-    float v[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (r >= 0 && r < n && c >= 0 && c < n) {
-      const SlotState& sl = slots[s0 + q];
-      // the six fields of B at (r, c) of slot s0 + q (same forms as the single-slice stencil)
-      const int i = ii + 1, j = jj + 1;
-      const bool r_lo = r >= 1, r_hi = r <= n - 2, c_lo = c >= 1, c_hi = c <= n - 2;
-      auto X = [&](int a, int b) { return S.T[a][b][q]; };
-      float u[6];
-      u[0] = c_lo ? X(i, j) - X(i, j - 1) : 0.f;
-      u[1] = r_lo ? X(i, j) - X(i - 1, j) : 0.f;
-      u[2] = (c_lo ? -(X(i, j) - X(i, j - 1)) : 0.f) + (c_hi ? X(i, j + 1) - X(i, j) : 0.f);
-      u[3] = c_lo ? ((r_lo ? -(X(i, j) - X(i, j - 1)) : 0.f) +
-                     (r_hi ? X(i + 1, j) - X(i + 1, j - 1) : 0.f))
-                  : 0.f;
-      u[4] = (r_lo ? -(X(i, j) - X(i - 1, j)) : 0.f) + (r_hi ? X(i + 1, j) - X(i, j) : 0.f);
-      u[5] = r_lo ? ((c_lo ? -(X(i, j) - X(i - 1, j)) : 0.f) +
-                     (c_hi ? X(i, j + 1) - X(i - 1, j + 1) : 0.f))
-                  : 0.f;
-      const float n1 = u[0] * u[0] + u[1] * u[1];
-      const float n2 = u[2] * u[2] + u[3] * u[3] + u[4] * u[4] + u[5] * u[5];
-      const float s1 = sl.lambda1 / fmaxf(sqrtf(n1), sl.eps);
-      const float s2 = sl.lambda2 / fmaxf(sqrtf(n2), sl.eps);
-      v[0] = s1 * u[0];
-      v[1] = s1 * u[1];
-      v[2] = s2 * u[2];
-      v[3] = s2 * u[3];
-      v[4] = s2 * u[4];
-      v[5] = s2 * u[5];
-    }
-#pragma unroll
-    for (int f = 0; f < 6; ++f) S.V[f][ii][jj][q] = v[f];
-  }
-  __syncthreads();
-  const int col = tid % BST_C, q = tid / BST_C;
-  const SlotState& sl = slots[s0 + q];
-  const bool part = mode == 2 ? sl.fresh : (sl.active && !sl.done);
-  float reg = 0.f;
-#pragma unroll
-  for (int ii = 0; ii < BST_R; ++ii) {
-    const int r = r0 + ii, c = c0 + col;
-    if (part && r < n && c < n) {
-      const int i = ii + 1, j = col + 1;
-      const bool r_lo = r >= 1, r_hi = r <= n - 2, c_lo = c >= 1, c_hi = c <= n - 2;
-      auto W = [&](int f, int a, int b) { return S.V[f][a][b][q]; };
-      float gsum = 0.f;
-      if (c_lo) gsum += W(0, i, j);
-      if (c_hi) gsum -= W(0, i, j + 1);
-      if (r_lo) gsum += W(1, i, j);
-      if (r_hi) gsum -= W(1, i + 1, j);
-      // u3-form of v3, u6-form of v4, u5-form of v5, u4-form of v6
-      gsum += (c_lo ? -(W(2, i, j) - W(2, i, j - 1)) : 0.f) + (c_hi ? W(2, i, j + 1) - W(2, i, j) : 0.f);
-      gsum += r_lo ? ((c_lo ? -(W(3, i, j) - W(3, i - 1, j)) : 0.f) +
-                      (c_hi ? W(3, i, j + 1) - W(3, i - 1, j + 1) : 0.f))
-                   : 0.f;
-      gsum += (r_lo ? -(W(4, i, j) - W(4, i - 1, j)) : 0.f) + (r_hi ? W(4, i + 1, j) - W(4, i, j) : 0.f);
-      gsum += c_lo ? ((r_lo ? -(W(5, i, j) - W(5, i, j - 1)) : 0.f) +
-                      (r_hi ? W(5, i + 1, j) - W(5, i + 1, j - 1) : 0.f))
-                   : 0.f;
-      gR[(size_t)(r * n + c) * Kp + s0 + q] = gsum;
-      if (want_reg) {
-        auto Kf = [&](int a, int b) { return S.K[a][b][q]; };
-        const int a = ii + 2, b = col + 2;
-        float u[6];
-        u[0] = c_lo ? Kf(a, b) - Kf(a, b - 1) : 0.f;
-        u[1] = r_lo ? Kf(a, b) - Kf(a - 1, b) : 0.f;
-        u[2] = (c_lo ? -(Kf(a, b) - Kf(a, b - 1)) : 0.f) + (c_hi ? Kf(a, b + 1) - Kf(a, b) : 0.f);
-        u[3] = c_lo ? ((r_lo ? -(Kf(a, b) - Kf(a, b - 1)) : 0.f) +
-                       (r_hi ? Kf(a + 1, b) - Kf(a + 1, b - 1) : 0.f))
-                    : 0.f;
-        u[4] = (r_lo ? -(Kf(a, b) - Kf(a - 1, b)) : 0.f) + (r_hi ? Kf(a + 1, b) - Kf(a, b) : 0.f);
-        u[5] = r_lo ? ((c_lo ? -(Kf(a, b) - Kf(a - 1, b)) : 0.f) +
-                       (c_hi ? Kf(a, b + 1) - Kf(a - 1, b + 1) : 0.f))
-                    : 0.f;
-        const float n1 = u[0] * u[0] + u[1] * u[1];
-        const float n2 = u[2] * u[2] + u[3] * u[3] + u[4] * u[4] + u[5] * u[5];
-        reg += sl.lambda1 * s_eps_f(n1, sl.eps) + sl.lambda2 * s_eps_f(n2, sl.eps);
-      }
-    }
-  }
-  __syncthreads();  // the tile buffers are reused by the next item
-  return reg;
+// A lane gathers the slots gathered_slot + i * GSTRIDE .. + 3, i < Q/4 (so
+// that a quarter warp's 16-byte loads are consecutive: one pass each), and
+// owns the E slots from owned_slot after the reduction.
+template <int W>
+__device__ __forceinline__ int gathered_slot(int lane) {
+  return 4 * (lane % Team<W>::L);
 }
+template <int W>
+__device__ __forceinline__ int owned_slot(int lane) {
+  using T = Team<W>;
+  const int g = lane % T::LANES / T::L;
+  if constexpr (T::Q == 4) return gathered_slot<W>(lane) + 2 * (g & 1) + (g >> 1);
+  return gathered_slot<W>(lane) + T::GSTRIDE * (g & 1) + T::E * (g >> 1);
+}
+
+// One row of M (row < 0: none) times the columns of X ([cols][stride]): each
+// lane ends with the sums of the E slots from owned_slot.  A lane gathers NZ
+// (2 or 4) entries of a pack per step while the columns and values of the
+// next pack are in flight; `on`: some of the lane's gathered slots is wanted.
+// All lanes of the warp take part.
+template <int W, bool BF16, int NZ>
+__device__ __forceinline__ void team_dot(const DevCSR& M, int row, const float* __restrict__ X,
+                                         int stride, int lane, bool on, uint64_t pol,
+                                         float (&out)[Team<W>::E]) {
+  using T = Team<W>;
+  constexpr int A = T::A, Q = T::Q, F = Q / 4, E = T::E;
+  const int g = lane % T::LANES / T::L;
+  int p = 0, cnt = 0;  // the lane's packs are g, g + G, ...: cnt of them from p
+  if (row >= 0 && on) {
+    const int s = __ldg(M.row_ptr + row);
+    const int npk = (__ldg(M.row_ptr + row + 1) - s) >> 2;
+    cnt = npk > g ? (npk - g + T::G - 1) / T::G : 0;
+    p = s + 4 * g;
+  }
+  const float* xl = X + gathered_slot<W>(lane);
+  float acc[A][Q];
+#pragma unroll
+  for (int i = 0; i < A; ++i)
+#pragma unroll
+    for (int q = 0; q < Q; ++q) acc[i][q] = 0.f;
+  int4 c = make_int4(0, 0, 0, 0);
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (cnt > 0) {
+    c = ld_stream_i4(M.col + p, pol);
+    v = ld_vals<BF16>(M, p, pol);
+  }
+  auto pack = [&](float (&a)[Q], bool more) {
+    const int cc[4] = {c.x, c.y, c.z, c.w};
+    const float vv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int h = 0; h < 4; h += NZ) {
+      float4 x[NZ][F];
+#pragma unroll
+      for (int u = 0; u < NZ; ++u)
+#pragma unroll
+        for (int i = 0; i < F; ++i)
+          x[u][i] = __ldg(reinterpret_cast<const float4*>(xl + (unsigned)(cc[h + u] * stride)) +
+                          i * (T::GSTRIDE / 4));
+      if (h + NZ == 4 && more) {
+        p += 4 * T::G;
+        c = ld_stream_i4(M.col + p, pol);
+        v = ld_vals<BF16>(M, p, pol);
+      }
+#pragma unroll
+      for (int u = 0; u < NZ; ++u)
+#pragma unroll
+        for (int i = 0; i < F; ++i) {
+          a[4 * i] = fmaf(vv[h + u], x[u][i].x, a[4 * i]);
+          a[4 * i + 1] = fmaf(vv[h + u], x[u][i].y, a[4 * i + 1]);
+          a[4 * i + 2] = fmaf(vv[h + u], x[u][i].z, a[4 * i + 2]);
+          a[4 * i + 3] = fmaf(vv[h + u], x[u][i].w, a[4 * i + 3]);
+        }
+    }
+  };
+  int j = 0;
+  for (; j + A < cnt; j += A) {  // all A packs have a successor: no tests
+#pragma unroll
+    for (int i = 0; i < A; ++i) pack(acc[i], true);
+  }
+#pragma unroll
+  for (int i = 0; i < A; ++i)
+    if (j + i < cnt) pack(acc[i], j + i + 1 < cnt);
+  __syncwarp();
+  if constexpr (T::G == 4) {
+    const bool hi1 = g & 1, hi2 = g >> 1;
+    float q[2 * E];
+#pragma unroll
+    for (int t = 0; t < 2 * E; ++t)
+      q[t] = (hi1 ? acc[0][2 * E + t] : acc[0][t]) +
+             __shfl_xor_sync(0xffffffffu, hi1 ? acc[0][t] : acc[0][2 * E + t], T::L);
+#pragma unroll
+    for (int t = 0; t < E; ++t)
+      out[t] = (hi2 ? q[E + t] : q[t]) +
+               __shfl_xor_sync(0xffffffffu, hi2 ? q[t] : q[E + t], 2 * T::L);
+  } else {
+    static_assert(T::G == 2 || T::G == 4, "two or four groups");
+    const bool hi = g != 0;
+    float q[2][E];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int t = 0; t < E; ++t)
+        q[i][t] = (hi ? acc[i % A][E + t] : acc[i % A][t]) +
+                  __shfl_xor_sync(0xffffffffu, hi ? acc[i % A][t] : acc[i % A][E + t], T::L);
+#pragma unroll
+    for (int t = 0; t < E; ++t) out[t] = q[0][t] + q[1][t];
+  }
+}
+
+// Rows are dealt to teams in the order M.order.  The grid is described by its
+// virtual blocks of P_WARPS teams: virtual block vb's team w takes the rows at
+// order positions vb * P_WARPS + w + i * (all teams).  A block runs RW virtual
+// blocks, so which rows a team takes (and with it the grouping of the
+// objective's sums) does not depend on the team's width.
+template <int W>
+struct RowDeal {
+  int vb, w;      // this lane's virtual block and its team in it
+  int first, step, rounds;
+  __device__ __forceinline__ RowDeal(int rows, int nvb) {
+    constexpr int RW = Team<W>::RW;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int u = warp * RW + lane / Team<W>::LANES;
+    vb = blockIdx.x * RW + u / P_WARPS;
+    w = u % P_WARPS;
+    step = nvb * P_WARPS;
+    first = vb < nvb ? vb * P_WARPS + w : rows;
+    rounds = (rows + step - 1) / step;  // uniform over the grid
+  }
+  // row of round i, or -1
+  __device__ __forceinline__ int row(const DevCSR& M, int i) const {
+    const int q = first + i * step;
+    if (q >= M.rows || first >= M.rows) return -1;
+    return M.order ? __ldg(M.order + q) : q;
+  }
+};
 
 __device__ double bgn_t(int k, double a, double b, double omega) {
   return a * pow((double)k, omega) + b;
@@ -405,211 +260,344 @@ __device__ void bset_theta(SlotState& s, double theta) {
 
 // -------------------------------------------------------------- k_bforward
 
-// Shared memory of the forward phase: the per-slot objective partials of the
-// block, and with stencil blocks in the grid the stencil tiles.  A launch
-// without stencil blocks (the first projection, volume mode) leaves out the
-// stencil's ~40 KB, so more blocks fit per SM and more of the unified L1
-// serves the gathers of image rows.
-struct BFwdEpi {
-  float dhi[B_WARPS][MAXK];
-  float dlo[B_WARPS][MAXK];
-};
-template <bool ST>
-struct BFwdSmem {
-  BFwdEpi e;
-};
-template <>
-struct BFwdSmem<true> {
-  union {
-    BFwdEpi e;
-    BStencilSmem st;
-  };
-};
-
-// ST false: SpMV blocks only (grid n_spmv_blocks); ST true: the SpMV blocks
-// followed by the stencil blocks in one grid, so the stencil blocks fill the
-// SMs as the SpMV blocks finish.
-template <int V, bool BF16, bool ST, int GR>
-__global__ void __launch_bounds__(B_THREADS) k_bforward(BFwdArgs a) {
-  __shared__ __align__(16) int s_off[B_WARPS][32];
-  __shared__ __align__(16) float s_val[B_WARPS][32];
-  __shared__ BFwdSmem<ST> sm;
+// W: slots the launch works on (every live slot is below it); a.Kp: the row
+// stride of the slot-minor arrays, at least W.
+template <int W, bool BF16, int NZ>
+__global__ void __launch_bounds__(P_THREADS, 2) k_bforward(BFwdArgs a) {
+  using T = Team<W>;
+  constexpr int E = T::E;
+  __shared__ float dsum_hi[P_WARPS * T::RW][W], dsum_lo[P_WARPS * T::RW][W];
   BatchState* bs = a.bst;
   if (a.mode == 0 && bs->remaining == 0) return;  // uniform over the grid
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int Kp = a.Kp, n = a.n;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int Kp = a.Kp;
   const int G = bs->gstep;
-  const bool proj_only = a.mode == 1;
-  const float* f = proj_only ? a.f[(G + 2) % 3] : a.f[G % 3];
-  float* y_out = proj_only ? a.y[(G + 1) & 1] : a.y[G & 1];
+  const float* f = a.f[G % 3];
+  float* y_out = a.y[G & 1];
   const float* y_prev = a.y[(G + 1) & 1];
-  const bool want = !proj_only && a.track;
-  // which of this lane's slots take part: every slot (projection), the live
-  // slots (step), or the fresh slots (admission, where f^{k-1} = f^k so the
-  // extrapolated projection is y itself)
-  int on[V];
-  float th_h[V];
-  bool lane_on = false;
+  const bool want = a.track != 0;
+  // a first forward phase (of a run, or of admitted slots): f^{k-1} = f^k, so
+  // the extrapolated projection is y itself
+  const bool first = a.mode != 0;
+  auto live = [&](const SlotState& sl) {
+    return a.mode == 2 ? sl.fresh : (sl.active && !sl.done);
+  };
+  const int sl0 = owned_slot<W>(lane), gl0 = gathered_slot<W>(lane);
+  int on[E];
+  float th_h[E];
+  bool any_on = false, gather_on = false;
 #pragma unroll
-  for (int t = 0; t < V; ++t) {
-    const SlotState& sl = a.slots[lane * V + t];
-    on[t] = proj_only ? 1 : (a.mode == 2 ? sl.fresh : (sl.active && !sl.done));
-    th_h[t] = a.mode == 2 ? 0.f : sl.theta_hi;
-    lane_on = lane_on || on[t];
+  for (int t = 0; t < E; ++t) {
+    const SlotState& sl = a.slots[sl0 + t];
+    on[t] = live(sl);
+    th_h[t] = first ? 0.f : sl.theta_hi;
+    any_on = any_on || on[t];
   }
-  float dh[V], dl[V];
-  int hits[V];
 #pragma unroll
-  for (int t = 0; t < V; ++t) {
+  for (int t = 0; t < T::Q; ++t)
+    gather_on = gather_on || live(a.slots[gl0 + t % 4 + t / 4 * T::GSTRIDE]);
+  float dh[E], dl[E];
+  int hits[E];
+#pragma unroll
+  for (int t = 0; t < E; ++t) {
     dh[t] = 0.f;
     dl[t] = 0.f;
     hits[t] = 0;
   }
-  if (!ST || (int)blockIdx.x < a.n_spmv_blocks) {
-    const uint64_t pol = evict_first_policy();
-#if APPGA_BCONTIG_FW
-    // each block owns a contiguous run of rows (neighbouring rays share
-    // pixels, so the gathered image rows are reused from L1)
-    const int per = (a.A.rows + a.n_spmv_blocks - 1) / a.n_spmv_blocks;
-    const int r0 = blockIdx.x * per, r1 = min(a.A.rows, r0 + per);
-    for (int row = r0 + warp; row < r1; row += B_WARPS) {
-#else
-    const int stride = a.n_spmv_blocks * B_WARPS;
-    for (int row = blockIdx.x * B_WARPS + warp; row < a.A.rows; row += stride) {
-#endif
-      float acc[V];
-      brow_dot<V, BF16, GR>(a.A, row, f, Kp, lane, lane_on, pol, s_off[warp], s_val[warp], acc);
-      if (!lane_on) continue;
-      const size_t o = (size_t)row * Kp + lane * V;
-      float yp[V], gg[V], gm[V], yo[V], wo[V];
-      vload<V>(y_out + o, yo);
-      if (!proj_only) {
-        vload<V>(y_prev + o, yp);
-        vload<V>(a.g + o, gg);
-        vload<V>(a.gamma + o, gm);
-        vload<V>(a.w + o, wo);
-      }
+  const uint64_t pol = evict_first_policy();
+  const RowDeal<W> deal(a.A.rows, a.n_spmv_blocks);
+  for (int i = 0; i < deal.rounds; ++i) {
+    const int row = deal.row(a.A, i);
+    float acc[E];
+    team_dot<W, BF16, NZ>(a.A, row, f, Kp, lane, gather_on, pol, acc);
+    if (row < 0 || !any_on) continue;
+    const size_t o = (size_t)row * Kp + sl0;
+    float yp[E], gg[E], gm[E], wo[E];
+    if (first) {
 #pragma unroll
-      for (int t = 0; t < V; ++t) {
-        if (!on[t]) continue;
-        yo[t] = acc[t];
-        if (proj_only) continue;
-        // y~ = y + theta (y - y_prev); den = max(y~ + gamma, kappa gamma); w = (den - g)/den
-        const float yt = a.mode == 2 ? acc[t] : fmaf(th_h[t], acc[t] - yp[t], acc[t]);
-        float den = yt + gm[t];
-        const float fl = 1e-3f * gm[t];
-        if (den < fl) {
-          den = fl;
-          ++hits[t];
-        }
-        wo[t] = __fdiv_rn(den - gg[t], den);
-        if (want) {
-          // data term y - g ln(y + gamma) in double-float
-          df yg;
-          two_sum(acc[t], gm[t], yg.hi, yg.lo);
-          const df term = df_add_f(df_neg(df_mul_f(df_log(yg), gg[t])), acc[t]);
-          acc_add(dh[t], dl[t], term.hi, term.lo);
-        }
-      }
-      vstore<V>(y_out + o, yo);
-      if (!proj_only) vstore<V>(a.w + o, wo);
+      for (int t = 0; t < E; ++t) yp[t] = acc[t];
+    } else {
+      vload<E>(y_prev + o, yp);
     }
-  } else if constexpr (ST) {
-    if (!proj_only) {
-      // stencil items: (tile, 8-slot chunk) pairs, persistent over the stencil blocks
-      const int nsb = gridDim.x - a.n_spmv_blocks;
-      const int ntx = (n + BST_C - 1) / BST_C, nty = (n + BST_R - 1) / BST_R;
-      const int nchunks = Kp / BST_S;
-      const int ntiles = ntx * nty;
-      __shared__ float sreg_hi[MAXK], sreg_lo[MAXK];  // per-slot regulariser sums
-      __shared__ int chunk_on[MAXK / BST_S];
-      for (int s = tid; s < MAXK; s += blockDim.x) {
-        sreg_hi[s] = 0.f;
-        sreg_lo[s] = 0.f;
+    vload<E>(a.g + o, gg);
+    vload<E>(a.gamma + o, gm);
+#pragma unroll
+    for (int t = 0; t < E; ++t) {
+      wo[t] = 0.f;
+      if (!on[t]) continue;
+      // y~ = y + theta (y - y_prev); den = max(y~ + gamma, kappa gamma); w = (den - g)/den
+      const float yt = first ? acc[t] : fmaf(th_h[t], acc[t] - yp[t], acc[t]);
+      float den = yt + gm[t];
+      const float fl = 1e-3f * gm[t];
+      if (den < fl) {
+        den = fl;
+        ++hits[t];
       }
-      for (int c = tid; c < nchunks; c += blockDim.x) {
-        int any = 0;
-        for (int q = 0; q < BST_S; ++q) {
-          const SlotState& sl = a.slots[c * BST_S + q];
-          any |= a.mode == 2 ? sl.fresh : (sl.active && !sl.done);
-        }
-        chunk_on[c] = any;
-      }
-      __syncthreads();
-      // Each block owns the same tiles for every slot chunk, so a slot's
-      // regulariser sum is grouped the same way whatever its slot index.
-      for (int tile = blockIdx.x - a.n_spmv_blocks; tile < ntiles; tile += nsb)
-      for (int chunk = 0; chunk < nchunks; ++chunk) {
-        if (!chunk_on[chunk]) continue;  // uniform over the block
-        const int r0 = (tile / ntx) * BST_R, c0 = (tile % ntx) * BST_C;
-        const float reg = bstencil_item(sm.st, f, a.f[(G + 2) % 3], a.slots, Kp, r0, c0,
-                                        chunk * BST_S, n, a.gR, want, a.mode);
-        if (want) {
-          // warp q holds slot chunk*8 + q: fold the warp's 32 columns
-          float h = reg, l = 0.f;
-          warp_sum_acc(h, l);
-          if (lane == 0) {
-            const int s = chunk * BST_S + warp;
-            acc_add(sreg_hi[s], sreg_lo[s], h, l);
-          }
-        }
-      }
-      __syncthreads();
-      if (want && warp == 0) {
-        // hand the per-slot sums to the lanes that own the slots in warp 0
-  #pragma unroll
-        for (int t = 0; t < V; ++t) {
-          dh[t] = sreg_hi[lane * V + t];
-          dl[t] = sreg_lo[lane * V + t];
-        }
+      wo[t] = __fdiv_rn(den - gg[t], den);
+      if (want) {
+        // data term y - g ln(y + gamma) in double-float
+        df yg;
+        two_sum(acc[t], gm[t], yg.hi, yg.lo);
+        const df term = df_add_f(df_neg(df_mul_f(df_log(yg), gg[t])), acc[t]);
+        acc_add(dh[t], dl[t], term.hi, term.lo);
       }
     }
+    vstore_on<E>(y_out + o, acc, on);
+    vstore_on<E>(a.w + o, wo, on);
   }
-  if (!proj_only) {
 #pragma unroll
-    for (int t = 0; t < V; ++t)
-      if (hits[t]) atomicAdd(&a.slots[lane * V + t].guard_hits, (unsigned long long)hits[t]);
+  for (int t = 0; t < E; ++t)
+    if (hits[t]) atomicAdd(&a.slots[sl0 + t].guard_hits, (unsigned long long)hits[t]);
+  if (!want) return;
+  // one row of per-slot sums per virtual block (its teams in order), left for
+  // the pixel phase of this step; an admission pass writes only the fresh
+  // slots' columns
+  const int team = (tid >> 5) * T::RW + lane / T::LANES;
+#pragma unroll
+  for (int t = 0; t < E; ++t) {
+    dsum_hi[team][sl0 + t] = dh[t];
+    dsum_lo[team][sl0 + t] = dl[t];
+  }
+  __syncthreads();
+  for (int q = tid; q < T::RW * W; q += P_THREADS) {
+    const int s = q % W, vb = blockIdx.x * T::RW + q / W;
+    if (vb >= a.n_spmv_blocks || !live(a.slots[s])) continue;
+    float h = 0.f, l = 0.f;
+    for (int w = 0; w < P_WARPS; ++w)
+      acc_add(h, l, dsum_hi[q / W * P_WARPS + w][s], dsum_lo[q / W * P_WARPS + w][s]);
+    a.fpartial[(size_t)vb * Kp + s] = make_float2(h, l);
+  }
+}
+
+// -------------------------------------------------------------- k_bstencil
+
+// The six fields of B at a pixel from its 3 x 3 neighbourhood x[dr + 1][dc + 1]
+// (the forms of the single-slice stencil).
+struct BEdges {
+  bool r_lo, r_hi, c_lo, c_hi;
+};
+__device__ __forceinline__ void bfields(const float (&x)[3][3], const BEdges& e, float (&u)[6]) {
+  const float dc = x[1][1] - x[1][0], dr = x[1][1] - x[0][1];
+  u[0] = e.c_lo ? dc : 0.f;
+  u[1] = e.r_lo ? dr : 0.f;
+  u[2] = (e.c_lo ? -dc : 0.f) + (e.c_hi ? x[1][2] - x[1][1] : 0.f);
+  u[3] = e.c_lo ? ((e.r_lo ? -dc : 0.f) + (e.r_hi ? x[2][1] - x[2][0] : 0.f)) : 0.f;
+  u[4] = (e.r_lo ? -dr : 0.f) + (e.r_hi ? x[2][1] - x[1][1] : 0.f);
+  u[5] = e.r_lo ? ((e.c_lo ? -dr : 0.f) + (e.c_hi ? x[1][2] - x[0][2] : 0.f)) : 0.f;
+}
+
+// B^T grad phi~(B f~) of the current iterates and the regulariser's share of
+// Phi(f^k).  A thread owns one slot of one image column and marches down a run
+// of rows: the 3 x 3 neighbourhoods of f~ and f^k and the gradient fields of
+// its own column stay in registers, and a row's values for the neighbouring
+// columns pass through shared memory, slots fastest (no bank conflicts), with
+// one barrier per row (the fields of row s - 2 go out with f~ of row s).
+// Reading every operand of a point from shared memory instead took 15 passes
+// of the L1 pipe per point and slot warp: 255 us at 64 slots of 256 x 256.
+// blockIdx.y is the chunk of eight slots; blocks of one x own the same tiles,
+// so a slot's sum is grouped the same way whatever its index, and leave their
+// row of sums after the projector's.  Runs beside k_bforward (both read only
+// the iterates).
+__global__ void __launch_bounds__(B_THREADS, 4) k_bstencil(BFwdArgs a) {
+  // double-buffered rows: f~, f^k and the fields 0, 2, 3, 5
+  __shared__ float sT[2][BST_C + 2][BST_S], sK[2][BST_C + 2][BST_S];
+  __shared__ float sV[2][4][BST_C + 2][BST_S];
+  __shared__ float red_hi[B_THREADS / 32][BST_S], red_lo[B_THREADS / 32][BST_S];
+  BatchState* bs = a.bst;
+  if (a.mode == 0 && bs->remaining == 0) return;  // uniform over the grid
+  const int tid = threadIdx.x, q = tid % BST_S, col = tid / BST_S;
+  const int slot = blockIdx.y * BST_S + q, Kp = a.Kp, n = a.n, G = bs->gstep;
+  const SlotState& sl = a.slots[slot];
+  const bool part = a.mode == 2 ? sl.fresh : (sl.active && !sl.done);
+  if (!__syncthreads_or(part)) return;  // no live slot in the chunk
+  const bool want = a.track != 0;
+  const float* fk = a.f[G % 3] + slot;
+  const float* fkm = a.f[(G + 2) % 3] + slot;
+  float* gR = a.gR + slot;
+  // a first forward phase has f^{k-1} = f^k
+  const float th = a.mode != 0 ? 0.f : sl.theta_hi;
+  const float lam1 = sl.lambda1, lam2 = sl.lambda2, eps = sl.eps;
+  const int ntx = (n + BST_OUT - 1) / BST_OUT, nty = (n + BST_R - 1) / BST_R;
+  float reg_h = 0.f, reg_l = 0.f;
+  for (int tile = blockIdx.x; tile < ntx * nty; tile += gridDim.x) {
+    const int r0 = (tile / ntx) * BST_R, r1 = min(n, r0 + BST_R);
+    const int c = (tile % ntx) * BST_OUT - 2 + col;
+    const bool c_in = c >= 0 && c < n;
+    const bool out_col = part && c_in && col >= 2 && col < BST_C - 2;
+    float t[3][3] = {}, k[3][3] = {};  // f~ and f^k at rows s - 2 .. s, columns c - 1 .. c + 1
+    // fields of the own column (and the neighbours' where the adjoint reads
+    // them): v of row s - 1, w of row s - 2, x of row s - 3
+    float v[6] = {}, w0 = 0.f, w0r = 0.f, w1 = 0.f, w2 = 0.f, w2l = 0.f, w2r = 0.f, w3 = 0.f,
+          w3r = 0.f, w4 = 0.f, w5 = 0.f, w5l = 0.f;
+    float x3 = 0.f, x3r = 0.f, x4 = 0.f, x0 = 0.f, x0r = 0.f, x1 = 0.f, x2 = 0.f, x2l = 0.f,
+          x2r = 0.f, x5 = 0.f, x5l = 0.f, y3 = 0.f, y3r = 0.f, y4 = 0.f;
+    float nk = 0.f, nm = 0.f;  // the next row, in flight
+    auto fetch = [&](int r) {
+      nk = nm = 0.f;
+      if (c_in && r >= 0 && r < n) {
+        const size_t o = (size_t)(r * n + c) * Kp;
+        nk = fk[o];
+        nm = fkm[o];
+      }
+    };
+    fetch(r0 - 2);
+    for (int s = r0 - 2; s <= r1 + 2; ++s) {
+      const int b = s & 1;
+      const float vk = nk, vt = fmaf(th, nk - nm, nk);
+      sT[b][col + 1][q] = vt;
+      if (want) sK[b][col + 1][q] = vk;
+      // the fields of row s - 2, computed in the last step
+      sV[b][0][col + 1][q] = v[0];
+      sV[b][1][col + 1][q] = v[2];
+      sV[b][2][col + 1][q] = v[3];
+      sV[b][3][col + 1][q] = v[5];
+      if (s < r1 + 2) fetch(s + 1);
+      __syncthreads();
+      // rows move up: y is row s - 4, x row s - 3, w row s - 2
+      y3 = x3; y3r = x3r; y4 = x4;
+      x0 = w0; x0r = w0r; x1 = w1; x2 = w2; x2l = w2l; x2r = w2r;
+      x3 = w3; x3r = w3r; x4 = w4; x5 = w5; x5l = w5l;
+      w0 = v[0]; w1 = v[1]; w2 = v[2]; w3 = v[3]; w4 = v[4]; w5 = v[5];
+      w0r = sV[b][0][col + 2][q];
+      w2l = sV[b][1][col][q];
+      w2r = sV[b][1][col + 2][q];
+      w3r = sV[b][2][col + 2][q];
+      w5l = sV[b][3][col][q];
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        t[0][j] = t[1][j];
+        t[1][j] = t[2][j];
+        k[0][j] = k[1][j];
+        k[1][j] = k[2][j];
+      }
+      t[2][0] = sT[b][col][q];
+      t[2][1] = vt;
+      t[2][2] = sT[b][col + 2][q];
+      if (want) {
+        k[2][0] = sK[b][col][q];
+        k[2][1] = vk;
+        k[2][2] = sK[b][col + 2][q];
+      }
+      // grad phi~ at row i = s - 1
+      const int i = s - 1;
+      const BEdges e = {i >= 1, i <= n - 2, c >= 1, c <= n - 2};
+#pragma unroll
+      for (int f = 0; f < 6; ++f) v[f] = 0.f;
+      if (c_in && i >= 0 && i < n) {
+        bfields(t, e, v);
+        const float n1 = v[0] * v[0] + v[1] * v[1];
+        const float n2 = v[2] * v[2] + v[3] * v[3] + v[4] * v[4] + v[5] * v[5];
+        const float s1 = lam1 / fmaxf(sqrtf(n1), eps), s2 = lam2 / fmaxf(sqrtf(n2), eps);
+        v[0] *= s1;
+        v[1] *= s1;
+#pragma unroll
+        for (int f = 2; f < 6; ++f) v[f] *= s2;
+        if (want && out_col && i >= r0 && i < r1) {
+          float u[6];
+          bfields(k, e, u);
+          const float m1 = u[0] * u[0] + u[1] * u[1];
+          const float m2 = u[2] * u[2] + u[3] * u[3] + u[4] * u[4] + u[5] * u[5];
+          acc_add(reg_h, reg_l, lam1 * s_eps_f(m1, eps) + lam2 * s_eps_f(m2, eps), 0.f);
+        }
+      }
+      // the adjoint at row o = s - 3: rows o - 1 (y), o (x), o + 1 (w)
+      const int o = s - 3;
+      if (out_col && o >= r0 && o < r1) {
+        const bool r_lo = o >= 1, r_hi = o <= n - 2;
+        float sum = 0.f;
+        if (e.c_lo) sum += x0;
+        if (e.c_hi) sum -= x0r;
+        if (r_lo) sum += x1;
+        if (r_hi) sum -= w1;
+        sum += (e.c_lo ? -(x2 - x2l) : 0.f) + (e.c_hi ? x2r - x2 : 0.f);
+        sum += r_lo ? ((e.c_lo ? -(x3 - y3) : 0.f) + (e.c_hi ? x3r - y3r : 0.f)) : 0.f;
+        sum += (r_lo ? -(x4 - y4) : 0.f) + (r_hi ? w4 - x4 : 0.f);
+        sum += e.c_lo ? ((r_lo ? -(x5 - x5l) : 0.f) + (r_hi ? w5 - w5l : 0.f)) : 0.f;
+        gR[(size_t)(o * n + c) * Kp] = sum;
+      }
+    }
+    __syncthreads();  // the row buffers are refilled by the next tile
   }
   if (!want) return;
-  // block partial per slot (fixed order over warps), left for the pixel
-  // phase of this step; an admission pass writes only the fresh slots' columns
-  __syncthreads();
+  // the block's sum of each slot: four columns by shuffles, then the warps in order
 #pragma unroll
-  for (int t = 0; t < V; ++t) {
-    sm.e.dhi[warp][lane * V + t] = dh[t];
-    sm.e.dlo[warp][lane * V + t] = dl[t];
+  for (int o = BST_S; o < 32; o <<= 1)
+    acc_add(reg_h, reg_l, __shfl_xor_sync(0xffffffffu, reg_h, o),
+            __shfl_xor_sync(0xffffffffu, reg_l, o));
+  if (tid % 32 < BST_S) {
+    red_hi[tid / 32][q] = reg_h;
+    red_lo[tid / 32][q] = reg_l;
   }
   __syncthreads();
-  for (int s = tid; s < Kp; s += blockDim.x) {
-    const SlotState& sl = a.slots[s];
-    if (a.mode == 2 ? !sl.fresh : !(sl.active && !sl.done)) continue;
+  if (tid < BST_S && part) {
     float h = 0.f, l = 0.f;
-    for (int w = 0; w < B_WARPS; ++w) acc_add(h, l, sm.e.dhi[w][s], sm.e.dlo[w][s]);
-    a.fpartial[(size_t)blockIdx.x * Kp + s] = make_float2(h, l);
+    for (int w = 0; w < B_THREADS / 32; ++w) acc_add(h, l, red_hi[w][q], red_lo[w][q]);
+    a.fpartial[(size_t)(a.n_spmv_blocks + blockIdx.x) * Kp + slot] = make_float2(h, l);
   }
 }
 
 // --------------------------------------------------------------- k_bpixel
 
-template <int V, bool BF16, int GR>
-__global__ void __launch_bounds__(B_THREADS) k_bpixel(BPixArgs a) {
-  __shared__ __align__(16) int s_off[B_WARPS][32];
-  __shared__ __align__(16) float s_val[B_WARPS][32];
-  __shared__ float r_hi[MAXK], r_lo[MAXK], t_hi[MAXK], t_lo[MAXK];
+// Per-slot sums of the forward phase's rows in OBJ_GROUPS groups (rows g,
+// g + OBJ_GROUPS, ...), summed by the pixel phase's first blocks; the last
+// block adds the group sums.  Every sum runs in four parts combined in order,
+// whatever the grid and the slots' number.
+constexpr int OBJ_GROUPS = 64;
+constexpr int OBJ_PARTS = P_THREADS / MAXK;
+__device__ void sum_rows(const float2* rows, int first, int step, int count, int Kp,
+                         float (&r_hi)[P_THREADS], float (&r_lo)[P_THREADS]) {
+  const int s = threadIdx.x % MAXK, part = threadIdx.x / MAXK;
+  float h = 0.f, l = 0.f;
+  if (s < Kp) {
+#pragma unroll 4
+    for (int i = first + part * step; i < count; i += OBJ_PARTS * step) {
+      const float2 v = __ldcg(rows + (size_t)i * Kp + s);
+      acc_add(h, l, v.x, v.y);
+    }
+  }
+  __syncthreads();
+  r_hi[threadIdx.x] = h;
+  r_lo[threadIdx.x] = l;
+  __syncthreads();
+  if (threadIdx.x < MAXK) {
+    h = 0.f;
+    l = 0.f;
+    for (int q = 0; q < OBJ_PARTS; ++q) acc_add(h, l, r_hi[q * MAXK + s], r_lo[q * MAXK + s]);
+    r_hi[s] = h;
+    r_lo[s] = l;
+  }
+  __syncthreads();
+}
+
+template <int W, bool BF16, int NZ>
+__global__ void __launch_bounds__(P_THREADS, 2) k_bpixel(BPixArgs a) {
+  using T = Team<W>;
+  constexpr int E = T::E;
+  __shared__ float r_hi[P_THREADS], r_lo[P_THREADS];
+  __shared__ int s_last;
   BatchState* bs = a.bst;
   if (bs->remaining == 0) return;  // uniform over the grid
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31;
   const int Kp = a.Kp;
   const int G = bs->gstep;
   const float* fk = a.f[G % 3];
   const float* fkm = a.f[(G + 2) % 3];
   float* fn = a.f[(G + 1) % 3];
+  // every slot's Phi(f^k): the forward phase's rows, first because these
+  // blocks start first
+  if (a.track)
+    for (int g = blockIdx.x; g < OBJ_GROUPS; g += gridDim.x) {
+      sum_rows(a.fpartial, g, OBJ_GROUPS, a.n_fpartial, Kp, r_hi, r_lo);
+      if (tid < Kp) a.partial[(size_t)g * Kp + tid] = make_float2(r_hi[tid], r_lo[tid]);
+    }
   // this lane's slot parameters
-  float th[V], beta[V];
-  int live[V], kk[V], frz[V], back[V];
+  const int sl0 = owned_slot<W>(lane), gl0 = gathered_slot<W>(lane);
+  float th[E], beta[E];
+  int live[E], kk[E], frz[E], back[E];
+  bool gather_live = false;
 #pragma unroll
-  for (int t = 0; t < V; ++t) {
-    const SlotState& sl = a.slots[lane * V + t];
+  for (int t = 0; t < E; ++t) {
+    const SlotState& sl = a.slots[sl0 + t];
     th[t] = sl.theta_hi;
     beta[t] = sl.beta;
     live[t] = sl.active && !sl.done;
@@ -617,31 +605,27 @@ __global__ void __launch_bounds__(B_THREADS) k_bpixel(BPixArgs a) {
     frz[t] = sl.freeze_iter;
     back[t] = sl.rollback;
   }
-  bool lane_live = false;
 #pragma unroll
-  for (int t = 0; t < V; ++t) lane_live = lane_live || live[t];
+  for (int t = 0; t < T::Q; ++t) {
+    const SlotState& sl = a.slots[gl0 + t % 4 + t / 4 * T::GSTRIDE];
+    gather_live = gather_live || (sl.active && !sl.done);
+  }
   const uint64_t pol = evict_first_policy();
   int bad = 0;
-#if APPGA_BCONTIG_PX
-  // each block owns a contiguous run of pixels (neighbouring pixels lie on
-  // the same rays, so the gathered weight rows are reused from L1)
-  const int per = (a.At.rows + gridDim.x - 1) / gridDim.x;
-  const int j0 = blockIdx.x * per, j1 = min(a.At.rows, j0 + per);
-  for (int j = j0 + warp; j < j1; j += B_WARPS) {
-#else
-  const int stride = gridDim.x * B_WARPS;
-  for (int j = blockIdx.x * B_WARPS + warp; j < a.At.rows; j += stride) {
-#endif
-    float bp[V];
-    brow_dot<V, BF16, GR>(a.At, j, a.w, Kp, lane, lane_live, pol, s_off[warp], s_val[warp], bp);
-    const size_t o = (size_t)j * Kp + lane * V;
-    float vk[V], vm[V], gr[V], out[V];
-    vload<V>(fk + o, vk);
-    vload<V>(fkm + o, vm);
-    vload<V>(a.gR + o, gr);
+  const RowDeal<W> deal(a.At.rows, a.n_blocks);
+  for (int i = 0; i < deal.rounds; ++i) {
+    const int j = deal.row(a.At, i);
+    float bp[E];
+    team_dot<W, BF16, NZ>(a.At, j, a.w, Kp, lane, gather_live, pol, bp);
+    if (j < 0) continue;
+    const size_t o = (size_t)j * Kp + sl0;
+    float vk[E], vm[E], gr[E], out[E];
+    vload<E>(fk + o, vk);
+    vload<E>(fkm + o, vm);
+    vload<E>(a.gR + o, gr);
     const float il = __ldg(a.inv_lambda + j);
 #pragma unroll
-    for (int t = 0; t < V; ++t) {
+    for (int t = 0; t < E; ++t) {
       if (!live[t]) {
         // finished or empty slot: carry the image (the previous entry when
         // the slot stopped one step back)
@@ -662,26 +646,23 @@ __global__ void __launch_bounds__(B_THREADS) k_bpixel(BPixArgs a) {
       if (!isfinite(xv)) bad = 1;
       out[t] = fmaxf(xv, 0.f);
     }
-    vstore<V>(fn + o, out);
+    int on[E];
+#pragma unroll
+    for (int t = 0; t < E; ++t) on[t] = 1;
+    vstore_on<E>(fn + o, out, on);
   }
   if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(&bs->flags, APPGA_FLAG_NONFINITE);
-  // This block's share of every slot's Phi(f^k): forward partial rows
-  // b, b + G, ... (fixed order).
-  for (int s = tid; s < Kp; s += blockDim.x) {
-    float h = 0.f, l = 0.f;
-    if (a.track)
-      for (int i = blockIdx.x; i < a.n_fpartial; i += gridDim.x) {
-        const float2 v = a.fpartial[(size_t)i * Kp + s];
-        acc_add(h, l, v.x, v.y);
-      }
-    r_hi[s] = h;
-    r_lo[s] = l;
-  }
   // Finalise the step in the last block: Phi and the stopping test of every
   // live slot, then its next index and momentum; the global step advances.
+  __threadfence();
   __syncthreads();
-  if (grid_reduce_slots(a.partial, a.gtick, &bs->ticket_p, r_hi, r_lo, Kp, t_hi, t_lo)) {
-    __shared__ int s_rem[B_THREADS];
+  if (tid == 0) s_last = atomicAdd(&bs->ticket_p, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (s_last) {
+    __threadfence();
+    const float *t_hi = r_hi, *t_lo = r_lo;  // the slots' totals
+    if (a.track) sum_rows(a.partial, 0, 1, OBJ_GROUPS, Kp, r_hi, r_lo);
+    if (tid == 0) bs->ticket_p = 0;
     __shared__ int s_jstop;
     if (a.joint) {
       // volume: the slices are one problem; its objective is the sum of the
@@ -763,11 +744,9 @@ __global__ void __launch_bounds__(B_THREADS) k_bpixel(BPixArgs a) {
       }
       bset_theta(sl, th_next);
     }
-    s_rem[tid] = rem;
-    __syncthreads();
+    static_assert(P_THREADS >= MAXK, "one slot per thread");
+    const int tot = __syncthreads_count(rem);
     if (tid == 0) {
-      int tot = 0;
-      for (int i = 0; i < (int)blockDim.x; ++i) tot += s_rem[i];
       bs->gstep = G + 1;
       bs->remaining = tot;
     }
@@ -898,80 +877,58 @@ __global__ void __launch_bounds__(256) k_binit_image(const float* __restrict__ g
 
 int sm_count() { return current_sm_count(); }
 
-int bforward_grid_n(const BFwdArgs& a, int* n_spmv) {
-  const int sms = sm_count();
-  int nsp = (a.A.rows + B_WARPS - 1) / B_WARPS;
-  const int cap = sms * clamp_per_sm(a.spmv_per_sm, default_spmv_per_sm(a.Kp));
-  if (nsp > cap) nsp = cap;
-  int nst = 0;
-  if (a.mode != 1 && !a.no_stencil) {
-    // equal tile counts per stencil block
-    const int tiles = ((a.n + BST_C - 1) / BST_C) * ((a.n + BST_R - 1) / BST_R);
-    const int scap = sms * clamp_per_sm(a.stencil_per_sm, default_stencil_per_sm(a.Kp));
-    const int per = (tiles + scap - 1) / scap;
-    nst = (tiles + per - 1) / per;
-  }
-  if (n_spmv) *n_spmv = nsp;
-  return nsp + nst;
+// Virtual blocks of the forward phase's projector rows.
+int fw_blocks(const BFwdArgs& a) {
+  const int nb = (a.A.rows + P_WARPS - 1) / P_WARPS;
+  return std::min(nb, sm_count() * clamp_per_sm(a.spmv_per_sm, kSpmvPerSm));
+}
+// Stencil blocks per slot chunk: equal tile counts per block.
+int st_blocks(const BFwdArgs& a) {
+  if (a.no_stencil) return 0;
+  const int tiles = ((a.n + BST_OUT - 1) / BST_OUT) * ((a.n + BST_R - 1) / BST_R);
+  const int cap = sm_count() * clamp_per_sm(a.stencil_per_sm, kStencilPerSm);
+  const int per = (tiles + cap - 1) / cap;
+  return (tiles + per - 1) / per;
 }
 
-// Gather probe: the batched projectors' inner loop alone.  Every row of M
-// is reduced against the Kp-wide slot-minor rows of x by brow_dot, in the
-// row order of the projection it stands for (contig: a contiguous run of
-// rows per block, else rows dealt to the grid's warps in turn), with no
-// epilogue, stencil or pixel update: the time of the column/value stream and
-// the gathers by themselves.
-template <int V>
-__global__ void __launch_bounds__(B_THREADS) k_gather_probe(DevCSR M, const float* __restrict__ x,
-                                                            int Kp, int contig,
-                                                            float* __restrict__ sink) {
-  __shared__ __align__(16) int s_off[B_WARPS][32];
-  __shared__ __align__(16) float s_val[B_WARPS][32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// Gather probe: the batched projectors' inner loop alone.  Every row of M is
+// reduced against the W-wide slot-minor rows of x by team_dot, dealt to the
+// teams as in the projections, with no epilogue, stencil or pixel update.
+template <int W>
+__global__ void __launch_bounds__(P_THREADS, 2) k_gather_probe(DevCSR M, const float* __restrict__ x,
+                                                               int nvb, float* __restrict__ sink) {
+  const int lane = threadIdx.x & 31;
   const uint64_t pol = evict_first_policy();
-  const int per = (M.rows + gridDim.x - 1) / gridDim.x;
-  const int r0 = contig ? blockIdx.x * per : blockIdx.x * B_WARPS;
-  const int r1 = contig ? min(M.rows, r0 + per) : M.rows;
-  const int step = contig ? B_WARPS : gridDim.x * B_WARPS;
+  const RowDeal<W> deal(M.rows, nvb);
   float s = 0.f;
-  for (int row = r0 + warp; row < r1; row += step) {
-    float acc[V];
-    brow_dot<V, false>(M, row, x, Kp, lane, true, pol, s_off[warp], s_val[warp], acc);
+  for (int i = 0; i < deal.rounds; ++i) {
+    float acc[Team<W>::E];
+    team_dot<W, false, 4>(M, deal.row(M, i), x, W, lane, true, pol, acc);
 #pragma unroll
-    for (int t = 0; t < V; ++t) s += acc[t];
+    for (int t = 0; t < Team<W>::E; ++t) s += acc[t];
   }
   if (s == 1.0e38f) sink[blockIdx.x] = s;  // keeps the loads; the value is never used
 }
 
-template <int V>
-cudaError_t bforward_v(const BFwdArgs& a0, cudaStream_t s) {
-  BFwdArgs a = a0;
-  const int sms = sm_count();
-  (void)sms;
-  int nsp = 0;
-  const int grid = bforward_grid_n(a, &nsp);
-  a.n_spmv_blocks = nsp;
-  const bool st = grid > nsp, g4 = a.gather_rows == 4;
-  void (*kern)(BFwdArgs);
-  if (a.use_bf16)
-    kern = st ? (g4 ? k_bforward<V, true, true, 4> : k_bforward<V, true, true, 8>)
-              : (g4 ? k_bforward<V, true, false, 4> : k_bforward<V, true, false, 8>);
-  else
-    kern = st ? (g4 ? k_bforward<V, false, true, 4> : k_bforward<V, false, true, 8>)
-              : (g4 ? k_bforward<V, false, false, 4> : k_bforward<V, false, false, 8>);
-  kern<<<grid, B_THREADS, 0, s>>>(a);
+template <int W>
+int blocks_of(int nvb) {
+  return (nvb + Team<W>::RW - 1) / Team<W>::RW;
+}
+
+template <int W>
+cudaError_t bforward_w(const BFwdArgs& a, cudaStream_t s) {
+  const bool g4 = a.gather_rows == 4;
+  void (*kern)(BFwdArgs) = a.use_bf16 ? (g4 ? k_bforward<W, true, 2> : k_bforward<W, true, 4>)
+                                      : (g4 ? k_bforward<W, false, 2> : k_bforward<W, false, 4>);
+  kern<<<blocks_of<W>(a.n_spmv_blocks), P_THREADS, 0, s>>>(a);
   return cudaGetLastError();
 }
-template <int V>
-cudaError_t bpixel_v(const BPixArgs& a, cudaStream_t s) {
-  const int sms = sm_count();
-  int nb = (a.At.rows + B_WARPS - 1) / B_WARPS;
-  const int cap = sms * clamp_per_sm(a.blocks_per_sm, default_pixel_per_sm(a.Kp));
-  if (nb > cap) nb = cap;
+template <int W>
+cudaError_t bpixel_w(const BPixArgs& a, cudaStream_t s) {
   const bool g4 = a.gather_rows == 4;
-  void (*kern)(BPixArgs) = a.use_bf16 ? (g4 ? k_bpixel<V, true, 4> : k_bpixel<V, true, 8>)
-                                      : (g4 ? k_bpixel<V, false, 4> : k_bpixel<V, false, 8>);
-  kern<<<nb, B_THREADS, 0, s>>>(a);
+  void (*kern)(BPixArgs) = a.use_bf16 ? (g4 ? k_bpixel<W, true, 2> : k_bpixel<W, true, 4>)
+                                      : (g4 ? k_bpixel<W, false, 2> : k_bpixel<W, false, 4>);
+  kern<<<blocks_of<W>(a.n_blocks), P_THREADS, 0, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -981,7 +938,7 @@ cudaError_t bpixel_v(const BPixArgs& a, cudaStream_t s) {
 // stencil blocks per SM (the launchers clamp the tuned values).
 int batch_max_blocks() { return sm_count() * 2 * kMaxPerSm + 64; }
 
-int bforward_grid(const BFwdArgs& a) { return bforward_grid_n(a, nullptr); }
+int bforward_grid(const BFwdArgs& a) { return fw_blocks(a) + st_blocks(a); }
 
 cudaError_t launch_resolve_rollback(const BFwdArgs& a, cudaStream_t s) {
   const int len = a.n * a.n;
@@ -994,36 +951,53 @@ cudaError_t launch_resolve_rollback(const BFwdArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_bforward(const BFwdArgs& a, cudaStream_t s) {
+cudaError_t launch_bforward(const BFwdArgs& a0, cudaStream_t s) {
   cudaError_t e = ensure_tables();
   if (e != cudaSuccess) return e;
-  switch (a.Kp / 32) {
-    case 1: return bforward_v<1>(a, s);
-    case 2: return bforward_v<2>(a, s);
-    case 4: return bforward_v<4>(a, s);
+  BFwdArgs a = a0;
+  a.n_spmv_blocks = fw_blocks(a);
+  switch (a.width) {
+    case 8: return bforward_w<8>(a, s);
+    case 16: return bforward_w<16>(a, s);
+    case 32: return bforward_w<32>(a, s);
+    case 64: return bforward_w<64>(a, s);
+    case 128: return bforward_w<128>(a, s);
   }
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_gather_probe(const DevCSR& M, bool forward, const float* x, int Kp,
-                                float* sink, int blocks_per_sm, cudaStream_t s) {
+cudaError_t launch_bstencil(const BFwdArgs& a0, cudaStream_t s) {
+  BFwdArgs a = a0;
+  a.n_spmv_blocks = fw_blocks(a);
+  const int nst = st_blocks(a);
+  if (nst == 0) return cudaSuccess;
+  k_bstencil<<<dim3(nst, a.width / BST_S), B_THREADS, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_gather_probe(const DevCSR& M, const float* x, int Kp, float* sink,
+                                int blocks_per_sm, cudaStream_t s) {
   if (blocks_per_sm < 1 || blocks_per_sm > kMaxPerSm) return cudaErrorInvalidValue;
-  const int grid = sm_count() * blocks_per_sm;
-  const int contig = forward ? APPGA_BCONTIG_FW : APPGA_BCONTIG_PX;
-  switch (Kp / 32) {
-    case 1: k_gather_probe<1><<<grid, B_THREADS, 0, s>>>(M, x, Kp, contig, sink); break;
-    case 2: k_gather_probe<2><<<grid, B_THREADS, 0, s>>>(M, x, Kp, contig, sink); break;
-    case 4: k_gather_probe<4><<<grid, B_THREADS, 0, s>>>(M, x, Kp, contig, sink); break;
+  const int grid = std::min((M.rows + P_WARPS - 1) / P_WARPS, sm_count() * blocks_per_sm);
+  switch (Kp) {
+    case 32: k_gather_probe<32><<<grid, P_THREADS, 0, s>>>(M, x, grid, sink); break;
+    case 64: k_gather_probe<64><<<grid, P_THREADS, 0, s>>>(M, x, grid, sink); break;
+    case 128: k_gather_probe<128><<<grid, P_THREADS, 0, s>>>(M, x, grid, sink); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
 }
 
-cudaError_t launch_bpixel(const BPixArgs& a, cudaStream_t s) {
-  switch (a.Kp / 32) {
-    case 1: return bpixel_v<1>(a, s);
-    case 2: return bpixel_v<2>(a, s);
-    case 4: return bpixel_v<4>(a, s);
+cudaError_t launch_bpixel(const BPixArgs& a0, cudaStream_t s) {
+  BPixArgs a = a0;
+  a.n_blocks = std::min((a.At.rows + P_WARPS - 1) / P_WARPS,
+                        sm_count() * clamp_per_sm(a.blocks_per_sm, kPixelPerSm));
+  switch (a.width) {
+    case 8: return bpixel_w<8>(a, s);
+    case 16: return bpixel_w<16>(a, s);
+    case 32: return bpixel_w<32>(a, s);
+    case 64: return bpixel_w<64>(a, s);
+    case 128: return bpixel_w<128>(a, s);
   }
   return cudaErrorInvalidValue;
 }

@@ -18,6 +18,7 @@
 #include <cstring>
 #include <deque>
 #include <limits>
+#include <map>
 #include <memory>
 #include <unordered_map>
 #include <vector>
@@ -51,7 +52,7 @@ struct Pool {
   BatchWorkspace b;
   BFwdArgs fa{};
   BPixArgs pa{};
-  cudaGraphExec_t gexec = nullptr;
+  std::map<int, cudaGraphExec_t> gexec;  // a replay's graph, by the slots it works on
   cudaStream_t stream = nullptr;  // all of this pool's work
   cudaEvent_t ev_snap = nullptr;  // the slot-state copy after a replay has landed
   cudaEvent_t ev_start = nullptr; // start of the replay (timing)
@@ -73,6 +74,13 @@ struct Pool {
   int* h_ids = nullptr;   // pinned mirror
 
   int free_slots() const { return (int)slot_req.size() - used; }
+  // slots the kernels work on: every held slot is below it, the others are
+  // empty (a slot's arithmetic does not depend on it)
+  int width() const {
+    int top = (int)slot_req.size();
+    while (top > 0 && slot_req[top - 1] == -1) --top;
+    return slot_width(top);
+  }
   bool idle() const { return !inflight; }
 };
 
@@ -90,7 +98,7 @@ int64_t pool_bytes(const appga_matrix* M, int Kp) {
 void free_pool(Pool* P) {
   if (!P) return;
   if (P->stream) cudaStreamSynchronize(P->stream);
-  if (P->gexec) cudaGraphExecDestroy(P->gexec);
+  for (auto& kv : P->gexec) cudaGraphExecDestroy(kv.second);
   if (P->ev_snap) cudaEventDestroy(P->ev_snap);
   if (P->ev_start) cudaEventDestroy(P->ev_start);
   if (P->ev_out) cudaEventDestroy(P->ev_out);
@@ -104,7 +112,7 @@ void free_pool(Pool* P) {
   cudaFreeHost(P->h_in);
   cudaFreeHost(P->h_out);
   cudaFreeHost(P->h_ids);
-  P->gexec = nullptr;
+  P->gexec.clear();
   P->d_in = P->d_out = nullptr;
   P->h_in = P->h_out = nullptr;
   P->d_ids = P->h_ids = nullptr;
@@ -178,7 +186,7 @@ appga_status create_pool(appga_server* S, int geom, int Kp, Pool** out) {
     return cuda_fail(e, "server pool staging");
   }
   const bool bf16 = S->cfg.a_precision == APPGA_PREC_BF16;
-  make_batch_args(M->A, M->At, bf16 ? M->inv_lambda_bf16 : M->inv_lambda, M->n, P->b, bf16,
+  make_batch_args(M->A, M->At, bf16 ? M->inv_lambda_bf16 : M->inv_lambda, M->n, P->b, Kp, bf16,
                   true, tuned_schedule(M, Kp, bf16), &P->fa, &P->pa);
   cudaStream_t s = P->stream;
   // every slot starts empty; the ring starts at step 1
@@ -199,7 +207,6 @@ appga_status create_pool(appga_server* S, int geom, int Kp, Pool** out) {
     e = cudaMemsetAsync(P->b.y[i], 0, (size_t)M->m * Kp * sizeof(float), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(P->b.g, 0, (size_t)M->m * Kp * sizeof(float), s);
   if (e == cudaSuccess) e = launch_fill_slots(P->b.gamma, M->m, Kp, 0, Kp, 1.f, s);
-  if (e == cudaSuccess) e = capture_batch_graph(P->fa, P->pa, S->cfg.steps_per_launch, s, &P->gexec);
   if (e != cudaSuccess) {
     free_pool(P.get());
     return cuda_fail(e, "server pool setup");
@@ -336,7 +343,9 @@ appga_status admit(appga_server* S, Pool* P, int count) {
   CK(launch_binit_momentum(P->b.slots, Kp, true, s));
   BFwdArgs a = P->fa;
   a.mode = 2;
+  a.width = P->width();
   CK(launch_bforward(a, s));
+  CK(launch_bstencil(a, s));
   // every held slot is live at a step boundary (finished ones were retired)
   P->b.bst_host->remaining = P->used + K;
   CK(cudaMemcpyAsync(&P->b.bst->remaining, &P->b.bst_host->remaining, sizeof(int),
@@ -621,8 +630,15 @@ extern "C" appga_status appga_server_step(appga_server* S, int32_t* pending_out)
       launched = true;
       S->pool_slot_steps += (int64_t)q->b.Kp * S->cfg.steps_per_launch;
       S->live_slot_steps += (int64_t)q->used * S->cfg.steps_per_launch;
+      cudaGraphExec_t& exec = q->gexec[q->width()];
+      if (exec == nullptr) {
+        BFwdArgs fa = q->fa;
+        BPixArgs pa = q->pa;
+        fa.width = pa.width = q->width();
+        CK(capture_batch_graph(fa, pa, S->cfg.steps_per_launch, q->b, q->stream, &exec));
+      }
       CK(cudaEventRecord(q->ev_start, q->stream));
-      CK(cudaGraphLaunch(q->gexec, q->stream));
+      CK(cudaGraphLaunch(exec, q->stream));
       CK(cudaMemcpyAsync(q->b.slots_host, q->b.slots, q->b.Kp * sizeof(SlotState),
                          cudaMemcpyDeviceToHost, q->stream));
       CK(cudaMemcpyAsync(q->b.bst_host, q->b.bst, sizeof(BatchState), cudaMemcpyDeviceToHost,
