@@ -19,12 +19,14 @@ namespace appga {
 
 void free_batch_workspace(BatchWorkspace* bw) {
   if (!bw) return;
-  if (bw->gexec) cudaGraphExecDestroy(bw->gexec);
+  for (auto& kv : bw->gexec) cudaGraphExecDestroy(kv.second);
   for (auto& p : bw->f) cudaFree(p);
   for (auto& p : bw->y) cudaFree(p);
   cudaFree(bw->w);
   cudaFree(bw->gR);
   cudaFree(bw->pfreeze);
+  cudaFree(bw->delta);
+  cudaFree(bw->low);
   cudaFree(bw->g);
   cudaFree(bw->gamma);
   cudaFree(bw->slots);
@@ -48,7 +50,7 @@ void free_batch_workspace(BatchWorkspace* bw) {
 int64_t batch_workspace_bytes(int m, int d, int Kp) {
   const int64_t ngroups = batch_max_blocks() / 64 + 2;
   int64_t b = 0;
-  b += (int64_t)5 * d * Kp * sizeof(float);  // f ring, gR, pfreeze
+  b += (int64_t)7 * d * Kp * sizeof(float);  // f ring, gR, pfreeze, delta, low
   b += (int64_t)5 * m * Kp * sizeof(float);  // y ring, w, g, gamma
   b += (int64_t)Kp * sizeof(SlotState) + sizeof(BatchState);
   b += (2 * batch_max_blocks() + ngroups + 2) * Kp * (int64_t)sizeof(float2);
@@ -68,6 +70,8 @@ cudaError_t alloc_batch_workspace(BatchWorkspace& b, int m, int d, int Kp) {
   if (e == cudaSuccess) e = dalloc(&b.w, mm);
   if (e == cudaSuccess) e = dalloc(&b.gR, dd);
   if (e == cudaSuccess) e = dalloc(&b.pfreeze, dd);
+  if (e == cudaSuccess) e = dalloc(&b.delta, dd);
+  if (e == cudaSuccess) e = dalloc(&b.low, dd);
   if (e == cudaSuccess) e = dalloc(&b.g, mm);
   if (e == cudaSuccess) e = dalloc(&b.gamma, mm);
   if (e == cudaSuccess) e = dalloc(&b.slots, (size_t)Kp);
@@ -113,6 +117,8 @@ void make_batch_args(const DevCSR& A, const DevCSR& At, const float* inv_lambda,
   fa->track = track ? 1 : 0;
   fa->use_bf16 = bf16 ? 1 : 0;
   for (int i = 0; i < 3; ++i) fa->f[i] = b.f[i];
+  fa->delta = b.delta;
+  fa->low = b.low;
   fa->y[0] = b.y[0];
   fa->y[1] = b.y[1];
   fa->w = b.w;
@@ -131,6 +137,8 @@ void make_batch_args(const DevCSR& A, const DevCSR& At, const float* inv_lambda,
   pa->width = stride;
   pa->use_bf16 = bf16 ? 1 : 0;
   for (int i = 0; i < 3; ++i) pa->f[i] = b.f[i];
+  pa->delta = b.delta;
+  pa->low = b.low;
   pa->w = b.w;
   pa->gR = b.gR;
   pa->inv_lambda = inv_lambda;
@@ -236,7 +244,8 @@ namespace {
 appga_status batched_solve(appga_ctx* ctx, appga_matrix* M, int32_t K, const float* g,
                            const float* gamma, const float* f_init, const appga_params* params,
                            float* f_out, appga_stats* stats_host, const BatchSchedule& sch,
-                           void* stream, int min_width = 0, bool volume = false) {
+                           void* stream, int min_width = 0, bool volume = false,
+                           bool want_phi = true) {
   appga_status rc = APPGA_OK;
   // the workspace holds 32, 64 or 128 slots; the run uses as many as the
   // slices need, 8 or 16 among them, as its row stride
@@ -249,32 +258,28 @@ appga_status batched_solve(appga_ctx* ctx, appga_matrix* M, int32_t K, const flo
   const bool track = params->track_objective != 0 || params->rel_obj_tol > 0.0;
   const bool bf16 = params->a_precision == APPGA_PREC_BF16 && M->has_bf16;
 
-  // input checks (g >= 0, gamma > 0, f_init >= 0, all finite) over every slice
+  // slot-minor copies of the sinograms, checked on the way (g >= 0, gamma > 0,
+  // f_init >= 0, all finite); padding slots hold harmless data
   CK(cudaMemsetAsync(b.flag, 0, sizeof(int), s));
-  CK(launch_validate_inputs(g, gamma, K * m, f_init, K * d, b.flag, s));
-  CK(cudaMemcpyAsync(b.flag_host, b.flag, sizeof(int), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
-  if (*b.flag_host)
-    return fail(APPGA_EDOMAIN,
-                "inputs must satisfy: g finite and >= 0, gamma finite and > 0, f finite and >= 0");
-
-  // slot-minor copies of the sinograms; padding slots hold harmless data
-  CK(launch_to_slot_minor(g, K, m, b.g, Kp, 0, nullptr, s));
-  CK(launch_to_slot_minor(gamma, K, m, b.gamma, Kp, 0, nullptr, s));
-  CK(launch_fill_slots(b.g, m, Kp, K, Kp, 0.f, s));
-  CK(launch_fill_slots(b.gamma, m, Kp, K, Kp, 1.f, s));
+  CK(launch_to_slot_minor(g, K, m, b.g, Kp, 0, nullptr, s, 0.f, false, b.flag));
+  CK(launch_to_slot_minor(gamma, K, m, b.gamma, Kp, 0, nullptr, s, 1.f, true, b.flag));
 
   // f^0 = f^1 = f_init (or the per-slice initial image) in the ring slots of step G0
   const int G0 = 1;
   float* cur = b.f[G0 % 3];
   if (f_init) {
-    CK(launch_to_slot_minor(f_init, K, d, cur, Kp, 0, nullptr, s));
+    CK(launch_to_slot_minor(f_init, K, d, cur, Kp, 0, nullptr, s, 0.f, false, b.flag));
+    if (volume)
+      CK(cudaMemcpyAsync(b.f[(G0 + 2) % 3], cur, (size_t)d * Kp * sizeof(float),
+                         cudaMemcpyDeviceToDevice, s));
+    CK(cudaMemsetAsync(b.delta, 0, (size_t)d * Kp * sizeof(float), s));
+    CK(cudaMemsetAsync(b.low, 0, (size_t)d * Kp * sizeof(float), s));
   } else {
-    CK(launch_binit_image(g, gamma, m, n, M->na, M->npfov, K, Kp, 0, nullptr, cur, s));
+    CK(launch_binit_image(g, gamma, m, n, M->na, M->npfov, K, Kp, 0, nullptr, b.partial, cur,
+                          volume ? b.f[(G0 + 2) % 3] : nullptr, b.delta, b.low, s));
   }
-  CK(launch_fill_slots(cur, d, Kp, K, Kp, 0.f, s));
-  CK(cudaMemcpyAsync(b.f[(G0 + 2) % 3], cur, (size_t)d * Kp * sizeof(float),
-                     cudaMemcpyDeviceToDevice, s));
+  CK(cudaMemcpyAsync(b.flag_host, b.flag, sizeof(int), cudaMemcpyDeviceToHost, s));
+  CK(cudaEventRecord(b.ev_join, s));
 
   for (int i = 0; i < Kp; ++i) b.slots_host[i] = slot_from_params(params, 1, i < K);
   CK(cudaMemcpyAsync(b.slots, b.slots_host, Kp * sizeof(SlotState), cudaMemcpyHostToDevice, s));
@@ -334,6 +339,15 @@ appga_status batched_solve(appga_ctx* ctx, appga_matrix* M, int32_t K, const flo
     CK(launch_slices_to_slots(vb.va.gR, b.gR, d, Kp, K, b.bst, s));
   }
 
+  // the verdict on the inputs, while the first forward phase runs; nothing has
+  // been written to the caller's buffers
+  CK(cudaEventSynchronize(b.ev_join));
+  if (*b.flag_host) {
+    CK(cudaStreamSynchronize(s));
+    return fail(APPGA_EDOMAIN,
+                "inputs must satisfy: g finite and >= 0, gamma finite and > 0, f finite and >= 0");
+  }
+
   if (params->max_iters > 0) {
     const int S = params->graph_iters > 0 ? params->graph_iters : kBatchGraphIters;
     char key[256];
@@ -341,24 +355,32 @@ appga_status batched_solve(appga_ctx* ctx, appga_matrix* M, int32_t K, const flo
     std::snprintf(key, sizeof key, "%d|%d|%d|%d|%d|%d|%d|%d|%d|%d|%d", Kp, (int)track, (int)bf16,
                   S, sch.spmv_per_sm, sch.stencil_per_sm, sch.pixel_per_sm, sch.gather_rows_fw,
                   sch.gather_rows_px, (int)volume, volume ? K : 0);
-    if (b.gexec == nullptr || b.gkey != key) {
-      if (b.gexec) {
-        cudaGraphExecDestroy(b.gexec);
-        b.gexec = nullptr;
-      }
-      const cudaError_t e =
-          capture_batch_graph(fa, pa, S, b, s, &b.gexec, volume ? &vb : nullptr);
-      if (e != cudaSuccess) return cuda_fail(e, "batched graph capture");
+    if (b.gkey != key) {
+      for (auto& kv : b.gexec) cudaGraphExecDestroy(kv.second);
+      b.gexec.clear();
       b.gkey = key;
     }
-    const int reps = (params->max_iters + S - 1) / S;
+    // exactly max_iters maps: replays of S, then of the remainder's binary digits
+    const std::vector<int> plan = replay_plan(params->max_iters, S);
+    std::vector<cudaGraphExec_t> execs;
+    for (const int maps : plan) {
+      auto it = b.gexec.find(maps);
+      if (it == b.gexec.end()) {
+        cudaGraphExec_t x = nullptr;
+        const cudaError_t e = capture_batch_graph(fa, pa, maps, b, s, &x, volume ? &vb : nullptr);
+        if (e != cudaSuccess) return cuda_fail(e, "batched graph capture");
+        it = b.gexec.emplace(maps, x).first;
+      }
+      execs.push_back(it->second);
+    }
+    const int reps = (int)execs.size();
     if (params->rel_obj_tol > 0.0) {
       cudaEvent_t ev[2];
       CK(cudaEventCreateWithFlags(&ev[0], cudaEventDisableTiming));
       CK(cudaEventCreateWithFlags(&ev[1], cudaEventDisableTiming));
       appga_status prc = APPGA_OK;
       for (int r = 0; r < reps; ++r) {
-        cudaError_t e = cudaGraphLaunch(b.gexec, s);
+        cudaError_t e = cudaGraphLaunch(execs[r], s);
         if (e == cudaSuccess)
           e = cudaMemcpyAsync(&b.bst_host->remaining, &b.bst->remaining, sizeof(int),
                               cudaMemcpyDeviceToHost, s);
@@ -380,7 +402,7 @@ appga_status batched_solve(appga_ctx* ctx, appga_matrix* M, int32_t K, const flo
       cudaEventDestroy(ev[1]);
       if (prc != APPGA_OK) return prc;
     } else {
-      for (int r = 0; r < reps; ++r) CK(cudaGraphLaunch(b.gexec, s));
+      for (cudaGraphExec_t x : execs) CK(cudaGraphLaunch(x, s));
     }
   }
   // a slot stopped by the test in the last pixel phase has its result one
@@ -388,20 +410,31 @@ appga_status batched_solve(appga_ctx* ctx, appga_matrix* M, int32_t K, const flo
   CK(launch_resolve_rollback(fa, s));
   CK(cudaMemcpyAsync(b.bst_host, b.bst, sizeof(BatchState), cudaMemcpyDeviceToHost, s));
   CK(cudaMemcpyAsync(b.slots_host, b.slots, Kp * sizeof(SlotState), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
-  const int Gf = b.bst_host->gstep;
-  CK(launch_from_slot_minor(b.f[Gf % 3], K, d, Kp, 0, nullptr, f_out, s));
-  if (track) {
-    // the objective terms of every result image, in the arithmetic of
-    // appga_objective, with one host round trip for all of them (2-D: data
-    // term and regulariser per slice; volume: the data terms, the 3-D
-    // regulariser follows with the statistics)
-    if ((rc = objective_terms(M, K, f_out, g, gamma, params, !volume, b.vscal, s)) != APPGA_OK)
-      return rc;
-    CK(cudaMemcpyAsync(b.vscal_host, b.vscal, (size_t)2 * K * sizeof(double),
+  CK(launch_from_slot_minor(fa, K, 0, nullptr, f_out, s));
+  if (track && want_phi) {
+    // the objective terms of every result image, projections in double-float
+    // (2-D: data term and regulariser per slice; volume: the data terms and
+    // the 3-D regulariser of the volume)
+    CK(launch_bobjective(fa, K, b.vscal, s));
+    if (volume) {
+      Vol3Args va{};
+      va.n = n;
+      va.nz = K;
+      va.f[0] = f_out;
+      va.lam1 = (float)params->lambda1;
+      va.lam2 = (float)params->lambda2;
+      va.eps = (float)params->eps;
+      va.want_reg = 1;
+      va.pstride = K;
+      va.gR = b.gR;  // scratch: the workspace holds d * Kp >= d * K floats
+      va.partial = b.fpartial;
+      CK(launch_stencil3d(va, s));
+      CK(launch_sum_pairs(b.fpartial, stencil3d_grid(n, K), K, K, b.vscal + 2 * K, s));
+    }
+    CK(cudaMemcpyAsync(b.vscal_host, b.vscal, (size_t)(2 * K + 1) * sizeof(double),
                        cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
   }
+  CK(cudaStreamSynchronize(s));
   rc = APPGA_OK;
   if (b.bst_host->flags & APPGA_FLAG_NONFINITE) rc = fail(APPGA_ENUMERIC, "a non-finite value appeared");
   if (stats_host) {
@@ -443,7 +476,8 @@ appga_status batched_run(appga_ctx* ctx, appga_matrix* M, int32_t K, const float
                          float* f_out, appga_stats* stats_host, const BatchSchedule& sch,
                          void* stream) {
   if (sch.chunk <= 0 || sch.chunk >= K)
-    return batched_solve(ctx, M, K, g, gamma, f_init, params, f_out, stats_host, sch, stream);
+    return batched_solve(ctx, M, K, g, gamma, f_init, params, f_out, stats_host, sch, stream, 0,
+                         false, stats_host != nullptr);
   // every sub-batch (the last one too) runs at the chunk's width, so the
   // workspace and its captured graph are reused
   for (int c0 = 0; c0 < K; c0 += sch.chunk) {
@@ -451,7 +485,8 @@ appga_status batched_run(appga_ctx* ctx, appga_matrix* M, int32_t K, const float
     appga_status rc = batched_solve(
         ctx, M, kc, g + (size_t)c0 * M->m, gamma + (size_t)c0 * M->m,
         f_init ? f_init + (size_t)c0 * M->d : nullptr, params, f_out + (size_t)c0 * M->d,
-        stats_host ? stats_host + c0 : nullptr, sch, stream, sch.chunk);
+        stats_host ? stats_host + c0 : nullptr, sch, stream, sch.chunk, false,
+        stats_host != nullptr);
     if (rc != APPGA_OK) return rc;
   }
   return APPGA_OK;
@@ -468,13 +503,13 @@ appga_status check_slot_width(const appga_matrix* M, int Kp) {
 
 appga_status volume_solve(appga_ctx* ctx, appga_matrix* M, int32_t K, const float* g,
                           const float* gamma, const float* f_init, const appga_params* params,
-                          float* f_out, void* stream) {
+                          float* f_out, bool want_phi, void* stream) {
   const bool bf16 = params->a_precision == APPGA_PREC_BF16 && M->has_bf16;
   const int Kp = padded_width(K);
   const appga_status rc = check_slot_width(M, Kp);
   if (rc != APPGA_OK) return rc;
   return batched_solve(ctx, M, K, g, gamma, f_init, params, f_out, nullptr,
-                       tuned_schedule(M, Kp, bf16), stream, 0, true);
+                       tuned_schedule(M, Kp, bf16), stream, 0, true, want_phi);
 }
 
 }  // namespace appga

@@ -27,6 +27,7 @@ struct SlotState {
   float theta_hi, theta_lo;  // theta_k as a double-float pair
   float lambda1, lambda2, eps, beta;
   double theta, t_cur, phi_cur, phi_prev;
+  double theta_next, t_next;  // momentum of index k + 1 (set by the forward phase of k)
   double omega, a, b, rel_tol;
   unsigned long long guard_hits;
 };
@@ -46,7 +47,8 @@ struct BFwdArgs {
   int32_t Kp;     // row stride of the slot-minor arrays
   int32_t width;  // slots worked on: 8, 16, 32, 64 or 128, every live slot below it
   int32_t mode;   // 0: solver step; 1: first forward phase of a run (f^{k-1} = f^k);
-                  // 2: first forward phase of the fresh slots only (admission)
+                  // 2: first forward phase of the fresh slots only (admission);
+                  // 3: objective of every active slot's result
   int32_t track;
   int32_t use_bf16;
   int32_t n_spmv_blocks;  // virtual blocks of the projection, set by the launcher
@@ -55,6 +57,8 @@ struct BFwdArgs {
   int32_t no_stencil;     // volume mode: the 3-D stencil takes the 2-D one's place
   int32_t gather_rows;    // image rows a lane gathers per step: 8 (0: default) or 4; tuned
   float* f[3];
+  const float* delta;  // f^k - f^{k-1}, and what rounding f^k to FP32 left over
+  const float* low;
   float* y[2];
   float* w;
   const float* g;
@@ -75,6 +79,8 @@ struct BPixArgs {
   int32_t blocks_per_sm;  // 0: default; tuned by the autotuner
   int32_t gather_rows;    // weight rows a lane gathers per step: 8 (0: default) or 4; tuned
   float* f[3];
+  float* delta;  // as BFwdArgs, of the current step, replaced by the next step's
+  float* low;
   const float* w;
   const float* gR;
   const float* inv_lambda;
@@ -134,6 +140,10 @@ cudaError_t launch_bforward(const BFwdArgs& a, cudaStream_t s);
 // The forward phase's 2-D stencil, on the same arguments; independent of
 // launch_bforward (they may overlap).
 cudaError_t launch_bstencil(const BFwdArgs& a, cudaStream_t s);
+// Objective of the results in the current ring entry, slots 0 .. K - 1: the
+// data term of slot s into out[2 s], its regulariser into out[2 s + 1] (0 with
+// a.no_stencil).  Uses the objective rows (fpartial) and gR as scratch.
+cudaError_t launch_bobjective(const BFwdArgs& a, int K, double* out, cudaStream_t s);
 // The batched projectors' inner loop alone over M (rows reduced against the
 // Kp-wide rows of x, [cols][Kp]; no epilogue) with blocks_per_sm (1..16)
 // blocks per SM; sink: at least (SMs x 16) floats, written only in a case
@@ -151,15 +161,18 @@ cudaError_t launch_bpixel(const BPixArgs& a, cudaStream_t s);
 // Slot lists: where `ids` is given, slice k goes to slot ids[k] (a device
 // array of K ints); otherwise to slot s0 + k.
 cudaError_t launch_binit_momentum(SlotState* slots, int Kp, bool only_fresh, cudaStream_t s);
+// (fill: value of the padding slots when ids == NULL; flag, may be NULL: set
+// to 1 if a value is not finite, negative or, with positive, zero)
 cudaError_t launch_to_slot_minor(const float* in, int K, int len, float* out, int Kp, int s0,
-                                 const int* ids, cudaStream_t s);
-cudaError_t launch_from_slot_minor(const float* in, int K, int len, int Kp, int s0,
-                                   const int* ids, float* out, cudaStream_t s);
-cudaError_t launch_copy_slots(const float* src, float* dst, int len, int Kp, const int* ids,
-                              int K, cudaStream_t s);
+                                 const int* ids, cudaStream_t s, float fill = 0.f,
+                                 bool positive = false, int* flag = nullptr);
+// images (a.n^2 pixels) of K slots of the current ring entry, slice-major
+cudaError_t launch_from_slot_minor(const BFwdArgs& a, int K, int s0, const int* ids, float* out,
+                                   cudaStream_t s);
 cudaError_t launch_fill_slots(float* out, int len, int Kp, int s0, int s1, float v, cudaStream_t s);
 cudaError_t launch_binit_image(const float* g, const float* gamma, int m, int n, int n_angles,
                                long long npfov, int K, int Kp, int s0, const int* ids,
-                               float* f_out, cudaStream_t s);
+                               float2* scratch, float* f_cur, float* f_prev, float* delta,
+                               float* low, cudaStream_t s);
 
 }  // namespace appga

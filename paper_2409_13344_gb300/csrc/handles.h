@@ -85,6 +85,8 @@ struct BatchWorkspace {
   float* w = nullptr;                         // [m][Kp]
   float* gR = nullptr;                        // [d][Kp]
   float* pfreeze = nullptr;                   // [d][Kp]
+  float* delta = nullptr;                     // [d][Kp]: f^k - f^{k-1}
+  float* low = nullptr;                       // [d][Kp]: rounding remainder of f^k
   float* g = nullptr;                         // [m][Kp]
   float* gamma = nullptr;                     // [m][Kp]
   SlotState* slots = nullptr;                 // [Kp]
@@ -99,7 +101,9 @@ struct BatchWorkspace {
   float* gsm = nullptr;                         // volume mode: slice-major 3-D gradient
   double* vscal = nullptr;       // volume objective terms: [Kp] data terms, regulariser
   double* vscal_host = nullptr;  // pinned mirror
-  cudaGraphExec_t gexec = nullptr;
+  // replays of n maps (the replay length and powers of two below it) for the
+  // settings in gkey
+  std::map<int, cudaGraphExec_t> gexec;
   std::string gkey;
   // the stencil's branch of the captured step (a second stream forked from
   // and joined to the solver's stream by two events)
@@ -138,10 +142,12 @@ cudaError_t capture_batch_graph(const BFwdArgs& fa, const BPixArgs& pa, int S,
                                 const VolumeSteps* vb = nullptr);
 // APPGA on a volume of K <= 128 slices sharing the matrix (the batched solver
 // in volume mode): device buffers as in appga_reconstruct_batched; on return
-// the workspace's pinned slot and batch states hold the final states.
+// the workspace's pinned slot and batch states hold the final states and, for
+// a tracked run with want_phi, vscal_host the terms of the result's objective
+// (data terms in entries 2 z, the volume's regulariser in entry 2 K).
 appga_status volume_solve(appga_ctx* ctx, appga_matrix* M, int32_t K, const float* g,
                           const float* gamma, const float* f_init, const appga_params* params,
-                          float* f_out, void* stream);
+                          float* f_out, bool want_phi, void* stream);
 // The batched kernels stage the offset col * Kp of every gathered slot-minor
 // row in 32 bits: APPGA_OK when max(m, d) * Kp stays below 2^31, else
 // APPGA_EINVAL (with the library's error message set).
@@ -221,13 +227,9 @@ bool loop_gathers_copy();
 // Fills the loop's gather copy of f^k (tiled or folded pairs), if it has one.
 cudaError_t loop_gather_copy(const appga_matrix* M, const float* f, cudaStream_t s);
 
-// The objective terms of K slices (f [K][d], g and gamma [K][m]) enqueued on
-// s without a host round trip, in the arithmetic of appga_objective: slice
-// i's data term into dev_out[2i] (double-float projection) and, with_reg, its
-// SHOITV regulariser into dev_out[2i + 1].
-appga_status objective_terms(appga_matrix* M, int K, const float* f, const float* g,
-                             const float* gamma, const appga_params* p, bool with_reg,
-                             double* dev_out, cudaStream_t s);
+// Graph replays of a run of `total` maps: replays of S, then of the remainder's
+// binary digits.
+std::vector<int> replay_plan(int total, int S);
 
 // Orders ctx->stream after the caller's stream / the caller's after ctx->stream.
 appga_status enter_stream(appga_ctx* ctx, void* stream);

@@ -251,6 +251,19 @@ struct RowDeal {
 __device__ double bgn_t(int k, double a, double b, double omega) {
   return a * pow((double)k, omega) + b;
 }
+// theta_{k+1} (and Nesterov's t_{k+1}) of a slot at index k.
+__device__ void next_momentum(SlotState& s) {
+  double th = 0.0, t = s.t_cur;
+  if (s.momentum == APPGA_MOMENTUM_GN) {
+    th = (bgn_t(s.k, s.a, s.b, s.omega) - 1.0) / bgn_t(s.k + 1, s.a, s.b, s.omega);
+  } else if (s.momentum == APPGA_MOMENTUM_NESTEROV) {
+    const double tn = 0.5 * (1.0 + sqrt(1.0 + 4.0 * t * t));
+    th = (t - 1.0) / tn;
+    t = tn;
+  }
+  s.theta_next = th;
+  s.t_next = t;
+}
 __device__ void bset_theta(SlotState& s, double theta) {
   s.theta = theta;
   const float h = (float)theta;
@@ -259,6 +272,31 @@ __device__ void bset_theta(SlotState& s, double theta) {
 }
 
 // -------------------------------------------------------------- k_bforward
+
+// One row of per-slot sums per virtual block (its teams in order), in the
+// columns of the live slots.
+template <int W, class Live>
+__device__ __forceinline__ void store_row_sums(const BFwdArgs& a, const float (&dh)[Team<W>::E],
+                                               const float (&dl)[Team<W>::E], float (*sum_hi)[W],
+                                               float (*sum_lo)[W], const Live& live) {
+  using T = Team<W>;
+  const int tid = threadIdx.x, lane = tid & 31, sl0 = owned_slot<W>(lane);
+  const int team = (tid >> 5) * T::RW + lane / T::LANES;
+#pragma unroll
+  for (int t = 0; t < T::E; ++t) {
+    sum_hi[team][sl0 + t] = dh[t];
+    sum_lo[team][sl0 + t] = dl[t];
+  }
+  __syncthreads();
+  for (int q = tid; q < T::RW * W; q += P_THREADS) {
+    const int s = q % W, vb = blockIdx.x * T::RW + q / W;
+    if (vb >= a.n_spmv_blocks || !live(a.slots[s])) continue;
+    float h = 0.f, l = 0.f;
+    for (int w = 0; w < P_WARPS; ++w)
+      acc_add(h, l, sum_hi[q / W * P_WARPS + w][s], sum_lo[q / W * P_WARPS + w][s]);
+    a.fpartial[(size_t)vb * a.Kp + s] = make_float2(h, l);
+  }
+}
 
 // W: slots the launch works on (every live slot is below it); a.Kp: the row
 // stride of the slot-minor arrays, at least W.
@@ -303,6 +341,13 @@ __global__ void __launch_bounds__(P_THREADS, 2) k_bforward(BFwdArgs a) {
     dh[t] = 0.f;
     dl[t] = 0.f;
     hits[t] = 0;
+  }
+  // the momentum of the next index, so that the pixel phase's last block only
+  // copies it: its FP64 powers take about 5 us, here beside the projections
+  // of the block's other warps
+  if (blockIdx.x == 0 && tid >= P_THREADS - W) {
+    SlotState& sl = a.slots[tid - (P_THREADS - W)];
+    if (live(sl)) next_momentum(sl);
   }
   const uint64_t pol = evict_first_policy();
   const RowDeal<W> deal(a.A.rows, a.n_spmv_blocks);
@@ -349,24 +394,8 @@ __global__ void __launch_bounds__(P_THREADS, 2) k_bforward(BFwdArgs a) {
   for (int t = 0; t < E; ++t)
     if (hits[t]) atomicAdd(&a.slots[sl0 + t].guard_hits, (unsigned long long)hits[t]);
   if (!want) return;
-  // one row of per-slot sums per virtual block (its teams in order), left for
-  // the pixel phase of this step; an admission pass writes only the fresh
-  // slots' columns
-  const int team = (tid >> 5) * T::RW + lane / T::LANES;
-#pragma unroll
-  for (int t = 0; t < E; ++t) {
-    dsum_hi[team][sl0 + t] = dh[t];
-    dsum_lo[team][sl0 + t] = dl[t];
-  }
-  __syncthreads();
-  for (int q = tid; q < T::RW * W; q += P_THREADS) {
-    const int s = q % W, vb = blockIdx.x * T::RW + q / W;
-    if (vb >= a.n_spmv_blocks || !live(a.slots[s])) continue;
-    float h = 0.f, l = 0.f;
-    for (int w = 0; w < P_WARPS; ++w)
-      acc_add(h, l, dsum_hi[q / W * P_WARPS + w][s], dsum_lo[q / W * P_WARPS + w][s]);
-    a.fpartial[(size_t)vb * Kp + s] = make_float2(h, l);
-  }
+  // an admission pass writes only the fresh slots' columns
+  store_row_sums<W>(a, dh, dl, dsum_hi, dsum_lo, live);
 }
 
 // -------------------------------------------------------------- k_bstencil
@@ -399,8 +428,8 @@ __device__ __forceinline__ void bfields(const float (&x)[3][3], const BEdges& e,
 // row of sums after the projector's.  Runs beside k_bforward (both read only
 // the iterates).
 __global__ void __launch_bounds__(B_THREADS, 4) k_bstencil(BFwdArgs a) {
-  // double-buffered rows: f~, f^k and the fields 0, 2, 3, 5
-  __shared__ float sT[2][BST_C + 2][BST_S], sK[2][BST_C + 2][BST_S];
+  // double-buffered rows: f^k, f~ - f^k and the fields 0, 2, 3, 5
+  __shared__ float sK[2][BST_C + 2][BST_S], sD[2][BST_C + 2][BST_S];
   __shared__ float sV[2][4][BST_C + 2][BST_S];
   __shared__ float red_hi[B_THREADS / 32][BST_S], red_lo[B_THREADS / 32][BST_S];
   BatchState* bs = a.bst;
@@ -408,15 +437,15 @@ __global__ void __launch_bounds__(B_THREADS, 4) k_bstencil(BFwdArgs a) {
   const int tid = threadIdx.x, q = tid % BST_S, col = tid / BST_S;
   const int slot = blockIdx.y * BST_S + q, Kp = a.Kp, n = a.n, G = bs->gstep;
   const SlotState& sl = a.slots[slot];
-  const bool part = a.mode == 2 ? sl.fresh : (sl.active && !sl.done);
+  const bool part = a.mode == 3 ? sl.active
+                                : a.mode == 2 ? sl.fresh : (sl.active && !sl.done);
   if (!__syncthreads_or(part)) return;  // no live slot in the chunk
   const bool want = a.track != 0;
   const float* fk = a.f[G % 3] + slot;
-  const float* fkm = a.f[(G + 2) % 3] + slot;
+  const float *delta = a.delta + slot, *low = a.low + slot;
   float* gR = a.gR + slot;
-  // a first forward phase has f^{k-1} = f^k
-  const float th = a.mode != 0 ? 0.f : sl.theta_hi;
-  const float lam1 = sl.lambda1, lam2 = sl.lambda2, eps = sl.eps;
+  const float th = sl.theta_hi;
+  const float lam1 = sl.lambda1, lam2 = sl.lambda2, eps = sl.eps, eps2 = eps * eps;
   const int ntx = (n + BST_OUT - 1) / BST_OUT, nty = (n + BST_R - 1) / BST_R;
   float reg_h = 0.f, reg_l = 0.f;
   for (int tile = blockIdx.x; tile < ntx * nty; tile += gridDim.x) {
@@ -424,28 +453,31 @@ __global__ void __launch_bounds__(B_THREADS, 4) k_bstencil(BFwdArgs a) {
     const int c = (tile % ntx) * BST_OUT - 2 + col;
     const bool c_in = c >= 0 && c < n;
     const bool out_col = part && c_in && col >= 2 && col < BST_C - 2;
-    float t[3][3] = {}, k[3][3] = {};  // f~ and f^k at rows s - 2 .. s, columns c - 1 .. c + 1
+    // f^k and f~ - f^k = theta (f^k - f^{k-1}) + low at rows s - 2 .. s, columns
+    // c - 1 .. c + 1
+    float k[3][3] = {}, d[3][3] = {};
     // fields of the own column (and the neighbours' where the adjoint reads
     // them): v of row s - 1, w of row s - 2, x of row s - 3
     float v[6] = {}, w0 = 0.f, w0r = 0.f, w1 = 0.f, w2 = 0.f, w2l = 0.f, w2r = 0.f, w3 = 0.f,
           w3r = 0.f, w4 = 0.f, w5 = 0.f, w5l = 0.f;
     float x3 = 0.f, x3r = 0.f, x4 = 0.f, x0 = 0.f, x0r = 0.f, x1 = 0.f, x2 = 0.f, x2l = 0.f,
           x2r = 0.f, x5 = 0.f, x5l = 0.f, y3 = 0.f, y3r = 0.f, y4 = 0.f;
-    float nk = 0.f, nm = 0.f;  // the next row, in flight
+    float nk = 0.f, nd = 0.f, nl = 0.f;  // the next row, in flight
     auto fetch = [&](int r) {
-      nk = nm = 0.f;
+      nk = nd = nl = 0.f;
       if (c_in && r >= 0 && r < n) {
         const size_t o = (size_t)(r * n + c) * Kp;
         nk = fk[o];
-        nm = fkm[o];
+        nd = delta[o];
+        nl = low[o];
       }
     };
     fetch(r0 - 2);
     for (int s = r0 - 2; s <= r1 + 2; ++s) {
       const int b = s & 1;
-      const float vk = nk, vt = fmaf(th, nk - nm, nk);
-      sT[b][col + 1][q] = vt;
-      if (want) sK[b][col + 1][q] = vk;
+      const float vk = nk, vd = fmaf(th, nd, nl);
+      sK[b][col + 1][q] = vk;
+      sD[b][col + 1][q] = vd;
       // the fields of row s - 2, computed in the last step
       sV[b][0][col + 1][q] = v[0];
       sV[b][1][col + 1][q] = v[2];
@@ -465,36 +497,38 @@ __global__ void __launch_bounds__(B_THREADS, 4) k_bstencil(BFwdArgs a) {
       w5l = sV[b][3][col][q];
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
-        t[0][j] = t[1][j];
-        t[1][j] = t[2][j];
         k[0][j] = k[1][j];
         k[1][j] = k[2][j];
+        d[0][j] = d[1][j];
+        d[1][j] = d[2][j];
       }
-      t[2][0] = sT[b][col][q];
-      t[2][1] = vt;
-      t[2][2] = sT[b][col + 2][q];
-      if (want) {
-        k[2][0] = sK[b][col][q];
-        k[2][1] = vk;
-        k[2][2] = sK[b][col + 2][q];
-      }
+      k[2][0] = sK[b][col][q];
+      k[2][1] = vk;
+      k[2][2] = sK[b][col + 2][q];
+      d[2][0] = sD[b][col][q];
+      d[2][1] = vd;
+      d[2][2] = sD[b][col + 2][q];
       // grad phi~ at row i = s - 1
       const int i = s - 1;
       const BEdges e = {i >= 1, i <= n - 2, c >= 1, c <= n - 2};
 #pragma unroll
       for (int f = 0; f < 6; ++f) v[f] = 0.f;
       if (c_in && i >= 0 && i < n) {
-        bfields(t, e, v);
+        // B f~ = B f^k + B (f~ - f^k): f~ itself is never rounded to FP32, and
+        // B f^k also serves the regulariser
+        float u[6];
+        bfields(k, e, u);
+        bfields(d, e, v);
+#pragma unroll
+        for (int f = 0; f < 6; ++f) v[f] += u[f];
         const float n1 = v[0] * v[0] + v[1] * v[1];
         const float n2 = v[2] * v[2] + v[3] * v[3] + v[4] * v[4] + v[5] * v[5];
-        const float s1 = lam1 / fmaxf(sqrtf(n1), eps), s2 = lam2 / fmaxf(sqrtf(n2), eps);
+        const float s1 = lam1 * inv_norm(n1, eps, eps2), s2 = lam2 * inv_norm(n2, eps, eps2);
         v[0] *= s1;
         v[1] *= s1;
 #pragma unroll
         for (int f = 2; f < 6; ++f) v[f] *= s2;
         if (want && out_col && i >= r0 && i < r1) {
-          float u[6];
-          bfields(k, e, u);
           const float m1 = u[0] * u[0] + u[1] * u[1];
           const float m2 = u[2] * u[2] + u[3] * u[3] + u[4] * u[4] + u[5] * u[5];
           acc_add(reg_h, reg_l, lam1 * s_eps_f(m1, eps) + lam2 * s_eps_f(m2, eps), 0.f);
@@ -533,6 +567,104 @@ __global__ void __launch_bounds__(B_THREADS, 4) k_bstencil(BFwdArgs a) {
     float h = 0.f, l = 0.f;
     for (int w = 0; w < B_THREADS / 32; ++w) acc_add(h, l, red_hi[w][q], red_lo[w][q]);
     a.fpartial[(size_t)(a.n_spmv_blocks + blockIdx.x) * Kp + slot] = make_float2(h, l);
+  }
+}
+
+// ------------------------------------------------------------- k_bobjective
+
+// Data terms sum y - g ln(y + gamma) of the results of every active slot, with
+// y = A f accumulated in double-float as the single-slice objective does (one
+// pass over A for all slots: 64 slots of 256 x 256 took 64 projections of 46
+// us one by one).  The rows of sums lie as the forward phase's.
+template <int W, bool BF16>
+__global__ void __launch_bounds__(P_THREADS, 2) k_bobjective(BFwdArgs a) {
+  using T = Team<W>;
+  constexpr int E = T::E, Q = T::Q, F = Q / 4;
+  __shared__ float dsum_hi[P_WARPS * T::RW][W], dsum_lo[P_WARPS * T::RW][W];
+  const int lane = threadIdx.x & 31, g = lane % T::LANES / T::L;
+  const int sl0 = owned_slot<W>(lane), Kp = a.Kp;
+  const float* xl = a.f[a.bst->gstep % 3] + gathered_slot<W>(lane);
+  const uint64_t pol = evict_first_policy();
+  const RowDeal<W> deal(a.A.rows, a.n_spmv_blocks);
+  float dh[E], dl[E];
+#pragma unroll
+  for (int t = 0; t < E; ++t) dh[t] = dl[t] = 0.f;
+  for (int i = 0; i < deal.rounds; ++i) {
+    const int row = deal.row(a.A, i);
+    float hi[Q], lo[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) hi[q] = lo[q] = 0.f;
+    if (row >= 0) {
+      const int e = __ldg(a.A.row_ptr + row + 1);
+      for (int p = __ldg(a.A.row_ptr + row) + 4 * g; p < e; p += 4 * T::G) {
+        const int4 c = ld_stream_i4(a.A.col + p, pol);
+        const float4 v = ld_vals<BF16>(a.A, p, pol);
+        const int cc[4] = {c.x, c.y, c.z, c.w};
+        const float vv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int k = 0; k < F; ++k) {
+            const float4 x = *(reinterpret_cast<const float4*>(xl + (unsigned)(cc[u] * Kp)) +
+                               k * (T::GSTRIDE / 4));
+            acc_fma(hi[4 * k], lo[4 * k], vv[u], x.x);
+            acc_fma(hi[4 * k + 1], lo[4 * k + 1], vv[u], x.y);
+            acc_fma(hi[4 * k + 2], lo[4 * k + 2], vv[u], x.z);
+            acc_fma(hi[4 * k + 3], lo[4 * k + 3], vv[u], x.w);
+          }
+      }
+    }
+    __syncwarp();
+    // the groups' sums, halving the slots a lane keeps at each exchange
+    constexpr int H1 = Q / 2;
+    const bool up1 = g & 1;
+    float qh[H1], ql[H1];
+#pragma unroll
+    for (int t = 0; t < H1; ++t) {
+      qh[t] = up1 ? hi[H1 + t] : hi[t];
+      ql[t] = up1 ? lo[H1 + t] : lo[t];
+      acc_add(qh[t], ql[t], __shfl_xor_sync(0xffffffffu, up1 ? hi[t] : hi[H1 + t], T::L),
+              __shfl_xor_sync(0xffffffffu, up1 ? lo[t] : lo[H1 + t], T::L));
+    }
+    if constexpr (T::G == 4) {
+      const bool up2 = g >> 1;
+#pragma unroll
+      for (int t = 0; t < E; ++t) {
+        const float sh = __shfl_xor_sync(0xffffffffu, up2 ? qh[t] : qh[E + t], 2 * T::L);
+        const float sl = __shfl_xor_sync(0xffffffffu, up2 ? ql[t] : ql[E + t], 2 * T::L);
+        qh[t] = up2 ? qh[E + t] : qh[t];
+        ql[t] = up2 ? ql[E + t] : ql[t];
+        acc_add(qh[t], ql[t], sh, sl);
+      }
+    }
+    if (row < 0) continue;
+    float gg[E], gm[E];
+    vload<E>(a.g + (size_t)row * Kp + sl0, gg);
+    vload<E>(a.gamma + (size_t)row * Kp + sl0, gm);
+#pragma unroll
+    for (int t = 0; t < E; ++t) {
+      const df y = quick_renorm(qh[t], ql[t]);
+      const df term = df_add(y, df_neg(df_mul_f(df_log(df_add_f(y, gm[t])), gg[t])));
+      acc_add(dh[t], dl[t], term.hi, term.lo);
+    }
+  }
+  store_row_sums<W>(a, dh, dl, dsum_hi, dsum_lo, [](const SlotState& sl) { return sl.active; });
+}
+
+// out[2 s] = sum over the first n0 rows, out[2 s + 1] over the next n1 rows, of
+// column s (double-float pairs, row stride Kp), in FP64; one block per column.
+__global__ void __launch_bounds__(256) k_sum_columns(const float2* __restrict__ rows, int n0,
+                                                     int n1, int Kp, double* __restrict__ out) {
+  const int s = blockIdx.x;
+  for (int part = 0; part < 2; ++part) {
+    const int r0 = part ? n0 : 0, r1 = part ? n0 + n1 : n0;
+    float h = 0.f, l = 0.f;
+    for (int i = r0 + threadIdx.x; i < r1; i += blockDim.x) {
+      const float2 v = rows[(size_t)i * Kp + s];
+      acc_add(h, l, v.x, v.y);
+    }
+    const df t = block_sum_acc(h, l);
+    if (threadIdx.x == 0) out[2 * s + part] = (double)t.hi + (double)t.lo;
   }
 }
 
@@ -583,6 +715,7 @@ __global__ void __launch_bounds__(P_THREADS, 2) k_bpixel(BPixArgs a) {
   const float* fk = a.f[G % 3];
   const float* fkm = a.f[(G + 2) % 3];
   float* fn = a.f[(G + 1) % 3];
+  bool any_back = false;
   // every slot's Phi(f^k): the forward phase's rows, first because these
   // blocks start first
   if (a.track)
@@ -604,6 +737,7 @@ __global__ void __launch_bounds__(P_THREADS, 2) k_bpixel(BPixArgs a) {
     kk[t] = sl.k;
     frz[t] = sl.freeze_iter;
     back[t] = sl.rollback;
+    any_back = any_back || back[t];
   }
 #pragma unroll
   for (int t = 0; t < T::Q; ++t) {
@@ -619,9 +753,10 @@ __global__ void __launch_bounds__(P_THREADS, 2) k_bpixel(BPixArgs a) {
     team_dot<W, BF16, NZ>(a.At, j, a.w, Kp, lane, gather_live, pol, bp);
     if (j < 0) continue;
     const size_t o = (size_t)j * Kp + sl0;
-    float vk[E], vm[E], gr[E], out[E];
+    float vk[E], vd[E], lo[E], gr[E], out[E];
     vload<E>(fk + o, vk);
-    vload<E>(fkm + o, vm);
+    vload<E>(a.delta + o, vd);
+    vload<E>(a.low + o, lo);
     vload<E>(a.gR + o, gr);
     const float il = __ldg(a.inv_lambda + j);
 #pragma unroll
@@ -629,10 +764,9 @@ __global__ void __launch_bounds__(P_THREADS, 2) k_bpixel(BPixArgs a) {
       if (!live[t]) {
         // finished or empty slot: carry the image (the previous entry when
         // the slot stopped one step back)
-        out[t] = back[t] ? vm[t] : vk[t];
+        out[t] = vk[t];
         continue;
       }
-      const float ft = fmaf(th[t], vk[t] - vm[t], vk[t]);
       float pk = vk[t];
       if (frz[t] >= 0) {
         if (kk[t] == frz[t]) {
@@ -641,11 +775,27 @@ __global__ void __launch_bounds__(P_THREADS, 2) k_bpixel(BPixArgs a) {
           pk = a.pfreeze[o + t];
         }
       }
+      // f^{k+1} = max(f^k + step, 0), step = theta (f^k - f^{k-1}) - p (grad F +
+      // grad R): what rounding f^{k+1} to FP32 leaves over is kept in low, and
+      // the step itself is the next f^k - f^{k-1}
       const float p = beta[t] * pk * il;
-      const float xv = __fmaf_rn(-p, bp[t] + gr[t], ft);
+      const float step = __fmaf_rn(th[t], vd[t], -__fmul_rn(p, bp[t] + gr[t]));
+      const float full = __fadd_rn(vk[t], lo[t]);
+      float xv, rest;
+      two_sum(vk[t], __fadd_rn(lo[t], step), xv, rest);
       if (!isfinite(xv)) bad = 1;
-      out[t] = fmaxf(xv, 0.f);
+      const bool pos = xv > 0.f;
+      out[t] = pos ? xv : 0.f;
+      vd[t] = pos ? step : -full;
+      lo[t] = pos ? rest : 0.f;
     }
+    if (any_back) {
+#pragma unroll
+      for (int t = 0; t < E; ++t)
+        if (back[t]) out[t] = fkm[o + t];
+    }
+    vstore_on<E>(a.delta + o, vd, live);
+    vstore_on<E>(a.low + o, lo, live);
     int on[E];
 #pragma unroll
     for (int t = 0; t < E; ++t) on[t] = 1;
@@ -733,16 +883,8 @@ __global__ void __launch_bounds__(P_THREADS, 2) k_bpixel(BPixArgs a) {
       }
       const int k = sl.k;
       sl.k = k + 1;
-      double th_next = 0.0;
-      if (sl.momentum == APPGA_MOMENTUM_GN) {
-        th_next = (bgn_t(k, sl.a, sl.b, sl.omega) - 1.0) / bgn_t(k + 1, sl.a, sl.b, sl.omega);
-      } else if (sl.momentum == APPGA_MOMENTUM_NESTEROV) {
-        const double t = sl.t_cur;
-        const double tn = 0.5 * (1.0 + sqrt(1.0 + 4.0 * t * t));
-        th_next = (t - 1.0) / tn;
-        sl.t_cur = tn;
-      }
-      bset_theta(sl, th_next);
+      sl.t_cur = sl.t_next;
+      bset_theta(sl, sl.theta_next);
     }
     static_assert(P_THREADS >= MAXK, "one slot per thread");
     const int tot = __syncthreads_count(rem);
@@ -800,25 +942,38 @@ __device__ __forceinline__ int slot_of(const int* ids, int s0, int k) {
 }
 
 // [K][len] slice-major -> [len][Kp] slot-minor: out[i*Kp + slot(s)] = in[s*len + i].
-// Padding slots are written separately.
+// Without a slot list the padding slots K .. Kp - 1 get `fill`.  With flag set
+// the values are checked on the way: finite and at least 0, or (positive)
+// above 0, else *flag becomes 1.
 __global__ void k_to_slot_minor(const float* __restrict__ in, int K, int len, float* __restrict__ out,
-                                int Kp, int s0, const int* __restrict__ ids) {
+                                int Kp, int s0, const int* __restrict__ ids, float fill,
+                                int positive, int* flag) {
   __shared__ float tile[32][33];
   const int i0 = blockIdx.x * 32, k0 = blockIdx.y * 32;
+  int bad = 0;
   for (int r = threadIdx.y; r < 32; r += blockDim.y) {
     const int k = k0 + r, i = i0 + threadIdx.x;
-    tile[r][threadIdx.x] = (k < K && i < len) ? in[(size_t)k * len + i] : 0.f;
+    const bool in_range = k < K && i < len;
+    const float v = in_range ? in[(size_t)k * len + i] : fill;
+    if (in_range && !(isfinite(v) && (positive ? v > 0.f : v >= 0.f))) bad = 1;
+    tile[r][threadIdx.x] = v;
   }
-  __syncthreads();
+  if (__syncthreads_or(bad) && flag != nullptr && threadIdx.x == 0 && threadIdx.y == 0)
+    atomicOr(flag, 1);
+  const int top = ids ? K : Kp - s0;
   for (int r = threadIdx.y; r < 32; r += blockDim.y) {
     const int i = i0 + r, k = k0 + threadIdx.x;
-    if (i < len && k < K) out[(size_t)i * Kp + slot_of(ids, s0, k)] = tile[threadIdx.x][r];
+    if (i < len && k < top) out[(size_t)i * Kp + slot_of(ids, s0, k)] = tile[threadIdx.x][r];
   }
 }
-// out[s*len + i] = in[i*Kp + slot(s)] for s < K.
-__global__ void k_from_slot_minor(const float* __restrict__ in, int K, int len, int Kp, int s0,
+// out[s*len + i] = in[i*Kp + slot(s)] for s < K, in the ring entry of the
+// current global step.
+__global__ void k_from_slot_minor(const float* f0, const float* f1, const float* f2,
+                                  const BatchState* bst, int K, int len, int Kp, int s0,
                                   const int* __restrict__ ids, float* __restrict__ out) {
   __shared__ float tile[32][33];
+  const float* ring[3] = {f0, f1, f2};
+  const float* in = ring[bst->gstep % 3];
   const int i0 = blockIdx.x * 32, k0 = blockIdx.y * 32;
   for (int r = threadIdx.y; r < 32; r += blockDim.y) {
     const int i = i0 + r, k = k0 + threadIdx.x;
@@ -830,15 +985,6 @@ __global__ void k_from_slot_minor(const float* __restrict__ in, int K, int len, 
     if (k < K && i < len) out[(size_t)k * len + i] = tile[threadIdx.x][r];
   }
 }
-// Copies the listed columns of one [len][Kp] array into another.
-__global__ void k_copy_slots(const float* __restrict__ src, float* __restrict__ dst, int len,
-                             int Kp, const int* __restrict__ ids, int K) {
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < (size_t)len * K;
-       t += (size_t)gridDim.x * blockDim.x) {
-    const size_t o = (t / K) * Kp + __ldg(ids + t % K);
-    dst[o] = src[o];
-  }
-}
 // Sets column s of a [len][Kp] array to v for s in [s0, s1).
 __global__ void k_fill_slots(float* out, int len, int Kp, int s0, int s1, float v) {
   const int w = s1 - s0;
@@ -848,29 +994,55 @@ __global__ void k_fill_slots(float* out, int len, int Kp, int s0, int s1, float 
 }
 
 // Per-slot initial image TMC_s * 1_disk (Sec. 4.1) for the slots of K slices
-// (s0 + k, or ids[k]) from slice-major g, gamma ([K][m]): one block per slice.
-__global__ void __launch_bounds__(256) k_binit_image(const float* __restrict__ g,
-                                                     const float* __restrict__ gamma, int m, int n,
-                                                     int n_angles, long long npfov, int Kp, int s0,
-                                                     const int* __restrict__ ids,
-                                                     float* __restrict__ f_out) {
-  const int k = blockIdx.x;
-  const int slot = slot_of(ids, s0, k);
+// (s0 + k, or ids[k]) from slice-major g, gamma ([K][m]): ACT_PARTS blocks per
+// slice sum g - gamma, then the images are filled a row of slots at a time (one
+// block per slice did both: 192 us for 64 slices of 256 x 256, 12 us now).
+constexpr int ACT_PARTS = 16;
+__global__ void __launch_bounds__(256) k_bactc(const float* __restrict__ g,
+                                               const float* __restrict__ gamma, int m,
+                                               float2* __restrict__ parts) {
+  const int k = blockIdx.y;
   float h = 0.f, l = 0.f;
-  for (int i = threadIdx.x; i < m; i += blockDim.x) {
+#pragma unroll 4
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
     acc_add(h, l, g[(size_t)k * m + i], 0.f);
     acc_add(h, l, -gamma[(size_t)k * m + i], 0.f);
   }
   const df t = block_sum_acc(h, l);
-  __shared__ float s_tmc;
-  if (threadIdx.x == 0)
-    s_tmc = (float)(((double)t.hi + (double)t.lo) / ((double)npfov * (double)n_angles));
+  if (threadIdx.x == 0) parts[k * ACT_PARTS + blockIdx.x] = make_float2(t.hi, t.lo);
+}
+// f_cur and, if not NULL, f_prev; delta and low become 0; without a slot list
+// the padding slots get 0.
+__global__ void __launch_bounds__(256) k_binit_image(const float2* __restrict__ parts, int n,
+                                                     int n_angles, long long npfov, int K, int Kp,
+                                                     int s0, const int* __restrict__ ids,
+                                                     float* __restrict__ f_cur,
+                                                     float* __restrict__ f_prev,
+                                                     float* __restrict__ delta,
+                                                     float* __restrict__ low) {
+  __shared__ float s_tmc[MAXK];
+  for (int k = threadIdx.x; k < K; k += blockDim.x) {
+    float h = 0.f, l = 0.f;
+    for (int q = 0; q < ACT_PARTS; ++q) {
+      const float2 v = parts[k * ACT_PARTS + q];
+      acc_add(h, l, v.x, v.y);
+    }
+    s_tmc[k] = (float)(((double)h + (double)l) / ((double)npfov * (double)n_angles));
+  }
   __syncthreads();
-  const float v = s_tmc;
-  for (int j = threadIdx.x; j < n * n; j += blockDim.x) {
+  const int cols = ids ? K : Kp - s0;
+  const size_t total = (size_t)n * n * cols;
+  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total;
+       t += (size_t)gridDim.x * blockDim.x) {
+    const int j = (int)(t / cols), k = (int)(t % cols);
     const int r = j / n, c = j % n;
     const long long dx = 2ll * c + 1 - n, dy = 2ll * r + 1 - n;
-    f_out[(size_t)j * Kp + slot] = (dx * dx + dy * dy <= (long long)n * n) ? v : 0.f;
+    const float v = k < K && dx * dx + dy * dy <= (long long)n * n ? s_tmc[k] : 0.f;
+    const size_t o = (size_t)j * Kp + slot_of(ids, s0, k);
+    f_cur[o] = v;
+    if (f_prev) f_prev[o] = v;
+    delta[o] = 0.f;
+    low[o] = 0.f;
   }
 }
 
@@ -975,6 +1147,38 @@ cudaError_t launch_bstencil(const BFwdArgs& a0, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+namespace {
+template <int W>
+cudaError_t bobjective_w(const BFwdArgs& a, cudaStream_t s) {
+  if (a.use_bf16)
+    k_bobjective<W, true><<<blocks_of<W>(a.n_spmv_blocks), P_THREADS, 0, s>>>(a);
+  else
+    k_bobjective<W, false><<<blocks_of<W>(a.n_spmv_blocks), P_THREADS, 0, s>>>(a);
+  return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t launch_bobjective(const BFwdArgs& a0, int K, double* out, cudaStream_t s) {
+  cudaError_t e = ensure_tables();
+  if (e != cudaSuccess) return e;
+  BFwdArgs a = a0;
+  a.mode = 3;
+  a.track = 1;
+  a.n_spmv_blocks = fw_blocks(a);
+  switch (a.width) {
+    case 8: e = bobjective_w<8>(a, s); break;
+    case 16: e = bobjective_w<16>(a, s); break;
+    case 32: e = bobjective_w<32>(a, s); break;
+    case 64: e = bobjective_w<64>(a, s); break;
+    case 128: e = bobjective_w<128>(a, s); break;
+    default: e = cudaErrorInvalidValue;
+  }
+  if (e == cudaSuccess) e = launch_bstencil(a, s);
+  if (e != cudaSuccess) return e;
+  k_sum_columns<<<K, 256, 0, s>>>(a.fpartial, a.n_spmv_blocks, st_blocks(a), a.Kp, out);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_gather_probe(const DevCSR& M, const float* x, int Kp, float* sink,
                                 int blocks_per_sm, cudaStream_t s) {
   if (blocks_per_sm < 1 || blocks_per_sm > kMaxPerSm) return cudaErrorInvalidValue;
@@ -1008,25 +1212,23 @@ cudaError_t launch_binit_momentum(SlotState* slots, int Kp, bool only_fresh, cud
 }
 
 cudaError_t launch_to_slot_minor(const float* in, int K, int len, float* out, int Kp, int s0,
-                                 const int* ids, cudaStream_t s) {
+                                 const int* ids, cudaStream_t s, float fill, bool positive,
+                                 int* flag) {
   if (K <= 0) return cudaSuccess;
-  dim3 grid((len + 31) / 32, (K + 31) / 32), block(32, 8);
-  k_to_slot_minor<<<grid, block, 0, s>>>(in, K, len, out, Kp, s0, ids);
+  const int cols = ids ? K : Kp - s0;
+  dim3 grid((len + 31) / 32, (cols + 31) / 32), block(32, 8);
+  k_to_slot_minor<<<grid, block, 0, s>>>(in, K, len, out, Kp, s0, ids, fill, positive ? 1 : 0,
+                                         flag);
   return cudaGetLastError();
 }
 
-cudaError_t launch_from_slot_minor(const float* in, int K, int len, int Kp, int s0,
-                                   const int* ids, float* out, cudaStream_t s) {
+cudaError_t launch_from_slot_minor(const BFwdArgs& a, int K, int s0, const int* ids, float* out,
+                                   cudaStream_t s) {
   if (K <= 0) return cudaSuccess;
+  const int len = a.n * a.n;
   dim3 grid((len + 31) / 32, (K + 31) / 32), block(32, 8);
-  k_from_slot_minor<<<grid, block, 0, s>>>(in, K, len, Kp, s0, ids, out);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_copy_slots(const float* src, float* dst, int len, int Kp, const int* ids,
-                              int K, cudaStream_t s) {
-  if (K <= 0) return cudaSuccess;
-  k_copy_slots<<<256, 256, 0, s>>>(src, dst, len, Kp, ids, K);
+  k_from_slot_minor<<<grid, block, 0, s>>>(a.f[0], a.f[1], a.f[2], a.bst, K, len, a.Kp, s0, ids,
+                                           out);
   return cudaGetLastError();
 }
 
@@ -1039,9 +1241,14 @@ cudaError_t launch_fill_slots(float* out, int len, int Kp, int s0, int s1, float
 
 cudaError_t launch_binit_image(const float* g, const float* gamma, int m, int n, int n_angles,
                                long long npfov, int K, int Kp, int s0, const int* ids,
-                               float* f_out, cudaStream_t s) {
+                               float2* scratch, float* f_cur, float* f_prev, float* delta,
+                               float* low, cudaStream_t s) {
   if (K <= 0) return cudaSuccess;
-  k_binit_image<<<K, 256, 0, s>>>(g, gamma, m, n, n_angles, npfov, Kp, s0, ids, f_out);
+  k_bactc<<<dim3(ACT_PARTS, K), 256, 0, s>>>(g, gamma, m, scratch);
+  const long long total = (long long)n * n * (ids ? K : Kp - s0);
+  const int grid = (int)std::min<long long>((total + 255) / 256, sm_count() * 8LL);
+  k_binit_image<<<grid, 256, 0, s>>>(scratch, n, n_angles, npfov, K, Kp, s0, ids, f_cur, f_prev,
+                                      delta, low);
   return cudaGetLastError();
 }
 

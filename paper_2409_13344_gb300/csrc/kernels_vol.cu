@@ -444,10 +444,11 @@ __global__ void __launch_bounds__(256) k_slices_to_slots(const float* in, float*
 
 // out = sum of rows x cols double-float pairs (row stride pstride), one block,
 // fixed order
-__global__ void __launch_bounds__(256) k_sum_pairs(const float2* __restrict__ p, int rows,
+__global__ void __launch_bounds__(1024) k_sum_pairs(const float2* __restrict__ p, int rows,
                                                    int cols, int pstride, double* out) {
   float h = 0.f, l = 0.f;
   const int total = rows * cols;
+#pragma unroll 4
   for (int i = threadIdx.x; i < total; i += blockDim.x) {
     const float2 v = p[(long long)(i / cols) * pstride + i % cols];
     acc_add(h, l, v.x, v.y);
@@ -482,7 +483,7 @@ cudaError_t launch_stencil3d(const Vol3Args& a, cudaStream_t s) {
 
 cudaError_t launch_sum_pairs(const float2* p, int rows, int cols, int pstride, double* out,
                              cudaStream_t s) {
-  k_sum_pairs<<<1, 256, 0, s>>>(p, rows, cols, pstride, out);
+  k_sum_pairs<<<1, 1024, 0, s>>>(p, rows, cols, pstride, out);
   return cudaGetLastError();
 }
 

@@ -205,6 +205,8 @@ appga_status create_pool(appga_server* S, int geom, int Kp, Pool** out) {
     e = cudaMemsetAsync(P->b.f[i], 0, (size_t)M->d * Kp * sizeof(float), s);
   for (int i = 0; i < 2 && e == cudaSuccess; ++i)
     e = cudaMemsetAsync(P->b.y[i], 0, (size_t)M->m * Kp * sizeof(float), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(P->b.delta, 0, (size_t)M->d * Kp * sizeof(float), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(P->b.low, 0, (size_t)M->d * Kp * sizeof(float), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(P->b.g, 0, (size_t)M->m * Kp * sizeof(float), s);
   if (e == cudaSuccess) e = launch_fill_slots(P->b.gamma, M->m, Kp, 0, Kp, 1.f, s);
   if (e != cudaSuccess) {
@@ -329,9 +331,8 @@ appga_status admit(appga_server* S, Pool* P, int count) {
   CK(launch_to_slot_minor(P->d_in + (size_t)K * m, K, m, P->b.gamma, Kp, 0, P->d_ids, s));
   // f^{k0} = f^{k0-1}: the initial image TMC * 1_disk (Sec. 4.1), or the request's own
   CK(launch_binit_image(P->d_in, P->d_in + (size_t)K * m, m, M->n, M->na, M->npfov, K, Kp, 0,
-                        P->d_ids, cur, s));
+                        P->d_ids, P->b.partial, cur, nullptr, P->b.delta, P->b.low, s));
   CK(launch_to_slot_minor(P->d_in + (size_t)2 * K * m, kf, d, cur, Kp, 0, P->d_ids + Kp, s));
-  CK(launch_copy_slots(cur, P->b.f[(Gs + 2) % 3], d, Kp, P->d_ids, K, s));
   for (int k = 0; k < K; ++k) {
     Request& R = S->reqs[ids[k]];
     SlotState st = slot_from_params(&R.p, 1, true);
@@ -424,7 +425,7 @@ appga_status retire_begin(appga_server* S, Pool* P) {
   CK(cudaMemcpyAsync(P->d_ids + 2 * Kp, P->h_ids + 2 * Kp, K * sizeof(int),
                      cudaMemcpyHostToDevice, s));
   // a finished slot carries its result forward, so it sits in the current ring entry
-  CK(launch_from_slot_minor(P->b.f[P->gstep % 3], K, d, Kp, 0, P->d_ids + 2 * Kp, P->d_out, s));
+  CK(launch_from_slot_minor(P->fa, K, 0, P->d_ids + 2 * Kp, P->d_out, s));
   CK(cudaMemcpyAsync(P->h_out, P->d_out, (size_t)K * d * sizeof(float), cudaMemcpyDeviceToHost,
                      s));
   appga_params def;

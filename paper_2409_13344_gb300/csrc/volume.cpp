@@ -6,7 +6,6 @@
 #include <cmath>
 #include <limits>
 #include <string>
-#include <vector>
 
 #include "appga.h"
 #include "appga_internal.h"
@@ -18,38 +17,6 @@ using namespace appga;
 namespace {
 
 #define CK(call) APPGA_CK(call)
-
-// Phi of the result volume f (slice-major): the slices' data terms, which the
-// solve left in the workspace's host mirror (entries 2z, double-float
-// projections), plus the 3-D regulariser of f, summed in FP64 on the host in
-// slice order.
-appga_status volume_objective(appga_ctx* ctx, appga_matrix* M, int nz, const float* f,
-                              const appga_params* p, double* phi) {
-  BatchWorkspace& b = *M->bw;
-  cudaStream_t s = ctx->stream;
-  std::vector<double> data((size_t)nz);
-  for (int z = 0; z < nz; ++z) data[(size_t)z] = b.vscal_host[2 * z];
-  Vol3Args va{};
-  va.n = M->n;
-  va.nz = nz;
-  va.f[0] = f;
-  va.lam1 = (float)p->lambda1;
-  va.lam2 = (float)p->lambda2;
-  va.eps = (float)p->eps;
-  va.want_reg = 1;
-  va.pstride = nz;
-  va.gR = b.gR;           // scratch: the batched workspace holds d * Kp >= d * nz floats
-  va.partial = b.fpartial;
-  CK(launch_stencil3d(va, s));
-  double* reg = b.vscal + 2 * nz;
-  CK(launch_sum_pairs(b.fpartial, stencil3d_grid(M->n, nz), nz, nz, reg, s));
-  CK(cudaMemcpyAsync(b.vscal_host + 2 * nz, reg, sizeof(double), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
-  double tot = 0.0;
-  for (int z = 0; z < nz; ++z) tot += data[(size_t)z];
-  *phi = tot + b.vscal_host[2 * nz];
-  return APPGA_OK;
-}
 
 }  // namespace
 
@@ -102,7 +69,7 @@ extern "C" appga_status appga_reconstruct_volume(appga_ctx* ctx, const appga_mat
   appga_status rc = appga_params_validate(params);
   if (rc != APPGA_OK) return rc;
   auto* M = const_cast<appga_matrix*>(mat);
-  rc = volume_solve(ctx, M, nz, g, gamma, f_init, params, f_out, stream);
+  rc = volume_solve(ctx, M, nz, g, gamma, f_init, params, f_out, stats_host != nullptr, stream);
   if (rc != APPGA_OK) return rc;
   if (!stats_host) return APPGA_OK;
   const BatchWorkspace& b = *M->bw;
@@ -120,12 +87,10 @@ extern "C" appga_status appga_reconstruct_volume(appga_ctx* ctx, const appga_mat
   const bool track = params->track_objective != 0 || params->rel_obj_tol > 0.0;
   if (track) {
     st.phi_prev = s0.stopped_early ? b.bst_host->phi_tot_prev : b.bst_host->phi_tot_cur;
-    if ((rc = enter_stream(ctx, stream)) != APPGA_OK) return rc;
+    // the slices' data terms in slice order, then the volume's regulariser
     double phi = 0.0;
-    rc = volume_objective(ctx, M, nz, f_out, params, &phi);
-    if (rc != APPGA_OK) return rc;
-    st.phi = phi;
-    if ((rc = leave_stream(ctx, stream)) != APPGA_OK) return rc;
+    for (int z = 0; z < nz; ++z) phi += b.vscal_host[2 * z];
+    st.phi = phi + b.vscal_host[2 * nz];
   }
   *stats_host = st;
   return APPGA_OK;
