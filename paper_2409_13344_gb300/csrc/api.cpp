@@ -1009,6 +1009,8 @@ appga_status appga_matrix_destroy(appga_matrix* M) {
   free_sell(M->sell_t);
   free_sell(M->fold_a);
   free_sell(M->fold_t);
+  free_quad(M->quad_a);
+  free_quad(M->quad_t);
   free_csr(M->A);
   free_csr(M->At);
   cudaFree(M->inv_lambda);

@@ -83,6 +83,18 @@ struct DevCSR {
   uint16_t* val_bf16 = nullptr;  // nnz_padded (optional BF16 copy)
 };
 
+// Row-block layout of the batched projectors (quads.cu): the rows in blocks of
+// four along DevCSR::order, each block the union of its rows' columns in packs
+// of four, with the four rows' values per column (zero where a row has none).
+struct DevQuad {
+  int32_t blocks = 0;
+  int32_t* off = nullptr;   // blocks + 1 offsets in packs
+  int32_t* rows = nullptr;  // 4 per block, -1 past the last row
+  int4* cols = nullptr;     // the four columns of a pack
+  float4* vals = nullptr;   // 4 per pack: the four rows' values at one column
+  uint2* vals_bf16 = nullptr;
+};
+
 // Device-resident iteration state of one solve.  Kernels derive buffer
 // indices and the momentum scalar from it, so captured graphs replay
 // unchanged from one iteration to the next.

@@ -103,14 +103,15 @@ BatchSchedule tuned_schedule(const appga_matrix* M, int Kp, bool bf16) {
   return it == M->tuned.end() ? BatchSchedule() : it->second;
 }
 
-void make_batch_args(const DevCSR& A, const DevCSR& At, const float* inv_lambda, int n,
-                     BatchWorkspace& b, int stride, bool bf16, bool track,
+void make_batch_args(const appga_matrix* M, BatchWorkspace& b, int stride, bool bf16, bool track,
                      const BatchSchedule& sch, BFwdArgs* fa, BPixArgs* pa) {
+  const int n = M->n;
   *fa = BFwdArgs{};
   fa->spmv_per_sm = sch.spmv_per_sm;
   fa->stencil_per_sm = sch.stencil_per_sm;
   fa->gather_rows = sch.gather_rows_fw;
-  fa->A = A;
+  fa->QA = M->quad_a;
+  fa->A = M->A;
   fa->n = n;
   fa->Kp = stride;
   fa->width = stride;
@@ -131,7 +132,7 @@ void make_batch_args(const DevCSR& A, const DevCSR& At, const float* inv_lambda,
   *pa = BPixArgs{};
   pa->blocks_per_sm = sch.pixel_per_sm;
   pa->gather_rows = sch.gather_rows_px;
-  pa->At = At;
+  pa->QT = M->quad_t;
   pa->n = n;
   pa->Kp = stride;
   pa->width = stride;
@@ -141,7 +142,7 @@ void make_batch_args(const DevCSR& A, const DevCSR& At, const float* inv_lambda,
   pa->low = b.low;
   pa->w = b.w;
   pa->gR = b.gR;
-  pa->inv_lambda = inv_lambda;
+  pa->inv_lambda = bf16 ? M->inv_lambda_bf16 : M->inv_lambda;
   pa->pfreeze = b.pfreeze;
   pa->slots = b.slots;
   pa->bst = b.bst;
@@ -252,6 +253,7 @@ appga_status batched_solve(appga_ctx* ctx, appga_matrix* M, int32_t K, const flo
   if ((rc = ensure_batch_workspace(M, std::max(padded_width(K), min_width))) != APPGA_OK) return rc;
   const int Kp = std::max(slot_width(K), min_width);
   if ((rc = enter_stream(ctx, stream)) != APPGA_OK) return rc;
+  if ((rc = ensure_quads(M, ctx->stream)) != APPGA_OK) return rc;
   BatchWorkspace& b = *M->bw;
   cudaStream_t s = ctx->stream;
   const int m = M->m, d = M->d, n = M->n;
@@ -293,8 +295,7 @@ appga_status batched_solve(appga_ctx* ctx, appga_matrix* M, int32_t K, const flo
 
   BFwdArgs fa;
   BPixArgs pa;
-  make_batch_args(M->A, M->At, bf16 ? M->inv_lambda_bf16 : M->inv_lambda, n, b, Kp, bf16, track,
-                  sch, &fa, &pa);
+  make_batch_args(M, b, Kp, bf16, track, sch, &fa, &pa);
   // volume: the K slots are the slices of one volume.  The 3-D stencil runs
   // on slice-major copies of the iterates after the forward phase, leaves
   // its per-slice regulariser sums after the forward phase's rows, and its
@@ -532,14 +533,13 @@ namespace appga {
 namespace {
 // best gathered GB/s over launch shapes for the column stream `col` (nnz
 // entries) into the slot-minor block x of `width` floats per row
-appga_status probe_best(const DevCSR& M, const float* x, int width, float* sink, int launches,
+appga_status probe_best(const DevQuad& M, long long nnz, const float* x, int width, float* sink, int launches,
                         cudaStream_t s, double* best) {
-  const long long nnz = M.nnz_padded;
   *best = 0.0;
   cudaEvent_t ev[2] = {nullptr, nullptr};
   CK(cudaEventCreate(&ev[0]));
   cudaError_t e = cudaEventCreate(&ev[1]);
-  for (const int per_sm : {2, 4, 6, 8, 12}) {
+  for (const int per_sm : {2, 4, 8, 12, 16}) {
     for (int i = 0; i < 2 && e == cudaSuccess; ++i)
       e = launch_gather_probe(M, x, width, sink, per_sm, s);
     if (e == cudaSuccess) e = cudaEventRecord(ev[0], s);
@@ -582,8 +582,9 @@ extern "C" appga_status appga_gather_probe(appga_ctx* ctx, const appga_matrix* m
   // back-projection: A^T's columns into the weight block [m][width]
   CK(cudaMemsetAsync(b.f[0], 0, (size_t)M->d * width * sizeof(float), s));
   CK(cudaMemsetAsync(b.w, 0, (size_t)M->m * width * sizeof(float), s));
-  rc = probe_best(M->A, b.f[0], width, sink, launches, s, gbs_fwd);
-  if (rc == APPGA_OK) rc = probe_best(M->At, b.w, width, sink, launches, s, gbs_bwd);
+  if ((rc = ensure_quads(M, s)) != APPGA_OK) return rc;
+  rc = probe_best(M->quad_a, M->A.nnz_padded, b.f[0], width, sink, launches, s, gbs_fwd);
+  if (rc == APPGA_OK) rc = probe_best(M->quad_t, M->At.nnz_padded, b.w, width, sink, launches, s, gbs_bwd);
   return rc;
 }
 

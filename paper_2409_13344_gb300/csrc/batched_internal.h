@@ -42,7 +42,8 @@ struct BatchState {
 };
 
 struct BFwdArgs {
-  DevCSR A;
+  DevQuad QA;
+  DevCSR A;       // the objective's double-float projections
   int32_t n;
   int32_t Kp;     // row stride of the slot-minor arrays
   int32_t width;  // slots worked on: 8, 16, 32, 64 or 128, every live slot below it
@@ -70,7 +71,7 @@ struct BFwdArgs {
 };
 
 struct BPixArgs {
-  DevCSR At;
+  DevQuad QT;
   int32_t n;
   int32_t Kp;             // row stride of the slot-minor arrays
   int32_t width;          // slots worked on (as BFwdArgs)
@@ -148,7 +149,7 @@ cudaError_t launch_bobjective(const BFwdArgs& a, int K, double* out, cudaStream_
 // Kp-wide rows of x, [cols][Kp]; no epilogue) with blocks_per_sm (1..16)
 // blocks per SM; sink: at least (SMs x 16) floats, written only in a case
 // that does not arise.
-cudaError_t launch_gather_probe(const DevCSR& M, const float* x, int Kp, float* sink,
+cudaError_t launch_gather_probe(const DevQuad& M, const float* x, int Kp, float* sink,
                                 int blocks_per_sm, cudaStream_t s);
 // Slots the kernels work on for K slices: the narrowest of 8, 16, 32, 64 and
 // 128 that holds them.

@@ -116,10 +116,12 @@ void free_batch_workspace(BatchWorkspace* bw);
 int64_t batch_workspace_bytes(int m, int d, int Kp);
 // Allocates every array of a width-Kp workspace (frees what it made on error).
 cudaError_t alloc_batch_workspace(BatchWorkspace& b, int m, int d, int Kp);
+// The batched projectors' layout of M's matrices (quads.cu), built on first use.
+appga_status ensure_quads(appga_matrix* M, cudaStream_t s);
+void free_quad(DevQuad& q);
 // Kernel arguments of one batched step over workspace b, `stride` (at most
-// b.Kp) slots per row, with matrix arrays from (A, At, inv_lambda).
-void make_batch_args(const DevCSR& A, const DevCSR& At, const float* inv_lambda, int n,
-                     BatchWorkspace& b, int stride, bool bf16, bool track,
+// b.Kp) slots per row, of matrix M (after ensure_quads).
+void make_batch_args(const appga_matrix* M, BatchWorkspace& b, int stride, bool bf16, bool track,
                      const BatchSchedule& sch, BFwdArgs* fa, BPixArgs* pa);
 // Tuned schedule of matrix M for padded width Kp and precision (defaults if none).
 BatchSchedule tuned_schedule(const appga_matrix* M, int Kp, bool bf16);
@@ -177,6 +179,7 @@ struct appga_matrix {
   // was not turned off): the first m/2 rows of A with tiled columns, and
   // their transpose in orbit order, both sliced (off == NULL: not folded)
   appga::DevSell fold_a, fold_t;
+  appga::DevQuad quad_a, quad_t;  // the batched projectors' layout (off == NULL: not built)
   int32_t fold_nb = 0;  // bins per angle of the folded matrix
   float* inv_lambda = nullptr;       // 1/Lambda of the FP32 values
   float* inv_lambda_bf16 = nullptr;  // 1/Lambda of the BF16-rounded values

@@ -1,18 +1,16 @@
 // Batched CUDA kernels: K independent slices (slots) that share one system
 // matrix run the APPGA iteration together, so every nonzero of A and A^T is
-// read once per iteration for all K right-hand sides (CSR SpMM).
+// read once per iteration for all K right-hand sides (SpMM).
 //
 // Layout (slot-minor): images f[j][s], sinograms y[i][s], w[i][s], g[i][s],
-// rows of Kp slots.  A launch works on the first W = 8, 16, 32, 64 or 128 of
-// them; the lanes of a warp share a row's products as Team<W> says.  The bound
-// is the L1 pipe: each nonzero takes W/32 passes of 128 bytes for its gathered
-// row, plus its share of the matrix's broadcast loads.  Rows are dealt to
-// warps along a Z-order curve (pixels, or rays by angle and bin), so a block
-// gathers for neighbouring rows and half to three quarters of the sectors hit
-// L1 (64 slots of 256 x 256: 1.8 and 1.2 GB from L2 per projection, 3.5 and
-// 2.6 GB in row order).  The per-(row, slot) epilogues match the single-slice
-// kernels (Eq. APPGAiter, Eq. EM, Sec. 2.2); the SHOITV stencil is a kernel of
-// its own that runs beside the forward projection.
+// rows of Kp slots.  A launch works on as many slots as are held: 8, 16, 32, 64
+// or twice 64.  The projections take the matrices in blocks of four neighbouring
+// rows (DevQuad), so that a gathered row serves up to four of them from
+// registers; QTeam says how a warp shares a block and what bounds it.  Blocks
+// follow a Z-order curve (pixels, or rays by angle and bin), so the blocks of an
+// SM gather for neighbouring rows and meet in L1.  The per-(row, slot) epilogues
+// match the single-slice kernels (Eq. APPGAiter, Eq. EM, Sec. 2.2); the SHOITV
+// stencil is a kernel of its own that runs beside the forward projection.
 //
 // Every slot carries its own device state (iteration index, momentum scalar,
 // objective, stop flag, parameters), so slots may sit at different
@@ -24,6 +22,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "appga_internal.h"
 #include "batched_internal.h"
@@ -34,19 +33,24 @@ namespace {
 
 constexpr int B_THREADS = 256;               // stencil blocks (and set-up kernels)
 constexpr int MAXK = 128;                    // largest padded batch
-// Projector blocks: 16 warps, two blocks per SM (64 registers per thread).  A
-// block's warps work on a compact bundle of rows (DevCSR::order), so the wider
-// the block the more of its gathers meet in L1.
+// Projector blocks: four warps, four blocks per SM (128 registers per thread:
+// a step's gathers are in flight at once, which gains more than more warps with
+// half of them would; eight-warp blocks are slower, their last warps idle more).
+constexpr int Q_THREADS = 128;
+constexpr int Q_WARPS = Q_THREADS / 32;
+constexpr int Q_PER_SM = 4;
+// Blocks of the objective's double-float projections.
 constexpr int P_THREADS = 512;
 constexpr int P_WARPS = P_THREADS / 32;
 constexpr int kMaxPerSm = 16;                // upper bound of the tuned values
 __host__ __forceinline__ int clamp_per_sm(int v, int dflt) {
   return v <= 0 ? dflt : (v > kMaxPerSm ? kMaxPerSm : v);
 }
-// Row groups per SM when no tuned schedule is given: more than are resident
+// Virtual blocks per SM when no tuned schedule is given: more than are resident
 // at once, so the block scheduler levels the tail.
-constexpr int kSpmvPerSm = 8;
-constexpr int kPixelPerSm = 8;
+constexpr int kSpmvPerSm = 16;
+constexpr int kPixelPerSm = 16;
+constexpr int kObjectivePerSm = 8;
 constexpr int kStencilPerSm = 8;
 // Stencil blocks: 8 slots x 32 image columns (the outer two on each side are
 // halo), marching down runs of BST_R rows.
@@ -69,28 +73,54 @@ __device__ __forceinline__ void vload(const float* p, float (&x)[E]) {
     x[3] = t.w;
   }
 }
-// Stores the elements whose on[] is set (one vector store when all are).
-template <int E>
-__device__ __forceinline__ void vstore_on(float* p, const float (&x)[E], const int (&on)[E]) {
-  int all = 1;
-#pragma unroll
-  for (int t = 0; t < E; ++t) all &= on[t] ? 1 : 0;
-  if (all) {
-    if constexpr (E == 1) {
+__device__ __forceinline__ void prefetch_l2(const void* p) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+}
+// Stores the elements whose bit is set in `on` (one vector store when all are).
+template <int V>
+__device__ __forceinline__ void vstore(float* p, const float (&x)[V], unsigned on) {
+  if (on == (1u << V) - 1) {
+    if constexpr (V == 1) {
       *p = x[0];
-    } else if constexpr (E == 2) {
+    } else if constexpr (V == 2) {
       *reinterpret_cast<float2*>(p) = make_float2(x[0], x[1]);
     } else {
       *reinterpret_cast<float4*>(p) = make_float4(x[0], x[1], x[2], x[3]);
     }
   } else {
 #pragma unroll
-    for (int t = 0; t < E; ++t)
-      if (on[t]) p[t] = x[t];
+    for (int t = 0; t < V; ++t)
+      if (on >> t & 1) p[t] = x[t];
+  }
+}
+// Two FP32 values in one 64-bit register pair, and a += w x on both (each
+// rounded once, as fmaf).
+__device__ __forceinline__ unsigned long long pair_of(float a, float b) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void split(unsigned long long v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ void fma2(unsigned long long& a, unsigned long long w,
+                                     unsigned long long x) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a) : "l"(w), "l"(x));
+}
+// The four rows' values at union column o.
+template <bool BF16>
+__device__ __forceinline__ float4 ld_quad(const DevQuad& M, size_t o, uint64_t pol) {
+  if constexpr (BF16) {
+    const uint2 u = ld_stream_u2(M.vals_bf16 + o, pol);
+    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u),
+                       __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u));
+  } else {
+    return ld_stream_f4(reinterpret_cast<const float*>(M.vals + o), pol);
   }
 }
 
-// How the lanes of a warp share a row whose products fill W slots.  A lane
+// The objective's double-float projections take one row at a time from the
+// CSR: how the lanes of a warp share a row whose products fill W slots.  A lane
 // holds Q slots (Q/4 16-byte loads per gathered row), L lanes make a group
 // that covers the W slots, and the G groups of a row's team take the row's
 // 4-entry packs in turn.  The row's sum is always that of four partial sums,
@@ -106,7 +136,6 @@ struct Team {
   static constexpr int Q = W >= 16 ? 8 : 4;
   static constexpr int L = W / Q;
   static constexpr int G = L <= 8 ? 4 : 32 / L;
-  static constexpr int A = 4 / G;
   static constexpr int LANES = L * G;
   static constexpr int RW = 32 / LANES;
   static constexpr int E = Q / G;  // slots a lane owns after the reduction
@@ -127,99 +156,234 @@ __device__ __forceinline__ int owned_slot(int lane) {
   return gathered_slot<W>(lane) + T::GSTRIDE * (g & 1) + T::E * (g >> 1);
 }
 
-// One row of M (row < 0: none) times the columns of X ([cols][stride]): each
-// lane ends with the sums of the E slots from owned_slot.  A lane gathers NZ
-// (2 or 4) entries of a pack per step while the columns and values of the
-// next pack are in flight; `on`: some of the lane's gathered slots is wanted.
-// All lanes of the warp take part.
-template <int W, bool BF16, int NZ>
-__device__ __forceinline__ void team_dot(const DevCSR& M, int row, const float* __restrict__ X,
-                                         int stride, int lane, bool on, uint64_t pol,
-                                         float (&out)[Team<W>::E]) {
-  using T = Team<W>;
-  constexpr int A = T::A, Q = T::Q, F = Q / 4, E = T::E;
-  const int g = lane % T::LANES / T::L;
-  int p = 0, cnt = 0;  // the lane's packs are g, g + G, ...: cnt of them from p
-  if (row >= 0 && on) {
-    const int s = __ldg(M.row_ptr + row);
-    const int npk = (__ldg(M.row_ptr + row + 1) - s) >> 2;
-    cnt = npk > g ? (npk - g + T::G - 1) / T::G : 0;
-    p = s + 4 * g;
+// How the kernels' warps share the layout's blocks of four rows (DevQuad): a
+// lane holds Q slots, L lanes make a group that covers the W slots, and the S
+// groups of a block's team take the block's packs of four union columns in turn
+// (pack k: group k mod S), each summing all four rows.  The groups' sums are
+// added pairwise along the bits of the group's index, so the results do not
+// depend on W.  A narrow team is part of a warp, RW of them, a wide one NWQ
+// warps of GW groups.
+//
+// The L1 pipe bounds these kernels on large matrices (S = 4).  Per union column
+// it passes W/32 lines of the gathered row and, because a 16-byte load is
+// served in quarter warps even where its lanes share an address, a quarter pass
+// for the column and one for the four values (four groups, four passes a load).
+// A union column serves 2.0 pixels of the back-projection, or 1.5 rays of the
+// forward projection, so at 64 slots an entry costs 1.6 or 2.2 passes against
+// 3.0 with one row per warp: 64 slots of 256 x 256 take 167 and 216 us against
+// 247 and 257 us.  Small matrices have too few blocks to fill the chip and each
+// team's chain of packs is what they wait for: S = 16 quarters it.
+constexpr int QROWS = 4;
+template <int W, int S>
+struct QTeam {
+  static constexpr int Q = W >= 64 ? 8 : 4;
+  static constexpr int F = Q / 4;  // 16-byte pieces of a gathered row per lane
+  static constexpr int U = Q == 4 ? 2 : 1;  // packs a lane gathers per step (NZ = 4)
+  static constexpr int L = W / Q;
+  static constexpr int STRIDE = 4 * L;  // slots between a lane's pieces
+  static constexpr int GW = S < 32 / L ? S : 32 / L;
+  static constexpr int NWQ = S / GW;
+  static constexpr int LANES = GW * L;
+  static constexpr int RW = 32 / LANES;
+  static constexpr int TB = Q_WARPS / NWQ * RW;  // teams of a thread block
+  static constexpr int TV = S == 4 ? 4 : 1;      // teams of a virtual block
+  // after the reduction a lane owns E slots of one row, in pieces of V
+  static constexpr int EW = Q / (GW / 4);
+  static constexpr int E = EW / NWQ;
+  static constexpr int V = E < 4 ? E : 4;
+  static_assert(GW >= 4 && E >= 1 && TB % TV == 0, "two exchanges halve the rows");
+};
+// A lane's place in its team.
+template <int W, int S>
+struct QLane {
+  int lane, warp, team, g, wq, row, slot;  // team of the block; group in the warp; warp in the
+                                           // team; owned row and first owned slot
+  __device__ __forceinline__ QLane() {
+    using T = QTeam<W, S>;
+    lane = threadIdx.x & 31;
+    warp = threadIdx.x >> 5;
+    team = warp / T::NWQ * T::RW + lane / T::LANES;
+    g = lane % T::LANES / T::L;
+    wq = warp % T::NWQ;
+    row = 2 * (g & 1) + (g >> 1 & 1);
+    int raw = T::E * wq;
+    if (T::GW >= 8) raw += T::Q / 2 * (g >> 2 & 1);
+    if (T::GW >= 16) raw += T::Q / 4 * (g >> 3 & 1);
+    slot = gathered() + raw / 4 * T::STRIDE + raw % 4;
   }
-  const float* xl = X + gathered_slot<W>(lane);
-  float acc[A][Q];
-#pragma unroll
-  for (int i = 0; i < A; ++i)
-#pragma unroll
-    for (int q = 0; q < Q; ++q) acc[i][q] = 0.f;
-  int4 c = make_int4(0, 0, 0, 0);
-  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (cnt > 0) {
-    c = ld_stream_i4(M.col + p, pol);
-    v = ld_vals<BF16>(M, p, pol);
+  // first of the lane's gathered slots (pieces of four, STRIDE apart)
+  __device__ __forceinline__ int gathered() const { return 4 * (lane % QTeam<W, S>::L); }
+};
+
+// Block b (negative: none) of M times the columns of X ([cols][stride]): the
+// lane's group's sums of its gathered slots for the four rows, as pairs of
+// neighbouring slots for the two-wide FP32 FMA.  A lane gathers NZ (2 or 4)
+// columns per step; `on`: some of its slots is wanted.
+template <int W, int S, bool BF16, int NZ>
+__device__ __forceinline__ void quad_sums(const DevQuad& M, int b, const float* __restrict__ X,
+                                          int stride, const QLane<W, S>& me, bool on, uint64_t pol,
+                                          unsigned long long (&acc2)[QROWS][QTeam<W, S>::Q / 2]) {
+  using T = QTeam<W, S>;
+  constexpr int Q = T::Q, F = T::F;
+  int k = 0, e = 0;
+  if (b >= 0 && on) {
+    k = __ldg(M.off + b) + me.wq * T::GW + me.g;
+    e = __ldg(M.off + b + 1);
   }
-  auto pack = [&](float (&a)[Q], bool more) {
-    const int cc[4] = {c.x, c.y, c.z, c.w};
-    const float vv[4] = {v.x, v.y, v.z, v.w};
+  const float* xl = X + me.gathered();
+#pragma unroll
+  for (int r = 0; r < QROWS; ++r)
+#pragma unroll
+    for (int q = 0; q < Q / 2; ++q) acc2[r][q] = 0ull;
+  constexpr int U = NZ == 4 ? T::U : 1;  // (a pack's products stay in its entries' order)
+  int4 c[U];
+#pragma unroll
+  for (int p = 0; p < U; ++p) {
+    c[p] = make_int4(0, 0, 0, 0);
+    if (k + S * p < e) c[p] = ld_stream_i4(reinterpret_cast<const int32_t*>(M.cols + k + S * p), pol);
+  }
+  // one step: U packs' gathers, the next U packs' columns, the products
+  auto step = [&](auto full) {
+    // the stream is two steps ahead in L2 (the loads below would otherwise
+    // wait for DRAM: 207 us of back-projection at 64 slots of 256 x 256, 189 so)
+    prefetch_l2(M.vals + 4 * (size_t)(k + 2 * S * U));
+    prefetch_l2(M.cols + (k + 2 * S * U));
 #pragma unroll
     for (int h = 0; h < 4; h += NZ) {
-      float4 x[NZ][F];
+      ulonglong2 x[U][NZ][F];
+      float4 v[U][NZ];
 #pragma unroll
-      for (int u = 0; u < NZ; ++u)
+      for (int p = 0; p < U; ++p) {
+        if (!full.value && k + S * p >= e) continue;
+        const int cc[4] = {c[p].x, c[p].y, c[p].z, c[p].w};
 #pragma unroll
-        for (int i = 0; i < F; ++i)
-          x[u][i] = __ldg(reinterpret_cast<const float4*>(xl + (unsigned)(cc[h + u] * stride)) +
-                          i * (T::GSTRIDE / 4));
-      if (h + NZ == 4 && more) {
-        p += 4 * T::G;
-        c = ld_stream_i4(M.col + p, pol);
-        v = ld_vals<BF16>(M, p, pol);
+        for (int u = 0; u < NZ; ++u) {
+#pragma unroll
+          for (int i = 0; i < F; ++i)
+            x[p][u][i] =
+                __ldg(reinterpret_cast<const ulonglong2*>(xl + (unsigned)(cc[h + u] * stride)) +
+                      i * (T::STRIDE / 4));
+          v[p][u] = ld_quad<BF16>(M, 4 * (size_t)(k + S * p) + h + u, pol);
+        }
+      }
+      if (h + NZ == 4) {
+#pragma unroll
+        for (int p = 0; p < U; ++p)
+          if (k + S * (U + p) < e)
+            c[p] = ld_stream_i4(reinterpret_cast<const int32_t*>(M.cols + k + S * (U + p)), pol);
       }
 #pragma unroll
-      for (int u = 0; u < NZ; ++u)
+      for (int p = 0; p < U; ++p) {
+        if (!full.value && k + S * p >= e) continue;
 #pragma unroll
-        for (int i = 0; i < F; ++i) {
-          a[4 * i] = fmaf(vv[h + u], x[u][i].x, a[4 * i]);
-          a[4 * i + 1] = fmaf(vv[h + u], x[u][i].y, a[4 * i + 1]);
-          a[4 * i + 2] = fmaf(vv[h + u], x[u][i].z, a[4 * i + 2]);
-          a[4 * i + 3] = fmaf(vv[h + u], x[u][i].w, a[4 * i + 3]);
+        for (int u = 0; u < NZ; ++u) {
+          const float vv[QROWS] = {v[p][u].x, v[p][u].y, v[p][u].z, v[p][u].w};
+#pragma unroll
+          for (int r = 0; r < QROWS; ++r) {
+            const unsigned long long w = pair_of(vv[r], vv[r]);
+#pragma unroll
+            for (int i = 0; i < F; ++i) {
+              fma2(acc2[r][2 * i], w, x[p][u][i].x);
+              fma2(acc2[r][2 * i + 1], w, x[p][u][i].y);
+            }
+          }
         }
+      }
     }
+    k += S * U;
   };
-  int j = 0;
-  for (; j + A < cnt; j += A) {  // all A packs have a successor: no tests
+  while (k + S * (U - 1) < e) step(std::true_type{});
+  if (U > 1 && k < e) step(std::false_type{});
+}
+// The groups' sums added up: the lane's E owned slots of its row.  All threads of
+// the block take part; each exchange halves the rows, then the slots a lane
+// keeps.  s_x: shared, 2 x Q_WARPS x EW x 32 floats where teams span warps;
+// `parity` alternates between its halves.
+template <int W, int S>
+__device__ __forceinline__ void quad_reduce(
+    const unsigned long long (&acc2)[QROWS][QTeam<W, S>::Q / 2], const QLane<W, S>& me,
+    float* s_x, int parity, float (&out)[QTeam<W, S>::E]) {
+  using T = QTeam<W, S>;
+  constexpr int Q = T::Q, EW = T::EW;
+  float acc[QROWS][Q];
 #pragma unroll
-    for (int i = 0; i < A; ++i) pack(acc[i], true);
-  }
+  for (int r = 0; r < QROWS; ++r)
 #pragma unroll
-  for (int i = 0; i < A; ++i)
-    if (j + i < cnt) pack(acc[i], j + i + 1 < cnt);
+    for (int q = 0; q < Q / 2; ++q) split(acc2[r][q], acc[r][2 * q], acc[r][2 * q + 1]);
   __syncwarp();
-  if constexpr (T::G == 4) {
-    const bool hi1 = g & 1, hi2 = g >> 1;
-    float q[2 * E];
+  const bool up0 = me.g & 1, up1 = me.g >> 1 & 1, up2 = me.g >> 2 & 1, up3 = me.g >> 3 & 1;
+  float q[2][Q], v[Q];
 #pragma unroll
-    for (int t = 0; t < 2 * E; ++t)
-      q[t] = (hi1 ? acc[0][2 * E + t] : acc[0][t]) +
-             __shfl_xor_sync(0xffffffffu, hi1 ? acc[0][t] : acc[0][2 * E + t], T::L);
+  for (int r = 0; r < 2; ++r)
 #pragma unroll
-    for (int t = 0; t < E; ++t)
-      out[t] = (hi2 ? q[E + t] : q[t]) +
-               __shfl_xor_sync(0xffffffffu, hi2 ? q[t] : q[E + t], 2 * T::L);
+    for (int t = 0; t < Q; ++t)
+      q[r][t] = (up0 ? acc[2 + r][t] : acc[r][t]) +
+                __shfl_xor_sync(0xffffffffu, up0 ? acc[r][t] : acc[2 + r][t], T::L);
+#pragma unroll
+  for (int t = 0; t < Q; ++t)
+    v[t] = (up1 ? q[1][t] : q[0][t]) +
+           __shfl_xor_sync(0xffffffffu, up1 ? q[0][t] : q[1][t], 2 * T::L);
+  if constexpr (T::GW >= 8) {
+#pragma unroll
+    for (int t = 0; t < Q / 2; ++t)
+      v[t] = (up2 ? v[Q / 2 + t] : v[t]) +
+             __shfl_xor_sync(0xffffffffu, up2 ? v[t] : v[Q / 2 + t], 4 * T::L);
+  }
+  if constexpr (T::GW >= 16) {
+#pragma unroll
+    for (int t = 0; t < Q / 4; ++t)
+      v[t] = (up3 ? v[Q / 4 + t] : v[t]) +
+             __shfl_xor_sync(0xffffffffu, up3 ? v[t] : v[Q / 4 + t], 8 * T::L);
+  }
+  if constexpr (T::NWQ == 1) {
+#pragma unroll
+    for (int t = 0; t < T::E; ++t) out[t] = v[t];
   } else {
-    static_assert(T::G == 2 || T::G == 4, "two or four groups");
-    const bool hi = g != 0;
-    float q[2][E];
+    float* buf = s_x + parity * Q_WARPS * EW * 32;
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
+    for (int t = 0; t < EW; ++t) buf[(me.warp * EW + t) * 32 + me.lane] = v[t];
+    __syncthreads();
+    const int w0 = me.warp - me.wq;
 #pragma unroll
-      for (int t = 0; t < E; ++t)
-        q[i][t] = (hi ? acc[i % A][E + t] : acc[i % A][t]) +
-                  __shfl_xor_sync(0xffffffffu, hi ? acc[i % A][t] : acc[i % A][E + t], T::L);
+    for (int t = 0; t < T::E; ++t) {
+      float x[T::NWQ];
 #pragma unroll
-    for (int t = 0; t < E; ++t) out[t] = q[0][t] + q[1][t];
+      for (int w = 0; w < T::NWQ; ++w)
+        x[w] = buf[((w0 + w) * EW + T::E * me.wq + t) * 32 + me.lane];
+      out[t] = T::NWQ == 2 ? x[0] + x[1] : (x[0] + x[1]) + (x[2 % T::NWQ] + x[3 % T::NWQ]);
+    }
   }
 }
+template <int W, int S>
+constexpr int kReduceFloats = QTeam<W, S>::NWQ > 1 ? 2 * Q_WARPS * QTeam<W, S>::EW * 32 : 1;
+
+// Blocks of the layout are dealt to teams in order.  The grid is described by
+// its virtual blocks of TV teams: virtual block vb's team w takes blocks
+// vb TV + w + i (all teams).  A thread block runs TB / TV virtual blocks, so
+// which rows a team takes (and with it the grouping of the objective's sums)
+// does not depend on the team's width.
+template <int W, int S>
+struct QuadDeal {
+  int vb, first, step, rounds;
+  __device__ __forceinline__ QuadDeal(const QLane<W, S>& me, int blocks, int nvb) {
+    using T = QTeam<W, S>;
+    vb = blockIdx.x * (T::TB / T::TV) + me.team / T::TV;
+    step = nvb * T::TV;
+    first = vb < nvb ? vb * T::TV + me.team % T::TV : blocks;
+    rounds = (blocks + step - 1) / step;  // uniform over the grid
+  }
+  // starts the loads of the first block's extent and rows
+  __device__ __forceinline__ void warm(const DevQuad& M) const {
+    if (first < M.blocks) {
+      asm volatile("prefetch.global.L1 [%0];" ::"l"(M.off + first));
+      asm volatile("prefetch.global.L1 [%0];" ::"l"(M.rows + QROWS * first));
+    }
+  }
+  __device__ __forceinline__ int block(const DevQuad& M, int i) const {
+    const int q = first + i * step;
+    return first < M.blocks && q < M.blocks ? q : -1;
+  }
+};
 
 // Rows are dealt to teams in the order M.order.  The grid is described by its
 // virtual blocks of P_WARPS teams: virtual block vb's team w takes the rows at
@@ -298,104 +462,115 @@ __device__ __forceinline__ void store_row_sums(const BFwdArgs& a, const float (&
   }
 }
 
-// W: slots the launch works on (every live slot is below it); a.Kp: the row
-// stride of the slot-minor arrays, at least W.
-template <int W, bool BF16, int NZ>
-__global__ void __launch_bounds__(P_THREADS, 2) k_bforward(BFwdArgs a) {
-  using T = Team<W>;
-  constexpr int E = T::E;
-  __shared__ float dsum_hi[P_WARPS * T::RW][W], dsum_lo[P_WARPS * T::RW][W];
+// Slots are worked on W at a time: blockIdx.y takes those from y W on (every
+// live slot is below gridDim.y W); a.Kp: the row stride of the slot-minor
+// arrays.
+template <int W, int S, bool BF16, int NZ>
+__global__ void __launch_bounds__(Q_THREADS, Q_PER_SM) k_bforward(BFwdArgs a) {
+  using T = QTeam<W, S>;
+  constexpr int E = T::E, V = T::V;
+  __shared__ float s_th[W];
+  __shared__ float d_hi[T::TB * QROWS][W], d_lo[T::TB * QROWS][W];  // data terms by team and row
+  __shared__ float s_x[kReduceFloats<W, S>];
   BatchState* bs = a.bst;
-  if (a.mode == 0 && bs->remaining == 0) return;  // uniform over the grid
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int Kp = a.Kp;
-  const int G = bs->gstep;
-  const float* f = a.f[G % 3];
+  const int remaining = bs->remaining, G = bs->gstep;
+  const QLane<W, S> me;
+  const QuadDeal<W, S> deal(me, a.QA.blocks, a.n_spmv_blocks);
+  deal.warm(a.QA);
+  const int tid = threadIdx.x;
+  const int Kp = a.Kp, s0 = blockIdx.y * W;
+  const float* f = a.f[G % 3] + s0;
   float* y_out = a.y[G & 1];
   const float* y_prev = a.y[(G + 1) & 1];
   const bool want = a.track != 0;
   // a first forward phase (of a run, or of admitted slots): f^{k-1} = f^k, so
   // the extrapolated projection is y itself
   const bool first = a.mode != 0;
+  SlotState* slots = a.slots + s0;
   auto live = [&](const SlotState& sl) {
     return a.mode == 2 ? sl.fresh : (sl.active && !sl.done);
   };
-  const int sl0 = owned_slot<W>(lane), gl0 = gathered_slot<W>(lane);
-  int on[E];
-  float th_h[E];
-  bool any_on = false, gather_on = false;
+  unsigned on = 0;  // the lane's live owned slots
+  bool gather_on = false;
 #pragma unroll
-  for (int t = 0; t < E; ++t) {
-    const SlotState& sl = a.slots[sl0 + t];
-    on[t] = live(sl);
-    th_h[t] = first ? 0.f : sl.theta_hi;
-    any_on = any_on || on[t];
-  }
+  for (int t = 0; t < E; ++t)
+    on |= live(slots[me.slot + t / V * T::STRIDE + t % V]) ? 1u << t : 0u;
 #pragma unroll
   for (int t = 0; t < T::Q; ++t)
-    gather_on = gather_on || live(a.slots[gl0 + t % 4 + t / 4 * T::GSTRIDE]);
-  float dh[E], dl[E];
-  int hits[E];
+    gather_on = gather_on || live(slots[me.gathered() + t / 4 * T::STRIDE + t % 4]);
+  for (int t = tid; t < W; t += Q_THREADS) s_th[t] = first ? 0.f : slots[t].theta_hi;
+  if (a.mode == 0 && remaining == 0) return;  // uniform over the grid
+  float* my_hi = d_hi[me.team * QROWS + me.row];
+  float* my_lo = d_lo[me.team * QROWS + me.row];
 #pragma unroll
-  for (int t = 0; t < E; ++t) {
-    dh[t] = 0.f;
-    dl[t] = 0.f;
-    hits[t] = 0;
-  }
+  for (int t = 0; t < E; ++t)
+    my_hi[me.slot + t / V * T::STRIDE + t % V] = my_lo[me.slot + t / V * T::STRIDE + t % V] = 0.f;
+  __syncthreads();
   // the momentum of the next index, so that the pixel phase's last block only
   // copies it: its FP64 powers take about 5 us, here beside the projections
   // of the block's other warps
-  if (blockIdx.x == 0 && tid >= P_THREADS - W) {
-    SlotState& sl = a.slots[tid - (P_THREADS - W)];
-    if (live(sl)) next_momentum(sl);
-  }
+  if (blockIdx.x == 0 && tid >= Q_THREADS - W && live(slots[tid - (Q_THREADS - W)]))
+    next_momentum(slots[tid - (Q_THREADS - W)]);
   const uint64_t pol = evict_first_policy();
-  const RowDeal<W> deal(a.A.rows, a.n_spmv_blocks);
-  for (int i = 0; i < deal.rounds; ++i) {
-    const int row = deal.row(a.A, i);
+  for (int r = 0; r < deal.rounds; ++r) {
+    const int b = deal.block(a.QA, r);
+    unsigned long long sums[QROWS][T::Q / 2];
+    quad_sums<W, S, BF16, NZ>(a.QA, b, f, Kp, me, gather_on, pol, sums);
+    const int row = b >= 0 ? __ldg(a.QA.rows + QROWS * b + me.row) : -1;
     float acc[E];
-    team_dot<W, BF16, NZ>(a.A, row, f, Kp, lane, gather_on, pol, acc);
-    if (row < 0 || !any_on) continue;
-    const size_t o = (size_t)row * Kp + sl0;
-    float yp[E], gg[E], gm[E], wo[E];
-    if (first) {
+    quad_reduce<W, S>(sums, me, s_x, r & 1, acc);
+    if (row < 0 || on == 0) continue;
 #pragma unroll
-      for (int t = 0; t < E; ++t) yp[t] = acc[t];
-    } else {
-      vload<E>(y_prev + o, yp);
-    }
-    vload<E>(a.g + o, gg);
-    vload<E>(a.gamma + o, gm);
+    for (int i = 0; i < E / V; ++i) {
+      const int sl = me.slot + i * T::STRIDE;
+      const size_t o = (size_t)row * Kp + s0 + sl;
+      float yp[V], gg[V], gm[V], wo[V], yo[V];
+      if (!first) vload<V>(y_prev + o, yp);
+      vload<V>(a.g + o, gg);
+      vload<V>(a.gamma + o, gm);
 #pragma unroll
-    for (int t = 0; t < E; ++t) {
-      wo[t] = 0.f;
-      if (!on[t]) continue;
-      // y~ = y + theta (y - y_prev); den = max(y~ + gamma, kappa gamma); w = (den - g)/den
-      const float yt = first ? acc[t] : fmaf(th_h[t], acc[t] - yp[t], acc[t]);
-      float den = yt + gm[t];
-      const float fl = 1e-3f * gm[t];
-      if (den < fl) {
-        den = fl;
-        ++hits[t];
+      for (int j = 0; j < V; ++j) {
+        const int t = V * i + j;
+        const float y = acc[t];
+        yo[j] = y;
+        wo[j] = 0.f;
+        if (!(on >> t & 1)) continue;
+        // y~ = y + theta (y - y_prev); den = max(y~ + gamma, kappa gamma); w = (den - g)/den
+        const float yt = first ? y : fmaf(s_th[sl + j], y - yp[j], y);
+        float den = yt + gm[j];
+        const float fl = 1e-3f * gm[j];
+        if (den < fl) {
+          den = fl;
+          atomicAdd(&slots[sl + j].guard_hits, 1ull);
+        }
+        wo[j] = __fdiv_rn(den - gg[j], den);
+        if (want) {
+          // data term y - g ln(y + gamma) in double-float
+          df yg;
+          two_sum(y, gm[j], yg.hi, yg.lo);
+          const df term = df_add_f(df_neg(df_mul_f(df_log(yg), gg[j])), y);
+          acc_add(my_hi[sl + j], my_lo[sl + j], term.hi, term.lo);
+        }
       }
-      wo[t] = __fdiv_rn(den - gg[t], den);
-      if (want) {
-        // data term y - g ln(y + gamma) in double-float
-        df yg;
-        two_sum(acc[t], gm[t], yg.hi, yg.lo);
-        const df term = df_add_f(df_neg(df_mul_f(df_log(yg), gg[t])), acc[t]);
-        acc_add(dh[t], dl[t], term.hi, term.lo);
-      }
+      const unsigned m = on >> (V * i) & ((1u << V) - 1);
+      vstore<V>(y_out + o, yo, m);
+      vstore<V>(a.w + o, wo, m);
     }
-    vstore_on<E>(y_out + o, acc, on);
-    vstore_on<E>(a.w + o, wo, on);
   }
-#pragma unroll
-  for (int t = 0; t < E; ++t)
-    if (hits[t]) atomicAdd(&a.slots[sl0 + t].guard_hits, (unsigned long long)hits[t]);
   if (!want) return;
-  // an admission pass writes only the fresh slots' columns
-  store_row_sums<W>(a, dh, dl, dsum_hi, dsum_lo, live);
+  // One row of per-slot sums per virtual block, in the columns of the live
+  // slots: its teams' rows in order.  An admission pass writes only the fresh
+  // slots' columns.
+  __syncthreads();
+  constexpr int VBB = T::TB / T::TV;
+  for (int q = tid; q < VBB * W; q += Q_THREADS) {
+    const int s = q % W, vb = blockIdx.x * VBB + q / W;
+    if (vb >= a.n_spmv_blocks || !live(slots[s])) continue;
+    float h = 0.f, l = 0.f;
+    for (int r = 0; r < T::TV * QROWS; ++r)
+      acc_add(h, l, d_hi[q / W * T::TV * QROWS + r][s], d_lo[q / W * T::TV * QROWS + r][s]);
+    a.fpartial[(size_t)vb * Kp + s0 + s] = make_float2(h, l);
+  }
 }
 
 // -------------------------------------------------------------- k_bstencil
@@ -672,16 +847,16 @@ __global__ void __launch_bounds__(256) k_sum_columns(const float2* __restrict__ 
 
 // Per-slot sums of the forward phase's rows in OBJ_GROUPS groups (rows g,
 // g + OBJ_GROUPS, ...), summed by the pixel phase's first blocks; the last
-// block adds the group sums.  Every sum runs in four parts combined in order,
+// block adds the group sums.  Every sum runs in two parts combined in order,
 // whatever the grid and the slots' number.
 constexpr int OBJ_GROUPS = 64;
-constexpr int OBJ_PARTS = P_THREADS / MAXK;
+constexpr int OBJ_PARTS = Q_THREADS / MAXK;
 __device__ void sum_rows(const float2* rows, int first, int step, int count, int Kp,
-                         float (&r_hi)[P_THREADS], float (&r_lo)[P_THREADS]) {
+                         float (&r_hi)[Q_THREADS], float (&r_lo)[Q_THREADS]) {
   const int s = threadIdx.x % MAXK, part = threadIdx.x / MAXK;
   float h = 0.f, l = 0.f;
   if (s < Kp) {
-#pragma unroll 4
+#pragma unroll 16
     for (int i = first + part * step; i < count; i += OBJ_PARTS * step) {
       const float2 v = __ldcg(rows + (size_t)i * Kp + s);
       acc_add(h, l, v.x, v.y);
@@ -701,112 +876,116 @@ __device__ void sum_rows(const float2* rows, int first, int step, int count, int
   __syncthreads();
 }
 
-template <int W, bool BF16, int NZ>
-__global__ void __launch_bounds__(P_THREADS, 2) k_bpixel(BPixArgs a) {
-  using T = Team<W>;
-  constexpr int E = T::E;
-  __shared__ float r_hi[P_THREADS], r_lo[P_THREADS];
+template <int W, int S, bool BF16, int NZ>
+__global__ void __launch_bounds__(Q_THREADS, Q_PER_SM) k_bpixel(BPixArgs a) {
+  using T = QTeam<W, S>;
+  constexpr int E = T::E, V = T::V;
+  __shared__ float r_hi[Q_THREADS], r_lo[Q_THREADS];
+  __shared__ float s_th[W], s_beta[W];
+  __shared__ int s_frz[W];  // -1: P from f^k; 0: the same, kept as f^{K_P}; 1: P from f^{K_P}
+  __shared__ float s_x[kReduceFloats<W, S>];
   __shared__ int s_last;
   BatchState* bs = a.bst;
-  if (bs->remaining == 0) return;  // uniform over the grid
+  const int remaining = bs->remaining, G = bs->gstep;
+  const QLane<W, S> me;
+  const QuadDeal<W, S> deal(me, a.QT.blocks, a.n_blocks);
+  deal.warm(a.QT);
   const int tid = threadIdx.x, lane = tid & 31;
-  const int Kp = a.Kp;
-  const int G = bs->gstep;
+  const int Kp = a.Kp, s0 = blockIdx.y * W;
+  if (remaining == 0) return;  // uniform over the grid
   const float* fk = a.f[G % 3];
   const float* fkm = a.f[(G + 2) % 3];
   float* fn = a.f[(G + 1) % 3];
-  bool any_back = false;
   // every slot's Phi(f^k): the forward phase's rows, first because these
   // blocks start first
-  if (a.track)
+  if (a.track && blockIdx.y == 0)
     for (int g = blockIdx.x; g < OBJ_GROUPS; g += gridDim.x) {
       sum_rows(a.fpartial, g, OBJ_GROUPS, a.n_fpartial, Kp, r_hi, r_lo);
       if (tid < Kp) a.partial[(size_t)g * Kp + tid] = make_float2(r_hi[tid], r_lo[tid]);
     }
-  // this lane's slot parameters
-  const int sl0 = owned_slot<W>(lane), gl0 = gathered_slot<W>(lane);
-  float th[E], beta[E];
-  int live[E], kk[E], frz[E], back[E];
-  bool gather_live = false;
+  const SlotState* slots = a.slots + s0;
+  unsigned live = 0, back = 0;  // the lane's owned slots
+  bool gather_on = false;
+  int freeze = 0;
 #pragma unroll
   for (int t = 0; t < E; ++t) {
-    const SlotState& sl = a.slots[sl0 + t];
-    th[t] = sl.theta_hi;
-    beta[t] = sl.beta;
-    live[t] = sl.active && !sl.done;
-    kk[t] = sl.k;
-    frz[t] = sl.freeze_iter;
-    back[t] = sl.rollback;
-    any_back = any_back || back[t];
+    const SlotState& sl = slots[me.slot + t / V * T::STRIDE + t % V];
+    live |= sl.active && !sl.done ? 1u << t : 0u;
+    back |= sl.rollback ? 1u << t : 0u;
+    freeze |= sl.freeze_iter >= 0;
   }
 #pragma unroll
   for (int t = 0; t < T::Q; ++t) {
-    const SlotState& sl = a.slots[gl0 + t % 4 + t / 4 * T::GSTRIDE];
-    gather_live = gather_live || (sl.active && !sl.done);
+    const SlotState& sl = slots[me.gathered() + t / 4 * T::STRIDE + t % 4];
+    gather_on = gather_on || (sl.active && !sl.done);
   }
+  for (int t = tid; t < W; t += Q_THREADS) {
+    const SlotState& sl = slots[t];
+    s_th[t] = sl.theta_hi;
+    s_beta[t] = sl.beta;
+    s_frz[t] = sl.freeze_iter < 0 || sl.k < sl.freeze_iter ? -1 : sl.k > sl.freeze_iter;
+  }
+  __syncthreads();
   const uint64_t pol = evict_first_policy();
   int bad = 0;
-  const RowDeal<W> deal(a.At.rows, a.n_blocks);
-  for (int i = 0; i < deal.rounds; ++i) {
-    const int j = deal.row(a.At, i);
+  for (int r = 0; r < deal.rounds; ++r) {
+    const int b = deal.block(a.QT, r);
+    unsigned long long sums[QROWS][T::Q / 2];
+    quad_sums<W, S, BF16, NZ>(a.QT, b, a.w + s0, Kp, me, gather_on, pol, sums);
+    const int j = b >= 0 ? __ldg(a.QT.rows + QROWS * b + me.row) : -1;
     float bp[E];
-    team_dot<W, BF16, NZ>(a.At, j, a.w, Kp, lane, gather_live, pol, bp);
+    quad_reduce<W, S>(sums, me, s_x, r & 1, bp);
     if (j < 0) continue;
-    const size_t o = (size_t)j * Kp + sl0;
-    float vk[E], vd[E], lo[E], gr[E], out[E];
-    vload<E>(fk + o, vk);
-    vload<E>(a.delta + o, vd);
-    vload<E>(a.low + o, lo);
-    vload<E>(a.gR + o, gr);
     const float il = __ldg(a.inv_lambda + j);
 #pragma unroll
-    for (int t = 0; t < E; ++t) {
-      if (!live[t]) {
-        // finished or empty slot: carry the image (the previous entry when
-        // the slot stopped one step back)
-        out[t] = vk[t];
-        continue;
-      }
-      float pk = vk[t];
-      if (frz[t] >= 0) {
-        if (kk[t] == frz[t]) {
-          a.pfreeze[o + t] = vk[t];
-        } else if (kk[t] > frz[t]) {
-          pk = a.pfreeze[o + t];
+    for (int i = 0; i < E / V; ++i) {
+      const int sl = me.slot + i * T::STRIDE;
+      const size_t o = (size_t)j * Kp + s0 + sl;
+      float vk[V], vd[V], lo[V], gr[V], out[V];
+      vload<V>(fk + o, vk);
+      vload<V>(a.delta + o, vd);
+      vload<V>(a.low + o, lo);
+      vload<V>(a.gR + o, gr);
+#pragma unroll
+      for (int u = 0; u < V; ++u) {
+        const int t = V * i + u;
+        if (!(live >> t & 1)) {
+          // finished or empty slot: carry the image (the previous entry when
+          // the slot stopped one step back)
+          out[u] = back >> t & 1 ? fkm[o + u] : vk[u];
+          continue;
         }
+        float pk = vk[u];
+        if (freeze) {
+          if (s_frz[sl + u] == 0) a.pfreeze[o + u] = vk[u];
+          if (s_frz[sl + u] == 1) pk = a.pfreeze[o + u];
+        }
+        // f^{k+1} = max(f^k + step, 0), step = theta (f^k - f^{k-1}) - p (grad F +
+        // grad R): what rounding f^{k+1} to FP32 leaves over is kept in low, and
+        // the step itself is the next f^k - f^{k-1}
+        const float p = s_beta[sl + u] * pk * il;
+        const float step = __fmaf_rn(s_th[sl + u], vd[u], -__fmul_rn(p, bp[t] + gr[u]));
+        const float full = __fadd_rn(vk[u], lo[u]);
+        float xv, rest;
+        two_sum(vk[u], __fadd_rn(lo[u], step), xv, rest);
+        if (!isfinite(xv)) bad = 1;
+        const bool pos = xv > 0.f;
+        out[u] = pos ? xv : 0.f;
+        vd[u] = pos ? step : -full;
+        lo[u] = pos ? rest : 0.f;
       }
-      // f^{k+1} = max(f^k + step, 0), step = theta (f^k - f^{k-1}) - p (grad F +
-      // grad R): what rounding f^{k+1} to FP32 leaves over is kept in low, and
-      // the step itself is the next f^k - f^{k-1}
-      const float p = beta[t] * pk * il;
-      const float step = __fmaf_rn(th[t], vd[t], -__fmul_rn(p, bp[t] + gr[t]));
-      const float full = __fadd_rn(vk[t], lo[t]);
-      float xv, rest;
-      two_sum(vk[t], __fadd_rn(lo[t], step), xv, rest);
-      if (!isfinite(xv)) bad = 1;
-      const bool pos = xv > 0.f;
-      out[t] = pos ? xv : 0.f;
-      vd[t] = pos ? step : -full;
-      lo[t] = pos ? rest : 0.f;
+      const unsigned m = live >> (V * i) & ((1u << V) - 1);
+      vstore<V>(fn + o, out, (1u << V) - 1);
+      vstore<V>(a.delta + o, vd, m);
+      vstore<V>(a.low + o, lo, m);
     }
-    if (any_back) {
-#pragma unroll
-      for (int t = 0; t < E; ++t)
-        if (back[t]) out[t] = fkm[o + t];
-    }
-    vstore_on<E>(a.delta + o, vd, live);
-    vstore_on<E>(a.low + o, lo, live);
-    int on[E];
-#pragma unroll
-    for (int t = 0; t < E; ++t) on[t] = 1;
-    vstore_on<E>(fn + o, out, on);
   }
   if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(&bs->flags, APPGA_FLAG_NONFINITE);
   // Finalise the step in the last block: Phi and the stopping test of every
   // live slot, then its next index and momentum; the global step advances.
   __threadfence();
   __syncthreads();
-  if (tid == 0) s_last = atomicAdd(&bs->ticket_p, 1u) == gridDim.x - 1;
+  if (tid == 0) s_last = atomicAdd(&bs->ticket_p, 1u) == gridDim.x * gridDim.y - 1;
   __syncthreads();
   if (s_last) {
     __threadfence();
@@ -886,7 +1065,7 @@ __global__ void __launch_bounds__(P_THREADS, 2) k_bpixel(BPixArgs a) {
       sl.t_cur = sl.t_next;
       bset_theta(sl, sl.theta_next);
     }
-    static_assert(P_THREADS >= MAXK, "one slot per thread");
+    static_assert(Q_THREADS >= MAXK, "one slot per thread");
     const int tot = __syncthreads_count(rem);
     if (tid == 0) {
       bs->gstep = G + 1;
@@ -1049,10 +1228,18 @@ __global__ void __launch_bounds__(256) k_binit_image(const float2* __restrict__ 
 
 int sm_count() { return current_sm_count(); }
 
-// Virtual blocks of the forward phase's projector rows.
+// Small matrices run 16 groups per block of rows (a rule on the matrix alone, so
+// that a slice's result does not depend on its batch): below two teams per
+// resident warp at four groups a block.  5 slots of 128 x 128 (4.1 k blocks):
+// 37 us per map with four groups, 32.6 with 16.
+bool many_groups(const DevQuad& M) { return M.blocks < 2 * Q_PER_SM * Q_WARPS * sm_count(); }
+int virtual_blocks(const DevQuad& M, int per_sm) {
+  const int tv = many_groups(M) ? 1 : 4;
+  return std::min((M.blocks + tv - 1) / tv, sm_count() * per_sm);
+}
+// Virtual blocks of the forward phase's projection.
 int fw_blocks(const BFwdArgs& a) {
-  const int nb = (a.A.rows + P_WARPS - 1) / P_WARPS;
-  return std::min(nb, sm_count() * clamp_per_sm(a.spmv_per_sm, kSpmvPerSm));
+  return virtual_blocks(a.QA, clamp_per_sm(a.spmv_per_sm, kSpmvPerSm));
 }
 // Stencil blocks per slot chunk: equal tile counts per block.
 int st_blocks(const BFwdArgs& a) {
@@ -1064,43 +1251,72 @@ int st_blocks(const BFwdArgs& a) {
 }
 
 // Gather probe: the batched projectors' inner loop alone.  Every row of M is
-// reduced against the W-wide slot-minor rows of x by team_dot, dealt to the
-// teams as in the projections, with no epilogue, stencil or pixel update.
-template <int W>
-__global__ void __launch_bounds__(P_THREADS, 2) k_gather_probe(DevCSR M, const float* __restrict__ x,
-                                                               int nvb, float* __restrict__ sink) {
-  const int lane = threadIdx.x & 31;
+// reduced against the slot-minor rows of x by quad_dot, dealt to the teams as
+// in the projections, with no epilogue, stencil or pixel update.
+template <int W, int S>
+__global__ void __launch_bounds__(Q_THREADS, Q_PER_SM) k_gather_probe(DevQuad M,
+                                                                      const float* __restrict__ x,
+                                                                      int Kp, int nvb,
+                                                                      float* __restrict__ sink) {
+  __shared__ float s_x[kReduceFloats<W, S>];
   const uint64_t pol = evict_first_policy();
-  const RowDeal<W> deal(M.rows, nvb);
+  const QLane<W, S> me;
+  const QuadDeal<W, S> deal(me, M.blocks, nvb);
   float s = 0.f;
   for (int i = 0; i < deal.rounds; ++i) {
-    float acc[Team<W>::E];
-    team_dot<W, false, 4>(M, deal.row(M, i), x, W, lane, true, pol, acc);
+    float acc[QTeam<W, S>::E];
+    unsigned long long sums[QROWS][QTeam<W, S>::Q / 2];
+    quad_sums<W, S, false, 4>(M, deal.block(M, i), x + blockIdx.y * W, Kp, me, true, pol, sums);
+    quad_reduce<W, S>(sums, me, s_x, i & 1, acc);
 #pragma unroll
-    for (int t = 0; t < Team<W>::E; ++t) s += acc[t];
+    for (int t = 0; t < QTeam<W, S>::E; ++t) s += acc[t];
   }
   if (s == 1.0e38f) sink[blockIdx.x] = s;  // keeps the loads; the value is never used
 }
 
-template <int W>
-int blocks_of(int nvb) {
-  return (nvb + Team<W>::RW - 1) / Team<W>::RW;
+// Thread blocks of nvb virtual blocks over the slots of `width`, W at a time.
+template <int W, int S>
+dim3 grid_of(int nvb, int width) {
+  constexpr int vbb = QTeam<W, S>::TB / QTeam<W, S>::TV;
+  return dim3((nvb + vbb - 1) / vbb, width / W);
 }
 
 template <int W>
 cudaError_t bforward_w(const BFwdArgs& a, cudaStream_t s) {
-  const bool g4 = a.gather_rows == 4;
-  void (*kern)(BFwdArgs) = a.use_bf16 ? (g4 ? k_bforward<W, true, 2> : k_bforward<W, true, 4>)
-                                      : (g4 ? k_bforward<W, false, 2> : k_bforward<W, false, 4>);
-  kern<<<blocks_of<W>(a.n_spmv_blocks), P_THREADS, 0, s>>>(a);
+  if (many_groups(a.QA)) {
+    void (*kern)(BFwdArgs) = a.use_bf16 ? k_bforward<W, 16, true, 4> : k_bforward<W, 16, false, 4>;
+    kern<<<grid_of<W, 16>(a.n_spmv_blocks, a.width), Q_THREADS, 0, s>>>(a);
+  } else {
+    const bool g4 = a.gather_rows == 4;
+    void (*kern)(BFwdArgs) =
+        a.use_bf16 ? (g4 ? k_bforward<W, 4, true, 2> : k_bforward<W, 4, true, 4>)
+                   : (g4 ? k_bforward<W, 4, false, 2> : k_bforward<W, 4, false, 4>);
+    kern<<<grid_of<W, 4>(a.n_spmv_blocks, a.width), Q_THREADS, 0, s>>>(a);
+  }
   return cudaGetLastError();
 }
 template <int W>
 cudaError_t bpixel_w(const BPixArgs& a, cudaStream_t s) {
-  const bool g4 = a.gather_rows == 4;
-  void (*kern)(BPixArgs) = a.use_bf16 ? (g4 ? k_bpixel<W, true, 2> : k_bpixel<W, true, 4>)
-                                      : (g4 ? k_bpixel<W, false, 2> : k_bpixel<W, false, 4>);
-  kern<<<blocks_of<W>(a.n_blocks), P_THREADS, 0, s>>>(a);
+  if (many_groups(a.QT)) {
+    void (*kern)(BPixArgs) = a.use_bf16 ? k_bpixel<W, 16, true, 4> : k_bpixel<W, 16, false, 4>;
+    kern<<<grid_of<W, 16>(a.n_blocks, a.width), Q_THREADS, 0, s>>>(a);
+  } else {
+    const bool g4 = a.gather_rows == 4;
+    void (*kern)(BPixArgs) =
+        a.use_bf16 ? (g4 ? k_bpixel<W, 4, true, 2> : k_bpixel<W, 4, true, 4>)
+                   : (g4 ? k_bpixel<W, 4, false, 2> : k_bpixel<W, 4, false, 4>);
+    kern<<<grid_of<W, 4>(a.n_blocks, a.width), Q_THREADS, 0, s>>>(a);
+  }
+  return cudaGetLastError();
+}
+template <int W>
+cudaError_t probe_w(const DevQuad& M, const float* x, int Kp, float* sink, int per_sm,
+                    cudaStream_t s) {
+  const int nvb = virtual_blocks(M, per_sm);
+  if (many_groups(M))
+    k_gather_probe<W, 16><<<grid_of<W, 16>(nvb, Kp), Q_THREADS, 0, s>>>(M, x, Kp, nvb, sink);
+  else
+    k_gather_probe<W, 4><<<grid_of<W, 4>(nvb, Kp), Q_THREADS, 0, s>>>(M, x, Kp, nvb, sink);
   return cudaGetLastError();
 }
 
@@ -1132,8 +1348,8 @@ cudaError_t launch_bforward(const BFwdArgs& a0, cudaStream_t s) {
     case 8: return bforward_w<8>(a, s);
     case 16: return bforward_w<16>(a, s);
     case 32: return bforward_w<32>(a, s);
-    case 64: return bforward_w<64>(a, s);
-    case 128: return bforward_w<128>(a, s);
+    case 64:
+    case 128: return bforward_w<64>(a, s);
   }
   return cudaErrorInvalidValue;
 }
@@ -1150,10 +1366,11 @@ cudaError_t launch_bstencil(const BFwdArgs& a0, cudaStream_t s) {
 namespace {
 template <int W>
 cudaError_t bobjective_w(const BFwdArgs& a, cudaStream_t s) {
+  const int grid = (a.n_spmv_blocks + Team<W>::RW - 1) / Team<W>::RW;
   if (a.use_bf16)
-    k_bobjective<W, true><<<blocks_of<W>(a.n_spmv_blocks), P_THREADS, 0, s>>>(a);
+    k_bobjective<W, true><<<grid, P_THREADS, 0, s>>>(a);
   else
-    k_bobjective<W, false><<<blocks_of<W>(a.n_spmv_blocks), P_THREADS, 0, s>>>(a);
+    k_bobjective<W, false><<<grid, P_THREADS, 0, s>>>(a);
   return cudaGetLastError();
 }
 }  // namespace
@@ -1164,7 +1381,8 @@ cudaError_t launch_bobjective(const BFwdArgs& a0, int K, double* out, cudaStream
   BFwdArgs a = a0;
   a.mode = 3;
   a.track = 1;
-  a.n_spmv_blocks = fw_blocks(a);
+  a.n_spmv_blocks =
+      std::min((a.A.rows + P_WARPS - 1) / P_WARPS, sm_count() * kObjectivePerSm);
   switch (a.width) {
     case 8: e = bobjective_w<8>(a, s); break;
     case 16: e = bobjective_w<16>(a, s); break;
@@ -1173,35 +1391,36 @@ cudaError_t launch_bobjective(const BFwdArgs& a0, int K, double* out, cudaStream
     case 128: e = bobjective_w<128>(a, s); break;
     default: e = cudaErrorInvalidValue;
   }
-  if (e == cudaSuccess) e = launch_bstencil(a, s);
+  const int nst = st_blocks(a);
+  if (e == cudaSuccess && nst > 0) {
+    k_bstencil<<<dim3(nst, a.width / BST_S), B_THREADS, 0, s>>>(a);
+    e = cudaGetLastError();
+  }
   if (e != cudaSuccess) return e;
-  k_sum_columns<<<K, 256, 0, s>>>(a.fpartial, a.n_spmv_blocks, st_blocks(a), a.Kp, out);
+  k_sum_columns<<<K, 256, 0, s>>>(a.fpartial, a.n_spmv_blocks, nst, a.Kp, out);
   return cudaGetLastError();
 }
 
-cudaError_t launch_gather_probe(const DevCSR& M, const float* x, int Kp, float* sink,
+cudaError_t launch_gather_probe(const DevQuad& M, const float* x, int Kp, float* sink,
                                 int blocks_per_sm, cudaStream_t s) {
   if (blocks_per_sm < 1 || blocks_per_sm > kMaxPerSm) return cudaErrorInvalidValue;
-  const int grid = std::min((M.rows + P_WARPS - 1) / P_WARPS, sm_count() * blocks_per_sm);
   switch (Kp) {
-    case 32: k_gather_probe<32><<<grid, P_THREADS, 0, s>>>(M, x, grid, sink); break;
-    case 64: k_gather_probe<64><<<grid, P_THREADS, 0, s>>>(M, x, grid, sink); break;
-    case 128: k_gather_probe<128><<<grid, P_THREADS, 0, s>>>(M, x, grid, sink); break;
-    default: return cudaErrorInvalidValue;
+    case 32: return probe_w<32>(M, x, Kp, sink, blocks_per_sm, s);
+    case 64:
+    case 128: return probe_w<64>(M, x, Kp, sink, blocks_per_sm, s);
   }
-  return cudaGetLastError();
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_bpixel(const BPixArgs& a0, cudaStream_t s) {
   BPixArgs a = a0;
-  a.n_blocks = std::min((a.At.rows + P_WARPS - 1) / P_WARPS,
-                        sm_count() * clamp_per_sm(a.blocks_per_sm, kPixelPerSm));
+  a.n_blocks = virtual_blocks(a.QT, clamp_per_sm(a.blocks_per_sm, kPixelPerSm));
   switch (a.width) {
     case 8: return bpixel_w<8>(a, s);
     case 16: return bpixel_w<16>(a, s);
     case 32: return bpixel_w<32>(a, s);
-    case 64: return bpixel_w<64>(a, s);
-    case 128: return bpixel_w<128>(a, s);
+    case 64:
+    case 128: return bpixel_w<64>(a, s);
   }
   return cudaErrorInvalidValue;
 }

@@ -169,6 +169,11 @@ appga_status create_pool(appga_server* S, int geom, int Kp, Pool** out) {
   P->bytes = pool_bytes(M, Kp);
   cudaError_t e = alloc_batch_workspace(P->b, M->m, M->d, Kp);
   if (e != cudaSuccess) return cuda_fail(e, "server pool workspace");
+  const appga_status rq = ensure_quads(const_cast<appga_matrix*>(M), S->ctx->stream);
+  if (rq != APPGA_OK) {
+    free_pool(P.get());
+    return rq;
+  }
   const size_t in_len = (size_t)Kp * (2 * (size_t)M->m + M->d);
   const size_t out_len = (size_t)Kp * M->d;
   e = cudaStreamCreateWithFlags(&P->stream, cudaStreamNonBlocking);
@@ -186,8 +191,7 @@ appga_status create_pool(appga_server* S, int geom, int Kp, Pool** out) {
     return cuda_fail(e, "server pool staging");
   }
   const bool bf16 = S->cfg.a_precision == APPGA_PREC_BF16;
-  make_batch_args(M->A, M->At, bf16 ? M->inv_lambda_bf16 : M->inv_lambda, M->n, P->b, Kp, bf16,
-                  true, tuned_schedule(M, Kp, bf16), &P->fa, &P->pa);
+  make_batch_args(M, P->b, Kp, bf16, true, tuned_schedule(M, Kp, bf16), &P->fa, &P->pa);
   cudaStream_t s = P->stream;
   // every slot starts empty; the ring starts at step 1
   appga_params def;
