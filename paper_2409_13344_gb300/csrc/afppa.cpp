@@ -5,6 +5,7 @@
 
 #include <cmath>
 #include <cstring>
+#include <string>
 
 #include "afppa_internal.h"
 #include "appga.h"
@@ -15,8 +16,9 @@ namespace appga {
 
 void free_afppa_workspace(AfppaWorkspace* aw) {
   if (!aw) return;
-  for (auto& p : aw->b) cudaFree(p);
-  for (auto& p : aw->c) cudaFree(p);
+  for (auto& kv : aw->gexec) cudaGraphExecDestroy(kv.second);
+  cudaFree(aw->duals);
+  cudaFree(aw->partial);
   cudaFree(aw->norms);
   cudaFreeHost(aw->norms_host);
   *aw = AfppaWorkspace();
@@ -32,8 +34,12 @@ appga_status ensure_afppa_workspace(appga_matrix* M) {
   auto* aw = new AfppaWorkspace();
   const size_t d = (size_t)M->d;
   cudaError_t e = cudaSuccess;
-  for (int i = 0; i < 3 && e == cudaSuccess; ++i) e = dalloc(&aw->b[i], 2 * d, &M->bytes);
-  for (int i = 0; i < 3 && e == cudaSuccess; ++i) e = dalloc(&aw->c[i], 4 * d, &M->bytes);
+  if (e == cudaSuccess) e = dalloc(&aw->duals, 18 * d, &M->bytes);
+  for (int i = 0; i < 3; ++i) {
+    aw->b[i] = aw->duals + 2 * d * i;
+    aw->c[i] = aw->duals + 6 * d + 4 * d * i;
+  }
+  if (e == cudaSuccess) e = dalloc(&aw->partial, kAfppaResultBlocks, &M->bytes);
   if (e == cudaSuccess) e = dalloc(&aw->norms, 2);
   if (e == cudaSuccess) e = cudaMallocHost((void**)&aw->norms_host, 2 * sizeof(double));
   if (e != cudaSuccess) {
@@ -67,61 +73,42 @@ extern "C" appga_status appga_afppa_reconstruct(appga_ctx* ctx, const appga_matr
   cudaStream_t s = ctx->stream;
   Workspace& ws = M->ws;
   AfppaWorkspace& aw = *M->aw;
-  if ((rc = validate_inputs(M, g, gamma, f_init, s)) != APPGA_OK) return rc;
   const bool bf16 = bf16_requested(M, p);
   const int d = M->d;
   const size_t fb = (size_t)d * sizeof(float);
 
-  // f^0 = f^1 = f_init (or TMC * 1_disk); zero duals; B^T [b~; c~] = 0
+  // start state, momentum table, f^0 = f^1 = f_init (or TMC * 1_disk) and the
+  // check of the inputs on the device; zero duals; B^T [b~; c~] = 0
   const int k0 = 1;
-  float* cur = ws.f[k0 % 3];
+  appga_params q = *p;
+  q.track_objective = 0;
+  const SolverState h = start_state(k0, &q, g, gamma);
+  if ((rc = momentum_table(M, ws.st, k0, p, s, &h)) != APPGA_OK) return rc;
+  FwdArgs fa{};
+  PixArgs pa{};
+  fa.A = M->A;
+  // the APPGA loop's projection layout (tiled gathers, sliced or folded)
+  loop_layout(M, &fa, &pa);
+  float *cur = ws.f[k0 % 3], *prev = ws.f[(k0 + 2) % 3];
   if (f_init) {
+    CK(launch_check_inputs(g, gamma, M->m, f_init, nullptr, d, ws.st, s));
     CK(cudaMemcpyAsync(cur, f_init, fb, cudaMemcpyDeviceToDevice, s));
+    CK(cudaMemcpyAsync(prev, f_init, fb, cudaMemcpyDeviceToDevice, s));
+    CK(loop_gather_copy(M, cur, s));
   } else {
     CK(launch_initial_image(g, gamma, M->m, M->n, M->na, M->npfov, ws.partial_aux, ws.gtick,
-                            ws.st_scratch, cur, s));
+                            ws.st_scratch, cur, s, prev, pa.ft, ws.st, pa.fpair));
+    if (!loop_gathers_copy()) CK(loop_gather_copy(M, cur, s));
   }
-  CK(cudaMemcpyAsync(ws.f[(k0 + 2) % 3], cur, fb, cudaMemcpyDeviceToDevice, s));
-  for (int i = 0; i < 3; ++i) {
-    CK(cudaMemsetAsync(aw.b[i], 0, 2 * fb, s));
-    CK(cudaMemsetAsync(aw.c[i], 0, 4 * fb, s));
-  }
+  CK(cudaMemsetAsync(aw.duals, 0, 18 * fb, s));
   CK(cudaMemsetAsync(ws.gR, 0, fb, s));
 
-  SolverState h{};
-  h.k = k0;
-  h.k0 = k0;
-  h.k_last = k0 + p->max_iters - 1;
-  h.done = p->max_iters == 0 ? 1 : 0;
-  h.k_next = k0;
-  h.done_next = h.done;
-  h.result_k = k0;
-  CK(cudaMemcpyAsync(ws.st, &h, sizeof h, cudaMemcpyHostToDevice, s));
-  if ((rc = momentum_table(M, ws.st, k0, p, s)) != APPGA_OK) return rc;
-
-  // y^{k0-1} = A f^{k0-1}, then the first forward phase (y^{k0}, w^{k0})
-  FwdArgs init{};
-  init.A = M->A;
-  init.use_bf16 = bf16 ? 1 : 0;
-  init.f[0] = ws.f[(k0 + 2) % 3];
-  init.y[0] = ws.y[(k0 + 1) & 1];
-  init.g = g;
-  init.gamma = gamma;
-  init.st = ws.st_scratch;
-  init.partial = ws.partial_aux;
-  init.gtick = ws.gtick;
-  init.solver_acc = 1;
-  init.n = M->n;
-  CK(launch_forward(init, s));
-  FwdArgs fa{};
-  fa.A = M->A;
+  // the first forward phase (y^{k0}, w^{k0}); f^{k0-1} = f^{k0}
   fa.use_bf16 = bf16 ? 1 : 0;
   for (int i = 0; i < 3; ++i) fa.f[i] = ws.f[i];
   fa.y[0] = ws.y[0];
   fa.y[1] = ws.y[1];
   fa.w = ws.w;
-  fa.g = g;
-  fa.gamma = gamma;
   fa.st = ws.st;
   fa.partial = ws.partial_r;
   fa.gtick = ws.gtick;
@@ -131,11 +118,9 @@ extern "C" appga_status appga_afppa_reconstruct(appga_ctx* ctx, const appga_matr
   fa.n = M->n;
   fa.ip = iter_params(p, false);
   fa.theta_tab = ws.theta_tab;
-  // the APPGA loop's projection layout (tiled gathers, sliced or folded)
-  PixArgs pa{};
-  loop_layout(M, &fa, &pa);
-  CK(loop_gather_copy(M, ws.f[k0 % 3], s));
-  CK(launch_forward(fa, s));
+  FwdArgs first = fa;
+  first.fresh_first = 1;
+  CK(launch_forward(first, s));
 
   pa.At = M->At;
   pa.n = M->n;
@@ -150,6 +135,7 @@ extern "C" appga_status appga_afppa_reconstruct(appga_ctx* ctx, const appga_matr
   pa.ip = iter_params(p, false);
   pa.use_bf16 = bf16 ? 1 : 0;
   pa.want_pmax = 1;
+  pa.fuse_fin = 1;
   pa.theta_tab = ws.theta_tab;
   DualArgs da{};
   da.n = M->n;
@@ -162,38 +148,63 @@ extern "C" appga_status appga_afppa_reconstruct(appga_ctx* ctx, const appga_matr
   }
   da.gR = ws.gR;
   da.st = ws.st;
+  da.theta_tab = ws.theta_tab;
 
   if (p->max_iters > 0) {
     const int S = p->graph_iters > 0 ? p->graph_iters : kAfppaGraphSteps;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
-    CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e = cudaSuccess;
-    for (int i = 0; i < S && e == cudaSuccess; ++i) {
-      e = launch_pixel(pa, s);
-      if (e == cudaSuccess) e = launch_afppa_dual(da, s);
-      if (e == cudaSuccess) e = launch_forward(fa, s);
+    std::string key = graph_key(p, false, bf16, S);
+    key.append(reinterpret_cast<const char*>(&ws.theta_tab), sizeof ws.theta_tab);
+    if (aw.gkey != key) {
+      for (auto& kv : aw.gexec) cudaGraphExecDestroy(kv.second);
+      aw.gexec.clear();
+      aw.gkey = key;
     }
-    const cudaError_t e2 = cudaStreamEndCapture(s, &graph);
-    if (e == cudaSuccess) e = e2;
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
-    if (graph) cudaGraphDestroy(graph);
-    const int reps = (p->max_iters + S - 1) / S;
-    for (int r = 0; r < reps && e == cudaSuccess; ++r) e = cudaGraphLaunch(exec, s);
-    if (exec) cudaGraphExecDestroy(exec);
-    if (e != cudaSuccess) return cuda_fail(e, "AFPPA graph");
+    for (const int maps : replay_plan(p->max_iters, S)) {
+      auto it = aw.gexec.find(maps);
+      if (it == aw.gexec.end()) {
+        cudaGraph_t graph = nullptr;
+        cudaGraphExec_t exec = nullptr;
+        CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
+        cudaError_t e = cudaSuccess;
+        for (int i = 0; i < maps && e == cudaSuccess; ++i) {
+          e = launch_pixel(pa, s);
+          if (e == cudaSuccess) e = launch_afppa_dual(da, s);
+          if (e == cudaSuccess) e = launch_forward(fa, s);
+        }
+        const cudaError_t e2 = cudaStreamEndCapture(s, &graph);
+        if (e == cudaSuccess) e = e2;
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
+        if (graph) cudaGraphDestroy(graph);
+        if (e != cudaSuccess) return cuda_fail(e, "AFPPA graph");
+        it = aw.gexec.emplace(maps, exec).first;
+      }
+      CK(cudaGraphLaunch(it->second, s));
+    }
   }
+  // the result (the dual update of step K wrote b^{K+1}, c^{K+1}), its relative
+  // change and the final state, with one host round trip
+  AfppaResultArgs ra{};
+  ra.d = d;
+  for (int i = 0; i < 3; ++i) {
+    ra.f[i] = ws.f[i];
+    ra.b[i] = aw.b[i];
+    ra.c[i] = aw.c[i];
+  }
+  ra.st = ws.st;
+  ra.f_out = f_out;
+  ra.b_out = b_out;
+  ra.c_out = c_out;
+  ra.partial = aw.partial;
+  ra.norms = aw.norms;
+  CK(launch_afppa_result(ra, s));
   CK(cudaMemcpyAsync(ws.st_host, ws.st, sizeof(SolverState), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
-  const SolverState fin = *ws.st_host;
-  const int rk = fin.result_k;
-  CK(cudaMemcpyAsync(f_out, ws.f[rk % 3], fb, cudaMemcpyDeviceToDevice, s));
-  // the duals of the last map: the dual update of step K wrote b^{K+1}, c^{K+1}
-  if (b_out) CK(cudaMemcpyAsync(b_out, aw.b[rk % 3], 2 * fb, cudaMemcpyDeviceToDevice, s));
-  if (c_out) CK(cudaMemcpyAsync(c_out, aw.c[rk % 3], 4 * fb, cudaMemcpyDeviceToDevice, s));
-  CK(launch_norms2(d, ws.f[rk % 3], ws.f[(rk + 2) % 3], aw.norms, s));
   CK(cudaMemcpyAsync(aw.norms_host, aw.norms, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
+  const SolverState fin = *ws.st_host;
+  if (fin.flags & APPGA_FLAG_DOMAIN)
+    return fail(APPGA_EDOMAIN,
+                "inputs must satisfy: g finite and >= 0, gamma finite and > 0, f finite and >= 0");
+  const int rk = fin.result_k;
   if (stats) {
     std::memset(stats, 0, sizeof *stats);
     stats->iters = rk - k0;

@@ -126,13 +126,11 @@ void free_workspace(Workspace& ws) {
   cudaFree(ws.theta_tab);
   cudaFree(ws.st);
   cudaFree(ws.st_scratch);
-  cudaFree(ws.flag);
   cudaFree(ws.d_g);
   cudaFree(ws.d_gamma);
   cudaFree(ws.d_finit);
   cudaFree(ws.d_fout);
   cudaFreeHost(ws.st_host);
-  cudaFreeHost(ws.flag_host);
   cudaFreeHost(ws.scalars_host);
   ws = Workspace();
 }
@@ -204,9 +202,7 @@ appga_status ensure_workspace(appga_matrix* M) {
   if (e == cudaSuccess) e = dalloc(&ws.scalars, 8, b);
   if (e == cudaSuccess) e = dalloc(&ws.st, 1, b);
   if (e == cudaSuccess) e = dalloc(&ws.st_scratch, 1, b);
-  if (e == cudaSuccess) e = dalloc(&ws.flag, 1, b);
   if (e == cudaSuccess) e = cudaMallocHost((void**)&ws.st_host, sizeof(SolverState));
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&ws.flag_host, sizeof(int));
   if (e == cudaSuccess) e = cudaMallocHost((void**)&ws.scalars_host, 8 * sizeof(double));
   if (e == cudaSuccess) e = cudaMemset(ws.st, 0, sizeof(SolverState));
   if (e == cudaSuccess) e = cudaMemset(ws.st_scratch, 0, sizeof(SolverState));
@@ -301,7 +297,7 @@ std::string graph_key(const appga_params* p, bool track, bool bf16, int S) {
 // Device state of a run at its start (iteration index k0).  A run of zero
 // maps with the objective tracked starts at done = 2: its one forward phase
 // and the last finalisation still evaluate Phi(f^{k0}).
-SolverState start_state(int32_t k0, const appga_params* p) {
+SolverState start_state(int32_t k0, const appga_params* p, const float* g, const float* gamma) {
   const bool track = p->track_objective != 0 || p->rel_obj_tol > 0.0;
   SolverState h{};
   h.k = k0;
@@ -313,6 +309,8 @@ SolverState start_state(int32_t k0, const appga_params* p) {
   h.result_k = k0;
   h.phi_cur = std::numeric_limits<double>::quiet_NaN();
   h.phi_prev = h.phi_cur;
+  h.g = g;
+  h.gamma = gamma;
   return h;
 }
 
@@ -356,8 +354,6 @@ appga_status setup_run(appga_matrix* M, const float* g, const float* gamma, int3
   fa.y[0] = ws.y[0];
   fa.y[1] = ws.y[1];
   fa.w = ws.w;
-  fa.g = g;
-  fa.gamma = gamma;
   fa.st = ws.st;
   fa.partial = ws.partial_r;
   fa.gtick = ws.gtick;
@@ -454,8 +450,8 @@ std::vector<int> replay_plan(int total, int S) {
 // Runs the maps of a prepared run (setup_run) on ctx->stream, then the last
 // finalisation of a tracked run.  With a stopping tolerance the stop flag is
 // polled one replay behind, so the device never idles on the host.
-appga_status run_maps(appga_matrix* M, const float* g, const float* gamma,
-                      const appga_params* p, const appga::FwdArgs& fa, const appga::PixArgs& pa) {
+appga_status run_maps(appga_matrix* M, const appga_params* p, const appga::FwdArgs& fa,
+                      const appga::PixArgs& pa) {
   appga_ctx* ctx = M->ctx;
   Workspace& ws = M->ws;
   cudaStream_t s = ctx->stream;
@@ -463,10 +459,9 @@ appga_status run_maps(appga_matrix* M, const float* g, const float* gamma,
   const bool bf16 = bf16_requested(M, p);
   const int S = p->graph_iters > 0 ? p->graph_iters : kDefaultGraphIters;
   if (p->max_iters > 0) {
-    // the captured kernel arguments hold the g / gamma addresses
     KeyBytes kb;
     kb.s = graph_key(p, track, bf16, S);
-    kb.add(g).add(gamma).add(ws.theta_tab);
+    kb.add(ws.theta_tab);
     const std::string& key = kb.s;
     // the whole ladder (S and every power of two below it) is captured on
     // first use of these arguments, so later calls of any length find their
@@ -568,19 +563,6 @@ appga_status check_params_and_mat(appga_ctx* ctx, const appga_matrix* M, const a
   return appga_params_validate(p);
 }
 
-appga_status validate_inputs(appga_matrix* M, const float* g, const float* gamma, const float* f,
-                             cudaStream_t s) {
-  Workspace& ws = M->ws;
-  CK(cudaMemsetAsync(ws.flag, 0, sizeof(int), s));
-  CK(appga::launch_validate_inputs(g, gamma, M->m, f, M->d, ws.flag, s));
-  CK(cudaMemcpyAsync(ws.flag_host, ws.flag, sizeof(int), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
-  if (*ws.flag_host)
-    return fail(APPGA_EDOMAIN,
-                "inputs must satisfy: g finite and >= 0, gamma finite and > 0, f finite and >= 0");
-  return APPGA_OK;
-}
-
 }  // namespace appga
 
 using namespace appga;
@@ -661,7 +643,7 @@ appga_status solve_common(appga_ctx* ctx, appga_matrix* M, const float* g, const
   // one when `direct`, inside a call graph), the last finalisation, the
   // result and the state read-back.
   auto enqueue = [&](bool direct) -> appga_status {
-    const SolverState h = start_state(k0, p);
+    const SolverState h = start_state(k0, p, g, gamma);
     appga_status r = momentum_table(M, ws.st, k0, p, s, &h);
     if (r != APPGA_OK) return r;
     float* slot_cur = ws.f[k0 % 3];
@@ -692,7 +674,7 @@ appga_status solve_common(appga_ctx* ctx, appga_matrix* M, const float* g, const
         CK(appga::launch_forward(fa, s));
       }
       if (p->track_objective != 0) CK(appga::launch_finalize(pa, s));
-    } else if ((r = run_maps(M, g, gamma, p, fa, pa)) != APPGA_OK) {
+    } else if ((r = run_maps(M, p, fa, pa)) != APPGA_OK) {
       return r;
     }
     CK(appga::launch_copy_result(ws.st, ws.f, f_out, f_out_prev, M->d, s));
@@ -1204,7 +1186,7 @@ appga_status appga_kernel_times(appga_ctx* ctx, const appga_matrix* mat, const f
   appga_params q = *params;
   q.max_iters = n_iters;
   q.rel_obj_tol = 0.0;
-  const SolverState h = start_state(1, &q);
+  const SolverState h = start_state(1, &q, g, gamma);
   if ((rc = momentum_table(M, ws.st, 1, &q, s, &h)) != APPGA_OK) return rc;
   CK(appga::launch_initial_image(g, gamma, M->m, M->n, M->na, M->npfov, ws.partial_aux, ws.gtick,
                                  ws.st_scratch, ws.f[1], s, ws.f[0]));

@@ -126,12 +126,15 @@ struct SolverState {
   unsigned int ticket_r;
   unsigned int ticket_aux;
   int32_t done_next;  // run status for the next forward phase
-  // fixed-point proximity iteration (AFPPA): theta of the step just taken,
-  // the dual step sizes from the largest preconditioner entry of that step,
-  // and that largest entry as bits (positive floats order as integers)
-  float theta_prev;
+  // fixed-point proximity iteration (AFPPA): the dual step sizes from the
+  // largest preconditioner entry of the step, and that largest entry as bits
+  // (positive floats order as integers; reset by the forward phase)
   float rho1, rho2;
   unsigned int pmax_bits;
+  // the run's sinogram and background: the loop's kernels read the addresses
+  // here, so captured loops serve any buffers
+  const float* g;
+  const float* gamma;
 };
 
 // One momentum scalar of a run: the FP64 value and its double-float split.
@@ -156,7 +159,7 @@ struct FwdArgs {
   float2* y[2];        // loop: projection ring A f^k as double-float pairs (hi, lo)
   double* y_out;       // standalone: A f in FP64
   float* w;            // back-projection weight 1 - g/den (may be null)
-  const float* g;
+  const float* g;      // standalone (the loop takes them from st)
   const float* gamma;
   float* gR;           // loop: B^T grad phi~(B f~) of the current iterate
   SolverState* st;
@@ -241,8 +244,6 @@ cudaError_t launch_stencil(int n, const float* f_cur, const float* f_prev, float
 cudaError_t launch_reg_term(int n, const float* f, float lam1, float lam2, float eps,
                             float2* partial, unsigned int* gtick, SolverState* st, double* out,
                             cudaStream_t s);
-cudaError_t launch_validate_inputs(const float* g, const float* gamma, int m, const float* f,
-                                   int d, int* flag, cudaStream_t s);
 // Solver-run input check without a host round trip: on a bad g, gamma, fa or
 // fb (fa, fb may be NULL) sets APPGA_FLAG_DOMAIN in st->flags and st->done.
 cudaError_t launch_check_inputs(const float* g, const float* gamma, int m, const float* fa,

@@ -35,8 +35,6 @@ struct Workspace {
   SolverState* st = nullptr;
   SolverState* st_scratch = nullptr;
   SolverState* st_host = nullptr;  // pinned
-  int* flag = nullptr;
-  int* flag_host = nullptr;        // pinned
   double* scalars_host = nullptr;  // pinned
   // device staging for the host-buffer entry point
   float* d_g = nullptr;
@@ -71,8 +69,13 @@ struct BatchSchedule {
 
 // Dual fields of the AFPPA solver (per matrix, allocated lazily).
 struct AfppaWorkspace {
+  float* duals = nullptr;                     // the rings below, 18 d floats
   float* b[3] = {nullptr, nullptr, nullptr};  // [2][d] first-order duals, iterate ring
   float* c[3] = {nullptr, nullptr, nullptr};  // [4][d] second-order duals
+  float4* partial = nullptr;                  // the result's block sums
+  // replays of n steps (as Workspace::gexec) for the settings in gkey
+  std::map<int, cudaGraphExec_t> gexec;
+  std::string gkey;
   double* norms = nullptr;                    // device [2]
   double* norms_host = nullptr;               // pinned [2]
 };
@@ -214,10 +217,12 @@ appga_status ensure_workspace(appga_matrix* M);
 appga_status momentum_table(appga_matrix* M, SolverState* st, int k0, const appga_params* p,
                             cudaStream_t s, const SolverState* init = nullptr);
 IterParams iter_params(const appga_params* p, bool track);
+// Device state of a run at its start, iteration index k0.
+SolverState start_state(int32_t k0, const appga_params* p, const float* g, const float* gamma);
+// The settings a captured loop of replay length S depends on, as a cache key.
+std::string graph_key(const appga_params* p, bool track, bool bf16, int S);
 bool bf16_requested(const appga_matrix* M, const appga_params* p);
 appga_status check_params_and_mat(appga_ctx* ctx, const appga_matrix* M, const appga_params* p);
-appga_status validate_inputs(appga_matrix* M, const float* g, const float* gamma, const float* f,
-                             cudaStream_t s);
 void free_afppa_workspace(AfppaWorkspace* aw);
 
 // The solver loop's projection layout in fa / pa: the folded sliced

@@ -652,12 +652,13 @@ __device__ __forceinline__ void load_theta(SolverState* st, const ThetaEntry& e)
 // the loop y~ by linearity), the guarded weight w = 1 - g/den (returned, and
 // stored at w[row] if store_w), and adds the data term y - g ln(y + gamma) of
 // the objective to (acc_hi, acc_lo).
-__device__ __forceinline__ float forward_row(const FwdArgs& a, df th, int kk, int row, float hi,
-                                             float lo, int& hits, int& bad, float& acc_hi,
-                                             float& acc_lo, bool store_w = true) {
+__device__ __forceinline__ float forward_row(const FwdArgs& a, const float* __restrict__ g,
+                                             const float* __restrict__ gamma, df th, int kk,
+                                             int row, float hi, float lo, int& hits, int& bad,
+                                             float& acc_hi, float& acc_lo, bool store_w = true) {
   float wv = 0.f;
   const df y = quick_renorm(hi, lo);
-  const float gam = a.gamma[row], gg = a.g[row];
+  const float gam = gamma[row], gg = g[row];
   if (a.loop) {
     a.y[kk & 1][row] = make_float2(y.hi, y.lo);
   } else {
@@ -776,7 +777,10 @@ __global__ void FW_BOUNDS k_forward(FwdArgs a) {
   pdl_wait();
   int kk = 0;
   df th = {0.f, 0.f};
+  const float *g = a.g, *gamma = a.gamma;
   if (a.loop) {
+    g = st->g;
+    gamma = st->gamma;
     // this step's index and status, handed over by the previous step's
     // finalisation; block 0 publishes them for the pixel phase.  done == 2:
     // the last pixel phase has run and this forward phase only evaluates the
@@ -789,6 +793,7 @@ __global__ void FW_BOUNDS k_forward(FwdArgs a) {
       st->done = dn;
       st->k = kk;
       load_theta(st, te);
+      if (a.no_stencil) st->pmax_bits = 0u;  // AFPPA: for the next pixel phase
     }
     if (dn == 1) return;
   }
@@ -832,7 +837,7 @@ __global__ void FW_BOUNDS k_forward(FwdArgs a) {
               const float2 v = ysum[q];
               const int row =
                   partner ? fold_partner(brow0 + q, a.fold_half, a.fold_nb) : brow0 + q;
-              wv = forward_row(a, th, kk, row, partner ? v.y : v.x, 0.f, hits, bad, acc_hi,
+              wv = forward_row(a, g, gamma, th, kk, row, partner ? v.y : v.x, 0.f, hits, bad, acc_hi,
                                acc_lo, false);
             }
             const float wp = __shfl_down_sync(0xffffffffu, wv, 16);
@@ -842,7 +847,7 @@ __global__ void FW_BOUNDS k_forward(FwdArgs a) {
         } else {
           for (int q = lane; q < bn; q += 32) {
             const float2 v = ysum[q];
-            forward_row(a, th, kk, brow0 + q, v.x, v.y, hits, bad, acc_hi, acc_lo);
+            forward_row(a, g, gamma, th, kk, brow0 + q, v.x, v.y, hits, bad, acc_hi, acc_lo);
           }
         }
       }
@@ -867,11 +872,11 @@ __global__ void FW_BOUNDS k_forward(FwdArgs a) {
       const int brow0 = pb * BROWS, bn = min(BROWS, m - brow0);
       for (int q = lane; q < bn; q += 32) {
         const float2 v = ysum_csr[q];
-        forward_row(a, th, kk, brow0 + q, v.x, v.y, hits, bad, acc_hi, acc_lo);
+        forward_row(a, g, gamma, th, kk, brow0 + q, v.x, v.y, hits, bad, acc_hi, acc_lo);
       }
     }
 #else
-    if (lane < nrows) forward_row(a, th, kk, row0 + lane, hi, lo, hits, bad, acc_hi, acc_lo);
+    if (lane < nrows) forward_row(a, g, gamma, th, kk, row0 + lane, hi, lo, hits, bad, acc_hi, acc_lo);
 #endif
   } else {
     // SHOITV gradient at f~^kk and the regulariser of Phi(f^kk)
@@ -1098,8 +1103,7 @@ __global__ void PX_BOUNDS k_pixel(PixArgs a) {
 
 // Finalises a step after the pixel phase, in one block (so the pixel blocks
 // end without a grid-wide ticket): Phi(f^kk) from the forward phase's block
-// partials in a fixed order and the stopping test, the AFPPA dual step sizes,
-// then the next index and its momentum scalar from the run's table.
+// partials in a fixed order and the stopping test, then the next index and its momentum scalar from the run's table.
 constexpr int FIN_THREADS = 512;
 #ifndef APPGA_FIN_BATCH
 #define APPGA_FIN_BATCH 12
@@ -1150,17 +1154,6 @@ __global__ void __launch_bounds__(FIN_THREADS) k_finalize(PixArgs a) {
       return;
     }
   }
-  if (a.want_pmax) {
-    // dual step sizes of this step: rho1 = 1/(2*8*p_max), rho2 = 1/(2*64*p_max)
-    // (kept when every entry is zero: the all-zero iterate is absorbing)
-    const float pm = __uint_as_float(st->pmax_bits);
-    if (pm > 0.f) {
-      st->rho1 = (float)(1.0 / (16.0 * (double)pm));
-      st->rho2 = (float)(1.0 / (128.0 * (double)pm));
-    }
-    st->pmax_bits = 0u;
-  }
-  st->theta_prev = st->theta_hi;
   if (kk >= st->k_last) {
     // with the objective tracked, the forward phase of f^{kk+1} still runs
     // and a last finalisation turns its partials into Phi(f^{kk+1})
@@ -1241,23 +1234,6 @@ __global__ void __launch_bounds__(FW::THREADS) k_reg_term(int n, const float* __
   const df b = block_sum_acc(reg, 0.f);
   double tot = 0.0;
   if (grid_reduce(partial, gtick, &st->ticket_aux, b, &tot) && threadIdx.x == 0) *out = tot;
-}
-
-// Input validation: g finite and >= 0, gamma finite and > 0, f finite and >= 0.
-__global__ void k_validate(const float* __restrict__ g, const float* __restrict__ gamma, int m,
-                           const float* __restrict__ f, int d, int* flag) {
-  int bad = 0;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
-    const float gi = g[i], ci = gamma[i];
-    if (!(isfinite(gi) && gi >= 0.f && isfinite(ci) && ci > 0.f)) bad = 1;
-  }
-  if (f != nullptr) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < d; i += gridDim.x * blockDim.x) {
-      const float x = f[i];
-      if (!(isfinite(x) && x >= 0.f)) bad = 1;
-    }
-  }
-  if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(flag, 1);
 }
 
 // Input check of a solver run: marks the run state with APPGA_FLAG_DOMAIN and
@@ -1397,12 +1373,6 @@ cudaError_t launch_to_fold_pairs(const float* f, float2* fpair, int n, cudaStrea
   return cudaGetLastError();
 }
 
-// The solver loop's kernels are launched with programmatic stream
-// serialisation (1), so each may start while its predecessor drains; 0 gives
-// plain stream order.
-#ifndef APPGA_PDL
-#define APPGA_PDL 1
-#endif
 // Preferred shared-memory carveout of the projector kernels in percent of the
 // unified L1 / shared memory (-1: the driver's choice).  The projectors need
 // little shared memory; the rest serves as L1 for the gathered vectors.
@@ -1420,25 +1390,6 @@ template <class K>
 cudaError_t set_carveout(K kern, int percent) {
   if (percent < 0) return cudaSuccess;
   return cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, percent);
-}
-template <class... P, class... Args>
-cudaError_t launch_dep(void (*kern)(P...), int grid, int block, cudaStream_t s, Args... args) {
-#if APPGA_PDL
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = s;
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, args...);
-#else
-  kern<<<grid, block, 0, s>>>(args...);
-  return cudaGetLastError();
-#endif
 }
 }  // namespace
 
@@ -1560,12 +1511,6 @@ cudaError_t launch_reg_term(int n, const float* f, float lam1, float lam2, float
                             float2* partial, unsigned int* gtick, SolverState* st, double* out,
                             cudaStream_t s) {
   k_reg_term<<<st_tiles(n), FW::THREADS, 0, s>>>(n, f, lam1, lam2, eps, partial, gtick, st, out);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_validate_inputs(const float* g, const float* gamma, int m, const float* f,
-                                   int d, int* flag, cudaStream_t s) {
-  k_validate<<<256, 256, 0, s>>>(g, gamma, m, f, d, flag);
   return cudaGetLastError();
 }
 

@@ -10,12 +10,15 @@
 //                  u = 2 f^{k+1} - f~^k, group by group, and the term
 //                  B1^T b~^{k+1} + B2^T c~^{k+1} that the next pixel phase adds
 //                  to the gradient (b~, c~ the momentum extrapolations).
-//   k_norms2     : ||x - y||^2 and ||x||^2 (double-float), for the relative
-//                  error RE = ||f^{k+1} - f^k|| / ||f^{k+1}||.
+//   k_afppa_result : the result out of the rings, and ||f^{k+1} - f^k||^2 and
+//                  ||f^{k+1}||^2 (double-float) for the relative error RE =
+//                  ||f^{k+1} - f^k|| / ||f^{k+1}||.
 //
 // The forward and pixel phases are the APPGA kernels (the forward phase
 // without its smoothed-TV stencil; the pixel phase also reduces the largest
-// preconditioner entry, from which rho1 = 1/(16 p_max), rho2 = 1/(128 p_max)).
+// preconditioner entry, from which every block of k_afppa_dual takes rho1 =
+// 1/(16 p_max), rho2 = 1/(128 p_max): a one-block kernel between the two cost
+// 3 us a step).
 //
 // Tile: 4 x 32 pixels per block.  u is staged with a 2-pixel halo so that the
 // six difference fields, and so the new duals, are known on a 1-pixel halo,
@@ -48,10 +51,20 @@ __device__ __forceinline__ void ball_project(float (&z)[L], float r) {
 __global__ void __launch_bounds__(DT) k_afppa_dual(DualArgs a) {
   __shared__ float T[DR + 4][TWD];
   __shared__ float V[6][DR + 2][VWD];
-  const SolverState* st = a.st;
-  const int k1 = st->k;  // index of f^{k+1}, the iterate the pixel phase just wrote
-  const float th_k = st->theta_prev, th_k1 = st->theta_hi;
-  const float rho1 = st->rho1, rho2 = st->rho2;
+  SolverState* st = a.st;
+  pdl_trigger();
+  pdl_wait();
+  const int k1 = st->k + 1;  // index of f^{k+1}, the iterate the pixel phase just wrote
+  const float th_k = st->theta_hi, th_k1 = a.theta_tab[k1 - st->k0].hi;
+  // the step's dual step sizes (kept when every entry of P is zero: the
+  // all-zero iterate is absorbing)
+  const float pm = __uint_as_float(st->pmax_bits);
+  const float rho1 = pm > 0.f ? (float)(1.0 / (16.0 * (double)pm)) : st->rho1;
+  const float rho2 = pm > 0.f ? (float)(1.0 / (128.0 * (double)pm)) : st->rho2;
+  if (blockIdx.x == 0 && threadIdx.x == 0 && pm > 0.f) {
+    st->rho1 = rho1;  // other blocks read these only when pm == 0
+    st->rho2 = rho2;
+  }
   const int n = a.n, d = n * n, tid = threadIdx.x;
   const float* f1 = a.f[k1 % 3];
   const float* f0 = a.f[(k1 + 2) % 3];
@@ -138,20 +151,39 @@ __global__ void __launch_bounds__(DT) k_afppa_dual(DualArgs a) {
   }
 }
 
-// out[0] = ||x - y||^2, out[1] = ||x||^2 (one block, fixed order)
-__global__ void __launch_bounds__(1024) k_norms2(int d, const float* __restrict__ x,
-                                                 const float* __restrict__ y, double* out) {
+__global__ void __launch_bounds__(256) k_afppa_result(AfppaResultArgs a) {
+  pdl_trigger();
+  pdl_wait();
+  if (a.st->flags & APPGA_FLAG_DOMAIN) return;
+  const int rk = a.st->result_k;
+  const float *x = a.f[rk % 3], *y = a.f[(rk + 2) % 3], *b = a.b[rk % 3], *c = a.c[rk % 3];
   float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f;
-  for (int j = threadIdx.x; j < d; j += blockDim.x) {
+  const int stride = gridDim.x * blockDim.x;
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < a.d; j += stride) {
+    const float xj = x[j];
+    a.f_out[j] = xj;
     df e;
-    two_sum(x[j], -y[j], e.hi, e.lo);
+    two_sum(xj, -y[j], e.hi, e.lo);
     const df e2 = df_mul(e, e);
     acc_add(h0, l0, e2.hi, e2.lo);
-    const df xx = df_mul({x[j], 0.f}, {x[j], 0.f});
+    const df xx = df_mul({xj, 0.f}, {xj, 0.f});
     acc_add(h1, l1, xx.hi, xx.lo);
   }
+  if (a.b_out)
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < 2 * a.d; j += stride) a.b_out[j] = b[j];
+  if (a.c_out)
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < 4 * a.d; j += stride) a.c_out[j] = c[j];
   const df s0 = block_sum_acc(h0, l0);
   const df s1 = block_sum_acc(h1, l1);
+  if (threadIdx.x == 0) a.partial[blockIdx.x] = make_float4(s0.hi, s0.lo, s1.hi, s1.lo);
+}
+// The blocks' sums in a fixed order.
+__global__ void __launch_bounds__(kAfppaResultBlocks) k_afppa_norms(const float4* partial,
+                                                                    double* out) {
+  pdl_wait();
+  const float4 p = partial[threadIdx.x];
+  const df s0 = block_sum_acc(p.x, p.y);
+  const df s1 = block_sum_acc(p.z, p.w);
   if (threadIdx.x == 0) {
     out[0] = (double)s0.hi + (double)s0.lo;
     out[1] = (double)s1.hi + (double)s1.lo;
@@ -162,13 +194,13 @@ __global__ void __launch_bounds__(1024) k_norms2(int d, const float* __restrict_
 
 cudaError_t launch_afppa_dual(const DualArgs& a, cudaStream_t s) {
   const int tiles = ((a.n + DC - 1) / DC) * ((a.n + DR - 1) / DR);
-  k_afppa_dual<<<tiles, DT, 0, s>>>(a);
-  return cudaGetLastError();
+  return launch_dep(k_afppa_dual, tiles, DT, s, a);
 }
 
-cudaError_t launch_norms2(int d, const float* x, const float* y, double* out, cudaStream_t s) {
-  k_norms2<<<1, 1024, 0, s>>>(d, x, y, out);
-  return cudaGetLastError();
+cudaError_t launch_afppa_result(const AfppaResultArgs& a, cudaStream_t s) {
+  cudaError_t e = launch_dep(k_afppa_result, kAfppaResultBlocks, 256, s, a);
+  if (e != cudaSuccess) return e;
+  return launch_dep(k_afppa_norms, 1, kAfppaResultBlocks, s, (const float4*)a.partial, a.norms);
 }
 
 }  // namespace appga
