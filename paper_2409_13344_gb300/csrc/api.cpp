@@ -67,29 +67,31 @@ void free_csr(DevCSR& c) {
 
 void free_sell(DevSell& c) {
   cudaFree(c.off);
+  cudaFree(c.row);
   cudaFree(c.cols);
-  cudaFree(c.cols32);
   cudaFree(c.vals);
   cudaFree(c.vals_bf16);
   c = DevSell();
 }
 
-appga_status upload_sell(const appga::HostSell& h, bool bf16, DevSell* out, int64_t* bytes) {
+appga_status upload_sell(const appga::HostSell& h, const std::vector<int32_t>& row, int32_t rows,
+                         bool bf16, DevSell* out, int64_t* bytes) {
   DevSell c;
-  c.rows = h.rows;
+  c.rows = rows;
   c.slices = h.slices;
+  c.lanes = h.lanes;
   const size_t np = h.vals.size() / appga::PACK_ENTRIES;
   cudaError_t e = dalloc(&c.off, h.off.size(), bytes);
+  if (e == cudaSuccess) e = dalloc(&c.row, row.size(), bytes);
   if (e == cudaSuccess && !h.cols.empty()) e = dalloc(&c.cols, np, bytes);
-  if (e == cudaSuccess && !h.cols32.empty()) e = dalloc(&c.cols32, np, bytes);
   if (e == cudaSuccess) e = dalloc(&c.vals, np, bytes);
   if (e == cudaSuccess && bf16) e = dalloc(&c.vals_bf16, np, bytes);
   if (e == cudaSuccess)
     e = cudaMemcpy(c.off, h.off.data(), h.off.size() * 4, cudaMemcpyHostToDevice);
   if (e == cudaSuccess && !h.cols.empty())
     e = cudaMemcpy(c.cols, h.cols.data(), np * 8, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess && !h.cols32.empty())
-    e = cudaMemcpy(c.cols32, h.cols32.data(), np * 16, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess)
+    e = cudaMemcpy(c.row, row.data(), row.size() * 4, cudaMemcpyHostToDevice);
   if (e == cudaSuccess && np)
     e = cudaMemcpy(c.vals, h.vals.data(), np * 16, cudaMemcpyHostToDevice);
   if (e == cudaSuccess && bf16 && np) {
@@ -382,8 +384,7 @@ appga_status setup_run(appga_matrix* M, const float* g, const float* gamma, int3
   pa.fuse_fin = APPGA_FUSE_FIN;
   appga::loop_layout(M, &fa, &pa);
   if (!tiled_ready) CK(appga::loop_gather_copy(M, ws.f[k0 % 3], s));
-  pa.n_fwd_partial =
-      appga::forward_blocks(fa.S.off != nullptr ? fa.S.rows : M->m, M->n, fa.S.off != nullptr);
+  pa.n_fwd_partial = appga::forward_blocks(fa, M->n);
 
   // w^{k0}, y^{k0}, B^T grad phi~(B f~^{k0}) and Phi(f^{k0})
   appga::FwdArgs first = fa;
@@ -933,35 +934,69 @@ appga_status appga_matrix_create(appga_ctx* ctx, int32_t m, int32_t d, int32_t n
     cudaError_t e = dalloc(&M->A_tiled.col, ct.size(), &M->bytes);
     if (e == cudaSuccess && !ct.empty())
       e = cudaMemcpy(M->A_tiled.col, ct.data(), ct.size() * 4, cudaMemcpyHostToDevice);
-    // the solver loop's two projections in the sliced layout (both or neither)
+    // the solver loop's two projections in the sliced layout (both or neither):
+    // pixels by tiles and rays by tiles of (angle, bin), entries along the ray
     if (APPGA_PACK && e == cudaSuccess && !ct.empty() && !pt.col.empty()) {
+      appga::HostCSR along, pl;
+      appga::sort_along_rays(m, n_side, row_ptr_host, col_host, val_host, &along);
+      appga::pad_rows(m, d, row_ptr_host, along.col.data(), along.val.data(), appga::ROW_PAD, &pl);
+      along = appga::HostCSR();
+      for (auto& c : pl.col) c = appga::tiled_index(c / n_side, c % n_side, n_side);
+      auto rays = [&](int32_t rows, int lanes) {
+        std::vector<int32_t> order;
+        if (m % n_angles == 0) {
+          order = appga::zorder(rows / (m / n_angles), m / n_angles);
+        } else {
+          order.resize((size_t)rows);
+          for (int32_t i = 0; i < rows; ++i) order[(size_t)i] = i;
+        }
+        order.resize(((size_t)rows * lanes + 31) / 32 * (32 / lanes), -1);
+        return order;
+      };
+      const int la = appga::sell_lanes(m, false), lt = appga::sell_lanes(d, true);
+      std::vector<int32_t> oa = rays(m, la), ot = appga::zorder(n_side, n_side);
+      ot.resize(((size_t)d * lt + 31) / 32 * (32 / lt), -1);
       appga::HostSell ha, ht;
-      if (appga::build_sell(m, pa.row_ptr, ct, pa.val, &ha) &&
-          appga::build_sell(d, pt.row_ptr, pt.col, pt.val, &ht)) {
-        appga_status r1 = upload_sell(ha, want_bf16, &M->sell_a, &M->bytes);
-        if (r1 == APPGA_OK) r1 = upload_sell(ht, want_bf16, &M->sell_t, &M->bytes);
+      if (appga::build_sell(oa, la, pl.row_ptr, pl.col, pl.val, &ha) &&
+          appga::build_sell(ot, lt, pt.row_ptr, pt.col, pt.val, &ht)) {
+        appga_status r1 = upload_sell(ha, oa, m, want_bf16, &M->sell_a, &M->bytes);
+        if (r1 == APPGA_OK) r1 = upload_sell(ht, ot, d, want_bf16, &M->sell_t, &M->bytes);
         if (r1 != APPGA_OK) e = cudaErrorMemoryAllocation;
       }
-    }
-    // the folded loop: A's first half (its rows are a prefix of pa) and the
-    // transpose of that half in orbit order
-    if (M->sell_a.off != nullptr && e == cudaSuccess && (flags & APPGA_A_NO_FOLD) == 0 &&
-        appga::quarter_turn_symmetric(m, n_side, n_angles, row_ptr_host, col_host, val_host)) {
-      appga::HostCSR ft, pft;
-      appga::fold_transpose(at, m / 2, n_side, &ft);
-      appga::pad_rows(d, m / 2, ft.row_ptr.data(), ft.col.data(), ft.val.data(), appga::ROW_PAD,
-                      &pft);
-      appga::HostSell fa, fb;
-      if (!pft.col.empty() && appga::build_sell(m / 2, pa.row_ptr, ct, pa.val, &fa) &&
-          appga::build_sell(d, pft.row_ptr, pft.col, pft.val, &fb)) {
-        appga_status r1 = upload_sell(fa, want_bf16, &M->fold_a, &M->bytes);
-        if (r1 == APPGA_OK) r1 = upload_sell(fb, want_bf16, &M->fold_t, &M->bytes);
-        if (r1 != APPGA_OK) {
-          free_sell(M->fold_a);
-          free_sell(M->fold_t);
-          e = cudaErrorMemoryAllocation;
+      // the folded loop: A's first half (its rows are a prefix of pl) and the
+      // transpose of that half, orbits by tiles of the quadrant
+      if (M->sell_a.off != nullptr && e == cudaSuccess && (flags & APPGA_A_NO_FOLD) == 0 &&
+          appga::quarter_turn_symmetric(m, n_side, n_angles, row_ptr_host, col_host, val_host)) {
+        appga::HostCSR ft, pft;
+        appga::fold_transpose(at, m / 2, n_side, &ft);
+        appga::pad_rows(d, m / 2, ft.row_ptr.data(), ft.col.data(), ft.val.data(), appga::ROW_PAD,
+                        &pft);
+        const int fla = appga::sell_lanes(m / 2, false), flt = appga::sell_lanes(d, true);
+        const int per = 8 / flt;  // orbits of a slice
+        const std::vector<int32_t> foa = rays(m / 2, fla);
+        const std::vector<int32_t> orbits = appga::zorder(n_side / 2, n_side / 2);
+        std::vector<int32_t> rows(((size_t)d / 4 + per - 1) / per * per * 4, -1), pixel(rows);
+        for (size_t q = 0; q < rows.size(); ++q) {
+          const size_t slice = q / (4 * per), at_o = slice * per + q % per;
+          if (at_o >= orbits.size()) continue;
+          const int32_t member = (int32_t)(q % (4 * per) / per);
+          int32_t r, c;
+          appga::orbit_pixel(orbits[at_o], member, n_side, &r, &c);
+          rows[q] = 4 * orbits[at_o] + member;
+          pixel[q] = r * n_side + c;
         }
-        M->fold_nb = m / n_angles;
+        appga::HostSell fa, fb;
+        if (!pft.col.empty() && appga::build_sell(foa, fla, pl.row_ptr, pl.col, pl.val, &fa) &&
+            appga::build_sell(rows, flt, pft.row_ptr, pft.col, pft.val, &fb)) {
+          appga_status r1 = upload_sell(fa, foa, m / 2, want_bf16, &M->fold_a, &M->bytes);
+          if (r1 == APPGA_OK) r1 = upload_sell(fb, pixel, d, want_bf16, &M->fold_t, &M->bytes);
+          if (r1 != APPGA_OK) {
+            free_sell(M->fold_a);
+            free_sell(M->fold_t);
+            e = cudaErrorMemoryAllocation;
+          }
+          M->fold_nb = m / n_angles;
+        }
       }
     }
     if (e != cudaSuccess) rc = cuda_fail(e, "tiled column indices and sliced layout");
@@ -1022,7 +1057,7 @@ appga_status appga_matrix_get_info(const appga_matrix* M, appga_matrix_info* out
   out->has_bf16 = M->has_bf16;
   out->device_bytes = M->bytes;
   out->packed_columns = M->sell_t.cols != nullptr ? 1 : 0;
-  out->sliced_layout = (M->sell_t.cols != nullptr || M->sell_t.cols32 != nullptr) ? 1 : 0;
+  out->sliced_layout = M->sell_t.off != nullptr ? 1 : 0;
   out->quarter_turn_folded = M->fold_t.off != nullptr ? 1 : 0;
   return APPGA_OK;
 }

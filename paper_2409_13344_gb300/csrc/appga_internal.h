@@ -30,12 +30,13 @@ constexpr int32_t PACK_BASE_MAX = (1 << PACK_BASE_BITS) - 1;
 constexpr int32_t PACK_OFFSET_MAX = 8191;
 
 // Device copy of a HostSell (see below), with an optional BF16 copy of the
-// values (4 per pack, 8 bytes).
+// values (4 per pack, 8 bytes).  row holds what the kernels index by: the ray
+// or pixel of each row position (-1: none).
 struct DevSell {
-  int32_t rows = 0, slices = 0;
+  int32_t rows = 0, slices = 0, lanes = 0;
   int32_t* off = nullptr;
-  uint2* cols = nullptr;    // packed words (APPGA_SELL_PACK), or
-  int4* cols32 = nullptr;   // four 32-bit columns per pack
+  int32_t* row = nullptr;
+  uint2* cols = nullptr;    // packed words
   float4* vals = nullptr;
   uint2* vals_bf16 = nullptr;
 };
@@ -182,7 +183,7 @@ struct FwdArgs {
   // loop: theta_{k0+i} of the run (the forward phase takes theta_k from it)
   const ThetaEntry* theta_tab;
   // the sliced layout of A (solver projections with FP32 accumulation; its
-  // columns index ft); S.cols == NULL: the CSR A
+  // columns index ft); S.off == NULL: the CSR A
   DevSell S;
   // quarter-turn folded loop (fpair != NULL): S holds A's first fold_half
   // rows, the projector gathers fpair[t] = (f_j, f_{quarter_turn(j)}) at the
@@ -219,10 +220,11 @@ struct PixArgs {
   // 1: the pixel phase's first blocks finalise the step (Phi(f^k) from the
   // forward phase's partials, stopping test, next index); 0: k_finalize does
   int32_t fuse_fin;
-  // the sliced layout of A^T (S.cols == NULL: the CSR At)
+  // the sliced layout of A^T (S.off == NULL: the CSR At)
   DevSell S;
-  // quarter-turn folded loop (fpair != NULL): S holds the folded A^T (slice o
-  // = the four pixels of orbit o, columns the stored rows), w holds pairs
+  // quarter-turn folded loop (fpair != NULL): S holds the folded A^T (a slice
+  // of R rows: member q / (R/4) of orbit q % (R/4) at row position q; columns
+  // the stored rows), w holds pairs
   // (w_i, w_{fold_partner(i)}), and f^{k+1} is also written as the gather
   // pairs of the next forward phase
   float2* fpair;
@@ -230,8 +232,8 @@ struct PixArgs {
 
 // ---- launchers (kernels.cu) ----
 int stencil_tiles(int n);
-// grid of the solver-loop forward phase (sliced: A in the sliced layout)
-int forward_blocks(int m, int n, bool sliced);
+// grid of the solver-loop forward phase with these arguments
+int forward_blocks(const FwdArgs& a, int n);
 int max_partials(int m, int n);
 int max_group_tickets(int m, int n);
 
@@ -326,34 +328,34 @@ bool pack_columns(const std::vector<int32_t>& col, std::vector<uint64_t>* out);
 bool encode_pack(const int32_t* c, uint64_t* word);
 
 // Sliced layout of a row-padded CSR for the solver loop's projections
-// (sliced ELLPACK over 4-entry packs): rows in slices of SELL_ROWS; each row
-// owns SELL_LANES lanes of a warp, which take its packs in turn (pack k to
-// lane k mod SELL_LANES at step k / SELL_LANES); a slice runs for as many
-// steps as its longest row needs, and every step is one pack per lane, the
-// 32 packs of a step stored consecutively.  Positions are counted in packs;
-// padding packs have value 0 (and column 0).
-#ifndef APPGA_SELL_LANES
-#define APPGA_SELL_LANES 4
-#endif
-constexpr int SELL_LANES = APPGA_SELL_LANES;  // 1, 2, 4, 8, 16 or 32
-static_assert(SELL_LANES >= 1 && SELL_LANES <= 32 && 32 % SELL_LANES == 0, "lanes per row");
-constexpr int SELL_ROWS = 32 / SELL_LANES;
-// Columns of the sliced layout as packed words (1) or as four 32-bit
-// indices per pack (0).
-#ifndef APPGA_SELL_PACK
-#define APPGA_SELL_PACK 1
-#endif
+// (sliced ELLPACK over 4-entry packs): rows in slices of 32 / lanes; each row
+// owns `lanes` lanes of a warp, which take its packs in turn (pack k to lane
+// k mod lanes at step k / lanes); a slice runs for as many steps as its longest
+// row needs, and every step is one pack per lane, the 32 packs of a step stored
+// consecutively.  Positions are counted in packs; padding packs have value 0
+// (and column 0).
 struct HostSell {
-  int32_t rows = 0, slices = 0;
+  int32_t rows = 0, slices = 0, lanes = 0;
   std::vector<int32_t> off;    // slices + 1 pack offsets (a multiple of 32 apart)
-  std::vector<uint64_t> cols;  // one packed word per pack (APPGA_SELL_PACK)
-  std::vector<int32_t> cols32; // PACK_ENTRIES columns per pack (otherwise)
+  std::vector<uint64_t> cols;  // one packed word per pack
   std::vector<float> vals;     // PACK_ENTRIES values per pack
 };
-// false if some pack's columns do not fit the packed word or the layout
-// exceeds 2^31 packs
+// The rows `order` (row of each position, -1: none; a whole number of slices)
+// with `lanes` (1, 2, 4 or 8) lanes each.  false if some pack's columns do not
+// fit the packed word or the layout exceeds 2^31 packs.
+bool build_sell(const std::vector<int32_t>& order, int lanes, const std::vector<int32_t>& row_ptr,
+                const std::vector<int32_t>& col, const std::vector<float>& val, HostSell* out);
+// Lanes per row of a loop projection over `rows` rows of A, or of A^T (kernels.cu).
+int sell_lanes(int rows, bool transposed);
+// All rows in ascending order, four lanes each.
 bool build_sell(int32_t rows, const std::vector<int32_t>& row_ptr, const std::vector<int32_t>& col,
                 const std::vector<float>& val, HostSell* out);
+// The entries of every row in the order in which the ray crosses the n x n
+// image's longer extent (by column if the row's pixels span more columns than
+// rows, else by row), so that neighbouring rays' k-th entries are neighbouring
+// pixels.
+void sort_along_rays(int32_t rows, int32_t n, const int32_t* row_ptr, const int32_t* col,
+                     const float* val, HostCSR* out);
 
 void set_error(const std::string& msg);
 

@@ -4,6 +4,7 @@
 #include <cmath>
 #include <cstring>
 #include <string>
+#include <utility>
 
 #include "appga_internal.h"
 
@@ -120,48 +121,77 @@ bool pack_columns(const std::vector<int32_t>& col, std::vector<uint64_t>* out) {
   return true;
 }
 
-bool build_sell(int32_t rows, const std::vector<int32_t>& row_ptr, const std::vector<int32_t>& col,
-                const std::vector<float>& val, HostSell* out) {
-  constexpr int C = SELL_ROWS, L = SELL_LANES;
-  const int32_t ns = (rows + C - 1) / C;
-  out->rows = rows;
+bool build_sell(const std::vector<int32_t>& order, int lanes, const std::vector<int32_t>& row_ptr,
+                const std::vector<int32_t>& col, const std::vector<float>& val, HostSell* out) {
+  const int C = 32 / lanes, L = lanes;
+  const int32_t ns = (int32_t)(order.size() / C);
+  out->rows = (int32_t)order.size();
   out->slices = ns;
+  out->lanes = L;
   out->off.assign((size_t)ns + 1, 0);
+  auto packs = [&](int32_t r) { return r < 0 ? 0 : (row_ptr[r + 1] - row_ptr[r]) / PACK_ENTRIES; };
   // steps of a slice: the most packs of any of its rows, over the L lanes of a row
   int64_t total = 0;
   for (int32_t s = 0; s < ns; ++s) {
     int32_t most = 0;
-    for (int32_t r = s * C; r < std::min(rows, (s + 1) * C); ++r)
-      most = std::max(most, (row_ptr[r + 1] - row_ptr[r]) / PACK_ENTRIES);
+    for (int q = 0; q < C; ++q) most = std::max(most, packs(order[(size_t)s * C + q]));
     const int64_t steps = (most + L - 1) / L;
     total += steps * 32;
     if (total > (int64_t)INT32_MAX) return false;
     out->off[(size_t)s + 1] = (int32_t)total;
   }
-  if (APPGA_SELL_PACK)
-    out->cols.assign((size_t)total, 0ull);
-  else
-    out->cols32.assign((size_t)total * PACK_ENTRIES, 0);
+  out->cols.assign((size_t)total, 0ull);
   out->vals.assign((size_t)total * PACK_ENTRIES, 0.f);
   for (int32_t s = 0; s < ns; ++s) {
     const int64_t base = out->off[(size_t)s];
-    for (int32_t rr = 0; rr < C && s * C + rr < rows; ++rr) {
-      const int32_t r = s * C + rr;
-      const int32_t npk = (row_ptr[r + 1] - row_ptr[r]) / PACK_ENTRIES;
+    for (int q = 0; q < C; ++q) {
+      const int32_t r = order[(size_t)s * C + q], npk = packs(r);
       for (int32_t k = 0; k < npk; ++k) {
-        const int64_t pos = base + (int64_t)(k / L) * 32 + rr * L + (k % L);
+        const int64_t pos = base + (int64_t)(k / L) * 32 + q * L + (k % L);
         const int32_t e = row_ptr[r] + k * PACK_ENTRIES;
-        if (APPGA_SELL_PACK) {
-          if (!encode_pack(&col[(size_t)e], &out->cols[(size_t)pos])) return false;
-        }
-        for (int i = 0; i < PACK_ENTRIES; ++i) {
+        if (!encode_pack(&col[(size_t)e], &out->cols[(size_t)pos])) return false;
+        for (int i = 0; i < PACK_ENTRIES; ++i)
           out->vals[(size_t)pos * PACK_ENTRIES + i] = val[(size_t)e + i];
-          if (!APPGA_SELL_PACK) out->cols32[(size_t)pos * PACK_ENTRIES + i] = col[(size_t)e + i];
-        }
       }
     }
   }
   return true;
+}
+
+bool build_sell(int32_t rows, const std::vector<int32_t>& row_ptr, const std::vector<int32_t>& col,
+                const std::vector<float>& val, HostSell* out) {
+  std::vector<int32_t> order(((size_t)rows + 7) / 8 * 8, -1);
+  for (int32_t r = 0; r < rows; ++r) order[(size_t)r] = r;
+  if (!build_sell(order, 4, row_ptr, col, val, out)) return false;
+  out->rows = rows;
+  return true;
+}
+
+void sort_along_rays(int32_t rows, int32_t n, const int32_t* row_ptr, const int32_t* col,
+                     const float* val, HostCSR* out) {
+  out->rows = rows;
+  out->row_ptr.assign(row_ptr, row_ptr + rows + 1);
+  out->col.assign(col, col + row_ptr[rows]);
+  out->val.assign(val, val + row_ptr[rows]);
+  std::vector<std::pair<int32_t, int32_t>> key;  // (position along the ray, entry)
+  for (int32_t i = 0; i < rows; ++i) {
+    const int32_t s = row_ptr[i], e = row_ptr[i + 1];
+    int32_t c0 = n, c1 = -1, r0 = n, r1 = -1;
+    for (int32_t p = s; p < e; ++p) {
+      r0 = std::min(r0, col[p] / n);
+      r1 = std::max(r1, col[p] / n);
+      c0 = std::min(c0, col[p] % n);
+      c1 = std::max(c1, col[p] % n);
+    }
+    if (c1 - c0 <= r1 - r0) continue;  // ascending pixel indices are by row already
+    key.clear();
+    for (int32_t p = s; p < e; ++p) key.emplace_back(col[p] % n * n + col[p] / n, p);
+    std::sort(key.begin(), key.end());
+    for (int32_t k = 0; k < e - s; ++k) {
+      out->col[(size_t)(s + k)] = col[key[(size_t)k].second];
+      out->val[(size_t)(s + k)] = val[key[(size_t)k].second];
+    }
+  }
 }
 
 bool quarter_turn_symmetric(int32_t m, int32_t n, int32_t n_angles, const int32_t* row_ptr,

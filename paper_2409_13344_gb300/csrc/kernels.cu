@@ -20,11 +20,16 @@
 //                Eq. GNtheta)
 //
 // Projector layouts.  The solver loop streams its matrices in the sliced
-// layout (SellGroup): a warp owns a slice of SELL_ROWS rows, SELL_LANES lanes
-// per row take the row's 4-entry packs in turn (packed 2-byte columns and
-// value quads, PF steps in flight in registers, the next step's gathers
-// issued while the current one accumulates), and a butterfly leaves each
-// row's sum in all of its lanes.  When A has the quarter-turn symmetry the
+// layout (SellGroup): a warp owns a slice of 32 / L rows, L lanes per row take
+// the row's 4-entry packs in turn (packed 2-byte columns and value quads, PF
+// steps in flight in registers, the next step's gathers issued while the
+// current one accumulates), and a butterfly leaves each row's sum in all of its
+// lanes.  What a warp's gathers touch decides the speed (the L1 pipe is busy for
+// 57-64 % of a launch's cycles): slices hold neighbouring pixels, or rays of a
+// few bins and angles with their entries in order along the ray, and a row gets
+// as few lanes as still fill the chip (sell_lanes).  Rows in ascending order
+// with four lanes each took 38.1 us per folded map at 256^2, 32 now; 112 at
+// 400^2, 92 now.  When A has the quarter-turn symmetry the
 // loop streams only its folded halves (FOLD): each stored entry serves two
 // products, gathered as pairs (see fold_partner in appga_internal.h).  The
 // stand-alone projections and objective stream the row-padded CSR
@@ -87,26 +92,12 @@ struct Shape {
 #ifndef APPGA_PX_PF
 #define APPGA_PX_PF 3
 #endif
-// the sliced layout's step loop runs whole groups of steps without per-step
-// tests (1) or tests every step (0)
-#ifndef APPGA_SELL_PEEL
-#define APPGA_SELL_PEEL 1
-#endif
 // steps in flight per warp in the sliced layout's forward and pixel phases
 #ifndef APPGA_SELL_FW_PF
 #define APPGA_SELL_FW_PF 3
 #endif
 #ifndef APPGA_SELL_PX_PF
 #define APPGA_SELL_PX_PF 4
-#endif
-// Slices each warp of the sliced projections streams in turn (the loads of
-// the next slice are issued before the epilogue of the current one, which
-// hides that epilogue's latency); the grids shrink by the same factor.
-#ifndef APPGA_FW_SPW
-#define APPGA_FW_SPW 1
-#endif
-#ifndef APPGA_PX_SPW
-#define APPGA_PX_SPW 1
 #endif
 using FW = Shape<APPGA_FW_W, APPGA_FW_RPW, APPGA_FW_PF>;
 using PX = Shape<APPGA_PX_W, APPGA_PX_RPW, APPGA_PX_PF>;
@@ -130,9 +121,6 @@ using PX = Shape<APPGA_PX_W, APPGA_PX_RPW, APPGA_PX_PF>;
 #endif
 #ifndef APPGA_GPIPE
 #define APPGA_GPIPE 1
-#endif
-#ifndef APPGA_SFIRST
-#define APPGA_SFIRST 0
 #endif
 // forward epilogue once per block (1) or once per warp (0)
 #ifndef APPGA_FEPI
@@ -347,30 +335,17 @@ struct RowGroup {
 
 };
 
-// One slice of the sliced layout (DevSell) streamed by one warp: lane l
-// works on row l / SELL_LANES of the slice and takes every SELL_LANES-th pack
-// of it, so each step reads 32 consecutive packs (8-byte packed columns and
-// 16 values bytes per lane) and no lane has to find the row of its entries.
-// PF steps are kept in flight in registers and the gathers of the next step
-// are issued while the current one accumulates (two FP32 accumulators per
-// lane); the SELL_LANES partial sums of a row are combined by a butterfly,
-// which leaves the same row sum in each of its lanes.
-#if APPGA_SELL_PACK
-using SellCols = uint2;  // one packed word per pack
-__device__ __forceinline__ SellCols sell_cols_load(const DevSell& S, int pos, uint64_t pol) {
-  return ld_stream_u2(S.cols + pos, pol);
-}
-__device__ __forceinline__ int4 sell_cols(SellCols c) { return unpack_cols(c); }
-__device__ __forceinline__ SellCols sell_cols_zero() { return make_uint2(0u, 0u); }
-#else
-using SellCols = int4;  // four 32-bit columns per pack
-__device__ __forceinline__ SellCols sell_cols_load(const DevSell& S, int pos, uint64_t pol) {
-  return ld_stream_i4(reinterpret_cast<const int32_t*>(S.cols32 + pos), pol);
-}
-__device__ __forceinline__ int4 sell_cols(SellCols c) { return c; }
-__device__ __forceinline__ SellCols sell_cols_zero() { return make_int4(0, 0, 0, 0); }
-#endif
-
+// One slice of the sliced layout (DevSell) streamed by one warp: lane l works
+// on row position l / L of the slice and takes every L-th pack of it, so each
+// step reads 32 consecutive packs (8-byte packed columns and 16 values bytes
+// per lane) and no lane has to find the row of its entries.  The slice's rows
+// are neighbours (pixels of a tile, rays of a few bins and angles) whose k-th
+// entries are neighbours too, so a gather of the warp meets few lines.  PF
+// steps are kept in flight in registers and the gathers of the next step are
+// issued while the current one accumulates (at least eight FP32 accumulators per
+// row, so that long rows keep short chains of rounded sums);
+// the L partial sums of a row are combined by a butterfly, which leaves the
+// same row sum in each of its lanes.
 // The four gathered vector entries of a pack: one float each, or a pair
 // (the quarter-turn folded loop gathers two vectors at once).
 template <class V>
@@ -385,23 +360,17 @@ template <class V>
 __device__ __forceinline__ Quad<V> zero_quad() {
   return {V{}, V{}, V{}, V{}};
 }
-// Entries 0, 2 of a pack into a0 and 1, 3 into a1.
-__device__ __forceinline__ void fma_quad(float4 v, const Quad<float>& g, float& a0, float& a1) {
-  a0 = fmaf(v.x, g.x, a0);
-  a1 = fmaf(v.y, g.y, a1);
-  a0 = fmaf(v.z, g.z, a0);
-  a1 = fmaf(v.w, g.w, a1);
+__device__ __forceinline__ float fma_v(float v, float x, float a) { return fmaf(v, x, a); }
+__device__ __forceinline__ float2 fma_v(float v, float2 x, float2 a) {
+  return make_float2(fmaf(v, x.x, a.x), fmaf(v, x.y, a.y));
 }
-__device__ __forceinline__ void fma_quad(float4 v, const Quad<float2>& g, float2& a0,
-                                         float2& a1) {
-  a0.x = fmaf(v.x, g.x.x, a0.x);
-  a0.y = fmaf(v.x, g.x.y, a0.y);
-  a1.x = fmaf(v.y, g.y.x, a1.x);
-  a1.y = fmaf(v.y, g.y.y, a1.y);
-  a0.x = fmaf(v.z, g.z.x, a0.x);
-  a0.y = fmaf(v.z, g.z.y, a0.y);
-  a1.x = fmaf(v.w, g.w.x, a1.x);
-  a1.y = fmaf(v.w, g.w.y, a1.y);
+// The four entries of pack u into N accumulators in turn.
+template <int N, class V>
+__device__ __forceinline__ void fma_quad(float4 v, const Quad<V>& g, V (&a)[N], int u) {
+  a[(4 * u) % N] = fma_v(v.x, g.x, a[(4 * u) % N]);
+  a[(4 * u + 1) % N] = fma_v(v.y, g.y, a[(4 * u + 1) % N]);
+  a[(4 * u + 2) % N] = fma_v(v.z, g.z, a[(4 * u + 2) % N]);
+  a[(4 * u + 3) % N] = fma_v(v.w, g.w, a[(4 * u + 3) % N]);
 }
 __device__ __forceinline__ float add_v(float a, float b) { return a + b; }
 __device__ __forceinline__ float2 add_v(float2 a, float2 b) {
@@ -414,10 +383,10 @@ __device__ __forceinline__ float2 shfl_xor_v(float2 a, int o) {
   return make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
 }
 
-template <bool BF16, int PF>
+template <bool BF16, int PF, int L>
 struct SellGroup {
   int q0, steps;
-  SellCols c[PF];
+  uint2 c[PF];
   float4 v[PF];
 
   __device__ __forceinline__ static float4 vals(const DevSell& S, int pos, uint64_t pol) {
@@ -436,10 +405,10 @@ struct SellGroup {
     steps = (S.off[slice + 1] - S.off[slice]) >> 5;
 #pragma unroll
     for (int u = 0; u < PF; ++u) {
-      c[u] = sell_cols_zero();
+      c[u] = make_uint2(0u, 0u);
       v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (u < steps) {
-        c[u] = sell_cols_load(S, q0 + (u << 5), pol);
+        c[u] = ld_stream_u2(S.cols + q0 + (u << 5), pol);
         v[u] = vals(S, q0 + (u << 5), pol);
       }
     }
@@ -449,11 +418,13 @@ struct SellGroup {
   // (V = float2), in every lane of the row.
   template <class V>
   __device__ __forceinline__ V stream(const DevSell& S, const V* __restrict__ x, uint64_t pol) {
-    V a0{}, a1{};
+    constexpr int N = L < 4 ? 8 / L : 2;
+    V acc[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) acc[k] = V{};
     Quad<V> xg = zero_quad<V>();
-    if (steps > 0) xg = gather_quad(x, sell_cols(c[0]));
+    if (steps > 0) xg = gather_quad(x, unpack_cols(c[0]));
     int t0 = 0;
-#if APPGA_SELL_PEEL
     // whole groups of PF steps whose refills and next gathers all exist: no
     // per-step tests
     for (; t0 + 2 * PF <= steps; t0 += PF) {
@@ -461,14 +432,13 @@ struct SellGroup {
       for (int u = 0; u < PF; ++u) {
         const int t = t0 + u;
         const float4 vv = v[u];
-        c[u] = sell_cols_load(S, q0 + ((t + PF) << 5), pol);
+        c[u] = ld_stream_u2(S.cols + q0 + ((t + PF) << 5), pol);
         v[u] = vals(S, q0 + ((t + PF) << 5), pol);
         const Quad<V> xx = xg;
-        xg = gather_quad(x, sell_cols(c[(u + 1) % PF]));
-        fma_quad(vv, xx, a0, a1);
+        xg = gather_quad(x, unpack_cols(c[(u + 1) % PF]));
+        fma_quad(vv, xx, acc, u);
       }
     }
-#endif
     for (; t0 < steps; t0 += PF) {
 #pragma unroll
       for (int u = 0; u < PF; ++u) {
@@ -476,19 +446,23 @@ struct SellGroup {
         if (t < steps) {
           const float4 vv = v[u];
           if (t + PF < steps) {  // refill this slot with step t + PF
-            c[u] = sell_cols_load(S, q0 + ((t + PF) << 5), pol);
+            c[u] = ld_stream_u2(S.cols + q0 + ((t + PF) << 5), pol);
             v[u] = vals(S, q0 + ((t + PF) << 5), pol);
           }
           const Quad<V> xx = xg;
           // step t + 1 sits in slot (u + 1) % PF (refilled above when PF = 1)
-          if (t + 1 < steps) xg = gather_quad(x, sell_cols(c[(u + 1) % PF]));
-          fma_quad(vv, xx, a0, a1);
+          if (t + 1 < steps) xg = gather_quad(x, unpack_cols(c[(u + 1) % PF]));
+          fma_quad(vv, xx, acc, u);
         }
       }
     }
-    V r = add_v(a0, a1);
 #pragma unroll
-    for (int o = 1; o < SELL_LANES; o <<= 1) r = add_v(r, shfl_xor_v(r, o));
+    for (int h = N / 2; h > 0; h /= 2)
+#pragma unroll
+      for (int k = 0; k < h; ++k) acc[k] = add_v(acc[k], acc[k + h]);
+    V r = acc[0];
+#pragma unroll
+    for (int o = 1; o < L; o <<= 1) r = add_v(r, shfl_xor_v(r, o));
     return r;
   }
 };
@@ -695,37 +669,27 @@ __device__ __forceinline__ float forward_row(const FwdArgs& a, const float* __re
   return wv;
 }
 
-// Rows per forward block: FW::W warps of FW::R CSR rows, or of one slice of
-// SELL_ROWS rows in the sliced layout (per trip of the slice loop).
-template <bool SL>
-__host__ __device__ __forceinline__ constexpr int fw_block_rows() {
-  return SL ? FW::W * SELL_ROWS : FW::ROWS;
+// Projector blocks of the forward phase and blocks of the pixel phase: a warp
+// per CSR row group, or per slice.
+__host__ __device__ __forceinline__ int fw_proj_blocks(int rows, int slices) {
+  return slices > 0 ? (slices + FW::W - 1) / FW::W : (rows + FW::ROWS - 1) / FW::ROWS;
 }
-// Projector blocks of the forward phase over `rows` rows: CSR row groups, or
-// sliced with each warp taking APPGA_FW_SPW slices in turn.
-__host__ __device__ __forceinline__ int fw_proj_blocks(int rows, bool sliced) {
-  if (!sliced) return (rows + FW::ROWS - 1) / FW::ROWS;
-  const int ns = (rows + SELL_ROWS - 1) / SELL_ROWS;
-  return (ns + FW::W * APPGA_FW_SPW - 1) / (FW::W * APPGA_FW_SPW);
-}
-// Blocks of the pixel phase over d pixel rows (as fw_proj_blocks).
-__host__ __device__ __forceinline__ int px_blocks(int d, bool sliced) {
-  if (!sliced) return (d + PX::ROWS - 1) / PX::ROWS;
-  const int ns = (d + SELL_ROWS - 1) / SELL_ROWS;
-  return (ns + PX::W * APPGA_PX_SPW - 1) / (PX::W * APPGA_PX_SPW);
+__host__ __device__ __forceinline__ int px_blocks(int d, int slices) {
+  return slices > 0 ? (slices + PX::W - 1) / PX::W : (d + PX::ROWS - 1) / PX::ROWS;
 }
 
-// Blocks [0, nproj) project rows (CSR row groups, or slices of the sliced
-// layout when SL); in the solver loop the blocks after them run the stencil
-// tiles.
+// Blocks [0, nproj) project rows (CSR row groups if L == 0, else slices of the
+// sliced layout with L lanes per row); in the solver loop the blocks after them
+// run the stencil tiles.
 //
 // FOLD (quarter-turn folded loop, sliced): the slices hold A's first m/2
 // rows; each stored row i gathers the pairs fpair and yields y_i and
-// y_{fold_partner(i)}, so the block's 16 stored rows give 32 row epilogues,
-// one per lane of warp 0, and w is stored as the pairs the folded
-// back-projection gathers.
-template <bool BF16, bool DFA, bool SL, bool FOLD>
+// y_{fold_partner(i)}: two row epilogues, by two of the row's lanes where it has
+// them, and w is stored as the pairs the folded back-projection gathers.
+template <bool BF16, bool DFA, int L, bool FOLD>
 __global__ void FW_BOUNDS k_forward(FwdArgs a) {
+  constexpr bool SL = L > 0;
+  constexpr int LL = SL ? L : 1, SROWS = 32 / LL;
   __shared__ union {
     struct {
       float hi[FW::W][FW::R * SLOT_W];
@@ -739,32 +703,26 @@ __global__ void FW_BOUNDS k_forward(FwdArgs a) {
   pdl_trigger();
   SolverState* st = a.st;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // rows streamed (FOLD: the stored first half)
-  const int m = SL ? a.S.rows : a.A.rows;
-  constexpr int BROWS = fw_block_rows<SL>();
-  const int nproj = fw_proj_blocks(m, SL);
-  const int ns = SL ? a.S.slices : 0;
-#if APPGA_SFIRST
-  // stencil tiles take the first blocks, so the projector blocks end the grid
-  const int pb = (int)blockIdx.x - ((int)gridDim.x - nproj);
-  const int sb = blockIdx.x;
-#else
+  const int m = a.A.rows;
+  const int nproj = fw_proj_blocks(m, SL ? a.S.slices : 0);
   const int pb = blockIdx.x;
   const int sb = (int)blockIdx.x - nproj;
-#endif
-  const bool proj = pb >= 0 && pb < nproj;
-  // CSR: this warp's rows; sliced: this warp's first slice
-  const int row0 = SL ? (pb * FW::W + warp) * SELL_ROWS : pb * FW::ROWS + warp * FW::R;
-  const int nrows = proj ? max(0, min(SL ? SELL_ROWS : FW::R, m - row0)) : 0;
+  const bool proj = pb < nproj;
+  // CSR: this warp's rows; sliced: this warp's slice
+  const int slice = pb * FW::W + warp;
+  const int row0 = pb * FW::ROWS + warp * FW::R;
+  const int nrows = !proj ? 0 : (SL ? (slice < a.S.slices ? 1 : 0) : max(0, min(FW::R, m - row0)));
   // The warp's row bounds and first chunks of A: no kernel writes them, so
   // they are fetched before waiting for the previous kernel of the stream.
   RowGroup<BF16, DFA, FW::R, FW::PF> rg;
-  SellGroup<BF16, APPGA_SELL_FW_PF> sg;
+  SellGroup<BF16, APPGA_SELL_FW_PF, LL> sg;
   uint64_t pol = 0;
+  int srow = -1;  // sliced: the ray of this lane's row position
   if (proj) pol = evict_first_policy();
   if (nrows > 0) {
     if constexpr (SL) {
-      sg.prologue(a.S, pb * FW::W + warp, lane, pol);
+      sg.prologue(a.S, slice, lane, pol);
+      srow = __ldg(a.S.row + slice * SROWS + lane / LL);
     } else {
 #if APPGA_SBND
       rg.sb = reinterpret_cast<int*>(sm.slot.bnd[warp]);
@@ -800,59 +758,37 @@ __global__ void FW_BOUNDS k_forward(FwdArgs a) {
   float acc_hi = 0.f, acc_lo = 0.f;  // this thread's share of the objective
   int hits = 0, bad = 0;
   if (proj && SL) {
-    // slices pb*W + warp + t*G, t = 0, 1, ...: the block's trip t covers
-    // FW::W consecutive slices, whose row sums go to warp 0, so the
-    // double-float epilogue (with the logarithm of the data term) runs once
-    // per block trip; the next slice's loads are issued before it
+    // the block's row sums go to shared memory, so that the double-float row
+    // epilogues fill whole warps: FW::W * SROWS rows, and FOLD as many partners
+    constexpr int BR = FW::W * SROWS;
+    __shared__ float2 ysum[BR];
+    __shared__ int yrow[BR];
     const float* f = a.ft ? a.ft : (a.loop ? a.f[kk % 3] : a.f[0]);
-    const int G = nproj * FW::W;
-    __shared__ float2 ysum[BROWS];
-    for (int base = pb * FW::W; base < ns; base += G) {  // uniform over the block
-      const int sl = base + warp;
-      const int nr = sl < ns ? min(SELL_ROWS, m - sl * SELL_ROWS) : 0;
-      float2 yy = make_float2(0.f, 0.f);  // (y, 0), or FOLD (y, y of the partner row)
-      if (nr > 0) {
-        if constexpr (FOLD) {
-          yy = sg.stream(a.S, a.fpair, pol);
-        } else {
-          yy.x = sg.stream(a.S, f, pol);
-        }
+    float2 yy = make_float2(0.f, 0.f);
+    if (nrows > 0) {
+      if constexpr (FOLD) {
+        yy = sg.stream(a.S, a.fpair, pol);
+      } else {
+        yy.x = sg.stream(a.S, f, pol);
       }
-      if (APPGA_FW_SPW > 1 && sl + G < ns) sg.prologue(a.S, sl + G, lane, pol);
-      const int wrow = lane / SELL_LANES;
-      if ((lane % SELL_LANES) == 0 && wrow < nr) ysum[warp * SELL_ROWS + wrow] = yy;
-      __syncthreads();
-      if (warp == 0) {
-        const int brow0 = base * SELL_ROWS, bn = min(BROWS, m - brow0);
-        if constexpr (FOLD) {
-          static_assert(!FOLD || BROWS % 16 == 0, "folded row epilogues in passes of 16");
-          // per pass, lanes 0-15 take 16 stored rows and lanes 16-31 their
-          // partner rows
-#pragma unroll
-          for (int p0 = 0; p0 < BROWS; p0 += 16) {
-            const int q = p0 + lane % 16;
-            const bool partner = lane >= 16;
-            float wv = 0.f;
-            if (q < bn) {
-              const float2 v = ysum[q];
-              const int row =
-                  partner ? fold_partner(brow0 + q, a.fold_half, a.fold_nb) : brow0 + q;
-              wv = forward_row(a, g, gamma, th, kk, row, partner ? v.y : v.x, 0.f, hits, bad, acc_hi,
-                               acc_lo, false);
-            }
-            const float wp = __shfl_down_sync(0xffffffffu, wv, 16);
-            if (!partner && q < bn && a.w != nullptr)
-              reinterpret_cast<float2*>(a.w)[brow0 + q] = make_float2(wv, wp);
-          }
-        } else {
-          for (int q = lane; q < bn; q += 32) {
-            const float2 v = ysum[q];
-            forward_row(a, g, gamma, th, kk, brow0 + q, v.x, v.y, hits, bad, acc_hi, acc_lo);
-          }
-        }
+    }
+    if (lane % LL == 0) {
+      ysum[warp * SROWS + lane / LL] = yy;
+      yrow[warp * SROWS + lane / LL] = srow;
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < (FOLD ? 2 : 1) * BR; t += FW::THREADS) {
+      const int q = t % BR, i = yrow[q];
+      if (i < 0) continue;
+      if constexpr (FOLD) {
+        const bool partner = t >= BR;
+        const float wv =
+            forward_row(a, g, gamma, th, kk, partner ? fold_partner(i, a.fold_half, a.fold_nb) : i,
+                        partner ? ysum[q].y : ysum[q].x, 0.f, hits, bad, acc_hi, acc_lo, false);
+        if (a.w != nullptr) a.w[2 * i + (partner ? 1 : 0)] = wv;
+      } else {
+        forward_row(a, g, gamma, th, kk, i, ysum[q].x, 0.f, hits, bad, acc_hi, acc_lo);
       }
-      if (APPGA_FW_SPW == 1) break;  // one trip: the grid covers every slice
-      __syncthreads();  // ysum is refilled by the next trip
     }
   } else if (proj) {
     // the tiled copy when given (the solver's projections), else the image
@@ -865,6 +801,7 @@ __global__ void FW_BOUNDS k_forward(FwdArgs a) {
 #if APPGA_FEPI
     // the block's row sums go to warp 0, so the double-float epilogue runs
     // once per block, not once per warp
+    constexpr int BROWS = FW::ROWS;
     __shared__ float2 ysum_csr[BROWS];
     if (lane < nrows) ysum_csr[warp * FW::R + lane] = make_float2(hi, lo);
     __syncthreads();
@@ -1006,30 +943,35 @@ __device__ void fused_finalize(const PixArgs& a, SolverState* st, int kk) {
 }
 
 
-// FOLD (quarter-turn folded loop, sliced): warp o streams the folded A^T
-// rows of orbit o's four pixels q_r = turn^r(q_0), one per SELL_LANES lanes,
-// gathering the w pairs; (A^T w)_{q_r} = s1(q_r) + s2(q_{r-1}), the second
-// term from the lanes of member r-1, and f^{k+1} at q_r goes out with its
-// turned neighbour f^{k+1} at q_{r+1} as the next forward phase's pair.
-template <bool BF16, bool SL, bool FOLD>
+// FOLD (quarter-turn folded loop, sliced): a slice holds the folded A^T rows of
+// whole orbits (q_r = turn^r(q_0)), gathering the w pairs; (A^T w)_{q_r} =
+// s1(q_r) + s2(q_{r-1}), the second term from the lanes of member r-1, and
+// f^{k+1} at q_r goes out with its turned neighbour f^{k+1} at q_{r+1} as the
+// next forward phase's pair.
+template <bool BF16, int L, bool FOLD>
 __global__ void PX_BOUNDS k_pixel(PixArgs a) {
-  __shared__ float slot[PX::W][PX::R * SLOT_W];
+  constexpr bool SL = L > 0;
+  constexpr int LL = SL ? L : 1, SROWS = 32 / LL, ORB = SROWS / 4;
+  __shared__ float slot[PX::W][SL ? 1 : PX::R * SLOT_W];
   __shared__ int4 sbnd[PX::W][4];
-  static_assert(!FOLD || (SL && SELL_ROWS % 4 == 0), "a folded slice is whole orbits of four");
+  static_assert(!FOLD || (SL && SROWS % 4 == 0), "a folded slice is whole orbits of four");
   pdl_trigger();
   SolverState* st = a.st;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int d = a.At.rows;
   // CSR: this warp's pixel rows; sliced: this warp's slice
-  const int j0 = SL ? (blockIdx.x * PX::W + warp) * SELL_ROWS : blockIdx.x * PX::ROWS + warp * PX::R;
-  const int np = max(0, min(SL ? SELL_ROWS : PX::R, d - j0));
+  const int slice = blockIdx.x * PX::W + warp;
+  const int j0 = blockIdx.x * PX::ROWS + warp * PX::R;
+  const int np = SL ? (slice < a.S.slices ? 1 : 0) : max(0, min(PX::R, d - j0));
   // row bounds and first chunks of A^T before waiting (no kernel writes them)
   RowGroup<BF16, false, PX::R, PX::PF> rg;
-  SellGroup<BF16, APPGA_SELL_PX_PF> sg;
-  uint64_t pol = evict_first_policy();
+  SellGroup<BF16, APPGA_SELL_PX_PF, LL> sg;
+  const uint64_t pol = evict_first_policy();
+  int j = -1;  // sliced: the pixel of this lane's row position
   if (np > 0) {
     if constexpr (SL) {
-      sg.prologue(a.S, blockIdx.x * PX::W + warp, lane, pol);
+      sg.prologue(a.S, slice, lane, pol);
+      j = __ldg(a.S.row + slice * SROWS + lane / LL);
     } else {
 #if APPGA_SBND
       rg.sb = reinterpret_cast<int*>(sbnd[warp]);
@@ -1046,43 +988,24 @@ __global__ void PX_BOUNDS k_pixel(PixArgs a) {
   int bad = 0;
   float pmax = 0.f;  // largest preconditioner entry this lane met
   if constexpr (SL) {
-    // slices blockIdx.x * W + warp + t*G, t = 0, 1, ... (warp-uniform); the
-    // next slice's loads are issued before this slice's pixel updates
-    const int ns = a.S.slices, G = gridDim.x * PX::W;
-    for (int sl = blockIdx.x * PX::W + warp; sl < ns; sl += G) {
-      const int npr = min(SELL_ROWS, d - sl * SELL_ROWS);
-      float bp;
-      int j = -1;  // the pixel whose update this lane makes
-      int jr = 0, jc = 0;
+    if (np > 0) {
+      const int part = lane % LL;
+      float bp, fn = 0.f;
       if constexpr (FOLD) {
         const float2 sp = sg.stream(a.S, reinterpret_cast<const float2*>(a.w), pol);
-        if (APPGA_PX_SPW > 1 && sl + G < ns) sg.prologue(a.S, sl + G, lane, pol);
-        // row q of the slice is member q % 4 of orbit sl * SELL_ROWS / 4 + q / 4;
-        // member q - 1 (mod 4) of its orbit sits in row qm (a last slice may
-        // hold fewer orbits: npr rows)
-        const int q = lane / SELL_LANES, sub = lane % SELL_LANES;
-        const int qm = (q & ~3) | ((q + 3) & 3);
-        const float s2 = __shfl_sync(0xffffffffu, sp.y, qm * SELL_LANES + sub);
+        // member r of orbit o sits at row position r ORB + o: member r - 1 is
+        // ORB positions back, member r + 1 as many ahead (mod the slice)
+        const float s2 = __shfl_sync(0xffffffffu, sp.y, (lane + 32 - ORB * LL) & 31);
         bp = sp.x + s2;
-        if (sub == 0 && q < npr) {
-          orbit_pixel(sl * (SELL_ROWS / 4) + q / 4, q & 3, a.n, &jr, &jc);
-          j = jr * a.n + jc;
-        }
       } else {
         bp = sg.stream(a.S, a.w, pol);
-        if (APPGA_PX_SPW > 1 && sl + G < ns) sg.prologue(a.S, sl + G, lane, pol);
-        if ((lane % SELL_LANES) == 0 && lane / SELL_LANES < npr)
-          j = sl * SELL_ROWS + lane / SELL_LANES;
       }
-      float fn = 0.f;
-      if (j >= 0) pmax = fmaxf(pmax, pixel_update(a, kk, j, bp, bad, fn));
+      if (j >= 0 && part == 0) pmax = fmaxf(pmax, pixel_update(a, kk, j, bp, bad, fn));
       if constexpr (FOLD) {
-        // member q + 1 (mod 4) of the orbit: row qp
-        const int qp = ((lane / SELL_LANES) & ~3) | ((lane / SELL_LANES + 1) & 3);
-        const float fturn = __shfl_sync(0xffffffffu, fn, qp * SELL_LANES + lane % SELL_LANES);
-        if (j >= 0) a.fpair[tiled_index(jr, jc, a.n)] = make_float2(fn, fturn);
+        const float fturn = __shfl_sync(0xffffffffu, fn, (lane + ORB * LL) & 31);
+        if (j >= 0 && part == 0)
+          a.fpair[tiled_index(j / a.n, j % a.n, a.n)] = make_float2(fn, fturn);
       }
-      if (APPGA_PX_SPW == 1) break;  // one trip: the grid covers every slice
     }
   } else {
     float bp = 0.f, unused = 0.f;
@@ -1394,10 +1317,24 @@ cudaError_t set_carveout(K kern, int percent) {
 }  // namespace
 
 int stencil_tiles(int n) { return st_tiles(n); }
-int forward_blocks_of(int m, int n, bool sliced, bool stencil) {
-  return fw_proj_blocks(m, sliced) + (stencil ? st_tiles(n) : 0);
+int forward_blocks(const FwdArgs& a, int n) {
+  return fw_proj_blocks(a.A.rows, a.S.off != nullptr ? a.S.slices : 0) +
+         (a.no_stencil ? 0 : st_tiles(n));
 }
-int forward_blocks(int m, int n, bool sliced) { return forward_blocks_of(m, n, sliced, true); }
+
+// Lanes per row: the fewest (so that a warp's gathers lie closest together)
+// that still give 25 warps an SM to the back-projection, 52 to the forward
+// projection, whose grid also carries the row epilogues.  us per map at 256^2
+// folded (33 k rays, 65.5 k pixels) for forward/pixel lanes 8/2 (this rule):
+// 33; 4/2: 34; 8/4: 35; 4/4: 36; 2/2: 47; 4/1: 43.  At 400^2: 4/1 (this rule)
+// 92; 4/2: 94; 4/4: 99; 8/4: 104.  At 201^2 unfolded, BF16: 8/4 (this rule) 24;
+// 4/2: 30; 8/8: 26.
+int sell_lanes(int rows, bool transposed) {
+  const int warps = (transposed ? 25 : 52) * current_sm_count();
+  int lanes = 1;
+  while (lanes < 8 && (int64_t)rows * lanes / 32 < warps) lanes *= 2;
+  return lanes;
+}
 
 int max_partials(int m, int n) {
   const int a = proj_blocks<FW>(m) + st_tiles(n);
@@ -1407,6 +1344,41 @@ int max_partials(int m, int n) {
 }
 int max_group_tickets(int m, int n) { return max_partials(m, n) / RED_GROUP + 1; }
 
+namespace {
+template <int L>
+cudaError_t forward_sliced(const FwdArgs& a, cudaStream_t s) {
+  static PerDeviceOnce carve_once;
+  const cudaError_t carve = carve_once.run([] {
+    cudaError_t r = set_carveout(k_forward<true, false, L, false>, APPGA_CARVEOUT_FW);
+    if (r == cudaSuccess) r = set_carveout(k_forward<false, false, L, false>, APPGA_CARVEOUT_FW);
+    if (r == cudaSuccess) r = set_carveout(k_forward<true, false, L, true>, APPGA_CARVEOUT_FW);
+    if (r == cudaSuccess) r = set_carveout(k_forward<false, false, L, true>, APPGA_CARVEOUT_FW);
+    return r;
+  });
+  if (carve != cudaSuccess) return carve;
+  const int grid = fw_proj_blocks(a.A.rows, a.S.slices) + (a.loop && !a.no_stencil ? st_tiles(a.n) : 0);
+  void (*kern)(FwdArgs) =
+      a.fpair != nullptr ? (a.use_bf16 ? k_forward<true, false, L, true> : k_forward<false, false, L, true>)
+                         : (a.use_bf16 ? k_forward<true, false, L, false> : k_forward<false, false, L, false>);
+  return launch_dep(kern, grid, FW::THREADS, s, a);
+}
+template <int L>
+cudaError_t pixel_sliced(const PixArgs& a, cudaStream_t s) {
+  static PerDeviceOnce carve_once;
+  const cudaError_t carve = carve_once.run([] {
+    cudaError_t r = set_carveout(k_pixel<true, L, false>, APPGA_CARVEOUT_PX);
+    if (r == cudaSuccess) r = set_carveout(k_pixel<false, L, false>, APPGA_CARVEOUT_PX);
+    if (r == cudaSuccess) r = set_carveout(k_pixel<true, L, true>, APPGA_CARVEOUT_PX);
+    if (r == cudaSuccess) r = set_carveout(k_pixel<false, L, true>, APPGA_CARVEOUT_PX);
+    return r;
+  });
+  if (carve != cudaSuccess) return carve;
+  void (*kern)(PixArgs) = a.fpair != nullptr ? (a.use_bf16 ? k_pixel<true, L, true> : k_pixel<false, L, true>)
+                                             : (a.use_bf16 ? k_pixel<true, L, false> : k_pixel<false, L, false>);
+  return launch_dep(kern, px_blocks(a.At.rows, a.S.slices), PX::THREADS, s, a);
+}
+}  // namespace
+
 cudaError_t launch_forward(const FwdArgs& a, cudaStream_t s) {
   cudaError_t e = ensure_tables();
   if (e != cudaSuccess) return e;
@@ -1415,62 +1387,48 @@ cudaError_t launch_forward(const FwdArgs& a, cudaStream_t s) {
   // accumulates y in FP32; the stand-alone projection and objective calls
   // in double-float
   const bool dfa = (a.loop || a.solver_acc) ? APPGA_LOOP_DF != 0 : true;
+  // the sliced layout serves the solver's FP32-accumulated projections
+  if (a.S.off != nullptr && !dfa) {
+    switch (a.S.lanes) {
+      case 1: return forward_sliced<1>(a, s);
+      case 2: return forward_sliced<2>(a, s);
+      case 4: return forward_sliced<4>(a, s);
+      case 8: return forward_sliced<8>(a, s);
+    }
+    return cudaErrorInvalidValue;
+  }
+  if (a.fpair != nullptr) return cudaErrorInvalidValue;  // the folded loop is sliced
+  void (*kern)(FwdArgs) =
+      a.use_bf16 ? (dfa ? k_forward<true, true, 0, false> : k_forward<true, false, 0, false>)
+                 : (dfa ? k_forward<false, true, 0, false> : k_forward<false, false, 0, false>);
   static PerDeviceOnce carve_once;
   const cudaError_t carve = carve_once.run([] {
-    cudaError_t r = set_carveout(k_forward<true, true, false, false>, APPGA_CARVEOUT_FW);
-    if (r == cudaSuccess) r = set_carveout(k_forward<true, false, false, false>, APPGA_CARVEOUT_FW);
-    if (r == cudaSuccess) r = set_carveout(k_forward<false, true, false, false>, APPGA_CARVEOUT_FW);
-    if (r == cudaSuccess) r = set_carveout(k_forward<false, false, false, false>, APPGA_CARVEOUT_FW);
-    if (r == cudaSuccess) r = set_carveout(k_forward<true, false, true, false>, APPGA_CARVEOUT_FW);
-    if (r == cudaSuccess) r = set_carveout(k_forward<false, false, true, false>, APPGA_CARVEOUT_FW);
-    if (r == cudaSuccess) r = set_carveout(k_forward<true, false, true, true>, APPGA_CARVEOUT_FW);
-    if (r == cudaSuccess) r = set_carveout(k_forward<false, false, true, true>, APPGA_CARVEOUT_FW);
+    cudaError_t r = set_carveout(k_forward<true, true, 0, false>, APPGA_CARVEOUT_FW);
+    if (r == cudaSuccess) r = set_carveout(k_forward<true, false, 0, false>, APPGA_CARVEOUT_FW);
+    if (r == cudaSuccess) r = set_carveout(k_forward<false, true, 0, false>, APPGA_CARVEOUT_FW);
+    if (r == cudaSuccess) r = set_carveout(k_forward<false, false, 0, false>, APPGA_CARVEOUT_FW);
     return r;
   });
   if (carve != cudaSuccess) return carve;
-  // the sliced layout serves the solver's FP32-accumulated projections
-  if (a.S.off != nullptr && !dfa) {
-    const int sgrid = forward_blocks_of(a.S.rows, a.n, true, a.loop && !a.no_stencil);
-    if (a.fpair != nullptr)
-      return a.use_bf16 ? launch_dep(k_forward<true, false, true, true>, sgrid, FW::THREADS, s, a)
-                        : launch_dep(k_forward<false, false, true, true>, sgrid, FW::THREADS, s, a);
-    return a.use_bf16 ? launch_dep(k_forward<true, false, true, false>, sgrid, FW::THREADS, s, a)
-                      : launch_dep(k_forward<false, false, true, false>, sgrid, FW::THREADS, s, a);
-  }
-  if (a.fpair != nullptr) return cudaErrorInvalidValue;  // the folded loop is sliced
-  if (a.use_bf16)
-    return dfa ? launch_dep(k_forward<true, true, false, false>, grid, FW::THREADS, s, a)
-               : launch_dep(k_forward<true, false, false, false>, grid, FW::THREADS, s, a);
-  return dfa ? launch_dep(k_forward<false, true, false, false>, grid, FW::THREADS, s, a)
-             : launch_dep(k_forward<false, false, false, false>, grid, FW::THREADS, s, a);
+  return launch_dep(kern, grid, FW::THREADS, s, a);
 }
 
 cudaError_t launch_pixel(const PixArgs& a, cudaStream_t s) {
-  static PerDeviceOnce carve_once;
-  const cudaError_t carve = carve_once.run([] {
-    cudaError_t r = set_carveout(k_pixel<true, false, false>, APPGA_CARVEOUT_PX);
-    if (r == cudaSuccess) r = set_carveout(k_pixel<false, false, false>, APPGA_CARVEOUT_PX);
-    if (r == cudaSuccess) r = set_carveout(k_pixel<true, true, false>, APPGA_CARVEOUT_PX);
-    if (r == cudaSuccess) r = set_carveout(k_pixel<false, true, false>, APPGA_CARVEOUT_PX);
-    if (r == cudaSuccess) r = set_carveout(k_pixel<true, true, true>, APPGA_CARVEOUT_PX);
-    if (r == cudaSuccess) r = set_carveout(k_pixel<false, true, true>, APPGA_CARVEOUT_PX);
-    return r;
-  });
-  if (carve != cudaSuccess) return carve;
   const bool sl = a.S.off != nullptr;
-  const bool fold = a.fpair != nullptr;
-  if (fold && (!sl || a.S.rows != a.At.rows || a.n % 2 != 0)) return cudaErrorInvalidValue;
-  const int grid = px_blocks(a.At.rows, sl);
-  cudaError_t e;
-  if (fold)
-    e = a.use_bf16 ? launch_dep(k_pixel<true, true, true>, grid, PX::THREADS, s, a)
-                   : launch_dep(k_pixel<false, true, true>, grid, PX::THREADS, s, a);
-  else if (a.use_bf16)
-    e = sl ? launch_dep(k_pixel<true, true, false>, grid, PX::THREADS, s, a)
-           : launch_dep(k_pixel<true, false, false>, grid, PX::THREADS, s, a);
-  else
-    e = sl ? launch_dep(k_pixel<false, true, false>, grid, PX::THREADS, s, a)
-           : launch_dep(k_pixel<false, false, false>, grid, PX::THREADS, s, a);
+  if (a.fpair != nullptr && (!sl || a.S.rows != a.At.rows || a.n % 2 != 0))
+    return cudaErrorInvalidValue;
+  cudaError_t e = cudaErrorInvalidValue;
+  if (!sl) {
+    e = launch_dep(a.use_bf16 ? k_pixel<true, 0, false> : k_pixel<false, 0, false>,
+                   px_blocks(a.At.rows, 0), PX::THREADS, s, a);
+  } else {
+    switch (a.S.lanes) {
+      case 1: e = pixel_sliced<1>(a, s); break;
+      case 2: e = pixel_sliced<2>(a, s); break;
+      case 4: e = pixel_sliced<4>(a, s); break;
+      case 8: e = pixel_sliced<8>(a, s); break;
+    }
+  }
   if (e != cudaSuccess || a.theta_tab == nullptr || a.fuse_fin) return e;
   return launch_dep(k_finalize, 1, FIN_THREADS, s, a);
 }
