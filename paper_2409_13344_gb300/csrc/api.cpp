@@ -606,13 +606,14 @@ appga_status objective_on(appga_matrix* M, const float* f, const float* g, const
   a.data_out = ws.scalars;
   a.loop = 0;
   a.want_data = 1;
+  a.with_reg = 1;
+  a.ip = iter_params(p, false);
+  a.S = M->sell_a;
   a.n = M->n;
   CK(appga::launch_forward(a, s));
-  CK(appga::launch_reg_term(M->n, f, (float)p->lambda1, (float)p->lambda2, (float)p->eps,
-                            ws.partial_aux, ws.gtick, ws.st_scratch, ws.scalars + 1, s));
-  CK(cudaMemcpyAsync(ws.scalars_host, ws.scalars, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
+  CK(cudaMemcpyAsync(ws.scalars_host, ws.scalars, sizeof(double), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
-  *phi = ws.scalars_host[0] + ws.scalars_host[1];
+  *phi = ws.scalars_host[0];
   return APPGA_OK;
 }
 
@@ -1084,6 +1085,7 @@ appga_status appga_forward_ratio(appga_ctx* ctx, const appga_matrix* mat, const 
   a.data_out = data_out;
   a.loop = 0;
   a.want_data = data_out != nullptr ? 1 : 0;
+  a.S = M->sell_a;
   a.n = M->n;
   CK(appga::launch_forward(a, (cudaStream_t)stream));
   return APPGA_OK;
@@ -1096,7 +1098,7 @@ appga_status appga_backproject(appga_ctx* ctx, const appga_matrix* mat, const fl
   appga_status rc = ensure_workspace(M);
   if (rc != APPGA_OK) return rc;
   CK(cudaSetDevice(ctx->device));
-  CK(appga::launch_backproject(mat->At, w, out, 0, (cudaStream_t)stream));
+  CK(appga::launch_backproject(mat->At, mat->sell_t, w, out, (cudaStream_t)stream));
   return APPGA_OK;
 }
 
@@ -1131,12 +1133,13 @@ appga_status appga_pixel_update(appga_ctx* ctx, const appga_matrix* mat, const f
   h.theta_hi = (float)theta;
   h.theta_lo = (float)(theta - (double)h.theta_hi);
   h.t_cur = 1.0;
-  CK(cudaMemcpyAsync(M->ws.st_scratch, &h, sizeof h, cudaMemcpyHostToDevice, s));
+  CK(appga::launch_set_state(M->ws.st_scratch, h, s));
   // B^T grad phi~(B f~) of f~ = f_cur + theta (f_cur - f_prev)
   CK(appga::launch_stencil(M->n, f_cur, f_prev, (float)theta, (float)params->lambda1,
                            (float)params->lambda2, (float)params->eps, M->ws.gR, s));
   appga::PixArgs pa{};
   pa.At = M->At;
+  pa.S = M->sell_t;
   pa.n = M->n;
   pa.f[0] = const_cast<float*>(f_prev);
   pa.f[1] = const_cast<float*>(f_cur);
@@ -1152,6 +1155,7 @@ appga_status appga_pixel_update(appga_ctx* ctx, const appga_matrix* mat, const f
   q.precond_freeze_iter = -1;
   pa.ip = iter_params(&q, false);
   pa.use_bf16 = bf16_requested(M, params) ? 1 : 0;
+  pa.standalone = 1;
   CK(appga::launch_pixel(pa, s));
   return APPGA_OK;
 }

@@ -173,6 +173,7 @@ struct FwdArgs {
   int32_t want_data;   // evaluate the objective (data term; in the loop also the regulariser)
   int32_t use_bf16;
   int32_t no_stencil;  // solver loop without the SHOITV stencil blocks (AFPPA)
+  int32_t with_reg;    // standalone: data_out is the whole objective Phi(f)
   // loop: f^k in the 8 x 8-tiled pixel order; then A carries tiled column
   // indices (its projector gathers from ft, the stencil still reads f[])
   const float* ft;
@@ -182,8 +183,9 @@ struct FwdArgs {
   int32_t fresh_first;
   // loop: theta_{k0+i} of the run (the forward phase takes theta_k from it)
   const ThetaEntry* theta_tab;
-  // the sliced layout of A (solver projections with FP32 accumulation; its
-  // columns index ft); S.off == NULL: the CSR A
+  // the sliced layout of A (its columns are tiled; the solver's projections
+  // gather from ft, the double-float ones from the row-major image); S.off ==
+  // NULL: the CSR A
   DevSell S;
   // quarter-turn folded loop (fpair != NULL): S holds A's first fold_half
   // rows, the projector gathers fpair[t] = (f_j, f_{quarter_turn(j)}) at the
@@ -215,6 +217,7 @@ struct PixArgs {
   const ThetaEntry* theta_tab;
   IterParams ip;
   int32_t use_bf16;
+  int32_t standalone;  // one update outside the loop: compensated A^T w
   int32_t want_pmax;  // also reduce the largest preconditioner entry (AFPPA step sizes)
   float* ft;          // if set: f^{k+1} also written in the 8 x 8-tiled pixel order
   // 1: the pixel phase's first blocks finalise the step (Phi(f^k) from the
@@ -239,13 +242,12 @@ int max_group_tickets(int m, int n);
 
 cudaError_t launch_forward(const FwdArgs& a, cudaStream_t s);
 cudaError_t launch_pixel(const PixArgs& a, cudaStream_t s);
-cudaError_t launch_backproject(const DevCSR& At, const float* w, float* out, int use_bf16,
+// out = A^T w in FP32, through the sliced layout where there is one (S.off)
+cudaError_t launch_backproject(const DevCSR& At, const DevSell& S, const float* w, float* out,
                                cudaStream_t s);
+cudaError_t launch_set_state(SolverState* st, const SolverState& h, cudaStream_t s);
 cudaError_t launch_stencil(int n, const float* f_cur, const float* f_prev, float theta,
                            float lam1, float lam2, float eps, float* out, cudaStream_t s);
-cudaError_t launch_reg_term(int n, const float* f, float lam1, float lam2, float eps,
-                            float2* partial, unsigned int* gtick, SolverState* st, double* out,
-                            cudaStream_t s);
 // Solver-run input check without a host round trip: on a bad g, gamma, fa or
 // fb (fa, fb may be NULL) sets APPGA_FLAG_DOMAIN in st->flags and st->done.
 cudaError_t launch_check_inputs(const float* g, const float* gamma, int m, const float* fa,

@@ -146,6 +146,12 @@ bool build_sell(const std::vector<int32_t>& order, int lanes, const std::vector<
     const int64_t base = out->off[(size_t)s];
     for (int q = 0; q < C; ++q) {
       const int32_t r = order[(size_t)s * C + q], npk = packs(r);
+      // what is left of a row repeats a column of its last pack with zero
+      // values: no vector entry that the row does not meet is read for it
+      const int32_t steps = (out->off[(size_t)s + 1] - out->off[(size_t)s]) / 32;
+      for (int32_t k = npk; npk > 0 && k < steps * L; ++k)
+        out->cols[(size_t)(base + (int64_t)(k / L) * 32 + q * L + k % L)] =
+            (uint64_t)col[(size_t)row_ptr[r + 1] - PACK_ENTRIES];
       for (int32_t k = 0; k < npk; ++k) {
         const int64_t pos = base + (int64_t)(k / L) * 32 + q * L + (k % L);
         const int32_t e = row_ptr[r] + k * PACK_ENTRIES;

@@ -28,7 +28,7 @@
 // 57-64 % of a launch's cycles): slices hold neighbouring pixels, or rays of a
 // few bins and angles with their entries in order along the ray, and a row gets
 // as few lanes as still fill the chip (sell_lanes).  Rows in ascending order
-// with four lanes each took 38.1 us per folded map at 256^2, 32 now; 112 at
+// with four lanes each took 38.1 us per folded map at 256^2, 33 now; 112 at
 // 400^2, 92 now.  When A has the quarter-turn symmetry the
 // loop streams only its folded halves (FOLD): each stored entry serves two
 // products, gathered as pairs (see fold_partner in appga_internal.h).  The
@@ -52,6 +52,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <cfloat>
 #include <cmath>
 
 #include "appga_internal.h"
@@ -134,11 +135,6 @@ using PX = Shape<APPGA_PX_W, APPGA_PX_RPW, APPGA_PX_PF>;
 // row starts of a warp's group kept in shared memory instead of registers
 #ifndef APPGA_SBND
 #define APPGA_SBND 1
-#endif
-// accumulation of y = A f in the solver loop: 0 = FP32 (as the back-projection),
-// 1 = double-float per product
-#ifndef APPGA_LOOP_DF
-#define APPGA_LOOP_DF 0
 #endif
 
 constexpr int SLOT_W = 33;    // slot row stride: per-row sums read without bank conflicts
@@ -465,6 +461,76 @@ struct SellGroup {
     for (int o = 1; o < L; o <<= 1) r = add_v(r, shfl_xor_v(r, o));
     return r;
   }
+
+  // The same with each step's four products added to a compensated sum, for
+  // the stand-alone calls: no chain of rounded sums at any L.
+  __device__ __forceinline__ float stream_comp(const DevSell& S, const float* __restrict__ x,
+                                               uint64_t pol) {
+    float hi = 0.f, lo = 0.f;
+    float4 xg = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (steps > 0) xg = gather4(x, unpack_cols(c[0]));
+    for (int t0 = 0; t0 < steps; t0 += PF) {
+#pragma unroll
+      for (int u = 0; u < PF; ++u) {
+        const int t = t0 + u;
+        if (t < steps) {
+          const float4 vv = v[u], xx = xg;
+          if (t + PF < steps) {
+            c[u] = ld_stream_u2(S.cols + q0 + ((t + PF) << 5), pol);
+            v[u] = vals(S, q0 + ((t + PF) << 5), pol);
+          }
+          if (t + 1 < steps) xg = gather4(x, unpack_cols(c[(u + 1) % PF]));
+          acc_add(hi, lo, fmaf(vv.x, xx.x, fmaf(vv.y, xx.y, fmaf(vv.z, xx.z, vv.w * xx.w))), 0.f);
+        }
+      }
+    }
+#pragma unroll
+    for (int o = 1; o < L; o <<= 1)
+      acc_add(hi, lo, __shfl_xor_sync(0xffffffffu, hi, o), __shfl_xor_sync(0xffffffffu, lo, o));
+    return fabsf(hi) <= FLT_MAX ? hi + lo : hi;  // an infinite sum has no error term
+  }
+
+  // Row sums of the slice times the row-major n x n image x in double-float
+  // (hi, lo), in every lane of the row; the packed columns are 8 x 8-tiled.
+  __device__ __forceinline__ float2 stream_df(const DevSell& S, const float* __restrict__ x, int n,
+                                              uint64_t pol) {
+    const int nb = (n + 7) / 8;
+    const float inv = 1.f / (float)nb;
+    // tile / nb exactly: tiles below 2^14 (a packed column is below 2^20)
+    auto at = [&](int t) {
+      const int tile = t >> 6, tr = (int)(((float)tile + 0.5f) * inv);
+      return __ldg(x + (8 * tr + ((t >> 3) & 7)) * n + 8 * (tile - tr * nb) + (t & 7));
+    };
+    auto gather = [&](uint2 w) {
+      const int4 k = unpack_cols(w);
+      return make_float4(at(k.x), at(k.y), at(k.z), at(k.w));
+    };
+    float hi = 0.f, lo = 0.f;
+    float4 xg = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (steps > 0) xg = gather(c[0]);
+    for (int t0 = 0; t0 < steps; t0 += PF) {
+#pragma unroll
+      for (int u = 0; u < PF; ++u) {
+        const int t = t0 + u;
+        if (t < steps) {
+          const float4 vv = v[u], xx = xg;
+          if (t + PF < steps) {
+            c[u] = ld_stream_u2(S.cols + q0 + ((t + PF) << 5), pol);
+            v[u] = vals(S, q0 + ((t + PF) << 5), pol);
+          }
+          if (t + 1 < steps) xg = gather(c[(u + 1) % PF]);
+          acc_fma(hi, lo, vv.x, xx.x);
+          acc_fma(hi, lo, vv.y, xx.y);
+          acc_fma(hi, lo, vv.z, xx.z);
+          acc_fma(hi, lo, vv.w, xx.w);
+        }
+      }
+    }
+#pragma unroll
+    for (int o = 1; o < L; o <<= 1)
+      acc_add(hi, lo, __shfl_xor_sync(0xffffffffu, hi, o), __shfl_xor_sync(0xffffffffu, lo, o));
+    return make_float2(hi, lo);
+  }
 };
 
 // Sum of row `lane` of a streamed group in lanes 0..nrows-1 from the warp's
@@ -698,8 +764,7 @@ __global__ void FW_BOUNDS k_forward(FwdArgs a) {
     } slot;
     StencilSmem st;
   } sm;
-  static_assert(!(SL && DFA), "the sliced layout serves the FP32-accumulated projections");
-  static_assert(!FOLD || SL, "the folded loop streams the sliced layout");
+  static_assert(!FOLD || (SL && !DFA), "the folded loop streams the sliced layout");
   pdl_trigger();
   SolverState* st = a.st;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -768,6 +833,8 @@ __global__ void FW_BOUNDS k_forward(FwdArgs a) {
     if (nrows > 0) {
       if constexpr (FOLD) {
         yy = sg.stream(a.S, a.fpair, pol);
+      } else if constexpr (DFA) {
+        yy = sg.stream_df(a.S, a.f[0], a.n, pol);
       } else {
         yy.x = sg.stream(a.S, f, pol);
       }
@@ -780,6 +847,8 @@ __global__ void FW_BOUNDS k_forward(FwdArgs a) {
     for (int t = threadIdx.x; t < (FOLD ? 2 : 1) * BR; t += FW::THREADS) {
       const int q = t % BR, i = yrow[q];
       if (i < 0) continue;
+      // an empty ray's padding gathers pixel 0, whatever that holds
+      if (DFA && a.A.row_ptr[i] == a.A.row_ptr[i + 1]) ysum[q] = make_float2(0.f, 0.f);
       if constexpr (FOLD) {
         const bool partner = t >= BR;
         const float wv =
@@ -787,7 +856,7 @@ __global__ void FW_BOUNDS k_forward(FwdArgs a) {
                         partner ? ysum[q].y : ysum[q].x, 0.f, hits, bad, acc_hi, acc_lo, false);
         if (a.w != nullptr) a.w[2 * i + (partner ? 1 : 0)] = wv;
       } else {
-        forward_row(a, g, gamma, th, kk, i, ysum[q].x, 0.f, hits, bad, acc_hi, acc_lo);
+        forward_row(a, g, gamma, th, kk, i, ysum[q].x, ysum[q].y, hits, bad, acc_hi, acc_lo);
       }
     }
   } else if (proj) {
@@ -816,10 +885,12 @@ __global__ void FW_BOUNDS k_forward(FwdArgs a) {
     if (lane < nrows) forward_row(a, g, gamma, th, kk, row0 + lane, hi, lo, hits, bad, acc_hi, acc_lo);
 #endif
   } else {
-    // SHOITV gradient at f~^kk and the regulariser of Phi(f^kk)
+    // SHOITV gradient at f~^kk and the regulariser of Phi(f^kk); stand-alone
+    // objective: the regulariser of f alone
     const int b = sb;
     const int ntx = st_tiles_x(a.n);
-    const float reg = stencil_tile(sm.st, a.f[kk % 3], a.f[(kk + 2) % 3], th.hi,
+    const float reg = stencil_tile(sm.st, a.loop ? a.f[kk % 3] : a.f[0],
+                                   a.loop ? a.f[(kk + 2) % 3] : a.f[0], th.hi,
                                    (b / ntx) * ST_R, (b % ntx) * ST_C, a.n, a.ip.lambda1,
                                    a.ip.lambda2, a.ip.eps, a.gR, a.want_data != 0);
     acc_hi = reg;
@@ -948,7 +1019,10 @@ __device__ void fused_finalize(const PixArgs& a, SolverState* st, int kk) {
 // s1(q_r) + s2(q_{r-1}), the second term from the lanes of member r-1, and
 // f^{k+1} at q_r goes out with its turned neighbour f^{k+1} at q_{r+1} as the
 // next forward phase's pair.
-template <bool BF16, int L, bool FOLD>
+//
+// ONE (unfolded, sliced): a single update outside the loop, its A^T w summed
+// with compensation.
+template <bool BF16, int L, bool FOLD, bool ONE = false>
 __global__ void PX_BOUNDS k_pixel(PixArgs a) {
   constexpr bool SL = L > 0;
   constexpr int LL = SL ? L : 1, SROWS = 32 / LL, ORB = SROWS / 4;
@@ -998,7 +1072,9 @@ __global__ void PX_BOUNDS k_pixel(PixArgs a) {
         const float s2 = __shfl_sync(0xffffffffu, sp.y, (lane + 32 - ORB * LL) & 31);
         bp = sp.x + s2;
       } else {
-        bp = sg.stream(a.S, a.w, pol);
+        bp = ONE ? sg.stream_comp(a.S, a.w, pol) : sg.stream(a.S, a.w, pol);
+        // the padding of a pixel that no ray meets gathers w_0, whatever that holds
+        if (ONE && j >= 0 && a.At.row_ptr[j] == a.At.row_ptr[j + 1]) bp = 0.f;
       }
       if (j >= 0 && part == 0) pmax = fmaxf(pmax, pixel_update(a, kk, j, bp, bad, fn));
       if constexpr (FOLD) {
@@ -1119,7 +1195,6 @@ __global__ void k_theta_table(SolverState* st, ThetaEntry* tab, int k0, int n, i
 }
 
 // Standalone back-projection (step a3): out = A^T w.
-template <bool BF16>
 __global__ void __launch_bounds__(PX::THREADS) k_backproject(DevCSR At, const float* __restrict__ w,
                                                             float* __restrict__ out) {
   __shared__ float slot[PX::W][PX::R * SLOT_W];
@@ -1128,10 +1203,31 @@ __global__ void __launch_bounds__(PX::THREADS) k_backproject(DevCSR At, const fl
   const int row0 = blockIdx.x * PX::ROWS + warp * PX::R;
   const int nrows = max(0, min(PX::R, At.rows - row0));
   float s, unused;
-  warp_rows_dot<BF16, false, PX::R, PX::PF>(At, row0, nrows, w, lane, slot[warp], nullptr, s,
+  warp_rows_dot<false, false, PX::R, PX::PF>(At, row0, nrows, w, lane, slot[warp], nullptr, s,
                                             unused, reinterpret_cast<int*>(sbnd[warp]));
   if (lane < nrows) out[row0 + lane] = s;
 }
+
+// The same through the sliced A^T.
+template <int L>
+__global__ void __launch_bounds__(PX::THREADS) k_backproject_sliced(DevSell S,
+                                                                   const int32_t* row_ptr,
+                                                                   const float* __restrict__ w,
+                                                                   float* __restrict__ out) {
+  const int lane = threadIdx.x & 31, slice = blockIdx.x * PX::W + (threadIdx.x >> 5);
+  if (slice >= S.slices) return;
+  const uint64_t pol = evict_first_policy();
+  SellGroup<false, APPGA_SELL_PX_PF, L> sg;
+  sg.prologue(S, slice, lane, pol);
+  const int j = __ldg(S.row + slice * (32 / L) + lane / L);
+  const float s = sg.stream_comp(S, w, pol);
+  // the padding of an empty row gathers w_0, whatever that holds
+  if (j >= 0 && lane % L == 0) out[j] = row_ptr[j] == row_ptr[j + 1] ? 0.f : s;
+}
+
+// One state to *st (a kernel in the stream: a copy from pageable memory would
+// be staged and would leave the compute queue).
+__global__ void k_set_state(SolverState* st, SolverState h) { *st = h; }
 
 // Stencil kernel: gR = B^T grad phi~(B f~) with f~ = f_cur + theta (f_cur - f_prev)
 // (theta = 0, f_prev = f_cur: the plain SHOITV gradient, step a4).
@@ -1143,20 +1239,6 @@ __global__ void __launch_bounds__(FW::THREADS) k_stencil(int n, const float* __r
   const int ntx = st_tiles_x(n);
   stencil_tile(S, f_cur, f_prev, theta, (blockIdx.x / ntx) * ST_R, (blockIdx.x % ntx) * ST_C, n,
                lam1, lam2, eps, out, false);
-}
-
-// Regulariser term phi~(B f) (objective, step a6).
-__global__ void __launch_bounds__(FW::THREADS) k_reg_term(int n, const float* __restrict__ f,
-                                                         float lam1, float lam2, float eps,
-                                                         float2* partial, unsigned int* gtick,
-                                                         SolverState* st, double* out) {
-  __shared__ StencilSmem S;
-  const int ntx = st_tiles_x(n);
-  const float reg = stencil_tile(S, f, f, 0.f, (blockIdx.x / ntx) * ST_R,
-                                 (blockIdx.x % ntx) * ST_C, n, lam1, lam2, eps, nullptr, true);
-  const df b = block_sum_acc(reg, 0.f);
-  double tot = 0.0;
-  if (grid_reduce(partial, gtick, &st->ticket_aux, b, &tot) && threadIdx.x == 0) *out = tot;
 }
 
 // Input check of a solver run: marks the run state with APPGA_FLAG_DOMAIN and
@@ -1346,17 +1428,22 @@ int max_group_tickets(int m, int n) { return max_partials(m, n) / RED_GROUP + 1;
 
 namespace {
 template <int L>
-cudaError_t forward_sliced(const FwdArgs& a, cudaStream_t s) {
+cudaError_t forward_sliced(const FwdArgs& a, bool tiles, bool dfa, cudaStream_t s) {
   static PerDeviceOnce carve_once;
   const cudaError_t carve = carve_once.run([] {
     cudaError_t r = set_carveout(k_forward<true, false, L, false>, APPGA_CARVEOUT_FW);
     if (r == cudaSuccess) r = set_carveout(k_forward<false, false, L, false>, APPGA_CARVEOUT_FW);
     if (r == cudaSuccess) r = set_carveout(k_forward<true, false, L, true>, APPGA_CARVEOUT_FW);
     if (r == cudaSuccess) r = set_carveout(k_forward<false, false, L, true>, APPGA_CARVEOUT_FW);
+    if (r == cudaSuccess) r = set_carveout(k_forward<true, true, L, false>, APPGA_CARVEOUT_FW);
+    if (r == cudaSuccess) r = set_carveout(k_forward<false, true, L, false>, APPGA_CARVEOUT_FW);
     return r;
   });
   if (carve != cudaSuccess) return carve;
-  const int grid = fw_proj_blocks(a.A.rows, a.S.slices) + (a.loop && !a.no_stencil ? st_tiles(a.n) : 0);
+  const int grid = fw_proj_blocks(a.A.rows, a.S.slices) + (tiles ? st_tiles(a.n) : 0);
+  if (dfa)
+    return launch_dep(a.use_bf16 ? k_forward<true, true, L, false> : k_forward<false, true, L, false>,
+                      grid, FW::THREADS, s, a);
   void (*kern)(FwdArgs) =
       a.fpair != nullptr ? (a.use_bf16 ? k_forward<true, false, L, true> : k_forward<false, false, L, true>)
                          : (a.use_bf16 ? k_forward<true, false, L, false> : k_forward<false, false, L, false>);
@@ -1373,8 +1460,10 @@ cudaError_t pixel_sliced(const PixArgs& a, cudaStream_t s) {
     return r;
   });
   if (carve != cudaSuccess) return carve;
-  void (*kern)(PixArgs) = a.fpair != nullptr ? (a.use_bf16 ? k_pixel<true, L, true> : k_pixel<false, L, true>)
-                                             : (a.use_bf16 ? k_pixel<true, L, false> : k_pixel<false, L, false>);
+  void (*kern)(PixArgs) =
+      a.standalone ? (a.use_bf16 ? k_pixel<true, L, false, true> : k_pixel<false, L, false, true>)
+      : a.fpair != nullptr ? (a.use_bf16 ? k_pixel<true, L, true> : k_pixel<false, L, true>)
+                           : (a.use_bf16 ? k_pixel<true, L, false> : k_pixel<false, L, false>);
   return launch_dep(kern, px_blocks(a.At.rows, a.S.slices), PX::THREADS, s, a);
 }
 }  // namespace
@@ -1382,18 +1471,18 @@ cudaError_t pixel_sliced(const PixArgs& a, cudaStream_t s) {
 cudaError_t launch_forward(const FwdArgs& a, cudaStream_t s) {
   cudaError_t e = ensure_tables();
   if (e != cudaSuccess) return e;
-  const int grid = proj_blocks<FW>(a.A.rows) + (a.loop && !a.no_stencil ? st_tiles(a.n) : 0);
+  const bool tiles = a.loop ? a.no_stencil == 0 : a.with_reg != 0;
+  const int grid = proj_blocks<FW>(a.A.rows) + (tiles ? st_tiles(a.n) : 0);
   // the solver (its loop and its projection of the previous iterate)
   // accumulates y in FP32; the stand-alone projection and objective calls
   // in double-float
-  const bool dfa = (a.loop || a.solver_acc) ? APPGA_LOOP_DF != 0 : true;
-  // the sliced layout serves the solver's FP32-accumulated projections
-  if (a.S.off != nullptr && !dfa) {
+  const bool dfa = !(a.loop || a.solver_acc);
+  if (a.S.off != nullptr) {
     switch (a.S.lanes) {
-      case 1: return forward_sliced<1>(a, s);
-      case 2: return forward_sliced<2>(a, s);
-      case 4: return forward_sliced<4>(a, s);
-      case 8: return forward_sliced<8>(a, s);
+      case 1: return forward_sliced<1>(a, tiles, dfa, s);
+      case 2: return forward_sliced<2>(a, tiles, dfa, s);
+      case 4: return forward_sliced<4>(a, tiles, dfa, s);
+      case 8: return forward_sliced<8>(a, tiles, dfa, s);
     }
     return cudaErrorInvalidValue;
   }
@@ -1449,26 +1538,31 @@ cudaError_t launch_copy_result(const SolverState* st, float* const f[3], float* 
                     (const float*)f[2], out, out_prev, d);
 }
 
-cudaError_t launch_backproject(const DevCSR& At, const float* w, float* out, int use_bf16,
+cudaError_t launch_backproject(const DevCSR& At, const DevSell& S, const float* w, float* out,
                                cudaStream_t s) {
-  const int grid = proj_blocks<PX>(At.rows);
-  if (use_bf16)
-    k_backproject<true><<<grid, PX::THREADS, 0, s>>>(At, w, out);
-  else
-    k_backproject<false><<<grid, PX::THREADS, 0, s>>>(At, w, out);
+  const int blocks = px_blocks(At.rows, S.off != nullptr ? S.slices : 0);
+  if (S.off == nullptr) {
+    k_backproject<<<blocks, PX::THREADS, 0, s>>>(At, w, out);
+  } else {
+    switch (S.lanes) {
+      case 1: k_backproject_sliced<1><<<blocks, PX::THREADS, 0, s>>>(S, At.row_ptr, w, out); break;
+      case 2: k_backproject_sliced<2><<<blocks, PX::THREADS, 0, s>>>(S, At.row_ptr, w, out); break;
+      case 4: k_backproject_sliced<4><<<blocks, PX::THREADS, 0, s>>>(S, At.row_ptr, w, out); break;
+      case 8: k_backproject_sliced<8><<<blocks, PX::THREADS, 0, s>>>(S, At.row_ptr, w, out); break;
+      default: return cudaErrorInvalidValue;
+    }
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_set_state(SolverState* st, const SolverState& h, cudaStream_t s) {
+  k_set_state<<<1, 1, 0, s>>>(st, h);
   return cudaGetLastError();
 }
 
 cudaError_t launch_stencil(int n, const float* f_cur, const float* f_prev, float theta,
                            float lam1, float lam2, float eps, float* out, cudaStream_t s) {
   k_stencil<<<st_tiles(n), FW::THREADS, 0, s>>>(n, f_cur, f_prev, theta, lam1, lam2, eps, out);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_reg_term(int n, const float* f, float lam1, float lam2, float eps,
-                            float2* partial, unsigned int* gtick, SolverState* st, double* out,
-                            cudaStream_t s) {
-  k_reg_term<<<st_tiles(n), FW::THREADS, 0, s>>>(n, f, lam1, lam2, eps, partial, gtick, st, out);
   return cudaGetLastError();
 }
 

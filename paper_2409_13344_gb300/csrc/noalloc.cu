@@ -52,10 +52,6 @@ cudaError_t scratch_address(int device, void** out) {
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-__global__ void k_sum2(const double* parts, double* out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) *out = parts[0] + parts[1];
-}
-
 }  // namespace
 
 extern "C" appga_status appga_objective_noalloc(appga_ctx* ctx, const appga_matrix* mat,
@@ -68,13 +64,14 @@ extern "C" appga_status appga_objective_noalloc(appga_ctx* ctx, const appga_matr
   if (mat->ctx != ctx) return fail(APPGA_EINVAL, "matrix belongs to another context");
   appga_status rc = appga_params_validate(params);
   if (rc != APPGA_OK) return rc;
-  // scratch layout: partials | group tickets | state | two partial sums
+  // scratch layout: partials | group tickets | state | 16 spare bytes (part of
+  // the size limit that callers know)
   const int np = max_partials(mat->m, mat->n);
   const int ng = max_group_tickets(mat->m, mat->n);
   const size_t off_tick = align256((size_t)np * sizeof(float2));
   const size_t off_state = off_tick + align256((size_t)ng * sizeof(unsigned int));
-  const size_t off_sums = off_state + align256(sizeof(SolverState));
-  const size_t need = off_sums + 2 * sizeof(double);
+  const size_t off_end = off_state + align256(sizeof(SolverState));
+  const size_t need = off_end + 2 * sizeof(double);
   if (need > kScratchBytes)
     return fail(APPGA_EINVAL, "appga_objective_noalloc: this matrix needs " + std::to_string(need) +
                                   " bytes of scratch; the fixed scratch holds " +
@@ -88,10 +85,9 @@ extern "C" appga_status appga_objective_noalloc(appga_ctx* ctx, const appga_matr
   auto* partial = reinterpret_cast<float2*>(bytes);
   auto* gtick = reinterpret_cast<unsigned int*>(bytes + off_tick);
   auto* st = reinterpret_cast<SolverState*>(bytes + off_state);
-  auto* sums = reinterpret_cast<double*>(bytes + off_sums);
   cudaStream_t s = (cudaStream_t)stream;
   // the tickets and the state start at zero; partials are written before read
-  e = cudaMemsetAsync(gtick, 0, off_sums - off_tick, s);
+  e = cudaMemsetAsync(gtick, 0, off_end - off_tick, s);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(scratch)");
   FwdArgs a{};
   a.A = mat->A;
@@ -102,18 +98,14 @@ extern "C" appga_status appga_objective_noalloc(appga_ctx* ctx, const appga_matr
   a.st = st;
   a.partial = partial;
   a.gtick = gtick;
-  a.data_out = sums;
+  a.data_out = phi_out;
   a.loop = 0;
   a.want_data = 1;
+  a.with_reg = 1;
+  a.ip = iter_params(params, false);
+  a.S = mat->sell_a;
   a.n = mat->n;
   e = launch_forward(a, s);
-  if (e == cudaSuccess)
-    e = launch_reg_term(mat->n, f, (float)params->lambda1, (float)params->lambda2,
-                        (float)params->eps, partial, gtick, st, sums + 1, s);
-  if (e == cudaSuccess) {
-    k_sum2<<<1, 32, 0, s>>>(sums, phi_out);
-    e = cudaGetLastError();
-  }
   if (e != cudaSuccess) return cuda_fail(e, "appga_objective_noalloc launch");
   return APPGA_OK;
 }

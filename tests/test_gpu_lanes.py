@@ -86,3 +86,40 @@ def test_batched_groups_of_large_matrices(A, ctx, n, angles):
         ref = O.appga(O.Problem(Amat, sls[i].g, sls[i].gamma, n), O.Params(**PAR),
                       n_angles=angles, track_phi=False).f
         assert np.linalg.norm(whole[i] - ref) <= 5e-6 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("n,angles,bins", [(16, 10, 8), (178, 6, 253), (247, 5, 350),
+                                           (24, 3734, 34), (24, 7484, 34)])
+def test_single_projections_touch_only_their_entries(A, ctx, n, angles, bins):
+    # entries a row does not have are never read into it: an infinite vector
+    # entry reaches exactly the rows that hold it, an empty row stays zero, and
+    # the other rows keep the accuracy of double-float / compensated sums
+    geom = W.Geometry(n, angles, bins)
+    Amat = W.siddon_matrix(geom).astype(np.float64)
+    mat = A.Matrix(ctx, Amat.astype(np.float32), n, angles)
+    m, d = Amat.shape
+    rng = np.random.default_rng(2)
+    f = rng.random(d).astype(np.float32)
+    w = rng.standard_normal(m).astype(np.float32)
+    y_ref, b_ref = Amat @ f, Amat.T @ w
+    hit = np.asarray(Amat.sum(axis=1)).ravel() > 0
+    for x in (0, d // 2 + n // 2):
+        f[x] = np.inf
+        w[x % m] = np.inf
+        y = torch.empty(m, dtype=torch.float64, device=DEV)
+        one = torch.ones(m, dtype=torch.float32, device=DEV)
+        A.appga_forward_ratio(ctx.handle, mat.handle, torch.from_numpy(f).to(DEV), one, one, y)
+        out = torch.empty(d, dtype=torch.float32, device=DEV)
+        A.appga_backproject(ctx.handle, mat.handle, torch.from_numpy(w).to(DEV), out)
+        y, out = y.cpu().numpy(), out.cpu().numpy()
+        col = np.zeros(m, bool)
+        for xx in np.nonzero(~np.isfinite(f))[0]:
+            col |= Amat[:, [xx]].toarray().ravel() != 0
+        row = np.zeros(d, bool)
+        for xx in np.nonzero(~np.isfinite(w))[0]:
+            row |= Amat[[xx]].toarray().ravel() != 0
+        assert np.all(~np.isfinite(y[col])) and np.all(y[~hit] == 0)
+        assert np.all(np.abs(y - y_ref)[~col] <= 1e-11 * y_ref[~col])
+        assert not np.isfinite(out[row]).any()
+        bound = 3e-7 * (Amat.T @ np.where(np.isfinite(w), np.abs(w), 0))
+        assert np.all(np.abs(out - b_ref)[~row] <= bound[~row])
