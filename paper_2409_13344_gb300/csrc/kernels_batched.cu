@@ -246,7 +246,10 @@ __device__ __forceinline__ void quad_sums(const DevQuad& M, int b, const float* 
   auto step = [&](auto full) {
     // the stream is two steps ahead in L2 (the loads below would otherwise
     // wait for DRAM: 207 us of back-projection at 64 slots of 256 x 256, 189 so)
-    prefetch_l2(M.vals + 4 * (size_t)(k + 2 * S * U));
+    if constexpr (BF16)
+      prefetch_l2(M.vals_bf16 + 4 * (size_t)(k + 2 * S * U));
+    else
+      prefetch_l2(M.vals + 4 * (size_t)(k + 2 * S * U));
     prefetch_l2(M.cols + (k + 2 * S * U));
 #pragma unroll
     for (int h = 0; h < 4; h += NZ) {

@@ -113,7 +113,7 @@ appga_status build(const DevCSR& M, cudaStream_t s, DevQuad* out, int64_t* bytes
     // (the projectors' L2 prefetches run up to 64 packs past the end)
     if (e == cudaSuccess) e = dalloc(&q.cols, np + 64, bytes);
     if (e == cudaSuccess) e = dalloc(&q.vals, 4 * np + 256, bytes);
-    if (e == cudaSuccess && M.val_bf16) e = dalloc(&q.vals_bf16, 4 * np, bytes);
+    if (e == cudaSuccess && M.val_bf16) e = dalloc(&q.vals_bf16, 4 * np + 256, bytes);
   }
   if (e == cudaSuccess) {
     k_quad_fill<<<grid, 64, 0, s>>>(M, q);
