@@ -274,9 +274,11 @@ appga_status appga_reconstruct_host(appga_ctx* ctx, const appga_matrix* mat, con
  * does not depend on the other slices in the batch.  The projector
  * accumulation is FP32 in a different order from the single-slice path, so
  * results agree with appga_reconstruct to FP32 rounding.  Slices are held in
- * blocks of Kp = 32, 64 or 128 slots (the smallest that holds K); the
- * kernels index them with 32-bit offsets, so max(m, d) * Kp must stay below
- * 2^31 (else EINVAL).  EINVAL also for K outside [1, 128] or bad params;
+ * blocks of Kp = 32, 64 or 128 slots (the smallest that holds K), of which the
+ * kernels work on the first 8, 16, 32, 64 or 128 (again the smallest that
+ * holds K); they index slots with 32-bit offsets, so max(m, d) * Kp must stay
+ * below 2^31 (else EINVAL).  The first batched call of a matrix builds the
+ * layout that these kernels stream and keeps it with the matrix.  EINVAL also for K outside [1, 128] or bad params;
  * EDOMAIN for non-finite or negative g or f_init, or gamma <= 0.  Synchronises. */
 appga_status appga_reconstruct_batched(appga_ctx* ctx, const appga_matrix* mat, int32_t K,
                                        const float* g, const float* gamma, const float* f_init,
@@ -289,7 +291,7 @@ appga_status appga_reconstruct_batched(appga_ctx* ctx, const appga_matrix* mat, 
  * reduced against the width-float rows of a slot-minor block named by its
  * columns (the column/value stream and the gathers), in the projectors' row
  * order, with no epilogue, stencil or pixel update, for several grid sizes
- * (blocks per SM), and keeps the fastest.  *gbs_fwd: A's rows against an
+ * (virtual blocks of four warps per SM), and keeps the fastest.  *gbs_fwd: A's rows against an
  * image block [d][width] (the forward projection); *gbs_bwd: A^T's rows
  * against a weight block [m][width] (the back-projection); both host doubles,
  * gathered bytes (padded entries x width x 4) per second / 1e9.  width: 32,
@@ -345,11 +347,11 @@ appga_status appga_reconstruct_volume(appga_ctx* ctx, const appga_matrix* mat, i
  * Each trial runs 4 + 16 APPGA maps of every slice (after 4 warm-up maps)
  * and is timed with CUDA events on the library stream.  Tunables, searched
  * one after another from the kernels' defaults: the sub-batch width (run K
- * slices as several batches of 32 or 64), SpMV blocks per SM of the forward
- * phase, blocks per SM of the back-projection, stencil blocks per SM, and for
- * each projection the rows it gathers per step of its staged (column, value)
- * pairs (8, or 4: fewer loads in flight, fewer registers; separate kernel
- * instances).  The
+ * slices as several batches of 32 or 64), the shares per SM that the forward
+ * phase's rows, the back-projection's rows and the stencil's tiles are dealt
+ * into (four-warp blocks of the work list), and for each projection the
+ * gathers a team keeps in flight (8, or 4: half as many, fewer registers;
+ * separate kernel instances, for matrices of at least 4864 row blocks).  The
  * best schedule is kept in the matrix handle and used by later
  * appga_reconstruct_batched calls (and server pools) with the same padded
  * width (32, 64 or 128) and precision.  out_host (may be NULL) receives the
@@ -365,8 +367,8 @@ typedef struct {
   int32_t stencil_per_sm; /* 0 = kernel default */
   int32_t pixel_per_sm;   /* 0 = kernel default */
   int32_t chunk;          /* slices per sub-batch; 0 = the whole batch */
-  int32_t gather_rows_fw; /* image rows the forward projection gathers per step: 8 or 4 (0 = 8) */
-  int32_t gather_rows_px; /* weight rows the back-projection gathers per step: 8 or 4 (0 = 8) */
+  int32_t gather_rows_fw; /* forward projection's gathers in flight: 8, or 4 for half (0 = 8) */
+  int32_t gather_rows_px; /* back-projection's gathers in flight: 8, or 4 for half (0 = 8) */
   double us_per_slice_iter;         /* chosen schedule, microseconds per slice-iteration */
   double us_per_slice_iter_default; /* the default schedule */
 } appga_batch_tuning;

@@ -38,9 +38,10 @@
  * A request's result does not depend on which slot it runs in, on the other
  * requests of its pool, or on when it was admitted: every slot runs the same
  * per-slot arithmetic, so the same request gives the same image alone and in
- * any mix with the same pool width and precision.  (With adaptive widths a
- * request's pool width depends on the load, and images of the same request
- * agree to FP32 rounding across widths.)
+ * any mix with the same precision.  A row's sum is the same whatever the
+ * number of slots the kernels run, so it does not depend on the pool's width,
+ * nor on how many of the pool's slots are live (a replay works on the first 8,
+ * 16, 32, 64 or 128 slots, the smallest that holds them).
  *
  * Streams: every pool has its own stream, so the replays of different pools
  * (and geometries) overlap on the device.  A scheduling round
