@@ -80,6 +80,7 @@ appga_status upload_sell(const appga::HostSell& h, const std::vector<int32_t>& r
   c.rows = rows;
   c.slices = h.slices;
   c.lanes = h.lanes;
+  c.packs = h.off.back();
   const size_t np = h.vals.size() / appga::PACK_ENTRIES;
   cudaError_t e = dalloc(&c.off, h.off.size(), bytes);
   if (e == cudaSuccess) e = dalloc(&c.row, row.size(), bytes);
@@ -1000,6 +1001,14 @@ appga_status appga_matrix_create(appga_ctx* ctx, int32_t m, int32_t d, int32_t n
         }
       }
     }
+    auto fetch_ahead = [](DevSell& a, DevSell& t) {
+      const int64_t packs = (int64_t)a.packs + t.packs;
+      for (int bf = 0; bf < 2; ++bf)
+        if (appga::sell_fetch_ahead(a, t, packs * (bf ? 16 : 24))) a.ahead |= 1 << bf;
+      t.ahead = a.ahead;
+    };
+    fetch_ahead(M->sell_a, M->sell_t);
+    fetch_ahead(M->fold_a, M->fold_t);
     if (e != cudaSuccess) rc = cuda_fail(e, "tiled column indices and sliced layout");
   }
   if (rc == APPGA_OK) {

@@ -34,6 +34,8 @@ constexpr int32_t PACK_OFFSET_MAX = 8191;
 // or pixel of each row position (-1: none).
 struct DevSell {
   int32_t rows = 0, slices = 0, lanes = 0;
+  int32_t packs = 0;
+  int32_t ahead = 0;  // slices fetched into L2 ahead (sell_fetch_ahead): bit 0 FP32, bit 1 BF16
   int32_t* off = nullptr;
   int32_t* row = nullptr;
   uint2* cols = nullptr;    // packed words
@@ -349,6 +351,7 @@ bool build_sell(const std::vector<int32_t>& order, int lanes, const std::vector<
                 const std::vector<int32_t>& col, const std::vector<float>& val, HostSell* out);
 // Lanes per row of a loop projection over `rows` rows of A, or of A^T (kernels.cu).
 int sell_lanes(int rows, bool transposed);
+bool sell_fetch_ahead(const DevSell& a, const DevSell& t, int64_t bytes);
 // All rows in ascending order, four lanes each.
 bool build_sell(int32_t rows, const std::vector<int32_t>& row_ptr, const std::vector<int32_t>& col,
                 const std::vector<float>& val, HostSell* out);

@@ -19,24 +19,26 @@
 //                the FP64 table k_theta_table fills once per run (step a6;
 //                Eq. GNtheta)
 //
-// Projector layouts.  The solver loop streams its matrices in the sliced
-// layout (SellGroup): a warp owns a slice of 32 / L rows, L lanes per row take
-// the row's 4-entry packs in turn (packed 2-byte columns and value quads, PF
-// steps in flight in registers, the next step's gathers issued while the
-// current one accumulates), and a butterfly leaves each row's sum in all of its
-// lanes.  What a warp's gathers touch decides the speed (the L1 pipe is busy for
-// 57-64 % of a launch's cycles): slices hold neighbouring pixels, or rays of a
-// few bins and angles with their entries in order along the ray, and a row gets
-// as few lanes as still fill the chip (sell_lanes).  Rows in ascending order
-// with four lanes each took 38.1 us per folded map at 256^2, 33 now; 112 at
-// 400^2, 92 now.  When A has the quarter-turn symmetry the
-// loop streams only its folded halves (FOLD): each stored entry serves two
-// products, gathered as pairs (see fold_partner in appga_internal.h).  The
-// stand-alone projections and objective stream the row-padded CSR
-// (RowGroup): a warp owns R consecutive rows, whose entries form one
-// contiguous range streamed in 128-entry chunks; lanes park per-row partials
-// in shared-memory slots and lane q sums row q.  No block-wide barrier sits
-// on either streaming path.
+// Projector layouts.  The solver loop and the single hot-path calls stream their
+// matrices in the sliced layout (SellGroup): a warp owns a slice of 32 / L rows,
+// L lanes per row take the row's 4-entry packs in turn (packed 2-byte columns
+// and value quads, PF steps in flight in registers, the next step's gathers
+// issued while the current one accumulates), and a butterfly leaves each row's
+// sum in all of its lanes.  What a warp's gathers touch decides the speed (the
+// L1 pipe is busy for 57-64 % of a launch's cycles): slices hold neighbouring
+// pixels, or rays of a few bins and angles with their entries in order along the
+// ray, and a row gets as few lanes as still fill the chip (sell_lanes).  Rows in
+// ascending order with four lanes each took 38.1 us per folded map at 256^2, 31
+// now (32 before slices were fetched ahead, sell_fetch_ahead); 112 at 400^2, 92
+// now.  When A has the quarter-turn symmetry the loop streams only its folded
+// halves (FOLD): each stored entry serves two products, gathered as pairs (see
+// fold_partner in appga_internal.h).  The single calls sum in double-float
+// (forward) or with compensation (back): 42 and 25 us at 256^2 unfolded, 45 and
+// 34 through the CSR.  Matrices whose columns do not fit the packed words stream
+// the row-padded CSR (RowGroup): a warp owns R consecutive rows, whose entries
+// form one contiguous range streamed in 128-entry chunks; lanes park per-row
+// partials in shared-memory slots and lane q sums row q.  No block-wide barrier
+// sits on either streaming path.
 //
 // The per-row epilogue runs on the FP32 pipe only: double-float (FP32 pair)
 // arithmetic for y, y~, the guarded denominator, and a double-float natural
@@ -379,6 +381,12 @@ __device__ __forceinline__ float2 shfl_xor_v(float2 a, int o) {
   return make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
 }
 
+// The next bytes of a matrix stream into L2, in one instruction (16-byte
+// aligned, a multiple of 16 bytes).
+__device__ __forceinline__ void bulk_prefetch_l2(const void* p, int bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes));
+}
+
 template <bool BF16, int PF, int L>
 struct SellGroup {
   int q0, steps;
@@ -395,10 +403,23 @@ struct SellGroup {
     }
   }
 
+  // the slice's steps past PF into L2 (q0 of lane 0 is the slice's start)
+  __device__ __forceinline__ void ahead(const DevSell& S) const {
+    if (steps <= PF) return;
+    const size_t p = (size_t)q0 + (PF << 5);
+    const int n = (steps - PF) << 5;
+    bulk_prefetch_l2(S.cols + p, n * 8);
+    if constexpr (BF16)
+      bulk_prefetch_l2(S.vals_bf16 + p, n * 8);
+    else
+      bulk_prefetch_l2(S.vals + p, n * 16);
+  }
+
   // before the kernel waits for its predecessor: the slice's first PF steps
   __device__ __forceinline__ void prologue(const DevSell& S, int slice, int lane, uint64_t pol) {
     q0 = S.off[slice] + lane;
     steps = (S.off[slice + 1] - S.off[slice]) >> 5;
+    if (lane == 0 && ((S.ahead >> (BF16 ? 1 : 0)) & 1)) ahead(S);
 #pragma unroll
     for (int u = 0; u < PF; ++u) {
       c[u] = make_uint2(0u, 0u);
@@ -494,12 +515,14 @@ struct SellGroup {
   // (hi, lo), in every lane of the row; the packed columns are 8 x 8-tiled.
   __device__ __forceinline__ float2 stream_df(const DevSell& S, const float* __restrict__ x, int n,
                                               uint64_t pol) {
+    // pixel of tiled index t: tile / nb by a multiplication, exact for the tiles
+    // below 2^14 and nb <= 2^7 that a packed column can name (20 bits)
     const int nb = (n + 7) / 8;
-    const float inv = 1.f / (float)nb;
-    // tile / nb exactly: tiles below 2^14 (a packed column is below 2^20)
+    const unsigned inv = nb > 1 ? 0xffffffffu / (unsigned)nb + 1u : 0u;
+    const int per_row = 8 * (n - nb);
     auto at = [&](int t) {
-      const int tile = t >> 6, tr = (int)(((float)tile + 0.5f) * inv);
-      return __ldg(x + (8 * tr + ((t >> 3) & 7)) * n + 8 * (tile - tr * nb) + (t & 7));
+      const int tr = (int)__umulhi((unsigned)t >> 6, inv);
+      return __ldg(x + (tr * per_row + ((t >> 3) & ~7) + ((t >> 3) & 7) * n + (t & 7)));
     };
     auto gather = [&](uint2 w) {
       const int4 k = unpack_cols(w);
@@ -1416,6 +1439,24 @@ int sell_lanes(int rows, bool transposed) {
   int lanes = 1;
   while (lanes < 8 && (int64_t)rows * lanes / 32 < warps) lanes *= 2;
   return lanes;
+}
+
+// Whether a loop's two sliced matrices (a: forward, t: pixel phase) are fetched
+// ahead: each slice whole into L2 before its kernel waits for its predecessor,
+// so that its loads hit L2.  That pays where both streams fit L2 and the pixel
+// phase's slices are (nearly) all resident at once, 34 warps an SM; with more
+// of them the fetches of late slices push out what the early ones stream.  us
+// for 40 maps, without / with: 256^2 folded (89 MB, 4096 slices) 1362 / 1296;
+// 201^2 (86 MB, 5051) 1139 / 1063; 255^2 BF16 (118 MB, 4065) 1572 / 1501; 280^2
+// folded (117 MB, 4900) 1825 / 1828; beyond the line 300^2 folded BF16 (96 MB,
+// 5625) 1841 / 1909; 320^2 folded (175 MB) 2262 / 2352; 400^2 folded (342 MB,
+// 100 maps) 3735 / 4281.
+bool sell_fetch_ahead(const DevSell& a, const DevSell& t, int64_t bytes) {
+  int dev = 0, l2 = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess)
+    return false;
+  return a.off != nullptr && bytes <= (int64_t)l2 && t.slices <= 34 * current_sm_count();
 }
 
 int max_partials(int m, int n) {

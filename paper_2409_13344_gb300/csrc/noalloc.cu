@@ -1,7 +1,6 @@
 // appga_objective_noalloc: the FP64 objective Phi(f) computed with all of
-// its scratch memory (block partials of the grid reductions, their tickets,
-// a scratch iteration state and two partial sums) in one fixed, file-scope
-// device array instead of device memory the library allocates.
+// its scratch memory (block partials of the grid reductions, their tickets and
+// a scratch iteration state) in one fixed, file-scope device array instead of device memory the library allocates.
 //
 // Some callers cannot let a library allocate device memory after start-up:
 // processes that hand the whole device memory to their own pool at launch
