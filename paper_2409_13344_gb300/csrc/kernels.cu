@@ -1449,8 +1449,8 @@ int sell_lanes(int rows, bool transposed) {
 // for 40 maps, without / with: 256^2 folded (89 MB, 4096 slices) 1362 / 1296;
 // 201^2 (86 MB, 5051) 1139 / 1063; 255^2 BF16 (118 MB, 4065) 1572 / 1501; 280^2
 // folded (117 MB, 4900) 1825 / 1828; beyond the line 300^2 folded BF16 (96 MB,
-// 5625) 1841 / 1909; 320^2 folded (175 MB) 2262 / 2352; 400^2 folded (342 MB,
-// 100 maps) 3735 / 4281.
+// 5625) 1841 / 1909; 320^2 folded (175 MB) 2262 / 2352; 400^2 folded (342 MB)
+// 3735 / 4281.
 bool sell_fetch_ahead(const DevSell& a, const DevSell& t, int64_t bytes) {
   int dev = 0, l2 = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
