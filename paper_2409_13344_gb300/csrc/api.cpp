@@ -1001,14 +1001,8 @@ appga_status appga_matrix_create(appga_ctx* ctx, int32_t m, int32_t d, int32_t n
         }
       }
     }
-    auto fetch_ahead = [](DevSell& a, DevSell& t) {
-      const int64_t packs = (int64_t)a.packs + t.packs;
-      for (int bf = 0; bf < 2; ++bf)
-        if (appga::sell_fetch_ahead(a, t, packs * (bf ? 16 : 24))) a.ahead |= 1 << bf;
-      t.ahead = a.ahead;
-    };
-    fetch_ahead(M->sell_a, M->sell_t);
-    fetch_ahead(M->fold_a, M->fold_t);
+    appga::sell_fetch_ahead(M->sell_a, M->sell_t);
+    appga::sell_fetch_ahead(M->fold_a, M->fold_t);
     if (e != cudaSuccess) rc = cuda_fail(e, "tiled column indices and sliced layout");
   }
   if (rc == APPGA_OK) {

@@ -1441,22 +1441,35 @@ int sell_lanes(int rows, bool transposed) {
   return lanes;
 }
 
-// Whether a loop's two sliced matrices (a: forward, t: pixel phase) are fetched
-// ahead: each slice whole into L2 before its kernel waits for its predecessor,
-// so that its loads hit L2.  That pays where both streams fit L2 and the pixel
-// phase's slices are (nearly) all resident at once, 34 warps an SM; with more
-// of them the fetches of late slices push out what the early ones stream.  us
-// for 40 maps, without / with: 256^2 folded (89 MB, 4096 slices) 1362 / 1296;
-// 201^2 (86 MB, 5051) 1139 / 1063; 255^2 BF16 (118 MB, 4065) 1572 / 1501; 280^2
-// folded (117 MB, 4900) 1825 / 1828; beyond the line 300^2 folded BF16 (96 MB,
-// 5625) 1841 / 1909; 320^2 folded (175 MB) 2262 / 2352; 400^2 folded (342 MB)
-// 3735 / 4281.
-bool sell_fetch_ahead(const DevSell& a, const DevSell& t, int64_t bytes) {
+// Which of a loop's two sliced matrices (a: forward, t: pixel phase) are fetched
+// ahead, each slice whole into L2 before its kernel waits for its predecessor,
+// so that its loads hit L2.  That pays while the pixel phase's slices are
+// (nearly) all resident at once, 34 warps an SM: for both where the streams fit
+// L2, for the forward phase alone up to half as much again; with more bytes or
+// slices the fetches of late slices push out what the early ones stream.  us
+// for 40 maps without / forward only / both:
+//   256^2 folded      (89 MB, 4096 slices)    1362 / 1414 / 1296
+//   201^2             (86 MB, 5051)           1139 / 1140 / 1063
+//   255^2 BF16        (118 MB, 4065)          1572 / 1539 / 1501
+//   280^2 folded      (117 MB, 4900)          1825 / 1867 / 1828
+//   350^2 folded BF16 (152 MB, 3829)          2754 / 2735 / 2656
+//   255^2             (177 MB, 4065)          1769 / 1676 / 1772
+// and beyond the lines
+//   300^2 folded BF16 (96 MB, 5625)           1841 / 1853 / 1909
+//   320^2 folded      (175 MB, 6400)          2262 / 2276 / 2352
+//   400^2 folded      (342 MB, 5000)          3496 / 3664 / 4281 (both: with a tolerance)
+// The whole 256^2 matrices (185 MB) run at 43.6 us a map without, 40.6 so.
+void sell_fetch_ahead(DevSell& a, DevSell& t) {
   int dev = 0, l2 = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess)
-    return false;
-  return a.off != nullptr && bytes <= (int64_t)l2 && t.slices <= 34 * current_sm_count();
+    return;
+  if (a.off == nullptr || t.slices > 34 * current_sm_count()) return;
+  for (int bf = 0; bf < 2; ++bf) {
+    const int64_t bytes = ((int64_t)a.packs + t.packs) * (bf ? 16 : 24);
+    if (2 * bytes <= 3 * (int64_t)l2) a.ahead |= 1 << bf;
+    if (bytes <= (int64_t)l2) t.ahead |= 1 << bf;
+  }
 }
 
 int max_partials(int m, int n) {
