@@ -120,14 +120,13 @@ __device__ __forceinline__ float4 ld_quad(const DevQuad& M, size_t o, uint64_t p
 }
 
 // The objective's double-float projections take one row at a time from the
-// CSR: how the lanes of a warp share a row whose products fill W slots.  A lane
-// holds Q slots (Q/4 16-byte loads per gathered row), L lanes make a group
-// that covers the W slots, and the G groups of a row's team take the row's
-// 4-entry packs in turn.  The row's sum is always that of four partial sums,
-// p_i over the packs k = i (mod 4) in order, as (p0 + p1) + (p2 + p3), so the
-// results do not depend on W: the widest team holds several of the four in
-// one lane (A), the narrow ones work on RW rows of the warp at a time.
-// Eight slots per lane because the load of a pack's columns or values, which
+// CSR: how the lanes of a warp share a row whose products fill W <= 64 slots (a
+// grid of two in y covers 128).  A lane holds Q slots (Q/4 16-byte loads per
+// gathered row), L lanes make a group that covers the W slots, and the four
+// groups of a row's team take the row's 4-entry packs in turn, RW rows of the
+// warp at a time.  The row's sum is that of four partial sums, p_i over the
+// packs k = i (mod 4) in order, as (p0 + p1) + (p2 + p3), so the results do not
+// depend on W.  Eight slots per lane because the load of a pack's columns or values, which
 // a group's lanes make at one address, still takes the L1 pipe four passes
 // (a 16-byte load is served in quarter warps): with four groups a warp those
 // passes feed 16 entries.
@@ -135,11 +134,12 @@ template <int W>
 struct Team {
   static constexpr int Q = W >= 16 ? 8 : 4;
   static constexpr int L = W / Q;
-  static constexpr int G = L <= 8 ? 4 : 32 / L;
+  static constexpr int G = 4;
   static constexpr int LANES = L * G;
   static constexpr int RW = 32 / LANES;
   static constexpr int E = Q / G;  // slots a lane owns after the reduction
   static constexpr int GSTRIDE = 4 * L;
+  static_assert(LANES <= 32, "a team is part of a warp");
 };
 // A lane gathers the slots gathered_slot + i * GSTRIDE .. + 3, i < Q/4 (so
 // that a quarter warp's 16-byte loads are consecutive: one pass each), and
@@ -455,13 +455,14 @@ __device__ __forceinline__ void store_row_sums(const BFwdArgs& a, const float (&
     sum_lo[team][sl0 + t] = dl[t];
   }
   __syncthreads();
+  const int s0 = blockIdx.y * W;
   for (int q = tid; q < T::RW * W; q += P_THREADS) {
     const int s = q % W, vb = blockIdx.x * T::RW + q / W;
-    if (vb >= a.n_spmv_blocks || !live(a.slots[s])) continue;
+    if (vb >= a.n_spmv_blocks || !live(a.slots[s0 + s])) continue;
     float h = 0.f, l = 0.f;
     for (int w = 0; w < P_WARPS; ++w)
       acc_add(h, l, sum_hi[q / W * P_WARPS + w][s], sum_lo[q / W * P_WARPS + w][s]);
-    a.fpartial[(size_t)vb * a.Kp + s] = make_float2(h, l);
+    a.fpartial[(size_t)vb * a.Kp + s0 + s] = make_float2(h, l);
   }
 }
 
@@ -753,15 +754,16 @@ __global__ void __launch_bounds__(B_THREADS, 4) k_bstencil(BFwdArgs a) {
 // Data terms sum y - g ln(y + gamma) of the results of every active slot, with
 // y = A f accumulated in double-float as the single-slice objective does (one
 // pass over A for all slots: 64 slots of 256 x 256 took 64 projections of 46
-// us one by one).  The rows of sums lie as the forward phase's.
+// us one by one).  The rows of sums lie as the forward phase's; blockIdx.y takes
+// the slots from y W on.
 template <int W, bool BF16>
 __global__ void __launch_bounds__(P_THREADS, 2) k_bobjective(BFwdArgs a) {
   using T = Team<W>;
   constexpr int E = T::E, Q = T::Q, F = Q / 4;
   __shared__ float dsum_hi[P_WARPS * T::RW][W], dsum_lo[P_WARPS * T::RW][W];
   const int lane = threadIdx.x & 31, g = lane % T::LANES / T::L;
-  const int sl0 = owned_slot<W>(lane), Kp = a.Kp;
-  const float* xl = a.f[a.bst->gstep % 3] + gathered_slot<W>(lane);
+  const int s0 = blockIdx.y * W, sl0 = s0 + owned_slot<W>(lane), Kp = a.Kp;
+  const float* xl = a.f[a.bst->gstep % 3] + s0 + gathered_slot<W>(lane);
   const uint64_t pol = evict_first_policy();
   const RowDeal<W> deal(a.A.rows, a.n_spmv_blocks);
   float dh[E], dl[E];
@@ -804,16 +806,14 @@ __global__ void __launch_bounds__(P_THREADS, 2) k_bobjective(BFwdArgs a) {
       acc_add(qh[t], ql[t], __shfl_xor_sync(0xffffffffu, up1 ? hi[t] : hi[H1 + t], T::L),
               __shfl_xor_sync(0xffffffffu, up1 ? lo[t] : lo[H1 + t], T::L));
     }
-    if constexpr (T::G == 4) {
-      const bool up2 = g >> 1;
+    const bool up2 = g >> 1;
 #pragma unroll
-      for (int t = 0; t < E; ++t) {
-        const float sh = __shfl_xor_sync(0xffffffffu, up2 ? qh[t] : qh[E + t], 2 * T::L);
-        const float sl = __shfl_xor_sync(0xffffffffu, up2 ? ql[t] : ql[E + t], 2 * T::L);
-        qh[t] = up2 ? qh[E + t] : qh[t];
-        ql[t] = up2 ? ql[E + t] : ql[t];
-        acc_add(qh[t], ql[t], sh, sl);
-      }
+    for (int t = 0; t < E; ++t) {
+      const float sh = __shfl_xor_sync(0xffffffffu, up2 ? qh[t] : qh[E + t], 2 * T::L);
+      const float sl = __shfl_xor_sync(0xffffffffu, up2 ? ql[t] : ql[E + t], 2 * T::L);
+      qh[t] = up2 ? qh[E + t] : qh[t];
+      ql[t] = up2 ? ql[E + t] : ql[t];
+      acc_add(qh[t], ql[t], sh, sl);
     }
     if (row < 0) continue;
     float gg[E], gm[E];
@@ -1369,7 +1369,7 @@ cudaError_t launch_bstencil(const BFwdArgs& a0, cudaStream_t s) {
 namespace {
 template <int W>
 cudaError_t bobjective_w(const BFwdArgs& a, cudaStream_t s) {
-  const int grid = (a.n_spmv_blocks + Team<W>::RW - 1) / Team<W>::RW;
+  const dim3 grid((a.n_spmv_blocks + Team<W>::RW - 1) / Team<W>::RW, a.width / W);
   if (a.use_bf16)
     k_bobjective<W, true><<<grid, P_THREADS, 0, s>>>(a);
   else
@@ -1390,8 +1390,8 @@ cudaError_t launch_bobjective(const BFwdArgs& a0, int K, double* out, cudaStream
     case 8: e = bobjective_w<8>(a, s); break;
     case 16: e = bobjective_w<16>(a, s); break;
     case 32: e = bobjective_w<32>(a, s); break;
-    case 64: e = bobjective_w<64>(a, s); break;
-    case 128: e = bobjective_w<128>(a, s); break;
+    case 64:
+    case 128: e = bobjective_w<64>(a, s); break;
     default: e = cudaErrorInvalidValue;
   }
   const int nst = st_blocks(a);
