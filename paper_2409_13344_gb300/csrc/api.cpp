@@ -928,9 +928,8 @@ appga_status appga_matrix_create(appga_ctx* ctx, int32_t m, int32_t d, int32_t n
     rc = upload_order(appga::zorder(n_angles, m / n_angles), &M->A, &M->bytes);
   if (rc == APPGA_OK) {
     // A's column indices in the 8 x 8-tiled pixel order (row_ptr and values shared)
-    std::vector<int32_t> ct(pa.col.size());
-    for (size_t q = 0; q < ct.size(); ++q)
-      ct[q] = appga::tiled_index(pa.col[q] / n_side, pa.col[q] % n_side, n_side);
+    std::vector<int32_t> ct = pa.col;
+    appga::tile_columns(n_side, &ct);
     M->A_tiled = M->A;
     M->A_tiled.col = nullptr;
     cudaError_t e = dalloc(&M->A_tiled.col, ct.size(), &M->bytes);
@@ -939,11 +938,8 @@ appga_status appga_matrix_create(appga_ctx* ctx, int32_t m, int32_t d, int32_t n
     // the solver loop's two projections in the sliced layout (both or neither):
     // pixels by tiles and rays by tiles of (angle, bin), entries along the ray
     if (APPGA_PACK && e == cudaSuccess && !ct.empty() && !pt.col.empty()) {
-      appga::HostCSR along, pl;
-      appga::sort_along_rays(m, n_side, row_ptr_host, col_host, val_host, &along);
-      appga::pad_rows(m, d, row_ptr_host, along.col.data(), along.val.data(), appga::ROW_PAD, &pl);
-      along = appga::HostCSR();
-      for (auto& c : pl.col) c = appga::tiled_index(c / n_side, c % n_side, n_side);
+      appga::HostCSR pl;
+      appga::ray_packs(m, n_side, row_ptr_host, col_host, val_host, &pl);
       auto rays = [&](int32_t rows, int lanes) {
         std::vector<int32_t> order;
         if (m % n_angles == 0) {

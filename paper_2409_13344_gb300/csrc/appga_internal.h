@@ -317,6 +317,9 @@ bool quarter_turn_symmetric(int32_t m, int32_t n, int32_t n_angles, const int32_
 // from the stable transpose `at` of the whole A.
 void fold_transpose(const HostCSR& at, int32_t half, int32_t n, HostCSR* out);
 
+// Pixel indices of an n x n image to their 8 x 8-tiled positions, in place.
+void tile_columns(int32_t n, std::vector<int32_t>* col);
+
 // The points (y, x) of an ny x nx grid, as y * nx + x, along the Z-order curve:
 // every aligned run of 16 (64, ...) of the full square is a 4 x 4 (8 x 8, ...)
 // tile, so consecutive rows of a projector are neighbouring pixels, or rays
@@ -355,12 +358,13 @@ void sell_fetch_ahead(DevSell& a, DevSell& t);
 // All rows in ascending order, four lanes each.
 bool build_sell(int32_t rows, const std::vector<int32_t>& row_ptr, const std::vector<int32_t>& col,
                 const std::vector<float>& val, HostSell* out);
-// The entries of every row in the order in which the ray crosses the n x n
+// A with its rows padded to whole packs and its columns in the 8 x 8-tiled order,
+// the entries of every row in the order in which the ray crosses the n x n
 // image's longer extent (by column if the row's pixels span more columns than
 // rows, else by row), so that neighbouring rays' k-th entries are neighbouring
 // pixels.
-void sort_along_rays(int32_t rows, int32_t n, const int32_t* row_ptr, const int32_t* col,
-                     const float* val, HostCSR* out);
+void ray_packs(int32_t rows, int32_t n, const int32_t* row_ptr, const int32_t* col,
+               const float* val, HostCSR* out);
 
 void set_error(const std::string& msg);
 
