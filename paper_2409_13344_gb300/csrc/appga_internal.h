@@ -362,7 +362,8 @@ bool build_sell(int32_t rows, const std::vector<int32_t>& row_ptr, const std::ve
 // the entries of every row in the order in which the ray crosses the n x n
 // image's longer extent (by column if the row's pixels span more columns than
 // rows, else by row), so that neighbouring rays' k-th entries are neighbouring
-// pixels.
+// pixels.  A row whose packs do not fit the packed word in that order (a strip of
+// 32 pixels or more at 256 x 256) keeps the given one.
 void ray_packs(int32_t rows, int32_t n, const int32_t* row_ptr, const int32_t* col,
                const float* val, HostCSR* out);
 

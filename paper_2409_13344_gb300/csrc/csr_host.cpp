@@ -268,11 +268,23 @@ void ray_packs(int32_t rows, int32_t n, const int32_t* row_ptr, const int32_t* c
       }
       int32_t* pc = &out->col[(size_t)out->row_ptr[i]];
       float* pv = &out->val[(size_t)out->row_ptr[i]];
-      for (int32_t k = 0; k < len; ++k) {
-        pc[k] = tiled_index(at[order[k]].first, at[order[k]].second, n);
-        pv[k] = val[s + order[k]];
+      const int32_t padded = out->row_ptr[i + 1] - out->row_ptr[i];
+      auto place = [&] {
+        for (int32_t k = 0; k < len; ++k) {
+          pc[k] = tiled_index(at[order[k]].first, at[order[k]].second, n);
+          pv[k] = val[s + order[k]];
+        }
+        for (int32_t k = len; k < padded; ++k) pc[k] = pc[len - 1];
+      };
+      place();
+      // a row that covers a wide strip steps too far from one column to the next
+      bool fits = true;
+      uint64_t word;
+      for (int32_t k = 0; fits && k < padded; k += PACK_ENTRIES) fits = encode_pack(pc + k, &word);
+      if (!fits) {
+        for (int32_t k = 0; k < len; ++k) order[k] = k;
+        place();
       }
-      for (int32_t k = len; k < out->row_ptr[i + 1] - out->row_ptr[i]; ++k) pc[k] = pc[len - 1];
     }
   });
 }
