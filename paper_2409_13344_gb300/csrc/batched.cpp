@@ -47,15 +47,17 @@ void free_batch_workspace(BatchWorkspace* bw) {
   *bw = BatchWorkspace();
 }
 
+// Rows of BatchWorkspace::partial: the objective's 64 group sums, the set-up's 16
+// sums a slice, or the gather probe's sink (16 floats an SM).
+constexpr int kPartialRows = 128;
+
 int64_t batch_workspace_bytes(int m, int d, int Kp) {
-  const int64_t ngroups = batch_max_blocks() / 64 + 2;
   int64_t b = 0;
   b += (int64_t)7 * d * Kp * sizeof(float);  // f ring, gR, pfreeze, delta, low
   b += (int64_t)5 * m * Kp * sizeof(float);  // y ring, w, g, gamma
   b += (int64_t)Kp * sizeof(SlotState) + sizeof(BatchState);
-  b += (2 * batch_max_blocks() + ngroups + 2) * Kp * (int64_t)sizeof(float2);
-  b += ngroups * (int64_t)sizeof(unsigned int) + (int64_t)sizeof(int);
-  b += (int64_t)(Kp + 2) * sizeof(double);
+  b += (int64_t)(batch_max_blocks() + kPartialRows) * Kp * sizeof(float2);
+  b += (int64_t)sizeof(int) + (int64_t)(2 * Kp + 2) * sizeof(double);
   return b;
 }
 
@@ -63,7 +65,6 @@ cudaError_t alloc_batch_workspace(BatchWorkspace& b, int m, int d, int Kp) {
   b = BatchWorkspace();
   const size_t dd = (size_t)d * Kp, mm = (size_t)m * Kp;
   const int maxb = batch_max_blocks();
-  const int ngroups = maxb / 64 + 2;
   cudaError_t e = cudaSuccess;
   for (int i = 0; i < 3 && e == cudaSuccess; ++i) e = dalloc(&b.f[i], dd);
   for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = dalloc(&b.y[i], mm);
@@ -76,7 +77,7 @@ cudaError_t alloc_batch_workspace(BatchWorkspace& b, int m, int d, int Kp) {
   if (e == cudaSuccess) e = dalloc(&b.gamma, mm);
   if (e == cudaSuccess) e = dalloc(&b.slots, (size_t)Kp);
   if (e == cudaSuccess) e = dalloc(&b.bst, 1);
-  if (e == cudaSuccess) e = dalloc(&b.partial, (size_t)(maxb + ngroups + 2) * Kp);
+  if (e == cudaSuccess) e = dalloc(&b.partial, (size_t)kPartialRows * Kp);
   if (e == cudaSuccess) e = dalloc(&b.fpartial, (size_t)maxb * Kp);
   if (e == cudaSuccess) e = dalloc(&b.flag, 1);
   if (e == cudaSuccess) e = dalloc(&b.vscal, (size_t)2 * Kp + 2);

@@ -96,7 +96,7 @@ struct BatchWorkspace {
   SlotState* slots_host = nullptr;            // pinned [Kp]
   BatchState* bst = nullptr;
   BatchState* bst_host = nullptr;             // pinned
-  float2* partial = nullptr;                  // (blocks + groups) x Kp
+  float2* partial = nullptr;                  // kPartialRows x Kp
   float2* fpartial = nullptr;                 // forward-phase objective partials, blocks x Kp
   int* flag = nullptr;
   int* flag_host = nullptr;

@@ -66,10 +66,9 @@ struct Pool {
   int used = 0;
   int gstep = 0;  // global step of the pool, as last read back
   int64_t bytes = 0;
-  float* d_in = nullptr;  // [Kp][2m + d]: g, gamma, f_init of admitted slices
-  float* h_in = nullptr;  // pinned mirror
-  float* d_out = nullptr; // [Kp][d]: retired images
-  float* h_out = nullptr; // pinned mirror
+  float* d_in = nullptr;  // [Kp][2m]: g, gamma of admitted slices
+  float* h_in = nullptr;  // pinned [Kp][2m + d]: g, gamma, f_init
+  float* h_out = nullptr; // pinned [Kp][d]: retired images
   int* d_ids = nullptr;   // [3 Kp]: admitted slots | slots with f_init | retired slots
   int* h_ids = nullptr;   // pinned mirror
 
@@ -82,6 +81,11 @@ struct Pool {
     return slot_width(top);
   }
   bool idle() const { return !inflight; }
+  // Room for Kp images between replays, for those retired and then for the
+  // f_init of those admitted: the ring entry that the next step writes, which
+  // holds nothing until then.  The pool's stream orders the copies out of it
+  // before the next replay.
+  float* d_images() const { return b.f[(gstep + 1) % 3]; }
 };
 
 struct Geometry {
@@ -91,7 +95,7 @@ struct Geometry {
 
 int64_t pool_bytes(const appga_matrix* M, int Kp) {
   return batch_workspace_bytes(M->m, M->d, Kp) +
-         (int64_t)Kp * (2LL * M->m + 2LL * M->d) * (int64_t)sizeof(float) +
+         (int64_t)Kp * 2LL * M->m * (int64_t)sizeof(float) +
          3LL * Kp * (int64_t)sizeof(int);
 }
 
@@ -107,13 +111,12 @@ void free_pool(Pool* P) {
   P->ev_snap = P->ev_out = P->ev_start = nullptr;
   free_batch_workspace(&P->b);
   cudaFree(P->d_in);
-  cudaFree(P->d_out);
   cudaFree(P->d_ids);
   cudaFreeHost(P->h_in);
   cudaFreeHost(P->h_out);
   cudaFreeHost(P->h_ids);
   P->gexec.clear();
-  P->d_in = P->d_out = nullptr;
+  P->d_in = nullptr;
   P->h_in = P->h_out = nullptr;
   P->d_ids = P->h_ids = nullptr;
 }
@@ -180,8 +183,7 @@ appga_status create_pool(appga_server* S, int geom, int Kp, Pool** out) {
   if (e == cudaSuccess) e = cudaEventCreate(&P->ev_snap);
   if (e == cudaSuccess) e = cudaEventCreate(&P->ev_start);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&P->ev_out, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = dalloc(&P->d_in, in_len);
-  if (e == cudaSuccess) e = dalloc(&P->d_out, out_len);
+  if (e == cudaSuccess) e = dalloc(&P->d_in, (size_t)Kp * 2 * (size_t)M->m);
   if (e == cudaSuccess) e = dalloc(&P->d_ids, (size_t)3 * Kp);
   if (e == cudaSuccess) e = cudaMallocHost((void**)&P->h_in, in_len * sizeof(float));
   if (e == cudaSuccess) e = cudaMallocHost((void**)&P->h_out, out_len * sizeof(float));
@@ -328,15 +330,18 @@ appga_status admit(appga_server* S, Pool* P, int count) {
   }
   const int Gs = P->gstep;
   float* cur = P->b.f[Gs % 3];
-  CK(cudaMemcpyAsync(P->d_in, P->h_in, ((size_t)2 * K * m + (size_t)kf * d) * sizeof(float),
-                     cudaMemcpyHostToDevice, s));
+  CK(cudaMemcpyAsync(P->d_in, P->h_in, (size_t)2 * K * m * sizeof(float), cudaMemcpyHostToDevice,
+                     s));
+  if (kf > 0)
+    CK(cudaMemcpyAsync(P->d_images(), P->h_in + (size_t)2 * K * m, (size_t)kf * d * sizeof(float),
+                       cudaMemcpyHostToDevice, s));
   CK(cudaMemcpyAsync(P->d_ids, P->h_ids, (size_t)2 * Kp * sizeof(int), cudaMemcpyHostToDevice, s));
   CK(launch_to_slot_minor(P->d_in, K, m, P->b.g, Kp, 0, P->d_ids, s));
   CK(launch_to_slot_minor(P->d_in + (size_t)K * m, K, m, P->b.gamma, Kp, 0, P->d_ids, s));
   // f^{k0} = f^{k0-1}: the initial image TMC * 1_disk (Sec. 4.1), or the request's own
   CK(launch_binit_image(P->d_in, P->d_in + (size_t)K * m, m, M->n, M->na, M->npfov, K, Kp, 0,
                         P->d_ids, P->b.partial, cur, nullptr, P->b.delta, P->b.low, s));
-  CK(launch_to_slot_minor(P->d_in + (size_t)2 * K * m, kf, d, cur, Kp, 0, P->d_ids + Kp, s));
+  CK(launch_to_slot_minor(P->d_images(), kf, d, cur, Kp, 0, P->d_ids + Kp, s));
   for (int k = 0; k < K; ++k) {
     Request& R = S->reqs[ids[k]];
     SlotState st = slot_from_params(&R.p, 1, true);
@@ -429,9 +434,9 @@ appga_status retire_begin(appga_server* S, Pool* P) {
   CK(cudaMemcpyAsync(P->d_ids + 2 * Kp, P->h_ids + 2 * Kp, K * sizeof(int),
                      cudaMemcpyHostToDevice, s));
   // a finished slot carries its result forward, so it sits in the current ring entry
-  CK(launch_from_slot_minor(P->fa, K, 0, P->d_ids + 2 * Kp, P->d_out, s));
-  CK(cudaMemcpyAsync(P->h_out, P->d_out, (size_t)K * d * sizeof(float), cudaMemcpyDeviceToHost,
-                     s));
+  CK(launch_from_slot_minor(P->fa, K, 0, P->d_ids + 2 * Kp, P->d_images(), s));
+  CK(cudaMemcpyAsync(P->h_out, P->d_images(), (size_t)K * d * sizeof(float),
+                     cudaMemcpyDeviceToHost, s));
   appga_params def;
   appga_params_default(&def);
   P->ret_ids.resize(K);
