@@ -25,8 +25,10 @@
  *    geometry at the next step boundary, while the pool's other slots keep
  *    iterating (continuous batching).  A new pool is created only when its
  *    device memory fits both the free device memory minus hbm_reserve_bytes
- *    and hbm_budget_bytes minus what the server's pools already hold; when it
- *    does not, empty pools of other geometries are released first, and
+ *    and hbm_budget_bytes minus what the server's pools already hold (with the
+ *    first pool of a matrix, the free memory also has to hold the layout that
+ *    the batched kernels stream, which stays with the matrix and does not count
+ *    against the budget); when it does not, empty pools of other geometries are released first, and
  *    otherwise the request waits until memory frees up.
  *  - Retirement.  A slot whose problem reached max_iters maps or its
  *    relative-objective stopping test is copied out at the step boundary

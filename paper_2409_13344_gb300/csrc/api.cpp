@@ -45,7 +45,10 @@ appga_status fail(appga_status s, const std::string& msg) {
 
 appga_status cuda_fail(cudaError_t e, const char* what) {
   g_last_error = std::string(what) + ": " + cudaGetErrorString(e);
-  if (e == cudaErrorMemoryAllocation) return APPGA_ENOMEM;
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();  // or the check after the next launch would report it
+    return APPGA_ENOMEM;
+  }
   if (e == cudaErrorNoDevice || e == cudaErrorInvalidDevice || e == cudaErrorInsufficientDriver)
     return APPGA_ENODEV;
   return APPGA_ECUDA;

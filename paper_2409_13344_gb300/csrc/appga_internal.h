@@ -91,9 +91,10 @@ struct DevCSR {
 // of four, with the four rows' values per column (zero where a row has none).
 struct DevQuad {
   int32_t blocks = 0;
-  int32_t* off = nullptr;   // blocks + 1 offsets in packs
+  int32_t packs = 0;
+  int32_t* off = nullptr;   // blocks + 1 offsets in packs (NULL: not counted yet)
   int32_t* rows = nullptr;  // 4 per block, -1 past the last row
-  int4* cols = nullptr;     // the four columns of a pack
+  int4* cols = nullptr;     // the four columns of a pack (NULL: not built yet)
   float4* vals = nullptr;   // 4 per pack: the four rows' values at one column
   uint2* vals_bf16 = nullptr;
 };

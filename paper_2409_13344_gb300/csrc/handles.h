@@ -121,6 +121,9 @@ int64_t batch_workspace_bytes(int m, int d, int Kp);
 cudaError_t alloc_batch_workspace(BatchWorkspace& b, int m, int d, int Kp);
 // The batched projectors' layout of M's matrices (quads.cu), built on first use.
 appga_status ensure_quads(appga_matrix* M, cudaStream_t s);
+// Device bytes that ensure_quads has still to allocate (counts the blocks' packs
+// on first use, which allocates 20 bytes a block).
+appga_status quad_bytes_missing(appga_matrix* M, cudaStream_t s, int64_t* bytes);
 void free_quad(DevQuad& q);
 // Kernel arguments of one batched step over workspace b, `stride` (at most
 // b.Kp) slots per row, of matrix M (after ensure_quads).
@@ -182,7 +185,7 @@ struct appga_matrix {
   // was not turned off): the first m/2 rows of A with tiled columns, and
   // their transpose in orbit order, both sliced (off == NULL: not folded)
   appga::DevSell fold_a, fold_t;
-  appga::DevQuad quad_a, quad_t;  // the batched projectors' layout (off == NULL: not built)
+  appga::DevQuad quad_a, quad_t;  // the batched projectors' layout
   int32_t fold_nb = 0;  // bins per angle of the folded matrix
   float* inv_lambda = nullptr;       // 1/Lambda of the FP32 values
   float* inv_lambda_bf16 = nullptr;  // 1/Lambda of the BF16-rounded values

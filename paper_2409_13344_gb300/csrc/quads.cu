@@ -123,15 +123,19 @@ __global__ void __launch_bounds__(128) k_quad_fill(DevCSR M, DevQuad Q) {
   }
 }
 
-appga_status build(const DevCSR& M, cudaStream_t s, DevQuad* out, int64_t* bytes) {
+// 32 blocks of rows per thread block
+int grid_of(const DevQuad& q) { return (q.blocks + 31) / 32; }
+
+// The blocks of M: their rows' places and the packs of each, without the packs.
+appga_status count(const DevCSR& M, cudaStream_t s, DevQuad* out, int64_t* bytes) {
   DevQuad q;
+  int64_t held = 0;
   q.blocks = (M.rows + 3) / 4;
   std::vector<int32_t> off((size_t)q.blocks + 1);
-  cudaError_t e = dalloc(&q.off, (size_t)q.blocks + 1, bytes);
-  if (e == cudaSuccess) e = dalloc(&q.rows, (size_t)4 * q.blocks, bytes);
-  const int grid = (q.blocks + 31) / 32;  // 32 blocks of rows per thread block
+  cudaError_t e = dalloc(&q.off, (size_t)q.blocks + 1, &held);
+  if (e == cudaSuccess) e = dalloc(&q.rows, (size_t)4 * q.blocks, &held);
   if (e == cudaSuccess) {
-    k_quad_count<<<grid, 128, 0, s>>>(M, q.blocks, q.off + 1);
+    k_quad_count<<<grid_of(q), 128, 0, s>>>(M, q.blocks, q.off + 1);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess)
@@ -140,16 +144,8 @@ appga_status build(const DevCSR& M, cudaStream_t s, DevQuad* out, int64_t* bytes
   if (e == cudaSuccess) {
     off[0] = 0;
     for (int b = 0; b < q.blocks; ++b) off[b + 1] += off[b];  // packs <= entries / 2: fits
-    const size_t np = (size_t)off[q.blocks];
+    q.packs = off[q.blocks];
     e = cudaMemcpyAsync(q.off, off.data(), off.size() * 4, cudaMemcpyHostToDevice, s);
-    // (the projectors' L2 prefetches run up to 64 packs past the end)
-    if (e == cudaSuccess) e = dalloc(&q.cols, np + 64, bytes);
-    if (e == cudaSuccess) e = dalloc(&q.vals, 4 * np + 256, bytes);
-    if (e == cudaSuccess && M.val_bf16) e = dalloc(&q.vals_bf16, 4 * np + 256, bytes);
-  }
-  if (e == cudaSuccess) {
-    k_quad_fill<<<grid, 128, 0, s>>>(M, q);
-    e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {
@@ -157,6 +153,32 @@ appga_status build(const DevCSR& M, cudaStream_t s, DevQuad* out, int64_t* bytes
     return cuda_fail(e, "batched matrix layout");
   }
   *out = q;
+  *bytes += held;
+  return APPGA_OK;
+}
+
+// Packs allocated (the projectors' L2 prefetches run up to 64 past the end).
+size_t packs_held(const DevQuad& q) { return (size_t)q.packs + 64; }
+
+appga_status fill(const DevCSR& M, cudaStream_t s, DevQuad* out, int64_t* bytes) {
+  DevQuad q = *out;
+  int64_t held = 0;
+  cudaError_t e = dalloc(&q.cols, packs_held(q), &held);
+  if (e == cudaSuccess) e = dalloc(&q.vals, 4 * packs_held(q), &held);
+  if (e == cudaSuccess && M.val_bf16) e = dalloc(&q.vals_bf16, 4 * packs_held(q), &held);
+  if (e == cudaSuccess) {
+    k_quad_fill<<<grid_of(q), 128, 0, s>>>(M, q);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) {
+    cudaFree(q.cols);
+    cudaFree(q.vals);
+    cudaFree(q.vals_bf16);
+    return cuda_fail(e, "batched matrix layout");
+  }
+  *out = q;
+  *bytes += held;
   return APPGA_OK;
 }
 
@@ -171,13 +193,30 @@ void free_quad(DevQuad& q) {
   q = DevQuad();
 }
 
-appga_status ensure_quads(appga_matrix* M, cudaStream_t s) {
-  if (M->quad_a.off == nullptr) {
-    const appga_status rc = build(M->A, s, &M->quad_a, &M->bytes);
-    if (rc != APPGA_OK) return rc;
-  }
-  if (M->quad_t.off == nullptr) return build(M->At, s, &M->quad_t, &M->bytes);
+namespace {
+appga_status ensure_counts(appga_matrix* M, cudaStream_t s) {
+  appga_status rc = APPGA_OK;
+  if (M->quad_a.off == nullptr) rc = count(M->A, s, &M->quad_a, &M->bytes);
+  if (rc == APPGA_OK && M->quad_t.off == nullptr) rc = count(M->At, s, &M->quad_t, &M->bytes);
+  return rc;
+}
+}  // namespace
+
+appga_status quad_bytes_missing(appga_matrix* M, cudaStream_t s, int64_t* bytes) {
+  const appga_status rc = ensure_counts(M, s);
+  if (rc != APPGA_OK) return rc;
+  *bytes = 0;
+  const int64_t pack = sizeof(int4) + 4 * (sizeof(float4) + (M->A.val_bf16 ? sizeof(uint2) : 0));
+  if (M->quad_a.cols == nullptr) *bytes += (int64_t)packs_held(M->quad_a) * pack;
+  if (M->quad_t.cols == nullptr) *bytes += (int64_t)packs_held(M->quad_t) * pack;
   return APPGA_OK;
+}
+
+appga_status ensure_quads(appga_matrix* M, cudaStream_t s) {
+  appga_status rc = ensure_counts(M, s);
+  if (rc == APPGA_OK && M->quad_a.cols == nullptr) rc = fill(M->A, s, &M->quad_a, &M->bytes);
+  if (rc == APPGA_OK && M->quad_t.cols == nullptr) rc = fill(M->At, s, &M->quad_t, &M->bytes);
+  return rc;
 }
 
 }  // namespace appga

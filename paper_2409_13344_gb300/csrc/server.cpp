@@ -260,7 +260,9 @@ int new_pool_width(const appga_server* S, int geom) {
 }
 
 // Whether a new pool of geometry `geom` and width Kp fits the pool cap and
-// device memory.
+// device memory, with the row-block layout of a matrix that has had no batched
+// call or pool yet (some 23 bytes per entry of A, 33 with BF16).  The layout stays
+// with the matrix, so the pools' budget leaves it out.
 bool pool_fits(appga_server* S, int geom, int Kp) {
   if (S->cfg.max_pools > 0 && live_pools(S) >= S->cfg.max_pools) return false;
   if (S->cfg.max_pools_per_geometry > 0) {
@@ -270,9 +272,12 @@ bool pool_fits(appga_server* S, int geom, int Kp) {
   }
   const int64_t need = pool_bytes(S->geoms[geom].M, Kp);
   if (S->cfg.hbm_budget_bytes > 0 && S->bytes + need > S->cfg.hbm_budget_bytes) return false;
+  auto* M = const_cast<appga_matrix*>(S->geoms[geom].M);
+  int64_t layout = 0;
+  if (quad_bytes_missing(M, S->ctx->stream, &layout) != APPGA_OK) return false;
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
-  return (int64_t)free_b - S->cfg.hbm_reserve_bytes >= need;
+  return (int64_t)free_b - S->cfg.hbm_reserve_bytes >= need + layout;
 }
 
 // Releases every pool that holds no request (other than `keep_geom`'s) and
@@ -401,6 +406,13 @@ appga_status admit_all(appga_server* S) {
           if (!pool_fits(S, gi, width)) break;
         }
         appga_status rc = create_pool(S, gi, width, &P);
+        // memory that others took since the check: as if it had not been free
+        // (with no pool left whose end frees some, the caller is told)
+        if (rc == APPGA_ENOMEM && live_pools(S) > 0) {
+          if (released || !release_empty_pools(S, gi)) break;
+          released = true;
+          continue;
+        }
         if (rc != APPGA_OK) return rc;
       }
       appga_status rc = admit(S, P, P->free_slots());

@@ -72,3 +72,33 @@ def test_a_pool_fits_seven_images_and_sinograms_a_slot(A, ctx, problem):
             if j == job:
                 np.testing.assert_array_equal(f, alone)
     mat.close()
+
+
+def test_the_first_pool_counts_the_matrix_layout(A, ctx, problem):
+    # with free memory that holds a pool's slots but not the layout its kernels
+    # stream (at least 10 bytes an entry: 20 a column of a block of four rows, A
+    # and A^T), the request waits, and runs once there is room
+    Amat, sls = problem
+    mat = A.Matrix(ctx, Amat, GEOM.n, GEOM.n_angles)
+    before = mat.info().device_bytes
+    hold = torch.empty(1 << 30, dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    free, _ = torch.cuda.mem_get_info()
+    srv = A.Server(ctx, slots_per_pool=32,
+                   hbm_reserve_bytes=free - budget(Amat, 32) - 5 * Amat.nnz)
+    gid = srv.add_geometry(mat)
+    rid = srv.submit(gid, sls[0].g, sls[0].gamma, A.default_params(max_iters=3, beta=0.1))
+    for _ in range(3):
+        assert srv.step() == 1
+    assert srv.summary().pools == 0
+    assert mat.info().device_bytes - before < 1 << 20
+    del hold
+    torch.cuda.empty_cache()
+    for _ in range(100):
+        if srv.step() == 0:
+            break
+    assert srv.summary().completed == 1 and srv.summary().pools == 1
+    assert mat.info().device_bytes - before >= 10 * Amat.nnz
+    srv.collect(rid)
+    srv.close()
+    mat.close()
