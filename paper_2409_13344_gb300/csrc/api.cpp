@@ -1000,8 +1000,8 @@ appga_status appga_matrix_create(appga_ctx* ctx, int32_t m, int32_t d, int32_t n
         }
       }
     }
-    appga::sell_fetch_ahead(M->sell_a, M->sell_t);
-    appga::sell_fetch_ahead(M->fold_a, M->fold_t);
+    appga::sell_fetch_ahead(M->sell_a, M->sell_t, false);
+    appga::sell_fetch_ahead(M->fold_a, M->fold_t, true);
     if (e != cudaSuccess) rc = cuda_fail(e, "tiled column indices and sliced layout");
   }
   if (rc == APPGA_OK) {

@@ -355,7 +355,7 @@ bool build_sell(const std::vector<int32_t>& order, int lanes, const std::vector<
                 const std::vector<int32_t>& col, const std::vector<float>& val, HostSell* out);
 // Lanes per row of a loop projection over `rows` rows of A, or of A^T (kernels.cu).
 int sell_lanes(int rows, bool transposed);
-void sell_fetch_ahead(DevSell& a, DevSell& t);
+void sell_fetch_ahead(DevSell& a, DevSell& t, bool folded);
 // All rows in ascending order, four lanes each.
 bool build_sell(int32_t rows, const std::vector<int32_t>& row_ptr, const std::vector<int32_t>& col,
                 const std::vector<float>& val, HostSell* out);

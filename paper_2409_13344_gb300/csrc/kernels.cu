@@ -1443,28 +1443,45 @@ int sell_lanes(int rows, bool transposed) {
 
 // Which of a loop's two sliced matrices (a: forward, t: pixel phase) are fetched
 // ahead, each slice whole into L2 before its kernel waits for its predecessor,
-// so that its loads hit L2.  That pays while the pixel phase's slices are
-// (nearly) all resident at once, 34 warps an SM: for both where the streams fit
-// L2, for the forward phase alone up to half as much again; with more bytes or
-// slices the fetches of late slices push out what the early ones stream.  us
-// for 40 maps without / forward only / both:
-//   256^2 folded      (89 MB, 4096 slices)    1362 / 1414 / 1296
-//   201^2             (86 MB, 5051)           1139 / 1140 / 1063
-//   255^2 BF16        (118 MB, 4065)          1572 / 1539 / 1501
-//   280^2 folded      (117 MB, 4900)          1825 / 1867 / 1828
-//   350^2 folded BF16 (152 MB, 3829)          2754 / 2735 / 2656
-//   255^2             (177 MB, 4065)          1769 / 1676 / 1772
-// and beyond the lines
-//   300^2 folded BF16 (96 MB, 5625)           1841 / 1853 / 1909
-//   320^2 folded      (175 MB, 6400)          2262 / 2276 / 2352
-//   400^2 folded      (342 MB, 5000)          3496 / 3664 / 4281 (both: with a tolerance)
-// The whole 256^2 matrices (185 MB) run at 43.6 us a map without, 40.6 so.
-void sell_fetch_ahead(DevSell& a, DevSell& t) {
-  int dev = 0, l2 = 0;
+// so that its loads hit L2: both where the streams fit L2, the forward phase alone
+// up to half as much again; with more bytes the fetches of late slices push out
+// what the early ones stream.  The lines in slices are measured, not derived: none
+// where a folded pixel phase of two lanes starts a second wave (28 warps an SM at
+// its registers), none above 34 slices an SM otherwise.  us for 40 maps, FP32 and
+// BF16, without / forward only / both (medians of nine, their spread below 1 %;
+// streams of 52 to 120 MB, 35 to 80 in BF16):
+//   folded, two lanes
+//     256^2 (4096 slices)  928 / 904 / 905     880 / 872 / 877
+//     260^2 (4225)        1235 / 1235 / 1236  1186 / 1153 / 1150
+//     264^2 (4356)        1484 / 1519 / 1524  1363 / 1371 / 1364
+//     272^2 (4624)        1517 / 1558 / 1580  1405 / 1422 / 1420
+//     284^2 (5041)        1506 / 1556 / 1543  1361 / 1394 / 1410
+//     300^2 (5625)        1247 / 1292 / 1272  1187 / 1200 / 1211
+//   folded, four lanes
+//     200^2 (5000)        1016 / 982 / 993     956 / 954 / 965
+//     216^2 (5832)        1129 / 1123 / 1114  1092 / 1078 / 1090
+//   folded, one lane
+//     360^2 (4050)        1301 / 1364 / 1286  1237 / 1228 / 1168
+//     410^2 (5254)        1313 / 1360 / 1289  1236 / 1226 / 1188
+//   whole, four lanes (36 resident warps an SM)
+//     201^2 (5051)        1210 / 1199 / 1210  1124 / 1114 / 1100
+//     245^2 (7504)        1118 / 1052 / 1039  1003 / 963 / 954
+//   whole, two lanes (32)
+//     264^2 (4356)        1025 / 1014 / 975    906 / 858 / 835
+//     345^2 (7440)        1093 / 1129 / 1053   996 / 978 / 953
+// (so whole matrices of up to 49 slices an SM would gain too), and where the
+// bytes draw the line, earlier and on other data:
+//     255^2 whole (177 MB)       1769 / 1676 / 1772
+//     400^2 folded (342 MB)      3496 / 3664 / 4281 (both: with a tolerance)
+void sell_fetch_ahead(DevSell& a, DevSell& t, bool folded) {
+  int dev = 0, l2 = 0, blocks = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess)
+      cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_pixel<false, 2, true>, PX::THREADS,
+                                                    0) != cudaSuccess)
     return;
-  if (a.off == nullptr || t.slices > 34 * current_sm_count()) return;
+  const int per_sm = folded && t.lanes == 2 ? blocks * (PX::THREADS / 32) : 34;
+  if (a.off == nullptr || t.slices > per_sm * current_sm_count()) return;
   for (int bf = 0; bf < 2; ++bf) {
     const int64_t bytes = ((int64_t)a.packs + t.packs) * (bf ? 16 : 24);
     if (2 * bytes <= 3 * (int64_t)l2) a.ahead |= 1 << bf;
