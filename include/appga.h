@@ -353,8 +353,10 @@ appga_status appga_reconstruct_volume(appga_ctx* ctx, const appga_matrix* mat, i
  * gathers a team keeps in flight (8, or 4: half as many, fewer registers;
  * separate kernel instances, for matrices of at least 4864 row blocks).  The
  * best schedule is kept in the matrix handle and used by later
- * appga_reconstruct_batched calls (and server pools) with the same padded
- * width (32, 64 or 128) and precision.  out_host (may be NULL) receives the
+ * appga_reconstruct_batched calls with the same slot width (8, 16, 32, 64 or
+ * 128, the smallest that holds K) and precision, and by server pools (the
+ * forward phase's and the stencil's shares of the pool's full width, the rest of
+ * the width that a replay works on).  out_host (may be NULL) receives the
  * choice and the measured times.  Synchronises; allocates a K x d scratch
  * image block for the trials.  A schedule never changes the image of a run
  * with a fixed number of maps (every slot's arithmetic is the same); the
@@ -375,7 +377,7 @@ typedef struct {
 appga_status appga_autotune_batched(appga_ctx* ctx, const appga_matrix* mat, int32_t K,
                                     const float* g, const float* gamma,
                                     const appga_params* params, appga_batch_tuning* out_host);
-/* Reads / sets the schedule kept for (tuning->K's padded width,
+/* Reads / sets the schedule kept for (tuning->K's slot width,
  * tuning->a_precision), e.g. to reuse a tuning saved by an earlier process;
  * only K, a_precision and the six schedule fields are used (values per SM
  * in [0, 16], 0 = default; chunk 0, 32 or 64; gather rows 0, 4 or 8).  get

@@ -99,8 +99,8 @@ cudaError_t alloc_batch_workspace(BatchWorkspace& b, int m, int d, int Kp) {
   return cudaSuccess;
 }
 
-BatchSchedule tuned_schedule(const appga_matrix* M, int Kp, bool bf16) {
-  auto it = M->tuned.find(Kp * 2 + (bf16 ? 1 : 0));
+BatchSchedule tuned_schedule(const appga_matrix* M, int K, bool bf16) {
+  auto it = M->tuned.find(slot_width(K) * 2 + (bf16 ? 1 : 0));
   return it == M->tuned.end() ? BatchSchedule() : it->second;
 }
 
@@ -511,7 +511,7 @@ appga_status volume_solve(appga_ctx* ctx, appga_matrix* M, int32_t K, const floa
   const appga_status rc = check_slot_width(M, Kp);
   if (rc != APPGA_OK) return rc;
   return batched_solve(ctx, M, K, g, gamma, f_init, params, f_out, nullptr,
-                       tuned_schedule(M, Kp, bf16), stream, 0, true, want_phi);
+                       tuned_schedule(M, K, bf16), stream, 0, true, want_phi);
 }
 
 }  // namespace appga
@@ -527,7 +527,7 @@ extern "C" appga_status appga_reconstruct_batched(appga_ctx* ctx, const appga_ma
   auto* M = const_cast<appga_matrix*>(mat);
   const bool bf16 = params->a_precision == APPGA_PREC_BF16 && M->has_bf16;
   return batched_run(ctx, M, K, g, gamma, f_init, params, f_out, stats_host,
-                     tuned_schedule(M, padded_width(K), bf16), stream);
+                     tuned_schedule(M, K, bf16), stream);
 }
 
 namespace appga {
@@ -685,7 +685,7 @@ extern "C" appga_status appga_autotune_batched(appga_ctx* ctx, const appga_matri
   for (auto& e : ev) cudaEventDestroy(e);
   cudaFree(f_scratch);
   if (rc != APPGA_OK) return rc;
-  M->tuned[Kp * 2 + (bf16 ? 1 : 0)] = best;
+  M->tuned[slot_width(K) * 2 + (bf16 ? 1 : 0)] = best;
   if (out_host) {
     std::memset(out_host, 0, sizeof *out_host);
     out_host->K = K;
@@ -706,8 +706,7 @@ extern "C" appga_status appga_batch_schedule_get(const appga_matrix* mat,
                                                  appga_batch_tuning* t) {
   if (!mat || !t) return fail(APPGA_EINVAL, "null argument");
   if (t->K < 1 || t->K > 128) return fail(APPGA_EINVAL, "K must be in [1, 128]");
-  const BatchSchedule sch =
-      tuned_schedule(mat, padded_width(t->K), t->a_precision == APPGA_PREC_BF16);
+  const BatchSchedule sch = tuned_schedule(mat, t->K, t->a_precision == APPGA_PREC_BF16);
   t->spmv_per_sm = sch.spmv_per_sm;
   t->stencil_per_sm = sch.stencil_per_sm;
   t->pixel_per_sm = sch.pixel_per_sm;
@@ -735,6 +734,6 @@ extern "C" appga_status appga_batch_schedule_set(appga_matrix* mat, const appga_
   sch.chunk = t->chunk;
   sch.gather_rows_fw = t->gather_rows_fw == 8 ? 0 : t->gather_rows_fw;
   sch.gather_rows_px = t->gather_rows_px == 8 ? 0 : t->gather_rows_px;
-  mat->tuned[padded_width(t->K) * 2 + (t->a_precision == APPGA_PREC_BF16 ? 1 : 0)] = sch;
+  mat->tuned[slot_width(t->K) * 2 + (t->a_precision == APPGA_PREC_BF16 ? 1 : 0)] = sch;
   return APPGA_OK;
 }

@@ -52,7 +52,9 @@ struct Workspace {
 };
 
 // Launch schedule of the batched kernels (0 = the kernels' defaults), as
-// picked by appga_autotune_batched for one padded width and precision.
+// picked by appga_autotune_batched for one slot width and precision.  (A width's
+// schedule serves no other: 40 maps of 5 slices took 1345 us at 128 x 128 and 5861
+// at 256 x 256 by the defaults, 1952 and 8270 by what was tuned with 32.)
 struct BatchSchedule {
   int spmv_per_sm = 0;     // forward-phase SpMV blocks per SM
   int stencil_per_sm = 0;  // stencil blocks per SM
@@ -129,8 +131,8 @@ void free_quad(DevQuad& q);
 // b.Kp) slots per row, of matrix M (after ensure_quads).
 void make_batch_args(const appga_matrix* M, BatchWorkspace& b, int stride, bool bf16, bool track,
                      const BatchSchedule& sch, BFwdArgs* fa, BPixArgs* pa);
-// Tuned schedule of matrix M for padded width Kp and precision (defaults if none).
-BatchSchedule tuned_schedule(const appga_matrix* M, int Kp, bool bf16);
+// Tuned schedule of matrix M for K slices' slot width and precision (defaults if none).
+BatchSchedule tuned_schedule(const appga_matrix* M, int K, bool bf16);
 // Slot state of a problem run with `p` from iterate index k0 (active), or an
 // empty slot that holds no problem (inactive).
 SlotState slot_from_params(const appga_params* p, int k0, bool active);
@@ -195,7 +197,7 @@ struct appga_matrix {
   appga::Workspace ws;
   appga::BatchWorkspace* bw = nullptr;  // batched workspace (one width at a time)
   appga::AfppaWorkspace* aw = nullptr;  // AFPPA dual fields
-  std::map<int, appga::BatchSchedule> tuned;  // key: padded width * 2 + BF16
+  std::map<int, appga::BatchSchedule> tuned;  // key: slot width * 2 + BF16
 };
 
 namespace appga {

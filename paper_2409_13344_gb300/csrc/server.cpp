@@ -657,6 +657,14 @@ extern "C" appga_status appga_server_step(appga_server* S, int32_t* pending_out)
         BFwdArgs fa = q->fa;
         BPixArgs pa = q->pa;
         fa.width = pa.width = q->width();
+        // the schedule of this width, but for the forward phase's and the
+        // stencil's shares: a replay's first pixel phase reads the objective's
+        // rows that another width's replay may have left
+        const BatchSchedule sch = tuned_schedule(S->geoms[q->geom].M, fa.width,
+                                                 S->cfg.a_precision == APPGA_PREC_BF16);
+        fa.gather_rows = sch.gather_rows_fw;
+        pa.gather_rows = sch.gather_rows_px;
+        pa.blocks_per_sm = sch.pixel_per_sm;
         CK(capture_batch_graph(fa, pa, S->cfg.steps_per_launch, q->b, q->stream, &exec));
       }
       CK(cudaEventRecord(q->ev_start, q->stream));
