@@ -388,17 +388,20 @@ __device__ __forceinline__ void diff_fields(const float (*X)[W], int i, int j, i
   u[5] = form_u6<W>(X, i, j, r_lo, c_lo, c_hi);
 }
 
-// 1 / max(||u||, eps) from the squared norm, eps2 = eps * eps: a reciprocal
+// 1 / max(||u||, eps) from the squared norm, eps2 = square_of(eps): a reciprocal
 // square root with one Newton step whose residual 1 - m r^2 is formed without
 // rounding m r (about half an ulp, as accurate as 1 / sqrtf by two rounded
 // operations at a third of the instructions).  FP32 squares hold norms from
-// 1.1e-19 to 1.8e19: an eps whose square is not a normal float takes the square
-// root (a branch that is uniform over the grid), and an infinite squared norm
-// gives zero, as there: its reciprocal root is zero, and the residual, formed
+// 1.1e-19 to 1.8e19: an eps whose square is not a normal float (square_of) takes
+// the square root (a branch that is uniform over the grid), and an infinite squared
+// norm gives zero, as there: its reciprocal root is zero, and the residual, formed
 // from the clamped norm, stays finite.
+__device__ __forceinline__ float square_of(float eps) {
+  const float s = eps * eps;
+  return s >= 1.17549435e-38f && s <= 3.402823466e38f ? s : 0.f;
+}
 __device__ __forceinline__ float inv_norm(float nrm2, float eps, float eps2) {
-  if (!(eps2 >= 1.17549435e-38f && eps2 <= 3.402823466e38f))
-    return 1.f / fmaxf(sqrtf(nrm2), eps);
+  if (eps2 == 0.f) return 1.f / fmaxf(sqrtf(nrm2), eps);
   const float any = fmaxf(nrm2, eps2), m = fminf(any, 3.402823466e38f);
   const float r = rsqrtf(any);
   const float t = __fmul_rn(m, r);

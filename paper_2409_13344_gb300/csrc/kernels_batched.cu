@@ -624,7 +624,7 @@ __global__ void __launch_bounds__(B_THREADS, 4) k_bstencil(BFwdArgs a) {
   const float *delta = a.delta + slot, *low = a.low + slot;
   float* gR = a.gR + slot;
   const float th = sl.theta_hi;
-  const float lam1 = sl.lambda1, lam2 = sl.lambda2, eps = sl.eps, eps2 = eps * eps;
+  const float lam1 = sl.lambda1, lam2 = sl.lambda2, eps = sl.eps, eps2 = square_of(eps);
   const int ntx = (n + BST_OUT - 1) / BST_OUT, nty = (n + BST_R - 1) / BST_R;
   float reg_h = 0.f, reg_l = 0.f;
   for (int tile = blockIdx.x; tile < ntx * nty; tile += gridDim.x) {
@@ -1178,7 +1178,7 @@ __global__ void k_fill_slots(float* out, int len, int Kp, int s0, int s1, float 
 // Per-slot initial image TMC_s * 1_disk (Sec. 4.1) for the slots of K slices
 // (s0 + k, or ids[k]) from slice-major g, gamma ([K][m]): ACT_PARTS blocks per
 // slice sum g - gamma, then the images are filled a row of slots at a time (one
-// block per slice did both: 192 us for 64 slices of 256 x 256, 12 us now).
+// block per slice did both: 192 us for 64 slices of 256 x 256, 13 + 25 us now).
 constexpr int ACT_PARTS = 16;
 __global__ void __launch_bounds__(256) k_bactc(const float* __restrict__ g,
                                                const float* __restrict__ gamma, int m,
@@ -1253,9 +1253,9 @@ int st_blocks(const BFwdArgs& a) {
   return (tiles + per - 1) / per;
 }
 
-// Gather probe: the batched projectors' inner loop alone.  Every row of M is
-// reduced against the slot-minor rows of x by quad_dot, dealt to the teams as
-// in the projections, with no epilogue, stencil or pixel update.
+// Gather probe: the batched projectors' inner loop alone.  Every block of rows of
+// M is reduced against the slot-minor rows of x by quad_sums and quad_reduce, dealt
+// to the teams as in the projections, with no epilogue, stencil or pixel update.
 template <int W, int S>
 __global__ void __launch_bounds__(Q_THREADS, Q_PER_SM) k_gather_probe(DevQuad M,
                                                                       const float* __restrict__ x,
