@@ -120,9 +120,11 @@ typedef struct {
   int32_t has_bf16;
   int64_t device_bytes; /* device memory held by the handle */
   int32_t packed_columns; /* 1 if the solver loop streams 2-byte packed column
-                             indices (every column below 2^20 and, within each
-                             4-entry pack of a row, within [-8192, 8191] of the
-                             pack's first column); 0: 4-byte indices */
+                             indices (every column, in 8 x 8 pixel tiles, below
+                             2^20 and, within each 4-entry pack of a row, within
+                             [-8192, 8191] of the pack's first column, with A's
+                             entries in order along the ray or, where a row does
+                             not fit so, as given); 0: 4-byte indices */
   int32_t sliced_layout;  /* 1 if the solver loop's projections stream A and
                              A^T in the sliced (ELLPACK-like) layout; 0: CSR */
   int32_t quarter_turn_folded; /* 1 if the solver loop streams the quarter-turn
@@ -287,15 +289,16 @@ appga_status appga_reconstruct_batched(appga_ctx* ctx, const appga_matrix* mat, 
 
 /* appga_gather_probe: the rate of the batched projectors' inner loop alone on
  * this matrix (a measurement utility; the paper has no counterpart).  It
- * times `launches` runs of a kernel that runs only that loop: every row
- * reduced against the width-float rows of a slot-minor block named by its
- * columns (the column/value stream and the gathers), in the projectors' row
- * order, with no epilogue, stencil or pixel update, for several grid sizes
- * (virtual blocks of four warps per SM), and keeps the fastest.  *gbs_fwd: A's rows against an
+ * times `launches` runs of a kernel that runs only that loop: every block of
+ * four rows reduced against the width-float rows of a slot-minor block named by
+ * the union of their columns (the column/value stream and the gathers), in the
+ * projectors' row order, with no epilogue, stencil or pixel update, for several
+ * grid sizes (virtual blocks of four warps per SM), and keeps the fastest.  *gbs_fwd: A's rows against an
  * image block [d][width] (the forward projection); *gbs_bwd: A^T's rows
  * against a weight block [m][width] (the back-projection); both host doubles,
- * gathered bytes (padded entries x width x 4) per second / 1e9.  width: 32,
- * 64 or 128 (max(m, d) * width below 2^31, else EINVAL); launches >= 1 per
+ * in matrix-entry terms: padded CSR entries x width x 4 bytes per second / 1e9
+ * (a gathered row serves the 1.5-2 entries that a block's rows have in its
+ * column, so fewer bytes move than that).  width: 32, 64 or 128 (max(m, d) * width below 2^31, else EINVAL); launches >= 1 per
  * grid size.  Uses the matrix's batched
  * workspace; synchronises. */
 appga_status appga_gather_probe(appga_ctx* ctx, const appga_matrix* mat, int32_t width,

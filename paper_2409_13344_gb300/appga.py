@@ -385,9 +385,9 @@ def appga_reconstruct_batched(ctx, mat, K, g, gamma, f_init, params, f_out, stre
 
 
 def appga_gather_probe(ctx, mat, width: int = 64, launches: int = 20):
-    """Rate (gathered GB/s) of the batched projectors' inner loop alone on
-    this matrix, forward projection and back-projection (see appga.h):
-    (fwd, bwd)."""
+    """Rate (GB/s, a gathered row counted per matrix entry) of the batched
+    projectors' inner loop alone on this matrix, forward projection and
+    back-projection (see appga.h): (fwd, bwd)."""
     fwd, bwd = ctypes.c_double(), ctypes.c_double()
     _check(load_library().appga_gather_probe(ctx, mat, width, launches, ctypes.byref(fwd),
                                              ctypes.byref(bwd)), "appga_gather_probe")

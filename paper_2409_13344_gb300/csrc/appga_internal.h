@@ -356,7 +356,7 @@ bool build_sell(const std::vector<int32_t>& order, int lanes, const std::vector<
 // Lanes per row of a loop projection over `rows` rows of A, or of A^T (kernels.cu).
 int sell_lanes(int rows, bool transposed);
 void sell_fetch_ahead(DevSell& a, DevSell& t, bool folded);
-// All rows in ascending order, four lanes each.
+// All rows in ascending order, four lanes each (the host tests' plain layout).
 bool build_sell(int32_t rows, const std::vector<int32_t>& row_ptr, const std::vector<int32_t>& col,
                 const std::vector<float>& val, HostSell* out);
 // A with its rows padded to whole packs and its columns in the 8 x 8-tiled order,

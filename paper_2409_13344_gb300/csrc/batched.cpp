@@ -532,10 +532,11 @@ extern "C" appga_status appga_reconstruct_batched(appga_ctx* ctx, const appga_ma
 
 namespace appga {
 namespace {
-// best gathered GB/s over launch shapes for the column stream `col` (nnz
-// entries) into the slot-minor block x of `width` floats per row
-appga_status probe_best(const DevQuad& M, long long nnz, const float* x, int width, float* sink, int launches,
-                        cudaStream_t s, double* best) {
+// best GB/s over launch shapes of the blocks M (of a matrix of nnz padded
+// entries) against the slot-minor block x of `width` floats per row, counted as a
+// gathered row per entry
+appga_status probe_best(const DevQuad& M, long long nnz, const float* x, int width, float* sink,
+                        int launches, cudaStream_t s, double* best) {
   *best = 0.0;
   cudaEvent_t ev[2] = {nullptr, nullptr};
   CK(cudaEventCreate(&ev[0]));

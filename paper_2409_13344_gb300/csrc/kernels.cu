@@ -1469,8 +1469,9 @@ int sell_lanes(int rows, bool transposed) {
 //   whole, two lanes (32)
 //     264^2 (4356)        1025 / 1014 / 975    906 / 858 / 835
 //     345^2 (7440)        1093 / 1129 / 1053   996 / 978 / 953
-// (so whole matrices of up to 49 slices an SM would gain too), and where the
-// bytes draw the line, earlier and on other data:
+// (so whole matrices of up to 49 slices an SM would gain too); 100 tracked maps at
+// 256^2 folded, 180 angles, FP32: 3356 / 3464 / 3266.  And where the
+// bytes draw the line, on other data:
 //     255^2 whole (177 MB)       1769 / 1676 / 1772
 //     400^2 folded (342 MB)      3496 / 3664 / 4281 (both: with a tolerance)
 void sell_fetch_ahead(DevSell& a, DevSell& t, bool folded) {
